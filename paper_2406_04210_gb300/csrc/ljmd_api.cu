@@ -1042,6 +1042,10 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
         uoff += n[r];
     }
     md_status st = [&]() -> md_status {
+        // before the first allocation: a pooling allocator may hand out memory
+        // that work queued on the caller's stream still uses, and the box
+        // clears and fills it on its own stream
+        CKS(enter(b));
         BoxDev& d = b->d;
         copy_reps_to(b, d);
         size_t np3 = 3 * (size_t)b->np;
@@ -1112,7 +1116,6 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
         CKS(dev_alloc(b, &b->d_type_user, std::max<int64_t>(1, ntot)));
         CK(b, cudaMemcpyAsync(b->d_rep, b->reps.data(), sizeof(RepDev) * b->reps.size(),
                               cudaMemcpyHostToDevice, b->stream));
-        CKS(enter(b));
         if (ntot > 0) {
             const void *dpos, *dvel = nullptr, *dtype = nullptr;
             size_t pb = sizeof(double) * 3 * (size_t)ntot;
