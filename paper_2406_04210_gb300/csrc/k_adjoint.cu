@@ -220,132 +220,217 @@ __global__ void __launch_bounds__(512) k_param_reduce(const double* part_g, int 
 // loss):  h_k = (1/N_r) sum_{i<j, r_ij < rmax} exp(-(r_ij - c_k)^2 / (2 w^2)),
 // c_k = (k + 1/2) rhist / nbins, per replica (N_r its particle count).  The
 // lists must have been built at the current positions with rl >= rmax, so
-// that they hold every pair below rmax.  Pairs are counted once (uid_i <
-// uid_j).  part_h[chunk * nbins + k]: per-chunk sums, reduced per replica.
+// that they hold every pair below rmax.  Pairs are counted once (from the
+// lower slot).  part_h[chunk * nbins + k]: per-chunk sums, reduced per replica.
+//
+// Bound: the special-function unit, one exponential per (pair, bin).  A warp
+// takes 32 entries of a particle's row at a time, one per lane, and compacts
+// the distances of the counted ones into shared memory; every 32 of them the
+// lanes turn to the bins: lane l owns bins l, l + 32, ... and adds each
+// distance (one broadcast load) to its own sums in registers, so a pair's
+// distance is computed once for all bins and nothing is shared between lanes.
+// Sums run in FP32 over 32 distances, then in double-single.  N = 32,000, 64
+// bins: 1703 us with a thread per particle that walked its row once per bin,
+// 61 us here.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(LJ_CHUNK) k_pair_hist(BoxDev b, int nbins, float rbin, float inv2w2,
-                                                        float rmax2, double* part_h)
+constexpr int kHistThreads = 256;
+constexpr int kHistWarps = kHistThreads / 32;
+
+// exp(-x^2) with x scaled by sqrt(log2 e): one special-function instruction
+__device__ __forceinline__ float exp2_neg_sq(float t)
 {
-    __shared__ double s_red[LJ_CHUNK / 32];
-    __shared__ float4 s_shift[32];
-    int cur_r = -1;
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(-t * t));
+    return y;
+}
+
+template <int NB>   // bins per lane
+__global__ void __launch_bounds__(kHistThreads) k_pair_hist(BoxDev b, int nbins, float rbin, float scale, float rmax2,
+                                                            double* part_h)
+{
+    __shared__ double s_sum[kHistWarps][32 * NB];
+    __shared__ __align__(16) float s_r[kHistWarps][64];   // distances waiting for the bins: < 32 + one chunk
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    float* const rr = s_r[warp];
+    float ck[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) ck[q] = ((float)(lane + 32 * q) + 0.5f) * rbin;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
         const int4 ch = b.chunk[w];
-        __syncthreads();
-        if (ch.x != cur_r && threadIdx.x < 32) {
-            const RepDev& R = b.rep[ch.x];
-            const int k = threadIdx.x;
-            s_shift[k] = k < 27 ? make_float4((float)(k % 3 - 1) * R.ellf[0], (float)((k / 3) % 3 - 1) * R.ellf[1],
-                                              (float)(k / 9 - 1) * R.ellf[2], 0.f)
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        cur_r = ch.x;
-        __syncthreads();
-        const int p = ch.y + (int)threadIdx.x;
-        const bool act = p < ch.z;
-        float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
-        int cnt = 0, ui = 0;
-        if (act) {
-            pi = b.posq[p];
-            cnt = min(b.nbr_count[p], b.K);
-            ui = b.uid[p];
-        }
-        const uint32_t* L = b.nbr + (size_t)b.K * p;
-        for (int k = 0; k < nbins; ++k) {
-            const float ck = ((float)k + 0.5f) * rbin;
-            float acc = 0.f;
-            for (int s = 0; s < cnt; ++s) {
-                const unsigned ent = L[s];
-                const int j = (int)(ent & LJ_IDX_MASK);
-                if (b.uid[j] <= ui) continue;
-                const float4 pj = b.posq[j];
-                const float4 sh = s_shift[entry_k(ent)];
-                const float dx = (pi.x - pj.x) - sh.x, dy = (pi.y - pj.y) - sh.y, dz = (pi.z - pj.z) - sh.z;
-                const float r2 = dx * dx + dy * dy + dz * dz;
-                if (!(r2 < rmax2)) continue;
-                const float dr = sqrtf(r2) - ck;
-                acc += __expf(-dr * dr * inv2w2);
+        const RepDev& R = b.rep[ch.x];
+        const float ex = R.ellf[0], ey = R.ellf[1], ez = R.ellf[2];
+        float hi[NB], lo[NB];
+#pragma unroll
+        for (int q = 0; q < NB; ++q) hi[q] = lo[q] = 0.f;
+        // 32 distances into the lane's bins
+        auto batch = [&]() {
+            float acc[NB];
+#pragma unroll
+            for (int q = 0; q < NB; ++q) acc[q] = 0.f;
+#pragma unroll 2
+            for (int u = 0; u < 32; u += 4) {
+                const float4 r4 = *reinterpret_cast<const float4*>(rr + u);
+#pragma unroll
+                for (int q = 0; q < NB; ++q) {
+                    acc[q] += exp2_neg_sq((r4.x - ck[q]) * scale);
+                    acc[q] += exp2_neg_sq((r4.y - ck[q]) * scale);
+                    acc[q] += exp2_neg_sq((r4.z - ck[q]) * scale);
+                    acc[q] += exp2_neg_sq((r4.w - ck[q]) * scale);
+                }
             }
-            double t = warp_sum_d((double)acc);
-            if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = t;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double q = 0.0;
-                for (int m = 0; m < LJ_CHUNK / 32; ++m) q += s_red[m];
-                part_h[(size_t)w * nbins + k] = q;
+#pragma unroll
+            for (int q = 0; q < NB; ++q) ds_add_f(hi[q], lo[q], acc[q]);
+        };
+        int wait = 0;   // distances in s_r (warp-uniform)
+        for (int p = ch.y + warp; p < ch.z; p += kHistWarps) {
+            const float4 pi = b.posq[p];
+            const int cnt = min(b.nbr_count[p], b.K);
+            const uint32_t* L = b.nbr + (size_t)b.K * p;
+            for (int s0 = 0; s0 < cnt; s0 += 32) {
+                const int s = s0 + lane;
+                bool keep = false;
+                float r2 = 0.f;
+                if (s < cnt) {
+                    const unsigned ent = L[s];
+                    const int j = (int)(ent & LJ_IDX_MASK);
+                    if (j > p) {
+                        const float4 pj = b.posq[j];
+                        const float dx = fmaf(-entry_unit(ent, 26), ex, pi.x - pj.x);
+                        const float dy = fmaf(-entry_unit(ent, 28), ey, pi.y - pj.y);
+                        const float dz = fmaf(-entry_unit(ent, 30), ez, pi.z - pj.z);
+                        r2 = dx * dx + dy * dy + dz * dz;
+                        keep = r2 < rmax2;
+                    }
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, keep);
+                if (keep) rr[wait + __popc(bal & lt)] = sqrtf(r2);
+                wait += __popc(bal);
+                __syncwarp();
+                if (wait >= 32) {
+                    batch();
+                    const float tail = rr[32 + lane];   // the rest to the front
+                    __syncwarp();
+                    rr[lane] = tail;
+                    wait -= 32;
+                    __syncwarp();
+                }
             }
-            __syncthreads();
+        }
+        if (wait > 0) {   // far points fill the last batch: their exponentials are 0
+            if (lane >= wait) rr[lane] = 1.0e30f;
+            __syncwarp();
+            batch();
+            __syncwarp();
+        }
+        __syncthreads();   // the previous chunk's sums are read
+#pragma unroll
+        for (int q = 0; q < NB; ++q) s_sum[warp][lane + 32 * q] = (double)hi[q] + (double)lo[q];
+        __syncthreads();
+        for (int k = threadIdx.x; k < nbins; k += kHistThreads) {
+            double t = 0.0;
+            for (int m = 0; m < kHistWarps; ++m) t += s_sum[m][k];
+            part_h[(size_t)w * nbins + k] = t;
         }
     }
 }
 
-// per-replica histogram from the chunk sums: h[r * nbins + k] = sum / n_r
-__global__ void k_hist_reduce(BoxDev b, int nbins, const double* part_h, double* h)
+// per-replica histogram from the chunk sums: h[r * nbins + k] = sum / n_r.
+// A block takes 32 bins of a replica, its 8 warps every eighth chunk each
+// (34 us with one thread per bin over all 250 chunks of N = 32,000,
+// 10 us here); the order of the sum is fixed.
+__global__ void __launch_bounds__(256) k_hist_reduce(BoxDev b, int nbins, const double* part_h, double* h)
 {
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < b.nrep * nbins; idx += gridDim.x * blockDim.x) {
-        const int r = idx / nbins, k = idx % nbins;
+    __shared__ double s_red[8][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nblk = (nbins + 31) / 32;
+    for (int it = blockIdx.x; it < b.nrep * nblk; it += gridDim.x) {
+        const int r = it / nblk, k = 32 * (it % nblk) + lane;
         const RepDev& R = b.rep[r];
         double s = 0.0;
-        for (int c = R.chunk_off; c < R.chunk_off + R.nchunk; ++c) s += part_h[(size_t)c * nbins + k];
-        h[idx] = R.n > 0 ? s / (double)R.n : 0.0;
+        if (k < nbins) {
+#pragma unroll 4
+            for (int c = R.chunk_off + warp; c < R.chunk_off + R.nchunk; c += 8) s += part_h[(size_t)c * nbins + k];
+        }
+        s_red[warp][lane] = s;
+        __syncthreads();
+        if (warp == 0 && k < nbins) {
+            for (int m = 1; m < 8; ++m) s += s_red[m][lane];
+            h[(size_t)r * nbins + k] = R.n > 0 ? s / (double)R.n : 0.0;
+        }
+        __syncthreads();
     }
 }
 
 // gradient of sum_k coef[r, k] h_{r,k} with respect to the positions (user
 // order, FP64): dh_k/dx_i = (1/N_r) sum_j g_k'(r_ij) d_ij / r_ij over i's
 // full list (every pair seen from both ends), g_k' = -(r - c_k)/w^2 g_k.
-__global__ void __launch_bounds__(LJ_CHUNK) k_pair_hist_grad(BoxDev b, int nbins, float rbin, float inv2w2,
-                                                             float inv_w2, float rmax2, const double* coef,
-                                                             double* grad)
+// Bound by the exponentials as k_pair_hist; LJ_TPP threads per particle, as
+// the force kernel, so that small boxes fill the chip (N = 32,000, 64 bins:
+// 123 us with one thread per particle, 73 us here).
+__global__ void __launch_bounds__(LJ_FORCE_THREADS) k_pair_hist_grad(BoxDev b, int nbins, float rbin, float scale,
+                                                                     double inv_w2, float rmax2, const double* coef,
+                                                                     double* grad)
 {
-    __shared__ float4 s_shift[32];
-    __shared__ float s_coef[256];
+    __shared__ float2 s_bin[256];   // c_k, -coef_k / (n w^2)
+    const int grp = threadIdx.x / LJ_TPP, l4 = threadIdx.x % LJ_TPP;
     int cur_r = -1;
+    float ex = 0.f, ey = 0.f, ez = 0.f;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
         const int4 ch = b.chunk[w];
-        __syncthreads();
-        if (ch.x != cur_r) {
+        if (ch.x != cur_r) {   // block-uniform
             const RepDev& R = b.rep[ch.x];
-            if (threadIdx.x < 32) {
-                const int k = threadIdx.x;
-                s_shift[k] = k < 27 ? make_float4((float)(k % 3 - 1) * R.ellf[0], (float)((k / 3) % 3 - 1) * R.ellf[1],
-                                                  (float)(k / 9 - 1) * R.ellf[2], 0.f)
-                                    : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+            ex = R.ellf[0];
+            ey = R.ellf[1];
+            ez = R.ellf[2];
+            __syncthreads();   // the previous replica's table is no longer read
             for (int k = threadIdx.x; k < nbins; k += blockDim.x)
-                s_coef[k] = (float)(coef[(size_t)ch.x * nbins + k] / (R.n > 0 ? (double)R.n : 1.0));
+                s_bin[k] = make_float2(((float)k + 0.5f) * rbin,
+                                       (float)(-inv_w2 * coef[(size_t)ch.x * nbins + k] / (R.n > 0 ? (double)R.n : 1.0)));
+            __syncthreads();
+            cur_r = ch.x;
         }
-        cur_r = ch.x;
-        __syncthreads();
-        const int p = ch.y + (int)threadIdx.x;
-        if (p >= ch.z) continue;
-        const float4 pi = b.posq[p];
-        const int cnt = min(b.nbr_count[p], b.K);
-        const uint32_t* L = b.nbr + (size_t)b.K * p;
-        float gx = 0.f, gy = 0.f, gz = 0.f;
-        for (int s = 0; s < cnt; ++s) {
-            const unsigned ent = L[s];
-            const int j = (int)(ent & LJ_IDX_MASK);
-            const float4 pj = b.posq[j];
-            const float4 sh = s_shift[entry_k(ent)];
-            const float dx = (pi.x - pj.x) - sh.x, dy = (pi.y - pj.y) - sh.y, dz = (pi.z - pj.z) - sh.z;
-            const float r2 = dx * dx + dy * dy + dz * dz;
-            if (!(r2 < rmax2)) continue;
-            const float r = sqrtf(r2);
-            float dg = 0.f;
-            for (int k = 0; k < nbins; ++k) {
-                const float dr = r - ((float)k + 0.5f) * rbin;
-                dg = fmaf(s_coef[k] * (-dr * inv_w2), __expf(-dr * dr * inv2w2), dg);
+        for (int base = ch.y; base < ch.z; base += LJ_FORCE_THREADS / LJ_TPP) {
+            const int p = base + grp;
+            const bool act = p < ch.z;
+            const float4 pi = b.posq[act ? p : ch.y];
+            const int cnt = act ? min(b.nbr_count[p], b.K) : 0;
+            const uint32_t* L = b.nbr + (size_t)b.K * p;
+            float gx = 0.f, gy = 0.f, gz = 0.f;
+            for (int s = l4; s < cnt; s += LJ_TPP) {
+                const unsigned ent = L[s];
+                const float4 pj = b.posq[ent & LJ_IDX_MASK];
+                const float dx = fmaf(-entry_unit(ent, 26), ex, pi.x - pj.x);
+                const float dy = fmaf(-entry_unit(ent, 28), ey, pi.y - pj.y);
+                const float dz = fmaf(-entry_unit(ent, 30), ez, pi.z - pj.z);
+                const float r2 = dx * dx + dy * dy + dz * dz;
+                if (!(r2 < rmax2)) continue;
+                const float r = sqrtf(r2);
+                float dg = 0.f;
+#pragma unroll 4
+                for (int k = 0; k < nbins; ++k) {
+                    const float2 c = s_bin[k];
+                    const float dr = r - c.x;
+                    dg = fmaf(c.y * dr, exp2_neg_sq(dr * scale), dg);
+                }
+                const float t = dg / r;
+                gx = fmaf(t, dx, gx);
+                gy = fmaf(t, dy, gy);
+                gz = fmaf(t, dz, gz);
             }
-            const float t = dg / r;
-            gx = fmaf(t, dx, gx);
-            gy = fmaf(t, dy, gy);
-            gz = fmaf(t, dz, gz);
+#pragma unroll
+            for (int o = LJ_TPP / 2; o > 0; o >>= 1) {
+                gx += __shfl_xor_sync(0xffffffffu, gx, o);
+                gy += __shfl_xor_sync(0xffffffffu, gy, o);
+                gz += __shfl_xor_sync(0xffffffffu, gz, o);
+            }
+            if (act && l4 == 0) {
+                const size_t gu = (size_t)b.uid[p];
+                grad[3 * gu + 0] = gx;
+                grad[3 * gu + 1] = gy;
+                grad[3 * gu + 2] = gz;
+            }
         }
-        const size_t gu = (size_t)b.uid[p];
-        grad[3 * gu + 0] = gx;
-        grad[3 * gu + 1] = gy;
-        grad[3 * gu + 2] = gz;
     }
 }
 
@@ -376,23 +461,26 @@ cudaError_t launch_param_reduce(const double* part_g, int nchunk, int twoP, cons
 cudaError_t launch_pair_hist(const BoxDev& b, int nbins, double rhist, double width, double rmax, double* part_h,
                              double* h, Launch l)
 {
-    float rbin = (float)(rhist / nbins);
-    float inv2w2 = (float)(1.0 / (2.0 * width * width));
-    k_pair_hist<<<l.grid, LJ_CHUNK, 0, l.s>>>(b, nbins, rbin, inv2w2, (float)(rmax * rmax), part_h);
+    const float rbin = (float)(rhist / nbins), rmax2 = (float)(rmax * rmax);
+    // exp(-x^2 / (2 w^2)) = 2^-(scale x)^2
+    const float scale = (float)sqrt(1.4426950408889634 / (2.0 * width * width));
+    const int nb = (nbins + 31) / 32;   // 1 .. 8 (nbins <= 256)
+    if (nb <= 1) k_pair_hist<1><<<l.grid, kHistThreads, 0, l.s>>>(b, nbins, rbin, scale, rmax2, part_h);
+    else if (nb <= 2) k_pair_hist<2><<<l.grid, kHistThreads, 0, l.s>>>(b, nbins, rbin, scale, rmax2, part_h);
+    else if (nb <= 4) k_pair_hist<4><<<l.grid, kHistThreads, 0, l.s>>>(b, nbins, rbin, scale, rmax2, part_h);
+    else k_pair_hist<8><<<l.grid, kHistThreads, 0, l.s>>>(b, nbins, rbin, scale, rmax2, part_h);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    int n = b.nrep * nbins;
-    k_hist_reduce<<<(n + 255) / 256, 256, 0, l.s>>>(b, nbins, part_h, h);
+    const int64_t items = (int64_t)b.nrep * nb;
+    k_hist_reduce<<<(int)(items < 4096 ? items : 4096), 256, 0, l.s>>>(b, nbins, part_h, h);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pair_hist_grad(const BoxDev& b, int nbins, double rhist, double width, double rmax,
                                   const double* coef, double* grad, Launch l)
 {
-    float rbin = (float)(rhist / nbins);
-    float inv2w2 = (float)(1.0 / (2.0 * width * width));
-    float inv_w2 = (float)(1.0 / (width * width));
-    k_pair_hist_grad<<<l.grid, LJ_CHUNK, 0, l.s>>>(b, nbins, rbin, inv2w2, inv_w2, (float)(rmax * rmax), coef,
-                                                   grad);
+    const float scale = (float)sqrt(1.4426950408889634 / (2.0 * width * width));
+    k_pair_hist_grad<<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b, nbins, (float)(rhist / nbins), scale,
+                                                           1.0 / (width * width), (float)(rmax * rmax), coef, grad);
     return cudaGetLastError();
 }
