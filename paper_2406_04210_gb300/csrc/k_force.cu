@@ -644,81 +644,180 @@ __global__ void __launch_bounds__(LJ_BRICK_THREADS + 32, 4) k_force_tile_f32(Box
     }
 }
 
-// FP64 pair force (MD_PREC_FP64), one thread per particle over 128-particle
-// chunks, FP64 cell-relative offsets gathered from global memory.
-template <bool ENERGY>
+// 1/x in FP64 for x > 0, normal: the hardware's 20-bit approximation and one
+// third-order step y (1 + e + e^2), e = 1 - x y, which leaves e^3 < 2^-57.
+__device__ __forceinline__ double rcp_f64(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// FP64 pair force (MD_PREC_FP64).  Bound: the FP64 pipe, 2 lanes per clock
+// and SM (64 times fewer than FP32), so what counts is the FP64 instructions
+// per list entry.  LJ_TPP threads per particle scan its row in blocks of 16
+// entries with the FP32 offsets and queue, in shared memory, the entries
+// whose FP32 distance can lie within the cutoff (28 % of a row with skin 0.3
+// does not); the same threads then take the queued entries in FP64: offsets
+// gathered from global memory, the reciprocal by rcp_f64, powers of r^-2 with
+// the pair constants folded, the cutoff decided on r^2's bits: 23 FP64
+// instructions per pair within the cutoff with energies, against ~35 per list
+// entry for a thread per particle with a division.  Work items are quarters
+// of a chunk (32 particles per block), so that 4,000 particles reach 125 SMs.
+// N = 256,000, energies: 1177 us -> 688 us; N = 4,000: a step 127 us -> 48 us.
+constexpr int kF64Parts = LJ_CHUNK * LJ_TPP / LJ_F64_THREADS;   // work items per chunk
+constexpr int kF64Own = LJ_CHUNK / kF64Parts;                   // particles of a work item
+constexpr int kF64Scan = 96;                                    // entries scanned between two drains of the queue
+constexpr int kF64Queue = kF64Scan + 4;                         // a particle's queue (stride 4 banks)
+static_assert(kF64Parts == LJ_F64_WARPS, "one (E_pot, W) share per work item fills a chunk's shares");
+template <bool MONO, bool ENERGY>
 __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
 {
-    __shared__ double s_sh[3][27];
+    __shared__ double s_ell[3][4];                     // digit (0, 1, 2) of an entry -> shift (-1, 0, 1) * edge
+    __shared__ uint32_t s_q[kF64Own * kF64Queue];
+    __shared__ double2 s_c[LJ_MAXT * LJ_MAXT];         // 48 eps sigma^12, 24 eps sigma^6
+    __shared__ double2 s_e[LJ_MAXT * LJ_MAXT];         // 4 eps sigma^12, 4 eps sigma^6
+    __shared__ double s_sh[LJ_MAXT * LJ_MAXT];         // energy shift
+    __shared__ unsigned long long s_rc2[LJ_MAXT * LJ_MAXT];   // rc^2 (its bits)
+    __shared__ float s_near[LJ_MAXT * LJ_MAXT];        // FP32 r^2 below which an entry is queued
+    __shared__ double s_red[2][LJ_F64_WARPS];
     const LJDev* lj = b.lj;
     const int nt = lj->nt;
     const int np = b.np;
+    for (int k = threadIdx.x; k < nt * nt; k += blockDim.x) {
+        const double s2 = lj->dsig2[k], s6 = s2 * s2 * s2, e4 = lj->deps4[k];
+        s_c[k] = make_double2(12.0 * e4 * s6 * s6, 6.0 * e4 * s6);
+        s_e[k] = make_double2(e4 * s6 * s6, e4 * s6);
+        s_sh[k] = lj->dshift[k];
+        s_rc2[k] = (unsigned long long)__double_as_longlong(lj->drc2[k]);
+        s_near[k] = (float)lj->drc2[k] + b.band;       // the margin of the list build's FP64 recheck
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int grp = threadIdx.x / LJ_TPP, l4 = threadIdx.x % LJ_TPP;
+    uint32_t* const q = s_q + grp * kF64Queue;
+    const float4* __restrict__ posq = b.posq;
     int cur_r = -1;
-    for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
+    float3 ell = make_float3(0.f, 0.f, 0.f);
+    for (int it = blockIdx.x; it < b.nchunk * kF64Parts; it += gridDim.x) {
+        const int w = it / kF64Parts, part = it % kF64Parts;
         const int4 ch = b.chunk[w];
         const int r = ch.x;
-        if (r != cur_r) {
-            __syncthreads();
-            if (threadIdx.x < 27) {
-                const RepDev& R = b.rep[r];
-                const int k = threadIdx.x;
-                s_sh[0][k] = (double)(k % 3 - 1) * R.ell[0];
-                s_sh[1][k] = (double)((k / 3) % 3 - 1) * R.ell[1];
-                s_sh[2][k] = (double)(k / 9 - 1) * R.ell[2];
-            }
+        __syncthreads();   // the tables are complete; the previous item's sums are read
+        if (r != cur_r) {  // block-uniform
+            const RepDev& R = b.rep[r];
+            ell = make_float3(R.ellf[0], R.ellf[1], R.ellf[2]);
+            if (threadIdx.x < 9) s_ell[threadIdx.x / 3][threadIdx.x % 3] = (double)((int)threadIdx.x % 3 - 1) * R.ell[threadIdx.x / 3];
             __syncthreads();
             cur_r = r;
         }
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && part == 0) {
             if (w == 0) *b.any_req = 0;
             if (w == b.rep[r].chunk_off) {
                 b.disp_max[r] = 0u;
                 b.rebuild_req[r] = 0;
             }
         }
-        const int p = ch.y + (int)threadIdx.x;
-        double e = 0.0, vir = 0.0;
-        if (p < ch.z) {
-            double xi = b.off[p], yi = b.off[np + p], zi = b.off[2 * np + p];
-            int ti = b.type[p];
-            int cnt = min(b.nbr_count[p], b.K);
-            const uint32_t* lp = b.nbr + (size_t)b.K * p;
-            double fx = 0.0, fy = 0.0, fz = 0.0;
-            for (int s = 0; s < cnt; ++s) {
-                unsigned ent = __ldcs(lp + s);
-                int j = (int)(ent & LJ_IDX_MASK);
-                int k = entry_k(ent);
-                double dx = (xi - __ldg(&b.off[j])) - s_sh[0][k];
-                double dy = (yi - __ldg(&b.off[np + j])) - s_sh[1][k];
-                double dz = (zi - __ldg(&b.off[2 * np + j])) - s_sh[2][k];
-                double r2 = dx * dx + dy * dy + dz * dz;
-                int pp = ti * nt + __ldg(&b.type[j]);
-                if (r2 < lj->drc2[pp]) {
-                    double r2i = 1.0 / r2;
-                    double s2 = lj->dsig2[pp] * r2i;
-                    double s6 = s2 * s2 * s2;
-                    double f = lj->deps48[pp] * r2i * s6 * (s6 - 0.5);
-                    fx += f * dx;
-                    fy += f * dy;
-                    fz += f * dz;
+        const int p = ch.y + part * kF64Own + grp;
+        const bool act = p < ch.z;
+        const int pa = act ? p : ch.y;
+        const float4 pi = posq[pa];
+        const double xi = b.off[pa], yi = b.off[np + pa], zi = b.off[2 * np + pa];
+        const int tb = MONO ? 0 : __float_as_int(pi.w) * nt;
+        const int cnt = act ? min(b.nbr_count[p], b.K) : 0;
+        const uint4* row = reinterpret_cast<const uint4*>(b.nbr + (size_t)b.K * pa) + l4;
+        double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0, vir = 0.0;
+        int npair = 0;   // MONO: pairs within the cutoff (the shift is added once, at the end)
+        // the warp's longest row bounds every lane's scans (the shuffles below are warp-wide)
+        const int top = __reduce_max_sync(0xffffffffu, cnt);
+        for (int s0 = 0; s0 < top; s0 += kF64Scan) {
+            int nq = 0;   // queued entries of the particle (the same in its four lanes)
+            for (int s = s0; s < min(s0 + kF64Scan, top); s += LJ_ROW_BLOCK) {
+                uint4 ent = make_uint4(0u, 0u, 0u, 0u);
+                const int lim = cnt - (s + 4 * l4);   // entries of this thread in the block
+                if (lim > 0) ent = __ldcs(row + s / 4);
+                const uint32_t en[4] = {ent.x, ent.y, ent.z, ent.w};
+                bool in[4];
+                int c = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    in[u] = false;
+                    if (u < lim) {
+                        const float4 pj = __ldg(posq + (en[u] & LJ_IDX_MASK));
+                        const float dx = fmaf(-entry_unit(en[u], 26), ell.x, pi.x - pj.x);
+                        const float dy = fmaf(-entry_unit(en[u], 28), ell.y, pi.y - pj.y);
+                        const float dz = fmaf(-entry_unit(en[u], 30), ell.z, pi.z - pj.z);
+                        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                        in[u] = r2 < s_near[MONO ? 0 : tb + __float_as_int(pj.w)];
+                    }
+                    c += in[u] ? 1 : 0;
+                }
+                int incl = c;
+#pragma unroll
+                for (int o = 1; o < LJ_TPP; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, incl, o, LJ_TPP);
+                    if (l4 >= o) incl += t;
+                }
+                int at = nq + incl - c;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (in[u]) q[at++] = en[u];
+                nq += __shfl_sync(0xffffffffu, incl, LJ_TPP - 1, LJ_TPP);
+            }
+            __syncwarp();
+            for (int t = l4; t < nq; t += LJ_TPP) {
+                const uint32_t ent = q[t];
+                const int j = (int)(ent & LJ_IDX_MASK);
+                const double dx = (xi - __ldg(&b.off[j])) - s_ell[0][(ent >> 26) & 3u];
+                const double dy = (yi - __ldg(&b.off[np + j])) - s_ell[1][(ent >> 28) & 3u];
+                const double dz = (zi - __ldg(&b.off[2 * np + j])) - s_ell[2][ent >> 30];
+                const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                const int pp = MONO ? 0 : tb + __ldg(&b.type[j]);
+                // r2 < rc2 on their bits (neither is negative), not on the FP64 pipe; a NaN fails
+                if ((unsigned long long)__double_as_longlong(r2) < s_rc2[pp]) {
+                    const double2 c = s_c[pp];
+                    const double r2i = rcp_f64(r2);
+                    const double r6i = r2i * r2i * r2i;
+                    const double g = r6i * fma(c.x, r6i, -c.y);   // f r^2
+                    const double f = r2i * g;
+                    fx = fma(f, dx, fx);
+                    fy = fma(f, dy, fy);
+                    fz = fma(f, dz, fz);
                     if (ENERGY) {
-                        e += lj->deps4[pp] * s6 * (s6 - 1.0) - lj->dshift[pp];
-                        vir += f * r2;
+                        const double2 ec = s_e[pp];
+                        vir += g;
+                        if (MONO) {
+                            e = fma(r6i, fma(ec.x, r6i, -ec.y), e);
+                            ++npair;
+                        } else {
+                            e += fma(r6i, fma(ec.x, r6i, -ec.y), -s_sh[pp]);
+                        }
                     }
                 }
             }
-            b.force64[p] = fx;
-            b.force64[np + p] = fy;
-            b.force64[2 * np + p] = fz;
-            if (!isfinite(fx + fy + fz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
+            __syncwarp();   // the queue is read before it fills again
         }
+#pragma unroll
+        for (int o = LJ_TPP / 2; o > 0; o >>= 1) {
+            fx += __shfl_xor_sync(0xffffffffu, fx, o);
+            fy += __shfl_xor_sync(0xffffffffu, fy, o);
+            fz += __shfl_xor_sync(0xffffffffu, fz, o);
+        }
+        if (act && l4 < 3) b.force64[(size_t)l4 * np + p] = l4 == 0 ? fx : (l4 == 1 ? fy : fz);
+        if (act && l4 == 3 && !isfinite(fx + fy + fz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
         if (ENERGY) {
-            // one (E_pot, W) share per warp and chunk (no block barrier)
-            double de = warp_sum_d(0.5 * e), dw = warp_sum_d(0.5 * vir);
-            if ((threadIdx.x & 31) == 0) {
-                const size_t q = (size_t)w * LJ_F64_WARPS + (threadIdx.x >> 5);
-                b.part_f[2 * q] = de;
-                b.part_f[2 * q + 1] = dw;
+            // one (E_pot, W) share per work item
+            if (MONO) e -= (double)npair * s_sh[0];
+            const double de = warp_sum_d(0.5 * e), dw = warp_sum_d(0.5 * vir);
+            if (lane == 0) {
+                s_red[0][warp] = de;
+                s_red[1][warp] = dw;
+            }
+            __syncthreads();
+            if (threadIdx.x < 2) {
+                double t = s_red[threadIdx.x][0];
+                for (int k = 1; k < LJ_F64_WARPS; ++k) t += s_red[threadIdx.x][k];
+                b.part_f[2 * (size_t)it + threadIdx.x] = t;
             }
         }
     }
@@ -1130,8 +1229,13 @@ cudaError_t launch_force(const BoxDev& b, int energy, Launch l)
         return cudaGetLastError();
     }
     if (b.prec == 2) {
-        if (energy) k_force_f64<true><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
-        else k_force_f64<false><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
+        if (b.nt == 1) {
+            if (energy) k_force_f64<true, true><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
+            else k_force_f64<true, false><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
+        } else {
+            if (energy) k_force_f64<false, true><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
+            else k_force_f64<false, false><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
+        }
     } else if (b.force_tiles) {
         cudaError_t e = tile_kernel_attrs();
         if (e != cudaSuccess) return e;

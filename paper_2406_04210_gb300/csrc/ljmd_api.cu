@@ -274,7 +274,8 @@ Launch lforce(md_box* b)
         return Launch{std::max(1, std::min((int)b->d.nbrick, b->nsm * force_tile_blocks_per_sm(b->d.nt == 1))), 0,
                       b->stream};
     int per_sm = b->force_per_sm > 0 ? b->force_per_sm : (b->prec == 2 ? 12 : 6);
-    const int items = b->all_pairs ? b->d.nchunk * std::max(1, b->d.ap_js) : b->d.nchunk;
+    // the FP64 list kernel's items are quarters of a chunk
+    const int items = b->d.nchunk * (b->all_pairs ? std::max(1, b->d.ap_js) : b->prec == MD_PREC_FP64 ? LJ_F64_WARPS : 1);
     return Launch{std::max(1, std::min(items, b->nsm * per_sm)), 0, b->stream};
 }
 Launch llist(md_box* b)

@@ -48,7 +48,7 @@
 #define LJ_THERMO_CHUNKS 256   // chunks of one energy-reduction item
 #define LJ_LIST_THREADS 256    // threads of the list-build kernel
 #define LJ_LANE_THREADS 128    // threads of the lane-per-particle list-build kernel
-#define LJ_F64_THREADS 128     // threads of the FP64 pair kernel (one per particle)
+#define LJ_F64_THREADS 128     // threads of the FP64 pair kernel (LJ_TPP per particle)
 #define LJ_F64_WARPS (LJ_F64_THREADS / 32)   // its (E_pot, W) shares per chunk
 #define LJ_TPP 4               // threads per particle in the pair kernels
 #define LJ_SEG_MAX_CELLS 16    // most cells in one segment
