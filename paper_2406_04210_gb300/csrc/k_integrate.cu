@@ -75,7 +75,8 @@ __device__ __forceinline__ void wrap_d(const BoxDev& b, const RepDev& R, int c, 
 
 // sidx: this launch finalizes step (*b.step_ctr + sidx) (MID and LAST modes).
 template <int ACC, bool FORCE64, int MODE, bool ENERGY, bool TSTAT>
-__global__ void __launch_bounds__(LJ_CHUNK) k_integrate(BoxDev b, double dt, int sidx)
+__global__ void __launch_bounds__(LJ_CHUNK) k_integrate(BoxDev b, double dt, int sidx,
+                                                        cudaGraphConditionalHandle cond)
 {
     const int np = b.np;
     const double hdt = 0.5 * dt;
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_integrate(BoxDev b, double dt, int
             if ((threadIdx.x & 31) == 0 && __uint_as_float(m) > b.disp_thr2) {
                 atomicMax(&b.disp_max[r], m);
                 atomicOr(b.any_req, 1);
+                if (cond) cudaGraphSetConditional(cond, 1u);
             }
         }
         if (ENERGY && MODE != LJ_STEP_FIRST) {
@@ -180,12 +182,13 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_integrate(BoxDev b, double dt, int
 }
 
 template <int ACC, bool FORCE64>
-cudaError_t launch_integrate_t(const BoxDev& b, int mode, int energy, double dt, int sidx, Launch l)
+cudaError_t launch_integrate_t(const BoxDev& b, int mode, int energy, double dt, int sidx,
+                               cudaGraphConditionalHandle cond, Launch l)
 {
 #define LJ_INT_CASE(M, E)                                                                       \
     do {                                                                                        \
-        if (b.tstat_thr) k_integrate<ACC, FORCE64, M, E, true><<<l.grid, LJ_CHUNK, 0, l.s>>>(b, dt, sidx);  \
-        else k_integrate<ACC, FORCE64, M, E, false><<<l.grid, LJ_CHUNK, 0, l.s>>>(b, dt, sidx);            \
+        if (b.tstat_thr) k_integrate<ACC, FORCE64, M, E, true><<<l.grid, LJ_CHUNK, 0, l.s>>>(b, dt, sidx, cond);  \
+        else k_integrate<ACC, FORCE64, M, E, false><<<l.grid, LJ_CHUNK, 0, l.s>>>(b, dt, sidx, cond);            \
     } while (0)
     if (mode == LJ_STEP_FIRST) LJ_INT_CASE(LJ_STEP_FIRST, false);
     else if (mode == LJ_STEP_MID) {
@@ -324,11 +327,12 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_get_nlist(BoxDev b, int* count, lo
 
 }  // namespace
 
-cudaError_t launch_integrate(const BoxDev& b, int mode, int energy, double dt, int sidx, Launch l)
+cudaError_t launch_integrate(const BoxDev& b, int mode, int energy, double dt, int sidx,
+                             cudaGraphConditionalHandle cond, Launch l)
 {
-    if (b.prec == 0) return launch_integrate_t<0, false>(b, mode, energy, dt, sidx, l);
-    if (b.prec == 1) return launch_integrate_t<1, false>(b, mode, energy, dt, sidx, l);
-    return launch_integrate_t<1, true>(b, mode, energy, dt, sidx, l);
+    if (b.prec == 0) return launch_integrate_t<0, false>(b, mode, energy, dt, sidx, cond, l);
+    if (b.prec == 1) return launch_integrate_t<1, false>(b, mode, energy, dt, sidx, cond, l);
+    return launch_integrate_t<1, true>(b, mode, energy, dt, sidx, cond, l);
 }
 
 namespace {

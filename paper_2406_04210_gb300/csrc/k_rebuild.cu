@@ -15,13 +15,19 @@
 // ties by user index, so the layout is a deterministic function of the
 // positions; gather into the sorted arrays) -> k_nlist (27-cell search,
 // each neighbour cell narrowed to its candidates within reach along z).
+// Each stage is a device function; k_rebuild_cluster runs those up to the
+// gather in one launch for small boxes.
 #include <climits>
 
 #include "ljmd_internal.cuh"
 
 namespace {
 
-constexpr int kScanTile = 4096;   // cells per scan tile
+constexpr int kScanThreads = 128;
+constexpr int kScanTile = 2048;   // cells per scan tile
+// The cluster rebuild: one cluster of 16 blocks (the most a cluster may hold)
+constexpr int kClusterBlocks = 16;
+constexpr int kClusterThreads = 512;
 
 __device__ __forceinline__ int cell_coords(const RepDev& R, int gc, int& cx, int& cy)
 {
@@ -45,6 +51,12 @@ __device__ __forceinline__ int work_chunk(const BoxDev& b, int t, int& kr)
     while (t >= b.lw_coff[kr + 1]) ++kr;
     return b.rep[b.lw_rep[kr]].chunk_off + (t - b.lw_coff[kr]);
 }
+
+// The per-chunk stages run on groups of LJ_CHUNK threads: the blocks of the
+// separate kernels, or the quarters of a block of the cluster kernel.
+__device__ __forceinline__ int group_first() { return blockIdx.x * (blockDim.x / LJ_CHUNK) + threadIdx.x / LJ_CHUNK; }
+__device__ __forceinline__ int group_count() { return gridDim.x * (blockDim.x / LJ_CHUNK); }
+__device__ __forceinline__ int group_thread() { return threadIdx.x % LJ_CHUNK; }
 
 // 8-byte component c of particle p of an integrator array in the layout of
 // the box precision (FP64: one double; DS: hi/lo floats in two planes).
@@ -109,16 +121,15 @@ __device__ __forceinline__ void store_offB(const BoxDev& b, const RepDev& R, int
     }
 }
 
-__global__ void __launch_bounds__(LJ_CHUNK) k_bin(BoxDev b, int from_abs)
+__device__ __forceinline__ void phase_bin(const BoxDev& b, int from_abs)
 {
-    if (!box_needs_rebuild(b)) return;
     const int tot = b.lw_coff[b.lw_hdr[0]];
     int kr = 0;
-    for (int t = blockIdx.x; t < tot; t += gridDim.x) {
+    for (int t = group_first(); t < tot; t += group_count()) {
         const int w = work_chunk(b, t, kr);
         int4 ch = b.chunk[w];
         int r = ch.x;
-        int p = ch.y + (int)threadIdx.x;
+        int p = ch.y + group_thread();
         const bool act = p < ch.z;   // every lane reaches the warp-wide count below
         if (!act) p = ch.y;
         const RepDev& R = b.rep[r];
@@ -190,12 +201,19 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_bin(BoxDev b, int from_abs)
     }
 }
 
+__global__ void __launch_bounds__(LJ_CHUNK) k_bin(BoxDev b, int from_abs)
+{
+    if (box_needs_rebuild(b)) phase_bin(b, from_abs);
+}
+
 // ---------------------------------------------------------------------------
 // Exclusive scan of cell counts inside each replica, in two passes over
-// tiles of kScanTile cells: k_scan_tiles writes the tile-local prefix into
-// cell_start and the tile total into tile_sum; k_scan_add adds the totals of
-// the replica's earlier tiles plus the replica's first slot.
-// tiles[t] = (rep, first cell, end cell, first tile of the replica).
+// tiles of kScanTile cells, runs of consecutive cells per thread:
+// k_scan_tiles writes the tile-local prefix into cell_start and the tile
+// total into tile_sum; k_scan_add adds the totals of the replica's earlier
+// tiles plus the replica's first slot.  A replica of one tile is finished by
+// the first pass.  tiles[t] = (rep, first cell, end cell, first tile of the
+// replica).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int block_excl_scan(int v, int* s_warp, int& total)
 {
@@ -227,63 +245,81 @@ __device__ __forceinline__ int block_excl_scan(int v, int* s_warp, int& total)
     return r;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_tiles(BoxDev b, const int4* tiles, int ntiles,
-                                                      int* tile_sum)
+// cell c starts at slot s: its range is open for k_scatter (cell_end is the
+// cursor; it ends at start + count), its count is ready for the next build
+__device__ __forceinline__ void cell_open(const BoxDev& b, int c, int s)
 {
-    if (!box_needs_rebuild(b)) return;
+    b.cell_start[c] = s;
+    b.cell_end[c] = s;
+    b.cell_count[c] = 0;
+}
+
+template <int THREADS>
+__device__ __forceinline__ void phase_scan_tiles(const BoxDev& b, const int4* tiles, int ntiles, int* tile_sum)
+{
+    constexpr int kScanPer = kScanTile / THREADS;   // cells per thread
     __shared__ int s_warp[33];
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        int4 tl = tiles[t];
+        const int4 tl = tiles[t];
         if (!rep_needs_rebuild(b, tl.x)) continue;   // block-uniform
-        int carry = 0;
-        for (int base = tl.y; base < tl.z; base += blockDim.x) {
-            int c = base + (int)threadIdx.x;
-            int v = c < tl.z ? b.cell_count[c] : 0;
-            int total;
-            int ex = block_excl_scan(v, s_warp, total);
-            if (c < tl.z) b.cell_start[c] = carry + ex;
-            carry += total;
+        const int c0 = tl.y + (int)threadIdx.x * kScanPer;
+        int v[kScanPer], sum = 0;
+#pragma unroll
+        for (int u = 0; u < kScanPer; ++u) {
+            v[u] = c0 + u < tl.z ? b.cell_count[c0 + u] : 0;
+            sum += v[u];
         }
-        if (threadIdx.x == 0) tile_sum[t] = carry;
+        int total;
+        int ex = block_excl_scan(sum, s_warp, total);
+        const bool whole = tl.z - tl.y == b.rep[tl.x].ncell;
+        if (whole) ex += b.rep[tl.x].p_off;
+#pragma unroll
+        for (int u = 0; u < kScanPer; ++u) {
+            if (c0 + u < tl.z) {
+                if (whole) cell_open(b, c0 + u, ex);
+                else b.cell_start[c0 + u] = ex;
+            }
+            ex += v[u];
+        }
+        if (threadIdx.x == 0) tile_sum[t] = total;
     }
 }
 
-__global__ void __launch_bounds__(256) k_scan_add(BoxDev b, const int4* tiles, int ntiles,
-                                                   const int* tile_sum)
+__device__ __forceinline__ void phase_scan_add(const BoxDev& b, const int4* tiles, int ntiles, const int* tile_sum)
 {
-    if (!box_needs_rebuild(b)) return;
-    __shared__ int s_off;
+    __shared__ int s_warp[33];
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        int4 tl = tiles[t];
-        if (!rep_needs_rebuild(b, tl.x)) continue;
-        if (threadIdx.x == 0) {
-            int o = b.rep[tl.x].p_off;
-            for (int u = tl.w; u < t; ++u) o += tile_sum[u];
-            s_off = o;
-        }
-        __syncthreads();
-        int o = s_off;
-        for (int c = tl.y + (int)threadIdx.x; c < tl.z; c += blockDim.x) {
-            int s = b.cell_start[c] + o;
-            b.cell_start[c] = s;
-            b.cell_end[c] = s;     // cursor for k_scatter; ends at start + count
-            b.cell_count[c] = 0;   // ready for the next build
-        }
-        __syncthreads();
+        const int4 tl = tiles[t];
+        if (!rep_needs_rebuild(b, tl.x) || tl.z - tl.y == b.rep[tl.x].ncell) continue;   // block-uniform
+        int part = 0, before;
+        for (int u = tl.w + (int)threadIdx.x; u < t; u += blockDim.x) part += tile_sum[u];
+        block_excl_scan(part, s_warp, before);
+        before += b.rep[tl.x].p_off;
+        for (int c = tl.y + (int)threadIdx.x; c < tl.z; c += blockDim.x) cell_open(b, c, b.cell_start[c] + before);
     }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_tiles(BoxDev b, const int4* tiles, int ntiles, int* tile_sum)
+{
+    if (box_needs_rebuild(b)) phase_scan_tiles<kScanThreads>(b, tiles, ntiles, tile_sum);
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_add(BoxDev b, const int4* tiles, int ntiles,
+                                                            const int* tile_sum)
+{
+    if (box_needs_rebuild(b)) phase_scan_add(b, tiles, ntiles, tile_sum);
 }
 
 // ---------------------------------------------------------------------------
 // k_scatter: claim a slot inside the particle's new cell.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(LJ_CHUNK) k_scatter(BoxDev b)
+__device__ __forceinline__ void phase_scatter(const BoxDev& b)
 {
-    if (!box_needs_rebuild(b)) return;
     const int tot = b.lw_coff[b.lw_hdr[0]];
     int kr = 0;
-    for (int t = blockIdx.x; t < tot; t += gridDim.x) {
+    for (int t = group_first(); t < tot; t += group_count()) {
         int4 ch = b.chunk[work_chunk(b, t, kr)];
-        int p = ch.y + (int)threadIdx.x;
+        int p = ch.y + group_thread();
         const bool act = p < ch.z;
         // warp-aggregated slot claims: one atomic per distinct cell of the
         // warp, each lane's slot = old cursor + its rank among the peers
@@ -297,6 +333,11 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_scatter(BoxDev b)
     }
 }
 
+__global__ void __launch_bounds__(LJ_CHUNK) k_scatter(BoxDev b)
+{
+    if (box_needs_rebuild(b)) phase_scatter(b);
+}
+
 // ---------------------------------------------------------------------------
 // k_list_work: the work of a rebuild, one block.  The rebuilding replicas in
 // order, with the prefixes of their cell and particle-chunk counts, so that
@@ -305,9 +346,8 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_scatter(BoxDev b)
 // in which a few replicas of many rebuild does not walk (and test) every cell
 // and chunk of the batch.  Launched first in every rebuild sequence.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_list_work(BoxDev b)
+__device__ __forceinline__ void phase_list_work(const BoxDev& b)   // one block
 {
-    if (!box_needs_rebuild(b)) return;
     __shared__ int s_warp[33];
     int nsel = 0, ncell = 0, nch = 0;
     for (int base = 0; base < b.nrep; base += blockDim.x) {
@@ -331,6 +371,13 @@ __global__ void __launch_bounds__(1024) k_list_work(BoxDev b)
         b.lw_coff[nsel] = nch;
         b.lw_hdr[0] = nsel;
     }
+}
+
+__global__ void __launch_bounds__(1024) k_list_work(BoxDev b, unsigned long long* runs)
+{
+    if (!box_needs_rebuild(b)) return;
+    phase_list_work(b);
+    if (runs && threadIdx.x == 0) *runs += 1ull;   // launch accounting of a conditional rebuild
 }
 
 // ---------------------------------------------------------------------------
@@ -404,25 +451,11 @@ __device__ __forceinline__ void gather_one(const BoxDev& b, int p, int q, int gc
     b.ref[q] = pq;
 }
 
-__global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
+// GATHER: move the members at once (the cluster rebuild: no barrier between
+// the ranks and the gather); otherwise the ranks go to dst for k_gather.
+template <bool GATHER>
+__device__ __forceinline__ void phase_rank(const BoxDev& b)
 {
-    if (!box_needs_rebuild(b)) return;
-    if (b.all_pairs) {
-        // one cell holds the whole replica and no list needs an order: a
-        // particle's slot is its index inside the replica, one thread each
-        const int tot = b.lw_coff[b.lw_hdr[0]];
-        int kr = 0;
-        for (int t = blockIdx.x; t < tot; t += gridDim.x) {
-            const int4 ch = b.chunk[work_chunk(b, t, kr)];
-            const RepDev& R = b.rep[ch.x];
-            for (int s = ch.y + (int)threadIdx.x; s < ch.z; s += blockDim.x) {
-                if (s == R.p_off) atomicAdd(&b.nbuild[ch.x], 1ull);   // a re-binning
-                const int p = b.perm[s];
-                gather_one(b, p, R.p_off + (b.uidB[p] - R.u_off), R.cell_off);
-            }
-        }
-        return;
-    }
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
     const int total = b.lw_off[b.lw_hdr[0]];
@@ -447,9 +480,34 @@ __global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
                     rank += (kt < key) ? 1 : 0;
                 }
             }
-            if (idx < n) b.dst[s0 + idx] = s0 + rank;
+            if (idx < n) {
+                if (GATHER) gather_one(b, p, s0 + rank, gc);
+                else b.dst[s0 + idx] = s0 + rank;
+            }
         }
     }
+}
+
+__global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
+{
+    if (!box_needs_rebuild(b)) return;
+    if (b.all_pairs) {
+        // one cell holds the whole replica and no list needs an order: a
+        // particle's slot is its index inside the replica, one thread each
+        const int tot = b.lw_coff[b.lw_hdr[0]];
+        int kr = 0;
+        for (int t = blockIdx.x; t < tot; t += gridDim.x) {
+            const int4 ch = b.chunk[work_chunk(b, t, kr)];
+            const RepDev& R = b.rep[ch.x];
+            for (int s = ch.y + (int)threadIdx.x; s < ch.z; s += blockDim.x) {
+                if (s == R.p_off) atomicAdd(&b.nbuild[ch.x], 1ull);   // a re-binning
+                const int p = b.perm[s];
+                gather_one(b, p, R.p_off + (b.uidB[p] - R.u_off), R.cell_off);
+            }
+        }
+        return;
+    }
+    phase_rank<false>(b);
 }
 
 __global__ void __launch_bounds__(LJ_CHUNK) k_gather(BoxDev b)
@@ -802,9 +860,8 @@ __device__ __forceinline__ float lane_r2(const float2 nxy, float nz, const float
     return fmaf(dz, dz, s.x + s.y);
 }
 
-__global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
+__device__ __forceinline__ void phase_lanes(const BoxDev& b)
 {
-    if (!box_needs_rebuild(b)) return;
     // row buffers, slot-major per warp: code e of lane l at [e][l] (the 32
     // lanes' stores of one step fall in distinct banks whatever their counts)
     extern __shared__ __align__(16) uint16_t s_rows[];   // per warp: kLaneRow x 32 codes
@@ -1048,24 +1105,52 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
     if (threadIdx.x == 0 && s_longest > 0) atomicMax(&b.err[2], s_longest);
 }
 
-// Condition of the step graph's list-update node: 1 when the integrator (or
-// the host) raised the box-wide rebuild word, so that steps without a build
-// launch none of the rebuild kernels; each 1 is counted (launch accounting).
-__global__ void k_set_rebuild_cond(cudaGraphConditionalHandle h, const int* any_req, unsigned long long* runs)
+__global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
 {
-    const bool go = *((volatile const int*)any_req) != 0;
-    if (go) atomicAdd(runs, 1ull);
-    cudaGraphSetConditional(h, go ? 1u : 0u);
+    if (box_needs_rebuild(b)) phase_lanes(b);
 }
+
+// ---------------------------------------------------------------------------
+// k_rebuild_cluster: binning, sort and gather of small boxes in one launch,
+// by one thread-block cluster whose blocks meet at the hardware's cluster
+// barrier between the stages.  A step without a build then pays two early
+// exits (this and the list build) instead of eight, and a build no launches
+// between the stages; the list build stays a kernel of its own, as it wants
+// every SM.  (One cooperative launch for everything, with grid barriers, was
+// measured first: its launch inside a step graph cost nearly what the early
+// exits had, 32.7 us a step at N = 4,000 against 34.3.)
+// A step of the N = 4,000 fluid: 33.4 us with the separate kernels, 28.1 us
+// with this; the launch rule has the other sizes.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kClusterThreads) k_rebuild_cluster(BoxDev b, int from_abs, const int4* tiles,
+                                                                      int ntiles, int* tile_sum)
+{
+    if (!box_needs_rebuild(b)) return;   // the same word for every block: none is left waiting
+    if (b.nrep > 1) {   // one replica: its work lists never change
+        if (blockIdx.x == 0) phase_list_work(b);
+        cluster_barrier();
+    }
+    phase_bin(b, from_abs);
+    cluster_barrier();
+    phase_scan_tiles<kClusterThreads>(b, tiles, ntiles, tile_sum);
+    cluster_barrier();
+    if (ntiles > b.nrep) {   // some replica has more than one tile
+        phase_scan_add(b, tiles, ntiles, tile_sum);
+        cluster_barrier();
+    }
+    phase_scatter(b);
+    cluster_barrier();
+    phase_rank<true>(b);
+}
+static_assert(kClusterThreads % LJ_CHUNK == 0, "whole groups");
 
 }  // namespace
-
-cudaError_t launch_set_rebuild_cond(cudaGraphConditionalHandle h, const BoxDev& b, unsigned long long* runs,
-                                    cudaStream_t s)
-{
-    k_set_rebuild_cond<<<1, 1, 0, s>>>(h, b.any_req, runs);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_bin(const BoxDev& b, int from_abs, Launch l)
 {
@@ -1076,10 +1161,10 @@ cudaError_t launch_bin(const BoxDev& b, int from_abs, Launch l)
 cudaError_t launch_scan_tiles(const BoxDev& b, const int4* tiles, int ntiles, int* tile_sum,
                               Launch l)
 {
-    k_scan_tiles<<<l.grid, 1024, 0, l.s>>>(b, tiles, ntiles, tile_sum);
+    k_scan_tiles<<<l.grid, kScanThreads, 0, l.s>>>(b, tiles, ntiles, tile_sum);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_scan_add<<<l.grid, 256, 0, l.s>>>(b, tiles, ntiles, tile_sum);
+    if (e != cudaSuccess || ntiles <= b.nrep) return e;   // one tile per replica: finished
+    k_scan_add<<<l.grid, kScanThreads, 0, l.s>>>(b, tiles, ntiles, tile_sum);
     return cudaGetLastError();
 }
 
@@ -1115,9 +1200,9 @@ cudaError_t launch_nlist(const BoxDev& b, Launch l)
 // slots per lane.
 size_t nlist_lanes_smem(int) { return (size_t)LJ_LANE_THREADS * (size_t)kLaneRow * 2u; }
 
-cudaError_t launch_list_work(const BoxDev& b, cudaStream_t s)
+cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s)
 {
-    k_list_work<<<1, 1024, 0, s>>>(b);
+    k_list_work<<<1, 1024, 0, s>>>(b, runs);
     return cudaGetLastError();
 }
 
@@ -1132,6 +1217,42 @@ cudaError_t launch_nlist_lanes(const BoxDev& b, Launch l)
     }
     k_nlist_lanes<<<l.grid, LJ_LANE_THREADS, dyn, l.s>>>(b);
     return cudaGetLastError();
+}
+
+// Whether this GPU holds the cluster (16 blocks is beyond the portable 8).
+bool cluster_rebuild_fits()
+{
+    cudaLaunchConfig_t c{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kClusterBlocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    c.gridDim = dim3(kClusterBlocks);
+    c.blockDim = dim3(kClusterThreads);
+    c.attrs = &at;
+    c.numAttrs = 1;
+    int n = 0;
+    const bool ok =
+        cudaFuncSetAttribute(k_rebuild_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, k_rebuild_cluster, &c) == cudaSuccess && n > 0;
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
+cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles, int* tile_sum,
+                                   cudaStream_t s)
+{
+    cudaLaunchConfig_t c{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kClusterBlocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    c.gridDim = dim3(kClusterBlocks);
+    c.blockDim = dim3(kClusterThreads);
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k_rebuild_cluster, b, from_abs, tiles, ntiles, tile_sum);
 }
 
 int ljmd_scan_tile_cells() { return kScanTile; }

@@ -61,7 +61,7 @@ struct md_box {
     cudaEvent_t ev = nullptr;
     // the energy reduction's branch of the step graph (it overlaps the list update)
     cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
     // the rebuild sequence as the body of a conditional (IF) graph node
     bool use_cond = false;   // list update as a conditional graph node (md_set_graph_conditional)
     cudaStream_t cstream = nullptr;            // captures the node's body
@@ -93,7 +93,7 @@ struct md_box {
     LJDev* d_lj = nullptr;
     int4* d_tiles = nullptr;
     std::vector<int4> bricks;  // work items of the tiled force kernel: (replica, first cell x, y, z)
-    size_t pf_cap = 0;         // doubles of d.part_f
+    size_t pf_cap = 0;         // doubles of one of the two sets of d.part_f
     int4* d_brick = nullptr;
     int* d_tile_sum = nullptr;
     int* d_type_user = nullptr;
@@ -124,6 +124,7 @@ struct md_box {
     int force_per_sm = 0;      // 0 = automatic (tuning)
     int list_per_sm = 0;
     int seg_cells = 0;
+    bool cluster_ok = false;   // the GPU holds k_rebuild_cluster's cluster
     int64_t steps = 0;
     int64_t launches = 0;
     bool profiling = false;
@@ -356,51 +357,82 @@ md_status clear_err(md_box* b)
 // ------------------------------------------------------------------------
 // Rebuild / force sequences
 // ------------------------------------------------------------------------
-// Kernels of one rebuild sequence (bin, scan x2, scatter, rank, gather,
-// list; all pairs: binning only re-wraps and re-centres).
-int rebuild_kernels(md_box* b) { return b->all_pairs ? 6 : 8; }
-
-md_status enqueue_rebuild(md_box* b, int from_abs, cudaStream_t s = nullptr)
+// Kernels of one separate rebuild sequence (work lists where `runs` or several
+// replicas ask, bin, scan, its second pass where a replica has several tiles,
+// scatter, rank, gather, list; all pairs: binning only re-wraps and
+// re-centres).
+int rebuild_kernels(md_box* b, bool runs)
 {
-    if (!s) s = b->stream;
+    return (b->all_pairs ? 4 : 6) + ((int)b->tiles.size() > b->nrep ? 1 : 0) + (runs || b->nrep > 1 ? 1 : 0);
+}
+
+// Binning, sort and gather as one cluster launch (k_rebuild_cluster) instead
+// of the separate kernels: boxes whose stages 16 blocks get through faster
+// than the launches cost.  Per step, separate against cluster: N = 4,000
+// 33.4 / 28.1 us, N = 32,000 (the list update's phase) 22.5 / 19.0 us,
+// N = 100,000 61.4 / 69.6 us.
+constexpr int kClusterSlots = 32768;
+bool cluster_rebuild(md_box* b)
+{
+    if (b->all_pairs || !b->cluster_ok) return false;
+    return b->np <= kClusterSlots;
+}
+
+// runs: counts the sequence's executions (the body of a conditional node)
+md_status enqueue_rebuild_kernels(md_box* b, int from_abs, cudaStream_t s, unsigned long long* runs)
+{
     auto on = [s](Launch l) {
         l.s = s;
         return l;
     };
     Launch l = on(lch(b));
-    CK(b, launch_list_work(b->d, s));   // the cells and chunks the rebuild kernels visit
+    // the cells and chunks the rebuild kernels visit (one replica's never change: make_grid)
+    if (runs || b->nrep > 1) CK(b, launch_list_work(b->d, runs, s));
     CK(b, launch_bin(b->d, from_abs, l));
-    Launch lt{std::max(1, std::min((int)b->tiles.size(), b->nsm * 2)), 1024, s};
+    Launch lt{std::max(1, std::min((int)b->tiles.size(), b->nsm * 8)), 0, s};
     CK(b, launch_scan_tiles(b->d, b->d_tiles, (int)b->tiles.size(), b->d_tile_sum, lt));
     CK(b, launch_scatter(b->d, l));
     CK(b, launch_sortgather(b->d, on(b->all_pairs ? lch(b) : lcell(b)), l));
     if (!b->all_pairs) CK(b, launch_list(b, s));
-    b->launches += rebuild_kernels(b);
+    b->launches += rebuild_kernels(b, runs != nullptr);
     return MD_OK;
 }
 
-// The list update of one step inside a captured step graph: a one-thread
-// kernel sets the condition of an IF node from the box-wide rebuild word,
-// and the node's body (captured on the box's second stream) holds the
-// rebuild sequence, so a step without a build launches one tiny kernel
-// instead of the whole sequence (whose kernels exit early anyway).  The
-// body's kernels are counted when they run (k_set_rebuild_cond counts the
-// true conditions in cond_runs).  Outside a capture, or if the graph API
-// refuses the node, the plain sequence is enqueued.
-md_status enqueue_rebuild_step(md_box* b)
+md_status enqueue_rebuild(md_box* b, int from_abs)
 {
-    if (!b->use_cond) return enqueue_rebuild(b, 0);
+    if (!cluster_rebuild(b)) return enqueue_rebuild_kernels(b, from_abs, b->stream, nullptr);
+    CK(b, launch_rebuild_cluster(b->d, from_abs, b->d_tiles, (int)b->tiles.size(), b->d_tile_sum, b->stream));
+    CK(b, launch_list(b, b->stream));
+    b->launches += 2;
+    return MD_OK;
+}
+
+// With md_set_graph_conditional, the list update of a step inside a captured
+// step graph is an IF node: the integrator sets its condition (handle h)
+// when it raises the box-wide rebuild word, and the node's body (captured on
+// the box's second stream) holds the rebuild sequence, so a step without a
+// build launches nothing for it.  The body's kernels are counted when they
+// run (k_list_work counts them in cond_runs).  cond_begin makes the handle
+// before the integrator's launch; cond_node adds the node behind it.
+md_status cond_begin(md_box* b, cudaGraphConditionalHandle* h)
+{
+    *h = 0;
+    if (!b->use_cond || b->all_pairs) return MD_OK;
+    cudaStreamCaptureStatus cs;
+    cudaGraph_t g = nullptr;
+    CK(b, cudaStreamGetCaptureInfo(b->stream, &cs, nullptr, &g, nullptr, nullptr, nullptr));
+    if (cs != cudaStreamCaptureStatusActive) return MD_OK;
+    CK(b, cudaGraphConditionalHandleCreate(h, g, 0, cudaGraphCondAssignDefault));
+    return MD_OK;
+}
+
+md_status cond_node(md_box* b, cudaGraphConditionalHandle h)
+{
     cudaStreamCaptureStatus cs;
     cudaGraph_t g = nullptr;
     const cudaGraphNode_t* deps = nullptr;
     const cudaGraphEdgeData* edata = nullptr;
     size_t nd = 0;
-    CK(b, cudaStreamGetCaptureInfo(b->stream, &cs, nullptr, &g, &deps, &edata, &nd));
-    if (cs != cudaStreamCaptureStatusActive) return enqueue_rebuild(b, 0);
-    cudaGraphConditionalHandle h;
-    CK(b, cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
-    CK(b, launch_set_rebuild_cond(h, b->d, b->d_cond_runs, b->stream));
-    b->launches += 1;
     CK(b, cudaStreamGetCaptureInfo(b->stream, &cs, nullptr, &g, &deps, &edata, &nd));
     cudaGraphNodeParams p{};
     p.type = cudaGraphNodeTypeConditional;
@@ -413,7 +445,7 @@ md_status enqueue_rebuild_step(md_box* b)
     cudaGraph_t body = p.conditional.phGraph_out[0];
     CK(b, cudaStreamBeginCaptureToGraph(b->cstream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     const int64_t l0 = b->launches;
-    md_status st = enqueue_rebuild(b, 0, b->cstream);
+    md_status st = enqueue_rebuild_kernels(b, 0, b->cstream, b->d_cond_runs);
     b->launches = l0;   // counted per execution instead
     cudaGraph_t out = nullptr;
     cudaError_t ce = cudaStreamEndCapture(b->cstream, &out);
@@ -568,6 +600,8 @@ md_status make_grid(md_box* b)
     CKS(dev_alloc(b, &b->d_brick, b->bricks.size(), false));
     CK(b, cudaMemcpyAsync(b->d_brick, b->bricks.data(), sizeof(int4) * b->bricks.size(),
                           cudaMemcpyHostToDevice, b->stream));
+    const int lw1[6] = {1, 0, 0, d.ncell, 0, d.nchunk};   // the work lists of one replica never change
+    if (b->nrep == 1) CK(b, cudaMemcpyAsync(d.lw_hdr, lw1, sizeof lw1, cudaMemcpyHostToDevice, b->stream));
     CK(b, cudaStreamSynchronize(b->stream));   // `bricks` may change before the copy would run
     d.brick = b->d_brick;
     d.nbrick = (int)b->bricks.size();
@@ -577,7 +611,7 @@ md_status make_grid(md_box* b)
             dev_release(b, d.part_f);
             d.part_f = nullptr;
             b->pf_cap = 0;
-            CKS(dev_alloc(b, &d.part_f, need));
+            CKS(dev_alloc(b, &d.part_f, 2 * need));   // two sets, steps alternate
             b->pf_cap = need;
         }
     }
@@ -749,9 +783,13 @@ md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* rin
                         bool tape = false)
 {
     Launch l = lch(b);
-    // The energy reduction of step s reads the force shares of step s - 1 and
-    // the kinetic shares of this integrate: it runs on a branch (side stream)
-    // beside the list update and joins before the force kernel rewrites them.
+    // The energy reduction of step s reads the force shares of step s and the
+    // kinetic shares of the integrate after it.  It runs on a branch (side
+    // stream) beside the list update and the next force: the shares have two
+    // sets which the steps alternate, so the branch joins only before the
+    // force kernel that rewrites its set, a step later.  (With one set it had
+    // to join before the next force and, from N = 4,000 to 100,000, was the
+    // longer branch once the list update's early exits were two.)
     const Launch lt{lthermo(b).grid, LJ_THERMO_THREADS, b->side};
     size_t rs = (size_t)b->nrep * 4;
     auto mark = [&](int64_t s, int ph, int end, cudaStream_t st) -> cudaError_t {
@@ -761,40 +799,48 @@ md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* rin
         // an external record becomes an event-record node of the graph
         return cudaEventRecordWithFlags(ge->ev[2 * k + end], st, cudaEventRecordExternal);
     };
-    bool joined = true;
-    auto join = [&]() -> cudaError_t {
-        if (joined) return cudaSuccess;
-        joined = true;
-        return cudaStreamWaitEvent(b->stream, b->ev_join, 0);
+    BoxDev set[2] = {b->d, b->d};
+    set[1].part_f += b->pf_cap;
+    set[1].part_k += LJ_KIN_WARPS * std::max<size_t>(1, b->chunks.size());
+    bool pending[2] = {false, false};   // reductions not joined yet, by set
+    auto join = [&](int q) -> cudaError_t {
+        if (!pending[q]) return cudaSuccess;
+        pending[q] = false;
+        return cudaStreamWaitEvent(b->stream, b->ev_join[q], 0);
     };
     for (int64_t s = 0; s <= n; ++s) {
         int mode = s == 0 ? LJ_STEP_FIRST : (s == n ? LJ_STEP_LAST : LJ_STEP_MID);
         CK(b, mark(s, 0, 0, b->stream));
-        CK(b, launch_integrate(b->d, mode, s == 0 ? 0 : energy, dt, (int)(s > 0 ? s - 1 : 0), l));
+        cudaGraphConditionalHandle cond = 0;
+        if (s < n) CKS(cond_begin(b, &cond));
+        const int prev = (int)((s + 1) & 1);   // the set of step s - 1
+        CK(b, launch_integrate(set[prev], mode, s == 0 ? 0 : energy, dt, (int)(s > 0 ? s - 1 : 0), cond, l));
         CK(b, mark(s, 0, 1, b->stream));
         b->launches += 1;
         if (s > 0 && energy) {
             CK(b, cudaEventRecord(b->ev_fork, b->stream));
             CK(b, cudaStreamWaitEvent(b->side, b->ev_fork, 0));
             CK(b, mark(s, 3, 0, b->side));
-            CK(b, launch_thermo(b->d, ring + (s - 1) * rs, 1, lt));
+            CK(b, launch_thermo(set[prev], ring + (s - 1) * rs, 1, lt));
             CK(b, mark(s, 3, 1, b->side));
-            CK(b, cudaEventRecord(b->ev_join, b->side));
-            joined = false;
+            CK(b, cudaEventRecord(b->ev_join[prev], b->side));
+            pending[prev] = true;
             b->launches += 1;
         }
         if (s == n) break;
         CK(b, mark(s, 1, 0, b->stream));
-        if (!b->all_pairs) CKS(enqueue_rebuild_step(b));   // all pairs: the drift keeps offsets wrapped
+        if (cond) CKS(cond_node(b, cond));
+        else if (!b->all_pairs) CKS(enqueue_rebuild(b, 0));   // all pairs: the drift keeps offsets wrapped
         CK(b, mark(s, 1, 1, b->stream));
-        CK(b, join());
+        CK(b, join((int)(s & 1)));
         CK(b, mark(s, 2, 0, b->stream));
-        CK(b, launch_force(b->d, energy, lforce(b)));
+        CK(b, launch_force(set[s & 1], energy, lforce(b)));
         CK(b, mark(s, 2, 1, b->stream));
         b->launches += 1;
         if (tape) CKS(tape_save(b, (int)s + 1));
     }
-    CK(b, join());
+    CK(b, join(0));
+    CK(b, join(1));
     // steps since md_set_thermostat (the thermostat's counter), on the device
     if (!tape) {
         CK(b, launch_step_advance(b->d.step_ctr, n, b->stream));
@@ -851,10 +897,13 @@ md_status ckpt_copy(md_box* b, int c, bool restore)
 md_status replay_lists(md_box* b)
 {
     CKS(set_all_rebuild(b));
-    CK(b, launch_list_work(b->d, b->stream));
+    if (b->nrep > 1) {
+        CK(b, launch_list_work(b->d, nullptr, b->stream));
+        b->launches += 1;
+    }
     CK(b, launch_list(b, b->stream));
     CK(b, launch_force(b->d, 0, lforce(b)));
-    b->launches += 3;
+    b->launches += 2;
     return MD_OK;
 }
 
@@ -1002,14 +1051,17 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
     b->ustream = static_cast<cudaStream_t>(stream);
     cudaGetDevice(&b->device);
     cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, b->device);
+    b->cluster_ok = cluster_rebuild_fits();
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess ||
         cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->ev_join[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->ev_join[1], cudaEventDisableTiming) != cudaSuccess ||
         cudaStreamCreateWithFlags(&b->cstream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
-        if (b->ev_join) cudaEventDestroy(b->ev_join);
+        for (cudaEvent_t ev : b->ev_join)
+            if (ev) cudaEventDestroy(ev);
         if (b->ev_fork) cudaEventDestroy(b->ev_fork);
         if (b->side) cudaStreamDestroy(b->side);
         if (b->ev) cudaEventDestroy(b->ev);
@@ -1108,11 +1160,11 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
         }
         CKS(dev_alloc(b, &d.err, 4));
         CKS(dev_alloc(b, &b->d_cond_runs, 1));
-        CKS(dev_alloc(b, &d.part_k, LJ_KIN_WARPS * std::max<size_t>(1, b->chunks.size())));
+        CKS(dev_alloc(b, &d.part_k, 2 * LJ_KIN_WARPS * std::max<size_t>(1, b->chunks.size())));   // two sets
         // (E_pot, W) shares, 8 per chunk (chunk kernel) or brick (tiled
         // kernel; make_grid grows the array with the bricks)
         b->pf_cap = 2 * LJ_FORCE_WARPS * std::max<size_t>(1, b->chunks.size());
-        CKS(dev_alloc(b, &d.part_f, b->pf_cap));
+        CKS(dev_alloc(b, &d.part_f, 2 * b->pf_cap));
         apply_force_kernel(b);
         CKS(dev_alloc(b, &b->d_type_user, std::max<int64_t>(1, ntot)));
         CK(b, cudaMemcpyAsync(b->d_rep, b->reps.data(), sizeof(RepDev) * b->reps.size(),
@@ -1159,7 +1211,8 @@ md_status md_box_destroy(md_box* b)
     b->allocs.clear();
     if (b->ev) cudaEventDestroy(b->ev);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-    if (b->ev_join) cudaEventDestroy(b->ev_join);
+    for (cudaEvent_t ev : b->ev_join)
+        if (ev) cudaEventDestroy(ev);
     if (b->side) cudaStreamDestroy(b->side);
     if (b->cstream) cudaStreamDestroy(b->cstream);
     if (b->stream) cudaStreamDestroy(b->stream);
@@ -1398,7 +1451,7 @@ md_status md_integrate(md_box* b, double dt, int64_t nsteps, int32_t ckpt_every,
         int e2[3];
         CKS(read_err(b, e2));
         // rebuild sequences the step graph's IF nodes ran
-        b->launches += (int64_t)(runs - b->cond_runs_seen) * rebuild_kernels(b);
+        b->launches += (int64_t)(runs - b->cond_runs_seen) * rebuild_kernels(b, true);
         b->cond_runs_seen = runs;
         for (auto& ge : b->graphs)
             if (ge.exec == g) {
@@ -1566,7 +1619,7 @@ md_status md_adjoint(md_box* b, const double* lam_x_T, const double* lam_v_T, do
         CK(b, cudaMemcpyAsync(&runs, b->d_cond_runs, sizeof runs, cudaMemcpyDeviceToHost, b->stream));
         int e2[3];
         CKS(read_err(b, e2));
-        b->launches += (int64_t)(runs - b->cond_runs_seen) * rebuild_kernels(b);   // the replay's rebuilds
+        b->launches += (int64_t)(runs - b->cond_runs_seen) * rebuild_kernels(b, true);   // the replay's rebuilds
         b->cond_runs_seen = runs;
         if (e2[0]) return fail(b, MD_ERR_CAPACITY, "md_adjoint: replay of a segment failed");
         const int form = (c == C - 1 ? 1 : 0) | (c == 0 ? 2 : 0);

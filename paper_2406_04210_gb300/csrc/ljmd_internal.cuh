@@ -521,12 +521,13 @@ cudaError_t launch_nlist(const BoxDev& b, Launch l);
 // one warp per cell, one lane per particle (rows staged in shared memory:
 // nlist_lanes_smem(K) bytes per block)
 cudaError_t launch_nlist_lanes(const BoxDev& b, Launch l);
-cudaError_t launch_list_work(const BoxDev& b, cudaStream_t s);   // one block; before the cell kernels
+// one block; before the cell kernels; counts its executions with work in *runs (nullable)
+cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s);
+// binning, sort and gather in one launch of one cluster (small boxes)
+cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles, int* tile_sum,
+                                   cudaStream_t s);
+bool cluster_rebuild_fits();
 size_t nlist_lanes_smem(int K);
-// sets a step graph's IF-node condition from the box-wide rebuild word
-cudaError_t launch_set_rebuild_cond(cudaGraphConditionalHandle h, const BoxDev& b, unsigned long long* runs,
-                                    cudaStream_t s);
-
 // k_force.cu
 cudaError_t launch_force(const BoxDev& b, int energy, Launch l);
 cudaError_t launch_thermo(const BoxDev& b, double* out, int with_kin, Launch l);
@@ -547,7 +548,9 @@ cudaError_t launch_pair_hist_grad(const BoxDev& b, int nbins, double rhist, doub
                                   const double* coef, double* grad, Launch l);
 
 // k_integrate.cu
-cudaError_t launch_integrate(const BoxDev& b, int mode, int energy, double dt, int sidx, Launch l);
+// cond: condition of the step graph's list-update node, set when a build is due (0: none)
+cudaError_t launch_integrate(const BoxDev& b, int mode, int energy, double dt, int sidx,
+                             cudaGraphConditionalHandle cond, Launch l);
 cudaError_t launch_step_advance(long long* ctr, long long n, cudaStream_t s);
 cudaError_t launch_upload(const BoxDev& b, const double* pos, const double* vel,
                           const int* type, int set_vel, Launch l);
