@@ -337,9 +337,10 @@ md_status md_get_list_kernel(md_box* b, int32_t* kind);
  * Verlet lists; Sec. 5 finds that kernel bound by fetching neighbour data).
  * Both give the forces, energy and virial of the same lists, equal up to
  * FP32 rounding:
- *   MD_FORCE_CHUNKS  work items of 128 consecutive particles, 4 threads per
- *                    particle, neighbour offsets gathered from global memory
- *                    through L1, the image shift decoded from each entry
+ *   MD_FORCE_CHUNKS  work items of 128 consecutive particles (16 in boxes of
+ *                    up to 512 such chunks), 4 threads per particle,
+ *                    neighbour offsets gathered from global memory through
+ *                    L1, the image shift decoded from each entry
  *   MD_FORCE_TILES   work items of up to 2 x 2 x 2 cells ("bricks"): a
  *                    producer warp stages the next brick's neighbourhood (up
  *                    to 4 x 4 x 4 cells, at most 2048 particles) into shared

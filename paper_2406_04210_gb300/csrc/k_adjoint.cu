@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const fl
         const int r = ch.x;
         if (r != cur_r) {                       // block-uniform
             const RepDev& R = b.rep[r];
-            ell = make_float3(R.ellf[0], R.ellf[1], R.ellf[2]);
+            ell = make_float3(R.ellf[0], 0.25f * R.ellf[1], 0.0625f * R.ellf[2]);   // edges in the digits' units
             cur_r = r;
         }
         if (!MONO) {   // per-chunk species-pair sums in shared memory
@@ -116,13 +116,13 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const fl
             float hx = 0.f, hy = 0.f, hz = 0.f;
             for (int s = l8; s < cnt; s += LJ_TPP) {
                 const unsigned ent = __ldcs(L + s);
-                const int j = (int)(ent & LJ_IDX_MASK);
+                const int j = (int)entry_slot(ent);
                 const float4 pj = __ldg(posq + j);
                 const float4 uj = __ldg(u_slot + j);
                 // d = (o_i - o_j) - (dx, dy, dz) * ell, one rounding per component
-                const float dx = fmaf(-entry_unit(ent, 26), ell.x, pi.x - pj.x);
-                const float dy = fmaf(-entry_unit(ent, 28), ell.y, pi.y - pj.y);
-                const float dz = fmaf(-entry_unit(ent, 30), ell.z, pi.z - pj.z);
+                const float dx = fmaf(-entry_unit<0>(ent), ell.x, pi.x - pj.x);
+                const float dy = fmaf(-entry_unit<1>(ent), ell.y, pi.y - pj.y);
+                const float dz = fmaf(-entry_unit<2>(ent), ell.z, pi.z - pj.z);
                 const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
                 float4 c, gg;
                 int pp = 0;
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kHistThreads) k_pair_hist(BoxDev b, int nbins,
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
         const int4 ch = b.chunk[w];
         const RepDev& R = b.rep[ch.x];
-        const float ex = R.ellf[0], ey = R.ellf[1], ez = R.ellf[2];
+        const float ex = R.ellf[0], ey = 0.25f * R.ellf[1], ez = 0.0625f * R.ellf[2];   // edges in the digits' units
         float hi[NB], lo[NB];
 #pragma unroll
         for (int q = 0; q < NB; ++q) hi[q] = lo[q] = 0.f;
@@ -293,12 +293,12 @@ __global__ void __launch_bounds__(kHistThreads) k_pair_hist(BoxDev b, int nbins,
                 float r2 = 0.f;
                 if (s < cnt) {
                     const unsigned ent = L[s];
-                    const int j = (int)(ent & LJ_IDX_MASK);
+                    const int j = (int)entry_slot(ent);
                     if (j > p) {
                         const float4 pj = b.posq[j];
-                        const float dx = fmaf(-entry_unit(ent, 26), ex, pi.x - pj.x);
-                        const float dy = fmaf(-entry_unit(ent, 28), ey, pi.y - pj.y);
-                        const float dz = fmaf(-entry_unit(ent, 30), ez, pi.z - pj.z);
+                        const float dx = fmaf(-entry_unit<0>(ent), ex, pi.x - pj.x);
+                        const float dy = fmaf(-entry_unit<1>(ent), ey, pi.y - pj.y);
+                        const float dz = fmaf(-entry_unit<2>(ent), ez, pi.z - pj.z);
                         r2 = dx * dx + dy * dy + dz * dz;
                         keep = r2 < rmax2;
                     }
@@ -381,8 +381,8 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_pair_hist_grad(BoxDev b, i
         if (ch.x != cur_r) {   // block-uniform
             const RepDev& R = b.rep[ch.x];
             ex = R.ellf[0];
-            ey = R.ellf[1];
-            ez = R.ellf[2];
+            ey = 0.25f * R.ellf[1];   // edges in the digits' units
+            ez = 0.0625f * R.ellf[2];
             __syncthreads();   // the previous replica's table is no longer read
             for (int k = threadIdx.x; k < nbins; k += blockDim.x)
                 s_bin[k] = make_float2(((float)k + 0.5f) * rbin,
@@ -399,10 +399,10 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_pair_hist_grad(BoxDev b, i
             float gx = 0.f, gy = 0.f, gz = 0.f;
             for (int s = l4; s < cnt; s += LJ_TPP) {
                 const unsigned ent = L[s];
-                const float4 pj = b.posq[ent & LJ_IDX_MASK];
-                const float dx = fmaf(-entry_unit(ent, 26), ex, pi.x - pj.x);
-                const float dy = fmaf(-entry_unit(ent, 28), ey, pi.y - pj.y);
-                const float dz = fmaf(-entry_unit(ent, 30), ez, pi.z - pj.z);
+                const float4 pj = b.posq[entry_slot(ent)];
+                const float dx = fmaf(-entry_unit<0>(ent), ex, pi.x - pj.x);
+                const float dy = fmaf(-entry_unit<1>(ent), ey, pi.y - pj.y);
+                const float dz = fmaf(-entry_unit<2>(ent), ez, pi.z - pj.z);
                 const float r2 = dx * dx + dy * dy + dz * dz;
                 if (!(r2 < rmax2)) continue;
                 const float r = sqrtf(r2);

@@ -43,26 +43,30 @@ __device__ __forceinline__ void block_sum2(double& a, double& c, double (*s)[32]
     __syncthreads();
 }
 
+// -d_ij of an FP32 pair: -d = (o_j - o_i) + (dx, dy, dz) * ell, one rounding
+// for the difference and one for the shift; x and y as FP32 pairs (a gathered
+// float4 holds them as a register pair).  ell is the cell edge in the digits'
+// units (x, y / 4, z / 16).
+__device__ __forceinline__ float2 neg_d_xy(unsigned ent, const float4& pj, const float4& pi, const float3& ell)
+{
+    const float2 u = __fadd2_rn(make_float2(entry_raw<0>(ent), entry_raw<1>(ent)),
+                                make_float2(-digit_one(0), -digit_one(1)));
+    const float2 t = __fadd2_rn(make_float2(pj.x, pj.y), make_float2(-pi.x, -pi.y));
+    return __ffma2_rn(u, make_float2(ell.x, ell.y), t);
+}
+
 // One pair term of the FP32 force: accumulates f d into (fx, fy, fz) and,
 // with ENERGY, the pair energy and virial; the term is masked (not branched)
-// by the cutoff test, so the threads of a particle never diverge.  Entries
-// past a row's count name the sentinel slot, whose distance fails the test.
+// by the cutoff test, so the threads of a particle never diverge.  (The tiled
+// kernel's path for a neighbourhood beyond its tile.)
 template <bool MONO, bool ENERGY>
 __device__ __forceinline__ void pair_f32(unsigned ent, const float4& pj, const float4& pi, int ti,
                                          const float3& ell, const float4* s_lj, const float* s_rc2,
                                          const float* s_esh, int nt, const float4& mlj, float mrc2,
                                          float mesh, float& fx, float& fy, float& fz, float& e, float& vir)
 {
-    // d = (o_i - o_j) - (dx, dy, dz) * ell, one rounding per component; the
-    // x and y parts as FP32 pairs (a gathered float4 holds them as a register
-    // pair), computed negated: -d = (o_j - o_i) + (dx, dy) * ell, exactly
-    // the negation of the scalar form
-    const float2 uxy = __fadd2_rn(make_float2(__uint_as_float(0x4B400000u | ((ent >> 26) & 3u)),
-                                              __uint_as_float(0x4B400000u | ((ent >> 28) & 3u))),
-                                  make_float2(-12582913.0f, -12582913.0f));
-    const float2 tq = __fadd2_rn(make_float2(pj.x, pj.y), make_float2(-pi.x, -pi.y));
-    const float2 dq = __ffma2_rn(uxy, make_float2(ell.x, ell.y), tq);
-    const float dz = fmaf(-entry_unit(ent, 30), ell.z, pi.z - pj.z);
+    const float2 dq = neg_d_xy(ent, pj, pi, ell);
+    const float dz = fmaf(-entry_unit<2>(ent), ell.z, pi.z - pj.z);
     const float2 sq = __fmul2_rn(dq, dq);
     const float r2 = fmaf(dz, dz, sq.x + sq.y);
     float4 c;
@@ -93,140 +97,233 @@ __device__ __forceinline__ void pair_f32(unsigned ent, const float4& pj, const f
     }
 }
 
-// FP32 pair force (Sec. 4/5), one 128-particle chunk per block pass, LJ_TPP
-// (4) threads per particle.  A particle's row is read in blocks of
-// LJ_ROW_BLOCK (16) entries, the last block's entries past the count
-// replaced by the sentinel slot; thread l8 of the particle takes entries
-// 4 l8 .. 4 l8 + 3 of each block with one 16-byte load (the next block's
-// load in flight while this one is computed), gathers the four neighbours'
-// FP32 offsets through L1 (four gathers in flight, two independent pair
-// chains) and the four threads combine their partial forces with shuffles.
-// The kernel is bound by gather latency: resident warps matter more than
-// gathers in flight per thread.  Six blocks of 256 per SM (40 registers, no
-// spills) measured 11 % faster than four (64 registers), and eight gathers
-// in flight at three blocks 9 % slower.  On the 4M-particle fluid 4 threads
-// per particle x 4 entries per thread measured fastest among 2/4/8 x 2/4/8.
+// Sums of k_force_f32 over a thread's pairs, in units of c12 = 48 eps sigma^12
+// for one species (applied at the end).  w = sum f r^2 (the virial).  The
+// energy needs no pair arithmetic of its own: with s6 = (sigma / r)^6,
+//   u = 4 eps (s6^2 - s6) - shift = (f r^2) / 12 - (2 eps s6 + shift),
+// so b sums the second term (one species: over 2 eps sigma^6).  Each is two
+// partial sums (the two pairs of pair2_f32), which also halves what each
+// rounds.
+struct PairSums {
+    float fx, fy, fz;
+    float2 w, b;
+};
+
+// Two pair terms: the separations one by one, everything from r^2 on as FP32
+// pairs.  The cutoff masks 1/r^2 (times 1 or 0), so that every term of a pair
+// beyond it, the sentinel's too, is 0.
+template <bool MONO, bool ENERGY>
+__device__ __forceinline__ void pair2_f32(unsigned e0, const float4& q0, unsigned e1, const float4& q1,
+                                          const float4& pi, int tb, const float3& ell, const float4* s_lj,
+                                          const float* s_rc2, float nh, float kap, float mrc2, PairSums& S)
+{
+    const float2 a0 = neg_d_xy(e0, q0, pi, ell), a1 = neg_d_xy(e1, q1, pi, ell);
+    const float2 az = make_float2(fmaf(entry_unit<2>(e0), ell.z, q0.z - pi.z), fmaf(entry_unit<2>(e1), ell.z, q1.z - pi.z));
+    const float2 s0 = __fmul2_rn(a0, a0), s1 = __fmul2_rn(a1, a1);
+    const float2 r2 = __ffma2_rn(az, az, make_float2(s0.x + s0.y, s1.x + s1.y));
+    float2 c12, nc6, rc2, hb, esh;
+    if (MONO) {
+        rc2 = make_float2(mrc2, mrc2);
+    } else {
+        const int p0 = tb + __float_as_int(q0.w), p1 = tb + __float_as_int(q1.w);
+        const float4 c0 = s_lj[p0], c1 = s_lj[p1];
+        c12 = make_float2(c0.x, c1.x);
+        nc6 = make_float2(c0.y, c1.y);
+        hb = make_float2(c0.z, c1.z);
+        esh = make_float2(c0.w, c1.w);
+        rc2 = make_float2(s_rc2[p0], s_rc2[p1]);
+    }
+    const float2 in = make_float2(r2.x < rc2.x ? 1.f : 0.f, r2.y < rc2.y ? 1.f : 0.f);
+    const float2 ri = __fmul2_rn(make_float2(rcp_approx(r2.x), rcp_approx(r2.y)), in);
+    const float2 r6 = __fmul2_rn(__fmul2_rn(ri, ri), ri);
+    const float2 g =   // f r^2
+        __fmul2_rn(r6, MONO ? __fadd2_rn(r6, make_float2(nh, nh)) : __ffma2_rn(c12, r6, nc6));
+    const float2 f = __fmul2_rn(ri, g);
+    S.fx = fmaf(f.x, a0.x, S.fx);   // of -d: the sums are negated at the end
+    S.fy = fmaf(f.x, a0.y, S.fy);
+    S.fz = fmaf(f.x, az.x, S.fz);
+    S.fx = fmaf(f.y, a1.x, S.fx);
+    S.fy = fmaf(f.y, a1.y, S.fy);
+    S.fz = fmaf(f.y, az.y, S.fz);
+    if (ENERGY) {
+        S.w = __fadd2_rn(S.w, g);
+        if (MONO) S.b = __fadd2_rn(S.b, __ffma2_rn(in, make_float2(kap, kap), r6));
+        else S.b = __ffma2_rn(esh, in, __ffma2_rn(hb, r6, S.b));
+    }
+}
+
+// One pair term, the same sums, in scalar arithmetic: more instructions, but it
+// fits the 32 registers of eight blocks of 256 per SM (packed operands and
+// constants take register pairs).
+template <bool MONO, bool ENERGY>
+__device__ __forceinline__ void pair1_f32(unsigned e0, const float4& q0, const float4& pi, int tb, const float3& ell,
+                                          const float4* s_lj, const float* s_rc2, float nh, float kap, float mrc2,
+                                          PairSums& S)
+{
+    const float2 a0 = neg_d_xy(e0, q0, pi, ell);
+    const float az = fmaf(entry_unit<2>(e0), ell.z, q0.z - pi.z);
+    const float2 s0 = __fmul2_rn(a0, a0);
+    const float r2 = fmaf(az, az, s0.x + s0.y);
+    float4 c = make_float4(1.f, nh, 0.f, 0.f);
+    float rc2 = mrc2;
+    if (!MONO) {
+        const int p0 = tb + __float_as_int(q0.w);
+        c = s_lj[p0];
+        rc2 = s_rc2[p0];
+    }
+    const bool in = r2 < rc2;
+    const float ri = in ? rcp_approx(r2) : 0.f;
+    const float r6 = ri * ri * ri;
+    const float g = r6 * (MONO ? r6 + nh : fmaf(c.x, r6, c.y));   // f r^2
+    const float f = ri * g;
+    S.fx = fmaf(f, a0.x, S.fx);   // of -d: the sums are negated at the end
+    S.fy = fmaf(f, a0.y, S.fy);
+    S.fz = fmaf(f, az, S.fz);
+    if (ENERGY) {
+        S.w.x += g;
+        if (MONO) S.b.x += r6 + (in ? kap : 0.f);
+        else S.b.x = fmaf(c.z, r6, S.b.x + (in ? c.w : 0.f));
+    }
+}
+
+// FP32 pair force (Sec. 4/5), LJ_TPP (4) threads per particle.  A particle's
+// row is read in blocks of LJ_ROW_BLOCK (16) entries, the last block's entries
+// past the count replaced by the sentinel slot; each thread takes four
+// consecutive entries of a block with one 16-byte load (the next block's load
+// in flight while this one is computed) and gathers the four neighbours' FP32
+// offsets through L1 (four gathers in flight); the four threads combine their
+// partial forces with shuffles.
+// Work items: chunks of 128 particles, two passes of 64 by a block of 256; or,
+// SPREAD, 16 particles by a block of 64 threads (the rule is at spread_force).
+// What bounds it.  Chunks: the L1 data pipe, ~10 wavefronts per gather (67 %
+// of peak over the launch, 79 % while active), which neither fewer
+// instructions (33.4 M -> 26.5 M with the packed pairs: 47.2 us against 45.6
+// at 256k, fewer resident warps), nor rows in the order of slot mod 8 (fewer
+// bank conflicts, more lines: 44.7 us, but 662 us against 588 at 4M) moved, so
+// resident warps matter most: 32 registers and eight blocks per SM for one
+// species, 40 and six for several.  With the digits below the slot and the
+// energy from sums the force needs anyway: 4M with energies 589 -> 573 us,
+// without 529 -> 515, the 256k mixture 78.6 -> 75.3.  SPREAD: the serial row
+// (five dependent blocks), on every SM instead of a few: N = 4,000 16.4 -> 9.0
+// us, N = 32,000 17.2 -> 12.8 us; packed pairs, as registers are free there.
 // MONO: a single species, its pair constants read from the kernel
 // parameters.  SINGLE (MONO and one replica): the cell edge from the
-// parameters too and one pair chain, 32 registers, eight blocks per SM.
+// parameters too.  One (E_pot, W) share per warp and item.
 static_assert(LJ_TPP * 4 == LJ_ROW_BLOCK, "a row block is one 16-byte load per thread of a particle");
-template <bool MONO, bool ENERGY, bool SINGLE>
-__global__ void __launch_bounds__(LJ_FORCE_THREADS, SINGLE ? 8 : 6) k_force_f32(BoxDev b)
+template <bool MONO, bool ENERGY, bool SINGLE, int THREADS, int RES>
+__global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
 {
-    __shared__ float4 s_lj[LJ_MAXT * LJ_MAXT];   // c12, c6, e12, e6
-    __shared__ float s_rc2[LJ_MAXT * LJ_MAXT];
-    __shared__ float s_esh[LJ_MAXT * LJ_MAXT];
-    const LJDev* lj = b.lj;
-    const int nt = lj->nt;
-    for (int k = threadIdx.x; k < nt * nt; k += blockDim.x) {
-        s_lj[k] = make_float4(lj->c12[k], lj->c6[k], lj->e12[k], lj->e6[k]);
-        s_rc2[k] = lj->rc2[k];
-        s_esh[k] = lj->shift[k];
+    constexpr int TPP = LJ_TPP;
+    constexpr bool SPREAD = THREADS == LJ_SPREAD_THREADS;
+    constexpr int PASS = THREADS / TPP;                       // particles of a pass
+    constexpr int PARTS = SPREAD ? LJ_CHUNK / PASS : 1;       // work items of a chunk
+    constexpr int OWN = LJ_CHUNK / PARTS;                     // particles of an item
+    __shared__ float4 s_lj[MONO ? 1 : LJ_MAXT * LJ_MAXT];     // c12, -c6, 2 eps sigma^6, shift
+    __shared__ float s_rc2[MONO ? 1 : LJ_MAXT * LJ_MAXT];
+    if (!MONO) {
+        const LJDev* lj = b.lj;
+        for (int k = threadIdx.x; k < b.nt * b.nt; k += blockDim.x) {
+            s_lj[k] = make_float4(lj->c12[k], -lj->c6[k], 0.5f * lj->e6[k], lj->shift[k]);
+            s_rc2[k] = lj->rc2[k];
+        }
+        __syncthreads();   // the pair tables are complete (the block's only barrier)
     }
-    __syncthreads();   // the pair tables are complete (the block's only barrier)
-    const float4 mlj = b.c1;
-    const float mrc2 = b.rc2_1;
-    const float mesh = b.esh_1;
+    // one species: f r^2 = c12 r6 (r6 + nh), the energy's second term (e6 / 2) (r6 + kap)
+    const float c12 = MONO ? b.c1.x : 1.f, nh = b.nh_1, kap = b.kap_1, mrc2 = b.rc2_1;
     const int K = b.K;
-    const int grp = threadIdx.x / LJ_TPP, l8 = threadIdx.x % LJ_TPP;
+    const int grp = threadIdx.x / TPP, lt = threadIdx.x % TPP;
     const float4* __restrict__ posq = b.posq;
     const unsigned sent = entry_make(13, b.np);
     int cur_r = -1;
-    float3 ell = make_float3(0.f, 0.f, 0.f);
-    for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
+    float3 ell = make_float3(b.ell1.x, 0.25f * b.ell1.y, 0.0625f * b.ell1.z);   // edges in the digits' units
+    for (int it = blockIdx.x; it < b.nchunk * PARTS; it += gridDim.x) {
+        const int w = it / PARTS, part = it % PARTS;
         const int4 ch = b.chunk[w];
         const int r = ch.x;
-        if (SINGLE) {
-            ell = b.ell1;
-        } else if (r != cur_r) {                // block-uniform
+        if (!SINGLE && r != cur_r) {            // block-uniform
             const RepDev& R = b.rep[r];
-            ell = make_float3(R.ellf[0], R.ellf[1], R.ellf[2]);
+            ell = make_float3(R.ellf[0], 0.25f * R.ellf[1], 0.0625f * R.ellf[2]);
             cur_r = r;
         }
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && part == 0) {
             if (w == 0) *b.any_req = 0;         // the list update of this step has run
             if (w == b.rep[r].chunk_off) {      // clear the replica's rebuild triggers
                 b.disp_max[r] = 0u;
                 b.rebuild_req[r] = 0;
             }
         }
-        float e = 0.f, vir = 0.f;
-        for (int base = ch.y; base < ch.z; base += LJ_FORCE_THREADS / LJ_TPP) {
+        PairSums S;
+        S.w = S.b = make_float2(0.f, 0.f);
+        const int first = ch.y + part * OWN, last = min(first + OWN, ch.z);
+        for (int base = first; base < last; base += PASS) {
             const int p = base + grp;
-            const bool act = p < ch.z;
+            const bool act = p < last;
             float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
             int cnt = 0;
-            const uint4* L = reinterpret_cast<const uint4*>(b.nbr + (size_t)K * p) + l8;
+            const uint4* L = reinterpret_cast<const uint4*>(b.nbr + (size_t)K * p) + lt;
             uint4 cur = make_uint4(0u, 0u, 0u, 0u);
             if (act) {
                 pi = posq[p];
                 cnt = min(b.nbr_count[p], K);
                 cur = __ldcs(L);   // the row's first block (K >= 16 slots), in flight with the count
             }
-            const int nblk = (cnt + LJ_ROW_BLOCK - 1) / LJ_ROW_BLOCK;
-            const int ti = __float_as_int(pi.w);
-            float fx = 0.f, fy = 0.f, fz = 0.f, fx2 = 0.f, fy2 = 0.f, fz2 = 0.f;
-            // the second pair chain: independent partial forces, or (SINGLE,
-            // registers for occupancy) the first chain itself
-            float& gx = SINGLE ? fx : fx2;
-            float& gy = SINGLE ? fy : fy2;
-            float& gz = SINGLE ? fz : fz2;
+            const int nblk = (cnt + 4 * TPP - 1) / (4 * TPP);
+            const int tb = MONO ? 0 : __float_as_int(pi.w) * b.nt;
+            S.fx = S.fy = S.fz = 0.f;
             // four entries: four gathers in flight
             auto block4 = [&](const uint4& q) {
-                const float4 p0 = __ldg(posq + (q.x & LJ_IDX_MASK));
-                const float4 p1 = __ldg(posq + (q.y & LJ_IDX_MASK));
-                const float4 p2 = __ldg(posq + (q.z & LJ_IDX_MASK));
-                const float4 p3 = __ldg(posq + (q.w & LJ_IDX_MASK));
-                pair_f32<MONO, ENERGY>(q.x, p0, pi, ti, ell, s_lj, s_rc2, s_esh, nt, mlj, mrc2, mesh,
-                                       fx, fy, fz, e, vir);
-                pair_f32<MONO, ENERGY>(q.y, p1, pi, ti, ell, s_lj, s_rc2, s_esh, nt, mlj, mrc2, mesh,
-                                       gx, gy, gz, e, vir);
-                pair_f32<MONO, ENERGY>(q.z, p2, pi, ti, ell, s_lj, s_rc2, s_esh, nt, mlj, mrc2, mesh,
-                                       fx, fy, fz, e, vir);
-                pair_f32<MONO, ENERGY>(q.w, p3, pi, ti, ell, s_lj, s_rc2, s_esh, nt, mlj, mrc2, mesh,
-                                       gx, gy, gz, e, vir);
+                const float4 p0 = __ldg(posq + entry_slot(q.x));
+                const float4 p1 = __ldg(posq + entry_slot(q.y));
+                const float4 p2 = __ldg(posq + entry_slot(q.z));
+                const float4 p3 = __ldg(posq + entry_slot(q.w));
+                if (SPREAD) {
+                    pair2_f32<MONO, ENERGY>(q.x, p0, q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
+                    pair2_f32<MONO, ENERGY>(q.z, p2, q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
+                } else {
+                    pair1_f32<MONO, ENERGY>(q.x, p0, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
+                    pair1_f32<MONO, ENERGY>(q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
+                    pair1_f32<MONO, ENERGY>(q.z, p2, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
+                    pair1_f32<MONO, ENERGY>(q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
+                }
             };
             if (nblk > 0) {
                 for (int blk = 1; blk < nblk; ++blk) {
-                    const uint4 nxt = __ldcs(L + blk * LJ_TPP);   // in flight during this block
+                    const uint4 nxt = __ldcs(L + blk * TPP);   // in flight during this block
                     block4(cur);
                     cur = nxt;
                 }
                 // the row's last block: entries past the count (stale or
                 // never written) name the sentinel slot
-                const int lim = cnt - ((nblk - 1) * LJ_ROW_BLOCK + 4 * l8);
+                const int lim = cnt - ((nblk - 1) * 4 * TPP + 4 * lt);
                 cur.x = lim > 0 ? cur.x : sent;
                 cur.y = lim > 1 ? cur.y : sent;
                 cur.z = lim > 2 ? cur.z : sent;
                 cur.w = lim > 3 ? cur.w : sent;
                 block4(cur);
             }
-            if (!SINGLE) {
-                fx += fx2;
-                fy += fy2;
-                fz += fz2;
-            }
 #pragma unroll
-            for (int o = LJ_TPP / 2; o > 0; o >>= 1) {
-                fx += __shfl_xor_sync(0xffffffffu, fx, o);
-                fy += __shfl_xor_sync(0xffffffffu, fy, o);
-                fz += __shfl_xor_sync(0xffffffffu, fz, o);
+            for (int o = TPP / 2; o > 0; o >>= 1) {
+                S.fx += __shfl_xor_sync(0xffffffffu, S.fx, o);
+                S.fy += __shfl_xor_sync(0xffffffffu, S.fy, o);
+                S.fz += __shfl_xor_sync(0xffffffffu, S.fz, o);
             }
-            if (act && l8 == 0) {
-                b.force4[p] = make_float4(fx, fy, fz, 0.f);
-                if (!isfinite(fx + fy + fz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
+            if (act && lt == 0) {
+                b.force4[p] = make_float4(-c12 * S.fx, -c12 * S.fy, -c12 * S.fz, 0.f);
+                if (!isfinite(S.fx + S.fy + S.fz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
             }
         }
         if (ENERGY) {
-            // one (E_pot, W) share per warp and chunk, no block barrier: the
-            // warps of a block run ahead into the next chunk independently.
+            // one (E_pot, W) share per warp and item, no block barrier: the
+            // warps of a block run ahead into the next item independently.
             // The warp sum is double-single (two FP32 words per partial
             // sum): FP64-class precision on the FP32 pipe, since FP64 adds
             // are scarce on this GPU.  The share is stored as the (hi, lo)
             // pair itself (pf_ds), halved exactly; the reduction converts
+            const float vir = c12 * (S.w.x + S.w.y);
+            const float e = fmaf(vir, 1.f / 12.f, (MONO ? -0.5f * b.c1.w : -1.f) * (S.b.x + S.b.y));
             const float2 de = warp_sum_ds2(e), dw = warp_sum_ds2(vir);
             if ((threadIdx.x & 31) == 0) {
-                const size_t q = (size_t)w * LJ_FORCE_WARPS + (threadIdx.x >> 5);
+                const size_t q = (size_t)it * (THREADS / 32) + (threadIdx.x >> 5);
                 reinterpret_cast<float4*>(b.part_f)[q] =
                     make_float4(0.5f * de.x, 0.5f * de.y, 0.5f * dw.x, 0.5f * dw.y);
             }
@@ -246,7 +343,7 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS, SINGLE ? 8 : 6) k_force_f32(
 // the brick's particles' list rows, LJ_TPP threads per particle, four
 // entries per thread and 16-entry row block.  An entry (stencil digits of neighbour cell k, slot j) names the
 // tile element j - start + base of the tile cell at the particle's cell plus
-// k: its byte address is (entry << 2) plus a table word of the particle's
+// k: its byte address is (entry >> 4) plus a table word of the particle's
 // cell indexed by the digits, which also cancels what the shift leaves of
 // the digits -- one shift-add per entry, no decode and no image shift per
 // pair.  Pairs are evaluated two at a time with FP32-pair arithmetic on
@@ -332,7 +429,7 @@ __device__ __forceinline__ void tile_pair2(uint32_t a0, uint32_t a1, const float
 }
 
 // tile address of entry e for the particle's address table D
-__device__ __forceinline__ uint32_t tile_addr(uint32_t e, const uint32_t* D) { return (e << 2) + D[e >> 26]; }
+__device__ __forceinline__ uint32_t tile_addr(uint32_t e, const uint32_t* D) { return (e >> 4) + D[e & 63u]; }
 
 static_assert(LJ_BRICK_WARPS == LJ_FORCE_WARPS, "per-brick shares in the chunk kernel's share stride");
 constexpr int kBrickThreads = LJ_BRICK_THREADS;          // consumer threads
@@ -510,9 +607,8 @@ __global__ void __launch_bounds__(LJ_BRICK_THREADS + 32, 4) k_force_tile_f32(Box
                     const int u = cl & sx, v = (cl >> sx) & sy, w = cl >> (sx + sy);
                     const uint32_t dxd = kk % 3, dyd = (kk / 3) % 3, dzd = kk / 9;
                     const int tc = (u + (int)dxd) + tx * (v + (int)dyd) + txy * (w + (int)dzd);
-                    // (entry << 2) = 4 j + (dx digit << 28) + (dy digit << 30) mod 2^32
-                    s_D[buf][cl][(dzd << 4) | (dyd << 2) | dxd] =
-                        Xb + 4u * (uint32_t)(s_tb[tc] - s_ts[tc]) - (dxd << 28) - (dyd << 30);
+                    // (entry >> 4) = 4 j + dz digit
+                    s_D[buf][cl][(dzd << 4) | (dyd << 2) | dxd] = Xb + 4u * (uint32_t)(s_tb[tc] - s_ts[tc]) - dzd;
                 }
             }
             mbar_arrive1(&s_full[buf]);   // every producer lane: its stores precede the arrival
@@ -592,6 +688,7 @@ __global__ void __launch_bounds__(LJ_BRICK_THREADS + 32, 4) k_force_tile_f32(Box
                     tile_pair2<MONO, ENERGY, PL>(a2, a3, nx, ny, nz, ti, nt, s_lj, s_rc2, s_esh, mlj, mrc2, mesh, A);
                 }
             } else {   // neighbourhood larger than the tile: gathers from global memory
+                const float3 ell_digit = make_float3(ell.x, 0.25f * ell.y, 0.0625f * ell.z);
                 float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f, vir = 0.f;
                 for (int blk = 0; blk < nblk; ++blk) {
                     const bool last = blk + 1 == nblk;
@@ -600,9 +697,9 @@ __global__ void __launch_bounds__(LJ_BRICK_THREADS + 32, 4) k_force_tile_f32(Box
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
                         const unsigned ek = (!last || lim > kk) ? q[kk] : sent_ent;
-                        const float4 pj = __ldg(posq + (ek & LJ_IDX_MASK));
-                        pair_f32<MONO, ENERGY>(ek, pj, pi, ti, ell, s_lj, s_rc2, s_esh, nt, mlj, mrc2, mesh, fx, fy,
-                                               fz, e, vir);
+                        const float4 pj = __ldg(posq + entry_slot(ek));
+                        pair_f32<MONO, ENERGY>(ek, pj, pi, ti, ell_digit, s_lj, s_rc2, s_esh, nt, mlj, mrc2, mesh, fx,
+                                               fy, fz, e, vir);
                     }
                     cur = nx1;
                     nx1 = nx2;
@@ -706,7 +803,7 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
         __syncthreads();   // the tables are complete; the previous item's sums are read
         if (r != cur_r) {  // block-uniform
             const RepDev& R = b.rep[r];
-            ell = make_float3(R.ellf[0], R.ellf[1], R.ellf[2]);
+            ell = make_float3(R.ellf[0], 0.25f * R.ellf[1], 0.0625f * R.ellf[2]);   // edges in the digits' units
             if (threadIdx.x < 9) s_ell[threadIdx.x / 3][threadIdx.x % 3] = (double)((int)threadIdx.x % 3 - 1) * R.ell[threadIdx.x / 3];
             __syncthreads();
             cur_r = r;
@@ -743,10 +840,10 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
                 for (int u = 0; u < 4; ++u) {
                     in[u] = false;
                     if (u < lim) {
-                        const float4 pj = __ldg(posq + (en[u] & LJ_IDX_MASK));
-                        const float dx = fmaf(-entry_unit(en[u], 26), ell.x, pi.x - pj.x);
-                        const float dy = fmaf(-entry_unit(en[u], 28), ell.y, pi.y - pj.y);
-                        const float dz = fmaf(-entry_unit(en[u], 30), ell.z, pi.z - pj.z);
+                        const float4 pj = __ldg(posq + entry_slot(en[u]));
+                        const float dx = fmaf(-entry_unit<0>(en[u]), ell.x, pi.x - pj.x);
+                        const float dy = fmaf(-entry_unit<1>(en[u]), ell.y, pi.y - pj.y);
+                        const float dz = fmaf(-entry_unit<2>(en[u]), ell.z, pi.z - pj.z);
                         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
                         in[u] = r2 < s_near[MONO ? 0 : tb + __float_as_int(pj.w)];
                     }
@@ -767,10 +864,10 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
             __syncwarp();
             for (int t = l4; t < nq; t += LJ_TPP) {
                 const uint32_t ent = q[t];
-                const int j = (int)(ent & LJ_IDX_MASK);
-                const double dx = (xi - __ldg(&b.off[j])) - s_ell[0][(ent >> 26) & 3u];
-                const double dy = (yi - __ldg(&b.off[np + j])) - s_ell[1][(ent >> 28) & 3u];
-                const double dz = (zi - __ldg(&b.off[2 * np + j])) - s_ell[2][ent >> 30];
+                const int j = (int)entry_slot(ent);
+                const double dx = (xi - __ldg(&b.off[j])) - s_ell[0][ent & 3u];
+                const double dy = (yi - __ldg(&b.off[np + j])) - s_ell[1][(ent >> 2) & 3u];
+                const double dz = (zi - __ldg(&b.off[2 * np + j])) - s_ell[2][(ent >> 4) & 3u];
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 const int pp = MONO ? 0 : tb + __ldg(&b.type[j]);
                 // r2 < rc2 on their bits (neither is negative), not on the FP64 pipe; a NaN fails
@@ -1248,15 +1345,27 @@ cudaError_t launch_force(const BoxDev& b, int energy, Launch l)
             if (energy) k_force_tile_f32<false, true><<<l.grid, th, dx, l.s>>>(b);
             else k_force_tile_f32<false, false><<<l.grid, th, dx, l.s>>>(b);
         }
+    } else if (b.force_spread) {
+        const int th = LJ_SPREAD_THREADS;
+        if (b.nt == 1 && b.nrep == 1) {
+            if (energy) k_force_f32<true, true, true, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+            else k_force_f32<true, false, true, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+        } else if (b.nt == 1) {
+            if (energy) k_force_f32<true, true, false, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+            else k_force_f32<true, false, false, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+        } else {
+            if (energy) k_force_f32<false, true, false, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+            else k_force_f32<false, false, false, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+        }
     } else if (b.nt == 1 && b.nrep == 1) {
-        if (energy) k_force_f32<true, true, true><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
-        else k_force_f32<true, false, true><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        if (energy) k_force_f32<true, true, true, LJ_FORCE_THREADS, 8><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        else k_force_f32<true, false, true, LJ_FORCE_THREADS, 8><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
     } else if (b.nt == 1) {
-        if (energy) k_force_f32<true, true, false><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
-        else k_force_f32<true, false, false><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        if (energy) k_force_f32<true, true, false, LJ_FORCE_THREADS, 8><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        else k_force_f32<true, false, false, LJ_FORCE_THREADS, 8><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
     } else {
-        if (energy) k_force_f32<false, true, false><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
-        else k_force_f32<false, false, false><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        if (energy) k_force_f32<false, true, false, LJ_FORCE_THREADS, 6><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        else k_force_f32<false, false, false, LJ_FORCE_THREADS, 6><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
     }
     return cudaGetLastError();
 }

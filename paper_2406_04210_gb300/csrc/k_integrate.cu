@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_get_nlist(BoxDev b, int* count, lo
             int m = cnt < b.K ? cnt : b.K;
             if ((long long)m > cap) m = (int)cap;
             const uint32_t* lp = b.nbr + (size_t)b.K * p;
-            for (int s = 0; s < m; ++s) nbr[gu * cap + s] = b.uid[lp[s] & LJ_IDX_MASK];
+            for (int s = 0; s < m; ++s) nbr[gu * cap + s] = b.uid[entry_slot(lp[s])];
         }
     }
 }

@@ -698,9 +698,9 @@ __global__ void __launch_bounds__(LJ_LIST_THREADS, 3) k_nlist(BoxDev b)
                 if (lane >= o) incl += t;
             }
             const int total = __shfl_sync(0xffffffffu, incl, 31);
-            // entry of tile index t from cell k: t + kent[k] (the shift digits
-            // above the slot, the slot being t minus the cell's tile offset)
-            if (lane < 27) kent[lane] = entry_make(lane, 0) - (uint32_t)rk.z;
+            // entry of tile index t from cell k: t above the digits + kent[k]
+            // (the slot being t minus the cell's tile offset)
+            if (lane < 27) kent[lane] = entry_make(lane, 0) - ((uint32_t)rk.z << LJ_DIGIT_BITS);
             const int self13 = p0q + __shfl_sync(0xffffffffu, rk.z, 13);   // tile index of the quad's first particle
             const int off = incl - len;
             int cnt[4] = {0, 0, 0, 0};
@@ -739,7 +739,7 @@ __global__ void __launch_bounds__(LJ_LIST_THREADS, 3) k_nlist(BoxDev b)
                         qx[h] = t < wn ? pj.x + sh.x : 1.0e38f;
                         qy[h] = pj.y + sh.y;
                         qz[h] = pj.z + sh.z;
-                        ent[h] = (uint32_t)idx + kent[k];
+                        ent[h] = ((uint32_t)idx << LJ_DIGIT_BITS) + kent[k];
                         // tile slices are disjoint, so the index alone finds the
                         // particle itself: quad slot idx - self13 (if in 0..3)
                         selfg[h] = idx - self13;
@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(LJ_LIST_THREADS, 3) k_nlist(BoxDev b)
                     uint32_t ent = 0;
                     if (s < c) {
                         ent = row[s];
-                        const int j = (int)(ent & LJ_IDX_MASK);
+                        const int j = (int)entry_slot(ent);
                         const int k = entry_k(ent);
                         const float4 pj = b.posq[j];
                         const float4 sh = s_shift[k];
@@ -806,6 +806,8 @@ __global__ void __launch_bounds__(LJ_LIST_THREADS, 3) k_nlist(BoxDev b)
             const int c = lane == 0 ? cnt[0] : lane == 1 ? cnt[1] : lane == 2 ? cnt[2] : cnt[3];
             if (lane < nq) {
                 b.nbr_count[p0q + lane] = c;
+                for (int s = c; s < b.K && (s & 3); ++s)   // the row's last piece of four is filled with the sentinel
+                    row0[(size_t)b.K * lane + s] = entry_make(13, b.np);
                 if (c > b.K) {
                     atomicOr(&b.err[0], LJ_ERRBIT_CAPACITY);
                     atomicMax(&b.err[1], c);
@@ -851,13 +853,12 @@ constexpr int kRing = 64;   // staged candidates per warp: < 32 waiting + one ch
 // with the capacity K.
 constexpr int kLaneRow = 48;
 
-// r^2 of the pair (i, candidate q = o_j + shift) from n = -o_i.
-__device__ __forceinline__ float lane_r2(const float2 nxy, float nz, const float4& q)
+// r^2 - rl^2 of the pair (i, candidate q = o_j + shift), rounded as in the
+// batches.
+__device__ __forceinline__ float lane_t(const float4& pi, const float4& q, float rl2)
 {
-    const float2 d = __fadd2_rn(make_float2(q.x, q.y), nxy);
-    const float dz = q.z + nz;
-    const float2 s = __fmul2_rn(d, d);
-    return fmaf(dz, dz, s.x + s.y);
+    const float dx = __fadd_rn(q.x, -pi.x), dy = __fadd_rn(q.y, -pi.y), dz = __fadd_rn(q.z, -pi.z);
+    return __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmaf_rn(dx, dx, -rl2)));
 }
 
 __device__ __forceinline__ void phase_lanes(const BoxDev& b)
@@ -884,9 +885,10 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
     float* const ry = s_cy[warp];
     float* const rz = s_cz[warp];
     uint32_t* const rc = s_cc[warp];
-    const float lo2 = b.rl2f - b.band, hi2 = b.rl2f + b.band;
-    const float rcull = hi2 + 1e-3f;   // staging margin for the rounding of the shifted offsets
+    const float rl2 = b.rl2f, band = b.band;
+    const float rcull = rl2 + band + 1e-3f;   // staging margin for the rounding of the shifted offsets
     const float4* __restrict__ posq = b.posq;
+    const uint32_t sent = entry_make(13, b.np);
     int longest = 0;
     const int nwarp = gridDim.x * kLaneWarps;
     const int total = b.lw_off[b.lw_hdr[0]];
@@ -929,8 +931,6 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
                 uz = fmaxf(uz, __shfl_xor_sync(0xffffffffu, uz, o));
             }
             if (!act) pi = make_float4(1.0e30f, 1.0e30f, 1.0e30f, 0.f);   // a far point: r^2 is inf
-            const float2 nxy = make_float2(-pi.x, -pi.y);
-            const float nz = -pi.z;
             const uint32_t self = (13u << LJ_TILE_BITS) | (uint32_t)(ib + lane);   // the particle itself
             int cnt = 0;                   // codes in the row buffer
             int flushed = 0;               // list entries already written out (a multiple of 16)
@@ -950,7 +950,7 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
                                 const uint32_t h = row[32 * (16 * q + 4 * e + u)];
-                                o[u] = base[h >> LJ_TILE_BITS] + (h & LJ_TILE_MASK);
+                                o[u] = base[h >> LJ_TILE_BITS] + ((h & LJ_TILE_MASK) << LJ_DIGIT_BITS);
                             }
                             dst[(flushed >> 2) + 4 * q + e] = make_uint4(o[0], o[1], o[2], o[3]);
                         }
@@ -962,70 +962,54 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
                 cnt = rest;
                 __syncwarp();
             };
-            // test the staged candidates [head, head + cnt) against the lane's
-            // particle and append the hits
-            auto batch = [&](int nb) {
+            // test the 32 staged candidates from head on against the lane's
+            // particle and append the hits (the buffer has room: flushed before)
+            auto batch = [&]() {
                 const int c0 = cnt;
                 const int h0 = (int)(head & (kRing - 1));
-                float m = 0.f;   // largest accepted r^2 of the batch
-                if (nb == 32) {   // the buffer has room for 32 more (flushed before the batch)
-                    // branch-free, two candidates per step with FP32-pair
-                    // arithmetic: every candidate's code is written to the
-                    // next free slot (32-bit shared address), which advances
-                    // only on a hit
-                    uint32_t wa = (uint32_t)__cvta_generic_to_shared(row + 32 * cnt);
-                    const float2 px = make_float2(nxy.x, nxy.x), py = make_float2(nxy.y, nxy.y),
-                                 pz = make_float2(nz, nz);
-                    // four candidates per step: one 16-byte broadcast load per
-                    // component and for the codes
-                    auto step2 = [&](float2 qx, float2 qy, float2 qz, uint32_t c0, uint32_t c1) {
-                        const float2 dx = __fadd2_rn(qx, px), dy = __fadd2_rn(qy, py), dz = __fadd2_rn(qz, pz);
-                        const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-                        const bool h1 = (r2.x < hi2) & (c0 != self);
-                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(wa), "h"((unsigned short)c0));
-                        wa += h1 ? 64u : 0u;
-                        m = fmaxf(m, h1 ? r2.x : 0.f);
-                        const bool h2 = (r2.y < hi2) & (c1 != self);
-                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(wa), "h"((unsigned short)c1));
-                        wa += h2 ? 64u : 0u;
-                        m = fmaxf(m, h2 ? r2.y : 0.f);
-                    };
+                // branch-free, two candidates per step with FP32-pair
+                // arithmetic on t = r^2 - rl^2: every candidate's code is
+                // written to the next free slot (32-bit shared address), which
+                // advances only on a hit
+                float near = 1.0e30f;   // smallest |t| of the batch
+                uint32_t wa = (uint32_t)__cvta_generic_to_shared(row + 32 * cnt);
+                const float2 px = make_float2(-pi.x, -pi.x), py = make_float2(-pi.y, -pi.y),
+                             pz = make_float2(-pi.z, -pi.z), nrl = make_float2(-rl2, -rl2);
+                // four candidates per step: one 16-byte broadcast load per
+                // component and for the codes
+                auto step2 = [&](float2 qx, float2 qy, float2 qz, uint32_t c0, uint32_t c1) {
+                    const float2 dx = __fadd2_rn(qx, px), dy = __fadd2_rn(qy, py), dz = __fadd2_rn(qz, pz);
+                    const float2 t = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __ffma2_rn(dx, dx, nrl)));
+                    near = fminf(fminf(near, fabsf(t.x)), fabsf(t.y));
+                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(wa), "h"((unsigned short)c0));
+                    if ((t.x < band) & (c0 != self)) wa += 64u;
+                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(wa), "h"((unsigned short)c1));
+                    if ((t.y < band) & (c1 != self)) wa += 64u;
+                };
 #pragma unroll 2
-                    for (int u = 0; u < 32; u += 4) {
-                        const float4 qx = *reinterpret_cast<const float4*>(rx + h0 + u);
-                        const float4 qy = *reinterpret_cast<const float4*>(ry + h0 + u);
-                        const float4 qz = *reinterpret_cast<const float4*>(rz + h0 + u);
-                        const uint4 cc = *reinterpret_cast<const uint4*>(rc + h0 + u);
-                        step2(make_float2(qx.x, qx.y), make_float2(qy.x, qy.y), make_float2(qz.x, qz.y), cc.x, cc.y);
-                        step2(make_float2(qx.z, qx.w), make_float2(qy.z, qy.w), make_float2(qz.z, qz.w), cc.z, cc.w);
-                    }
-                    asm volatile("" ::: "memory");   // the stores above stay above
-                    __syncwarp();                      // and are seen by the reads below
-                    cnt = (int)((wa - (uint32_t)__cvta_generic_to_shared(row)) >> 6);
-                } else {
-                    for (int u = 0; u < nb; ++u) {
-                        const float4 q = make_float4(rx[h0 + u], ry[h0 + u], rz[h0 + u], 0.f);
-                        const float r2 = lane_r2(nxy, nz, q);
-                        const uint32_t code = rc[h0 + u];
-                        if (r2 < hi2 && code != self) {
-                            row[32 * cnt] = (uint16_t)code;
-                            ++cnt;
-                            m = fmaxf(m, r2);
-                        }
-                    }
+                for (int u = 0; u < 32; u += 4) {
+                    const float4 qx = *reinterpret_cast<const float4*>(rx + h0 + u);
+                    const float4 qy = *reinterpret_cast<const float4*>(ry + h0 + u);
+                    const float4 qz = *reinterpret_cast<const float4*>(rz + h0 + u);
+                    const uint4 cc = *reinterpret_cast<const uint4*>(rc + h0 + u);
+                    step2(make_float2(qx.x, qx.y), make_float2(qy.x, qy.y), make_float2(qz.x, qz.y), cc.x, cc.y);
+                    step2(make_float2(qx.z, qx.w), make_float2(qy.z, qy.w), make_float2(qz.z, qz.w), cc.z, cc.w);
                 }
+                asm volatile("" ::: "memory");   // the stores above stay above
+                __syncwarp();                      // and are seen by the reads below
+                cnt = (int)((wa - (uint32_t)__cvta_generic_to_shared(row)) >> 6);
                 // FP64 decision of the batch's accepted pairs near rl (rare)
-                if (__any_sync(0xffffffffu, m >= lo2) && m >= lo2) {
+                if (near <= band) {
                     int w = c0;
                     const int e = cnt;
                     for (int q = c0; q < e; ++q) {
                         const uint32_t code = row[32 * q];
                         const int k = (int)(code >> LJ_TILE_BITS);
-                        const int j = (int)(s_base[warp][k] & LJ_IDX_MASK) + (int)(code & LJ_TILE_MASK);
+                        const int j = (int)entry_slot(s_base[warp][k]) + (int)(code & LJ_TILE_MASK);
                         const float4 pj = posq[j];
                         const float4 sh = s_sh[warp][k];
                         const float4 qj = make_float4(pj.x + sh.x, pj.y + sh.y, pj.z + sh.z, 0.f);
-                        if (lane_r2(nxy, nz, qj) < lo2 || exact_within(b, R, i, j)) row[32 * w++] = (uint16_t)code;
+                        if (lane_t(pi, qj, rl2) < -band || exact_within(b, R, i, j)) row[32 * w++] = (uint16_t)code;
                     }
                     cnt = w;
                 }
@@ -1067,25 +1051,28 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
                 __syncwarp();
                 if (tail - head >= 32) {
                     if (__any_sync(0xffffffffu, cnt > kLaneRow - 32)) flush();
-                    batch(32);
+                    batch();
                 }
                 __syncwarp();
             }
-            if (tail > head) {
+            if (tail > head) {   // far points fill the last batch
+                const int rem = (int)(tail - head);
+                if (lane >= rem) rx[(head + lane) & (kRing - 1)] = 1.0e30f;
+                __syncwarp();
                 if (__any_sync(0xffffffffu, cnt > kLaneRow - 32)) flush();
-                batch((int)(tail - head));
+                batch();
             }
             __syncwarp();
             const int c = flushed + cnt;
             if (act) {
                 // the buffer's codes -> list entries, 4 at a time, up to the capacity
                 const int cst = min(cnt, K - flushed);
-                for (int e = 0; 4 * e < cst; ++e) {   // rows end inside a block: masked by the count
+                for (int e = 0; 4 * e < cst; ++e) {   // the row's last piece of four is filled with the sentinel
                     uint32_t o[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const uint32_t h = row[32 * (4 * e + u)];
-                        o[u] = base[h >> LJ_TILE_BITS] + (h & LJ_TILE_MASK);
+                        o[u] = 4 * e + u < cst ? base[h >> LJ_TILE_BITS] + ((h & LJ_TILE_MASK) << LJ_DIGIT_BITS) : sent;
                     }
                     dst[(flushed >> 2) + e] = make_uint4(o[0], o[1], o[2], o[3]);
                 }

@@ -260,12 +260,30 @@ Launch lcell(md_box* b) { return Launch{std::max(1, std::min((b->d.ncell + 7) / 
 // kernels leave one double-single share per warp and chunk (chunk kernel)
 // or brick (tiled kernel, LJ_BRICK_WARPS = LJ_FORCE_WARPS), the FP64 one an
 // FP64 share per warp and chunk, the all-pairs kernels one per chunk.
+// Small work items of the FP32 list force (16 particles instead of 128): up
+// to 512 chunks, where the chunks leave SMs idle or a block's two serial
+// passes set the time.  In-graph with energies, chunks / small items: N =
+// 4,000 16.0 / 9.0 us, 32,000 18.9 / 12.8, 64,000 ~20 / 18.6; at 100,000 both
+// 24.6, and at 1,000,000 148 / 166.
+bool spread_force(md_box* b) { return b->chunks.size() <= 512; }
+
+// doubles of one set of the per-chunk (E_pot, W) shares
+size_t share_doubles(md_box* b)
+{
+    return 2 * (size_t)(spread_force(b) ? LJ_SPREAD_SHARES : LJ_FORCE_WARPS) * std::max<size_t>(1, b->chunks.size());
+}
+
 void apply_force_kernel(md_box* b)
 {
     const bool list32 = !b->all_pairs && b->prec != MD_PREC_FP64;
     const bool tiles = list32 && b->force_kernel == MD_FORCE_TILES;
     b->d.force_tiles = tiles ? 1 : 0;
-    b->d.pf_stride = b->all_pairs ? 1 : b->prec == MD_PREC_FP64 ? LJ_F64_WARPS : LJ_FORCE_WARPS;
+    const bool spread = list32 && !tiles && spread_force(b);
+    b->d.force_spread = spread ? 1 : 0;
+    b->d.pf_stride = b->all_pairs                ? 1
+                     : b->prec == MD_PREC_FP64 ? LJ_F64_WARPS
+                     : spread                    ? LJ_SPREAD_SHARES
+                                                 : LJ_FORCE_WARPS;
     b->d.pf_ds = list32 ? 1 : 0;
 }
 
@@ -274,6 +292,10 @@ Launch lforce(md_box* b)
     if (b->d.force_tiles)   // persistent: the resident blocks, bricks handed out in a grid stride
         return Launch{std::max(1, std::min((int)b->d.nbrick, b->nsm * force_tile_blocks_per_sm(b->d.nt == 1))), 0,
                       b->stream};
+    if (b->d.force_spread) {
+        const int items = b->d.nchunk * (LJ_CHUNK * LJ_TPP / LJ_SPREAD_THREADS);
+        return Launch{std::max(1, std::min(items, b->nsm * 32)), 0, b->stream};
+    }
     int per_sm = b->force_per_sm > 0 ? b->force_per_sm : (b->prec == 2 ? 12 : 6);
     // the FP64 list kernel's items are quarters of a chunk
     const int items = b->d.nchunk * (b->all_pairs ? std::max(1, b->d.ap_js) : b->prec == MD_PREC_FP64 ? LJ_F64_WARPS : 1);
@@ -605,8 +627,8 @@ md_status make_grid(md_box* b)
     CK(b, cudaStreamSynchronize(b->stream));   // `bricks` may change before the copy would run
     d.brick = b->d_brick;
     d.nbrick = (int)b->bricks.size();
-    {   // (E_pot, W) shares: 8 per chunk or per brick
-        const size_t need = 2 * LJ_FORCE_WARPS * std::max<size_t>(1, std::max(b->chunks.size(), b->bricks.size()));
+    {   // (E_pot, W) shares: 8 per chunk or per brick, or those of the small work items
+        const size_t need = std::max(2 * LJ_FORCE_WARPS * std::max<size_t>(1, b->bricks.size()), share_doubles(b));
         if (need > b->pf_cap) {
             dev_release(b, d.part_f);
             d.part_f = nullptr;
@@ -1163,7 +1185,7 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
         CKS(dev_alloc(b, &d.part_k, 2 * LJ_KIN_WARPS * std::max<size_t>(1, b->chunks.size())));   // two sets
         // (E_pot, W) shares, 8 per chunk (chunk kernel) or brick (tiled
         // kernel; make_grid grows the array with the bricks)
-        b->pf_cap = 2 * LJ_FORCE_WARPS * std::max<size_t>(1, b->chunks.size());
+        b->pf_cap = share_doubles(b);
         CKS(dev_alloc(b, &d.part_f, 2 * b->pf_cap));
         apply_force_kernel(b);
         CKS(dev_alloc(b, &b->d_type_user, std::max<int64_t>(1, ntot)));
@@ -1316,6 +1338,11 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
     b->d.c1 = make_float4(h.c12[0], h.c6[0], h.e12[0], h.e6[0]);
     b->d.rc2_1 = h.rc2[0];
     b->d.esh_1 = h.shift[0];
+    {
+        const double s2 = sigma[0] * sigma[0], s6 = s2 * s2 * s2;
+        b->d.nh_1 = (float)(-0.5 / s6);
+        b->d.kap_1 = (float)(h.dshift[0] / (2.0 * eps[0] * s6));
+    }
     b->skin = skin;
     b->rl = rl;
     BoxDev& d = b->d;
@@ -2139,7 +2166,9 @@ extern "C" md_status md_force_noalloc(md_box* b, double* force_out, double* epot
     if (!b) return MD_ERR_ARG;
     // the chunk kernels always (their shares are per warp, not per particle)
     BoxDev v = b->d;
-    v.force_tiles = 0;   // same share layout per chunk as the FP32 list kernels
+    // same share layout per chunk as the FP32 list kernels (small boxes' 16
+    // shares per chunk instead of 8 stay far inside the scratch)
+    v.force_tiles = 0;
     const size_t nchunk = b->chunks.size();
     const size_t nshare = 2 * (size_t)v.pf_stride * nchunk;   // (E_pot, W) shares
     const size_t need = nshare + 4 * (size_t)b->nrep;

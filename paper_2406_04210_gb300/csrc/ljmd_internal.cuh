@@ -15,11 +15,12 @@
 //     contiguous slot range, and the 27-cell neighbourhood of all its cells
 //     is the "tile": 9 rows x (S + 2) cells, i.e. at most 18 contiguous slot
 //     ranges ("pieces"), staged in shared memory.
-//   * Verlet lists (Sec. 3) are 32-bit entries: the image shift of j's cell
-//     relative to i's cell as three 2-bit digits (dz+1, dy+1, dx+1 in bits
-//     31-30, 29-28, 27-26) and the slot j in bits 25-0, so
+//   * Verlet lists (Sec. 3) are 32-bit entries: the slot j in bits 31-6 and the
+//     image shift of j's cell relative to i's cell as three 2-bit digits
+//     (dz+1, dy+1, dx+1 in bits 5-4, 3-2, 1-0), so
 //     d_ij = (o_i - o_j) - (dx, dy, dz) * cell edge, decoded with integer and
-//     FP32 arithmetic (no table).  The stencil code k = 9(dz+1) + 3(dy+1) +
+//     FP32 arithmetic (no table): low digits fall inside an FP32 mantissa by
+//     one and-or each, where digits above the slot took a shift more.  The stencil code k = 9(dz+1) + 3(dy+1) +
 //     (dx+1) orders the 27 cells.
 //     Entry s of particle p is nbr[p K + s] (K a multiple of 16): the FP32
 //     force kernel reads a row in blocks of 16 entries, one 16-byte load per
@@ -36,7 +37,7 @@
 
 #define LJ_MAXT 8
 #define LJ_IDX_BITS 26         // slot indices must stay below 2^26
-#define LJ_IDX_MASK ((1u << LJ_IDX_BITS) - 1u)
+#define LJ_DIGIT_BITS 6        // an entry's image-shift digits, below the slot
 #define LJ_TILE_BITS 11
 #define LJ_TILE_MAX (1 << LJ_TILE_BITS)
 #define LJ_TILE_MASK (LJ_TILE_MAX - 1)
@@ -44,6 +45,8 @@
 #define LJ_FORCE_THREADS 256   // threads of the FP32 pair-force kernel
 #define LJ_FORCE_WARPS (LJ_FORCE_THREADS / 32)   // its (E_pot, W) shares per chunk
 #define LJ_KIN_WARPS (LJ_CHUNK / 32)   // E_kin shares per chunk (one per warp of the integrator)
+#define LJ_SPREAD_THREADS 64   // threads of its small work items (16 particles)
+#define LJ_SPREAD_SHARES (LJ_CHUNK * 4 / 32)   // their (E_pot, W) shares per chunk: one per warp
 #define LJ_THERMO_THREADS 256  // threads of the energy reduction
 #define LJ_THERMO_CHUNKS 256   // chunks of one energy-reduction item
 #define LJ_LIST_THREADS 256    // threads of the list-build kernel
@@ -135,6 +138,7 @@ struct BoxDev {
     // kernel from the kernel parameters (no registers held for them)
     float4 c1;                 // c12, c6, e12, e6
     float rc2_1, esh_1;
+    float nh_1, kap_1;         // -c6 / c12, shift / (e6 / 2)
     float3 ell1;               // one replica (nrep == 1): its cell edge, FP32
     double rl2;
     const RepDev* rep;
@@ -196,6 +200,7 @@ struct BoxDev {
     long long* step_ctr;       // steps since md_set_thermostat (device word)
     int all_pairs;             // every cutoff infinite: forces over all pairs, no lists
     int force_tiles;           // FP32 list forces by the tiled kernel (k_force_tile_f32)
+    int force_spread;          // FP32 list forces by k_force_f32's small work items
     const int4* brick;         // its work items: (replica, first cell x, y, z) of bricks of up to
     int nbrick;                // rep.br[0] x br[1] x br[2] cells
     int order;                 // order inside a cell: 0 z runs (LJ_ORDER_ZRUN), 1 Morton sub-cells
@@ -306,18 +311,29 @@ __device__ __forceinline__ float rcp_approx(float x)
 // ---- list entries ----
 __host__ __device__ __forceinline__ uint32_t entry_make(int k, int j)
 {
-    return ((uint32_t)(k / 9) << 30) | ((uint32_t)((k / 3) % 3) << 28) | ((uint32_t)(k % 3) << 26) |
-           (uint32_t)j;
+    return ((uint32_t)j << LJ_DIGIT_BITS) | ((uint32_t)(k / 9) << 4) | ((uint32_t)((k / 3) % 3) << 2) |
+           (uint32_t)(k % 3);
 }
+__device__ __forceinline__ uint32_t entry_slot(uint32_t e) { return e >> LJ_DIGIT_BITS; }
 __device__ __forceinline__ int entry_k(uint32_t e)
 {
-    return 9 * (int)(e >> 30) + 3 * (int)((e >> 28) & 3u) + (int)((e >> 26) & 3u);
+    return 9 * (int)((e >> 4) & 3u) + 3 * (int)((e >> 2) & 3u) + (int)(e & 3u);
 }
-// The digit at bit `pos` minus one, as an exact FP32 value in {-1, 0, 1}:
-// 0x4B400000 is 1.5 * 2^23, whose mantissa's low bits take the digit.
-__device__ __forceinline__ float entry_unit(uint32_t e, int pos)
+// The digit of axis A as an FP32 number: 1.5 * 2^23 + 4^A * digit, exactly
+// (0x4B400000 is 1.5 * 2^23, whose mantissa's low bits take the digit where
+// it stands).  digit_one(A) is its value for digit 1 (no shift).
+template <int A>
+__device__ __forceinline__ float entry_raw(uint32_t e)
 {
-    return __uint_as_float(0x4B400000u | ((e >> pos) & 3u)) - 12582913.0f;
+    return __uint_as_float(0x4B400000u | (e & (3u << (2 * A))));
+}
+__host__ __device__ constexpr float digit_one(int A) { return 12582912.0f + (float)(1 << (2 * A)); }
+// The digit minus one, in units of 4^-A: multiply by the cell edge over 4^A
+// (exact scalings).
+template <int A>
+__device__ __forceinline__ float entry_unit(uint32_t e)
+{
+    return entry_raw<A>(e) - digit_one(A);
 }
 
 // ---- Philox4x32-10 (Salmon et al., SC'11), counter-based random numbers ----
