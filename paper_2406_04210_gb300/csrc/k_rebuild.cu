@@ -827,31 +827,38 @@ __global__ void __launch_bounds__(LJ_LIST_THREADS, 3) k_nlist(BoxDev b)
 }
 
 // ---------------------------------------------------------------------------
-// k_nlist_lanes: the same lists, one warp per cell and one lane per particle
-// of the cell.  The warp streams the candidates of the 27 neighbour cells
-// in chunks of 32: lane t loads candidate t of the chunk (coalesced, the
-// next chunk's load in flight while this one is used), adds the cell's
-// shift and drops it when its distance from the bounding box of the cell's
-// particles is beyond the list radius (at least a quarter of the 27-cell
-// block lies there); the kept
-// candidates (shifted FP32 offset and a 16-bit code: neighbour cell k and
-// index inside it) go to a per-warp ring in shared memory.  Every 32 staged
-// candidates, each lane tests them all against its own particle -- one
-// broadcast shared-memory load per candidate for the whole cell -- and
-// appends the codes of its hits to its own row in shared memory (no
-// ballots: every lane owns its row); at the end it writes the row out as
-// list entries with 16-byte stores.  Pairs within `band` of rl^2 are
-// re-decided in FP64 as in k_nlist (checked per batch of 32: the largest
-// accepted r^2 tells whether any accepted pair lies in the band).  The x and
-// y parts of d_ij and d_ij^2 are computed as FP32 pairs.
+// k_nlist_lanes: the same lists, one warp per pass of 32 / G particles of a
+// cell, G lanes per particle.  The warp streams the candidates of the 27
+// neighbour cells in chunks of 32: lane t loads candidate t of the chunk
+// (coalesced, the next chunk's load in flight while this one is used), adds
+// the cell's shift and drops it when its distance from the bounding box of
+// the pass's particles is beyond the list radius (at least a quarter of the
+// 27-cell block lies there); the kept candidates (shifted FP32 offset and
+// list entry) go to a per-warp ring in shared memory.  Every 32 staged
+// candidates, each lane tests its 32 / G of them against its particle -- one
+// broadcast shared-memory load per candidate and component -- and appends the
+// entries of its hits to its own row buffer in shared memory (no ballots:
+// every lane owns its buffer), from which whole pieces of four entries go out
+// with 16-byte stores.  Pairs within `band` of rl^2 are re-decided in FP64 as
+// in k_nlist (checked per batch: the smallest |r^2 - rl^2| tells whether any
+// pair lies in the band).  d_ij and r^2 are computed as FP32 pairs.
+// G = 1 where the cells fill the GPU (launch_list's rule); what bounds it
+// then: issue (74 % of peak) and the shared-memory pipe (65 %), ~310
+// instructions a warp and 64 wavefronts of loads and stores per batch of 32
+// candidates, which is why the buffers hold whole entries (a step's store is
+// one wavefront; 16-bit codes took two, and a base table on the way out).
+// G = 4 for small boxes: a cell's warp ran alone on its scheduler, ~10 cycles
+// per instruction; four warps take a cell's particles, each with a tighter
+// bounding box and a quarter of the tests per lane.
+// Forced update (binning, sort, lists, force) at N = 4,000 176 -> 134 us, at 4M
+// 3694 -> 3470 us (cell scale 1.15: 3215 -> 3016).
 // ---------------------------------------------------------------------------
 constexpr int kLaneWarps = LJ_LANE_THREADS / 32;
 constexpr int kRing = 64;   // staged candidates per warp: < 32 waiting + one chunk
-// Codes a lane holds in shared memory: fewer than 16 not yet written out plus
-// one batch of 32.  Full 16-code blocks go out to the list before a batch
-// that could overflow the buffer, so the rows' shared memory does not grow
-// with the capacity K.
-constexpr int kLaneRow = 48;
+// Entries a lane holds in shared memory: fewer than 4 not yet written out, and
+// a batch's 32 / G on top (flushed when less room is left), so the rows'
+// shared memory does not grow with the capacity K.
+constexpr int kLaneRow = 40;
 
 // r^2 - rl^2 of the pair (i, candidate q = o_j + shift), rounded as in the
 // batches.
@@ -861,46 +868,49 @@ __device__ __forceinline__ float lane_t(const float4& pi, const float4& q, float
     return __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmaf_rn(dx, dx, -rl2)));
 }
 
-__device__ __forceinline__ void phase_lanes(const BoxDev& b)
+template <int G>
+__global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
 {
-    // row buffers, slot-major per warp: code e of lane l at [e][l] (the 32
+    if (!box_needs_rebuild(b)) return;
+    constexpr int P = 32 / G;    // particles of a pass
+    constexpr int T = 32 / G;    // candidates of a batch that a lane tests
+    // row buffers, slot-major per warp: entry e of lane l at [e][l] (the 32
     // lanes' stores of one step fall in distinct banks whatever their counts)
-    extern __shared__ __align__(16) uint16_t s_rows[];   // per warp: kLaneRow x 32 codes
+    extern __shared__ __align__(16) uint32_t s_rows[];   // per warp: kLaneRow x 32 entries
     __shared__ __align__(16) float s_cx[kLaneWarps][kRing];   // staged candidates: o_j + shift(k),
     __shared__ __align__(16) float s_cy[kLaneWarps][kRing];   // one array per component (four
     __shared__ __align__(16) float s_cz[kLaneWarps][kRing];   // candidates load as one 16-byte word)
-    __shared__ __align__(16) uint32_t s_cc[kLaneWarps][kRing];   // and their codes
+    __shared__ __align__(16) uint32_t s_ce[kLaneWarps][kRing];   // and their list entries
     __shared__ int2 s_rng[kLaneWarps][27];                // neighbour cell k: (first slot, end slot)
-    __shared__ float4 s_sh[kLaneWarps][27];               // shift(k) = (dx, dy, dz) * cell edge
-    __shared__ uint32_t s_base[kLaneWarps][32];           // entry of the first slot of cell k (27 used;
-                                                          // stale codes past a row's end index up to 31)
+    __shared__ float4 s_sh[kLaneWarps][27];               // shift(k) = (dx, dy, dz) * cell edge; k's digits
     __shared__ int s_longest;
     if (threadIdx.x == 0) s_longest = 0;
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int pl = lane % P, sub = lane / P;   // the lane's particle of the pass, its share of the candidates
     const unsigned lt = (1u << lane) - 1u;
     const int K = b.K;
-    uint16_t* const row = s_rows + (size_t)warp * kLaneRow * 32 + lane;   // slot e at row[32 e]
+    uint32_t* const row = s_rows + (size_t)warp * kLaneRow * 32 + lane;   // entry e at row[32 e]
     float* const rx = s_cx[warp];
     float* const ry = s_cy[warp];
     float* const rz = s_cz[warp];
-    uint32_t* const rc = s_cc[warp];
+    uint32_t* const re = s_ce[warp];
     const float rl2 = b.rl2f, band = b.band;
     const float rcull = rl2 + band + 1e-3f;   // staging margin for the rounding of the shifted offsets
     const float4* __restrict__ posq = b.posq;
-    const uint32_t sent = entry_make(13, b.np);
     int longest = 0;
     const int nwarp = gridDim.x * kLaneWarps;
-    const int total = b.lw_off[b.lw_hdr[0]];
+    const int total = b.lw_off[b.lw_hdr[0]] * G;
     int kr = 0;
     for (int t = blockIdx.x * kLaneWarps + warp; t < total; t += nwarp) {
-        const int gc = work_cell(b, t, kr);
+        const int gc = work_cell(b, t / G, kr);
         const int r = b.lw_rep[kr];
         const RepDev& R = b.rep[r];
+        const int cs = b.cell_start[gc], n = b.cell_end[gc] - cs;
+        if (lane == 0 && t % G == 0 && gc == R.cell_off) atomicAdd(&b.nbuild[r], 1ull);
+        if (P * (t % G) >= n) continue;   // warp-uniform
         int cx, cy;
         const int cz = cell_coords(R, gc, cx, cy);
-        const int cs = b.cell_start[gc], n = b.cell_end[gc] - cs;
-        if (lane == 0 && gc == R.cell_off) atomicAdd(&b.nbuild[r], 1ull);
         __syncwarp();
         if (lane < 27) {
             const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
@@ -908,21 +918,21 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
                            R.nc[0] * (wrapi(cy + dy, R.nc[1]) + R.nc[1] * wrapi(cz + dz, R.nc[2]));
             const int js = b.cell_start[cn], je = b.cell_end[cn];
             s_rng[warp][lane] = make_int2(js, je);
-            s_sh[warp][lane] = make_float4((float)dx * R.ellf[0], (float)dy * R.ellf[1], (float)dz * R.ellf[2], 0.f);
-            s_base[warp][lane] = entry_make(lane, js);
-            if (je - js > LJ_TILE_MAX) atomicOr(&b.err[0], LJ_ERRBIT_TILE);   // the 11-bit index: never at LJ densities
+            s_sh[warp][lane] = make_float4((float)dx * R.ellf[0], (float)dy * R.ellf[1], (float)dz * R.ellf[2],
+                                           __uint_as_float(entry_make(lane, 0)));
+            if (je - js > LJ_TILE_MAX) atomicOr(&b.err[0], LJ_ERRBIT_TILE);   // refused: never at LJ densities
         }
         __syncwarp();
-        for (int ib = 0; ib < n; ib += 32) {
-            const bool act = ib + lane < n;
-            const int i = cs + (act ? ib + lane : 0);
+        for (int ib = P * (t % G); ib < n; ib += P * G) {
+            const bool act = ib + pl < n;
+            const int i = cs + (act ? ib + pl : 0);
             float4 pi = posq[i];
             // the box of this pass's particles (tighter than the cell: the
             // candidates to test are those within the list radius of it)
             float lx = act ? pi.x : 1.0e30f, ly = act ? pi.y : 1.0e30f, lz = act ? pi.z : 1.0e30f;
             float ux = act ? pi.x : -1.0e30f, uy = act ? pi.y : -1.0e30f, uz = act ? pi.z : -1.0e30f;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
+            for (int o = P / 2; o > 0; o >>= 1) {
                 lx = fminf(lx, __shfl_xor_sync(0xffffffffu, lx, o));
                 ly = fminf(ly, __shfl_xor_sync(0xffffffffu, ly, o));
                 lz = fminf(lz, __shfl_xor_sync(0xffffffffu, lz, o));
@@ -931,44 +941,51 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
                 uz = fmaxf(uz, __shfl_xor_sync(0xffffffffu, uz, o));
             }
             if (!act) pi = make_float4(1.0e30f, 1.0e30f, 1.0e30f, 0.f);   // a far point: r^2 is inf
-            const uint32_t self = (13u << LJ_TILE_BITS) | (uint32_t)(ib + lane);   // the particle itself
-            int cnt = 0;                   // codes in the row buffer
-            int flushed = 0;               // list entries already written out (a multiple of 16)
+            const uint32_t self = entry_make(13, i);   // the particle itself
+            int cnt = 0;                   // entries in the row buffer
+            int flushed = 0;               // the particle's entries already written out (a multiple of 4)
             unsigned head = 0, tail = 0;   // ring positions (free-running; head stays a multiple of 32)
             uint4* const dst = reinterpret_cast<uint4*>(b.nbr + (size_t)K * i);   // the particle's row
-            const uint32_t* const base = s_base[warp];
-            // full 16-code blocks out to the list (the entry of cell k's first
-            // slot + index), the rest to the buffer's front; entries past the
-            // capacity are counted, not written
-            auto flush = [&]() {
-                const int nbk = act ? (cnt >> 4) : 0;
-                for (int q = 0; q < nbk; ++q) {
-                    if (flushed + 16 * (q + 1) <= K) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            uint32_t o[4];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                const uint32_t h = row[32 * (16 * q + 4 * e + u)];
-                                o[u] = base[h >> LJ_TILE_BITS] + ((h & LJ_TILE_MASK) << LJ_DIGIT_BITS);
-                            }
-                            dst[(flushed >> 2) + 4 * q + e] = make_uint4(o[0], o[1], o[2], o[3]);
-                        }
-                    }
+            // x summed over the lanes of the particle before this one; all gets the sum over all of them
+            auto lanes_before = [&](int x, int& all) {
+                if (G == 1) {
+                    all = x;
+                    return 0;
                 }
-                const int rest = cnt - 16 * nbk;
-                for (int q = 0; q < rest; ++q) row[32 * q] = row[32 * (16 * nbk + q)];
-                flushed += 16 * nbk;
+                int incl = x;
+#pragma unroll
+                for (int o = P; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                all = __shfl_sync(0xffffffffu, incl, 32 - P + pl);
+                return incl - x;
+            };
+            // whole pieces of four entries out to the list, the rest to the
+            // buffer's front; entries past the capacity are counted, not
+            // written
+            auto flush = [&]() {
+                const int nq = act ? (cnt >> 2) : 0;
+                int all;
+                const int at = (flushed >> 2) + lanes_before(nq, all);
+                for (int q = 0; q < nq; ++q) {
+                    const uint4 o = make_uint4(row[32 * (4 * q)], row[32 * (4 * q + 1)], row[32 * (4 * q + 2)],
+                                               row[32 * (4 * q + 3)]);
+                    if (4 * (at + q + 1) <= K) dst[at + q] = o;
+                }
+                const int rest = cnt & 3;
+                for (int q = 0; q < rest; ++q) row[32 * q] = row[32 * (cnt - rest + q)];
+                flushed += 4 * all;
                 cnt = rest;
-                __syncwarp();
             };
             // test the 32 staged candidates from head on against the lane's
-            // particle and append the hits (the buffer has room: flushed before)
+            // particle and append the hits
             auto batch = [&]() {
+                if (__any_sync(0xffffffffu, cnt > kLaneRow - T)) flush();
                 const int c0 = cnt;
-                const int h0 = (int)(head & (kRing - 1));
+                const int h0 = (int)(head & (kRing - 1)) + T * sub;
                 // branch-free, two candidates per step with FP32-pair
-                // arithmetic on t = r^2 - rl^2: every candidate's code is
+                // arithmetic on t = r^2 - rl^2: every candidate's entry is
                 // written to the next free slot (32-bit shared address), which
                 // advances only on a hit
                 float near = 1.0e30f;   // smallest |t| of the batch
@@ -976,40 +993,39 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
                 const float2 px = make_float2(-pi.x, -pi.x), py = make_float2(-pi.y, -pi.y),
                              pz = make_float2(-pi.z, -pi.z), nrl = make_float2(-rl2, -rl2);
                 // four candidates per step: one 16-byte broadcast load per
-                // component and for the codes
-                auto step2 = [&](float2 qx, float2 qy, float2 qz, uint32_t c0, uint32_t c1) {
+                // component and for the entries
+                auto step2 = [&](float2 qx, float2 qy, float2 qz, uint32_t e0, uint32_t e1) {
                     const float2 dx = __fadd2_rn(qx, px), dy = __fadd2_rn(qy, py), dz = __fadd2_rn(qz, pz);
-                    const float2 t = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __ffma2_rn(dx, dx, nrl)));
-                    near = fminf(fminf(near, fabsf(t.x)), fabsf(t.y));
-                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(wa), "h"((unsigned short)c0));
-                    if ((t.x < band) & (c0 != self)) wa += 64u;
-                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(wa), "h"((unsigned short)c1));
-                    if ((t.y < band) & (c1 != self)) wa += 64u;
+                    const float2 t2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __ffma2_rn(dx, dx, nrl)));
+                    near = fminf(fminf(near, fabsf(t2.x)), fabsf(t2.y));
+                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(wa), "r"(e0));
+                    if ((t2.x < band) & (e0 != self)) wa += 128u;
+                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(wa), "r"(e1));
+                    if ((t2.y < band) & (e1 != self)) wa += 128u;
                 };
 #pragma unroll 2
-                for (int u = 0; u < 32; u += 4) {
+                for (int u = 0; u < T; u += 4) {
                     const float4 qx = *reinterpret_cast<const float4*>(rx + h0 + u);
                     const float4 qy = *reinterpret_cast<const float4*>(ry + h0 + u);
                     const float4 qz = *reinterpret_cast<const float4*>(rz + h0 + u);
-                    const uint4 cc = *reinterpret_cast<const uint4*>(rc + h0 + u);
-                    step2(make_float2(qx.x, qx.y), make_float2(qy.x, qy.y), make_float2(qz.x, qz.y), cc.x, cc.y);
-                    step2(make_float2(qx.z, qx.w), make_float2(qy.z, qy.w), make_float2(qz.z, qz.w), cc.z, cc.w);
+                    const uint4 qe = *reinterpret_cast<const uint4*>(re + h0 + u);
+                    step2(make_float2(qx.x, qx.y), make_float2(qy.x, qy.y), make_float2(qz.x, qz.y), qe.x, qe.y);
+                    step2(make_float2(qx.z, qx.w), make_float2(qy.z, qy.w), make_float2(qz.z, qz.w), qe.z, qe.w);
                 }
                 asm volatile("" ::: "memory");   // the stores above stay above
-                __syncwarp();                      // and are seen by the reads below
-                cnt = (int)((wa - (uint32_t)__cvta_generic_to_shared(row)) >> 6);
+                __syncwarp();
+                cnt = (int)((wa - (uint32_t)__cvta_generic_to_shared(row)) >> 7);
                 // FP64 decision of the batch's accepted pairs near rl (rare)
                 if (near <= band) {
                     int w = c0;
                     const int e = cnt;
                     for (int q = c0; q < e; ++q) {
-                        const uint32_t code = row[32 * q];
-                        const int k = (int)(code >> LJ_TILE_BITS);
-                        const int j = (int)entry_slot(s_base[warp][k]) + (int)(code & LJ_TILE_MASK);
+                        const uint32_t ent = row[32 * q];
+                        const int j = (int)entry_slot(ent);
                         const float4 pj = posq[j];
-                        const float4 sh = s_sh[warp][k];
+                        const float4 sh = s_sh[warp][entry_k(ent)];
                         const float4 qj = make_float4(pj.x + sh.x, pj.y + sh.y, pj.z + sh.z, 0.f);
-                        if (lane_t(pi, qj, rl2) < -band || exact_within(b, R, i, j)) row[32 * w++] = (uint16_t)code;
+                        if (lane_t(pi, qj, rl2) < -band || exact_within(b, R, i, j)) row[32 * w++] = ent;
                     }
                     cnt = w;
                 }
@@ -1024,8 +1040,9 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
             float4 raw = make_float4(0.f, 0.f, 0.f, 0.f);
             if (k < 27 && j0 + lane < s_rng[warp][k].y) raw = posq[j0 + lane];
             while (k < 27) {
-                const int kc = k, len = min(32, s_rng[warp][k].y - j0);
-                const int ic = j0 - s_rng[warp][k].x + lane;   // index of this lane's candidate in cell kc
+                const int len = min(32, s_rng[warp][k].y - j0);
+                const float4 sh = s_sh[warp][k];
+                const uint32_t ent = ((uint32_t)(j0 + lane) << LJ_DIGIT_BITS) | __float_as_uint(sh.w);
                 const float4 cur = raw;
                 j0 += 32;
                 while (k < 27 && j0 >= s_rng[warp][k].y) {
@@ -1034,48 +1051,46 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
                 }
                 if (k < 27 && j0 + lane < s_rng[warp][k].y) raw = posq[j0 + lane];   // next chunk, in flight
                 // stage: shift into the cell's frame, keep what can be within reach of the cell
-                const float4 sh = s_sh[warp][kc];
                 const float qx = cur.x + sh.x, qy = cur.y + sh.y, qz = cur.z + sh.z;
                 const float gx = fmaxf(fmaxf(lx - qx, qx - ux), 0.f), gy = fmaxf(fmaxf(ly - qy, qy - uy), 0.f),
                             gz = fmaxf(fmaxf(lz - qz, qz - uz), 0.f);
                 const bool keep = lane < len && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < rcull;
                 const unsigned bal = __ballot_sync(0xffffffffu, keep);
                 if (keep) {
-                    const int t = (int)((tail + __popc(bal & lt)) & (kRing - 1));
-                    rx[t] = qx;
-                    ry[t] = qy;
-                    rz[t] = qz;
-                    rc[t] = ((uint32_t)kc << LJ_TILE_BITS) | (uint32_t)ic;
+                    const int q = (int)((tail + __popc(bal & lt)) & (kRing - 1));
+                    rx[q] = qx;
+                    ry[q] = qy;
+                    rz[q] = qz;
+                    re[q] = ent;
                 }
                 tail += __popc(bal);
                 __syncwarp();
-                if (tail - head >= 32) {
-                    if (__any_sync(0xffffffffu, cnt > kLaneRow - 32)) flush();
-                    batch();
-                }
+                if (tail - head >= 32) batch();
                 __syncwarp();
             }
             if (tail > head) {   // far points fill the last batch
-                const int rem = (int)(tail - head);
-                if (lane >= rem) rx[(head + lane) & (kRing - 1)] = 1.0e30f;
+                if (lane >= (int)(tail - head)) rx[(head + lane) & (kRing - 1)] = 1.0e30f;
                 __syncwarp();
-                if (__any_sync(0xffffffffu, cnt > kLaneRow - 32)) flush();
                 batch();
             }
-            __syncwarp();
-            const int c = flushed + cnt;
-            if (act) {
-                // the buffer's codes -> list entries, 4 at a time, up to the capacity
-                const int cst = min(cnt, K - flushed);
-                for (int e = 0; 4 * e < cst; ++e) {   // the row's last piece of four is filled with the sentinel
-                    uint32_t o[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const uint32_t h = row[32 * (4 * e + u)];
-                        o[u] = 4 * e + u < cst ? base[h >> LJ_TILE_BITS] + ((h & LJ_TILE_MASK) << LJ_DIGIT_BITS) : sent;
-                    }
-                    dst[(flushed >> 2) + e] = make_uint4(o[0], o[1], o[2], o[3]);
-                }
+            // what the buffers still hold, up to the capacity
+            int c;
+            if (G == 1) {
+                c = flushed + cnt;
+                if (act)   // the last piece may hold stale entries past the count
+                    for (int q = 0; 4 * q < cnt && flushed + 4 * q < K; ++q)
+                        dst[(flushed >> 2) + q] = make_uint4(row[32 * (4 * q)], row[32 * (4 * q + 1)],
+                                                             row[32 * (4 * q + 2)], row[32 * (4 * q + 3)]);
+            } else {
+                flush();
+                int all;
+                const int at = flushed + lanes_before(act ? cnt : 0, all);
+                if (act)
+                    for (int q = 0; q < cnt; ++q)
+                        if (at + q < K) reinterpret_cast<uint32_t*>(dst)[at + q] = row[32 * q];
+                c = flushed + all;
+            }
+            if (act && sub == 0) {
                 b.nbr_count[i] = c;
                 if (c > K) {
                     atomicOr(&b.err[0], LJ_ERRBIT_CAPACITY);
@@ -1090,11 +1105,6 @@ __device__ __forceinline__ void phase_lanes(const BoxDev& b)
     if (lane == 0 && longest > 0) atomicMax(&s_longest, longest);
     __syncthreads();
     if (threadIdx.x == 0 && s_longest > 0) atomicMax(&b.err[2], s_longest);
-}
-
-__global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
-{
-    if (box_needs_rebuild(b)) phase_lanes(b);
 }
 
 // ---------------------------------------------------------------------------
@@ -1183,26 +1193,17 @@ cudaError_t launch_nlist(const BoxDev& b, Launch l)
     return cudaGetLastError();
 }
 
-// Shared memory of k_nlist_lanes (any capacity K): kLaneRow 16-bit code
-// slots per lane.
-size_t nlist_lanes_smem(int) { return (size_t)LJ_LANE_THREADS * (size_t)kLaneRow * 2u; }
-
 cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s)
 {
     k_list_work<<<1, 1024, 0, s>>>(b, runs);
     return cudaGetLastError();
 }
 
-cudaError_t launch_nlist_lanes(const BoxDev& b, Launch l)
+cudaError_t launch_nlist_lanes(const BoxDev& b, int per_particle, Launch l)
 {
-    static size_t attr = 0;
-    const size_t dyn = nlist_lanes_smem(b.K);
-    if (dyn > attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_nlist_lanes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        if (e != cudaSuccess) return e;
-        attr = dyn;
-    }
-    k_nlist_lanes<<<l.grid, LJ_LANE_THREADS, dyn, l.s>>>(b);
+    const size_t dyn = (size_t)LJ_LANE_THREADS * kLaneRow * sizeof(uint32_t);   // the row buffers: below 48 KB
+    if (per_particle == 4) k_nlist_lanes<4><<<l.grid, LJ_LANE_THREADS, dyn, l.s>>>(b);
+    else k_nlist_lanes<1><<<l.grid, LJ_LANE_THREADS, dyn, l.s>>>(b);
     return cudaGetLastError();
 }
 

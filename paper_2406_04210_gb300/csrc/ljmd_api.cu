@@ -317,10 +317,15 @@ bool lanes_list(md_box* b)
 cudaError_t launch_list(md_box* b, cudaStream_t s)
 {
     if (lanes_list(b)) {
-        const int per_sm = b->list_per_sm > 0 ? b->list_per_sm : 8;   // resident blocks (64 registers, 19.5 KB)
+        const int per_sm = b->list_per_sm > 0 ? b->list_per_sm : 8;   // resident blocks (64 registers, 27 KB)
         const int warps = LJ_LANE_THREADS / 32;
+        // four lanes per particle where a warp per cell leaves schedulers
+        // idle: forced update (with host overhead) at N = 4,000 160 -> 134 us,
+        // 32,000 (1,728 cells) 186 -> 178, 64,000 (4,096 cells) 175 -> 188
+        const int g = b->d.ncell <= 2048 ? 4 : 1;
         return launch_nlist_lanes(
-            b->d, Launch{std::max(1, std::min((b->d.ncell + warps - 1) / warps, b->nsm * per_sm)), LJ_LANE_THREADS, s});
+            b->d, g,
+            Launch{std::max(1, std::min((b->d.ncell * g + warps - 1) / warps, b->nsm * per_sm)), LJ_LANE_THREADS, s});
     }
     Launch l = llist(b);
     l.s = s;

@@ -534,16 +534,14 @@ int ljmd_scan_tile_cells();
 cudaError_t launch_scatter(const BoxDev& b, Launch l);
 cudaError_t launch_sortgather(const BoxDev& b, Launch l, Launch lg);   // rank (l), then gather (lg) unless all pairs
 cudaError_t launch_nlist(const BoxDev& b, Launch l);
-// one warp per cell, one lane per particle (rows staged in shared memory:
-// nlist_lanes_smem(K) bytes per block)
-cudaError_t launch_nlist_lanes(const BoxDev& b, Launch l);
+// one warp per cell (per_particle 1) or per quarter of its particles (4 lanes per particle)
+cudaError_t launch_nlist_lanes(const BoxDev& b, int per_particle, Launch l);
 // one block; before the cell kernels; counts its executions with work in *runs (nullable)
 cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s);
 // binning, sort and gather in one launch of one cluster (small boxes)
 cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles, int* tile_sum,
                                    cudaStream_t s);
 bool cluster_rebuild_fits();
-size_t nlist_lanes_smem(int K);
 // k_force.cu
 cudaError_t launch_force(const BoxDev& b, int energy, Launch l);
 cudaError_t launch_thermo(const BoxDev& b, double* out, int with_kin, Launch l);
