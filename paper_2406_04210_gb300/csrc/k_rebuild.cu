@@ -58,21 +58,6 @@ __device__ __forceinline__ int group_first() { return blockIdx.x * (blockDim.x /
 __device__ __forceinline__ int group_count() { return gridDim.x * (blockDim.x / LJ_CHUNK); }
 __device__ __forceinline__ int group_thread() { return threadIdx.x % LJ_CHUNK; }
 
-// 8-byte component c of particle p of an integrator array in the layout of
-// the box precision (FP64: one double; DS: hi/lo floats in two planes).
-__device__ __forceinline__ void copy_acc(const BoxDev& b, double* dst, const double* src, int c,
-                                         int q, int p)
-{
-    if (b.prec == 0) {
-        const float* s = reinterpret_cast<const float*>(src);
-        float* d = reinterpret_cast<float*>(dst);
-        d[c * b.np + q] = s[c * b.np + p];
-        d[3 * b.np + c * b.np + q] = s[3 * b.np + c * b.np + p];
-    } else {
-        dst[c * b.np + q] = src[c * b.np + p];
-    }
-}
-
 // ---------------------------------------------------------------------------
 // k_bin: new cell of every particle of a rebuilding replica, its offset from
 // the new cell's centre (offB, the state's layout), its wrapped FP64 position
@@ -87,13 +72,11 @@ __device__ __forceinline__ void copy_acc(const BoxDev& b, double* dst, const dou
 // x outside [0, L) at FP64 rounding, takes the FP64 path of a build from
 // positions: wrap x into [0, L), cell = floor(x / edge), offset = x - centre.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void bin_from_x(const BoxDev& b, const RepDev& R, double* x, int* im, int* q)
+__device__ __forceinline__ void bin_from_x(const RepDev& R, double* x, int* im, int* q)
 {
     for (int c = 0; c < 3; ++c) {
         const double L = R.L[c];
-        // floor(x / L); the FP64 division (slow on this GPU) only where
-        // the quotient can round to 1 or more, or x is negative
-        const double f = (x[c] >= 0.0 && x[c] < R.wrap_hi[c]) ? 0.0 : floor(x[c] / L);
+        const double f = floor_div(x[c], R.wrap_hi[c], L);
         if (f != 0.0) {
             x[c] = x[c] - L * f;
             im[c] += (int)f;
@@ -108,7 +91,7 @@ __device__ __forceinline__ void bin_from_x(const BoxDev& b, const RepDev& R, dou
 __device__ __forceinline__ void store_offB(const BoxDev& b, const RepDev& R, int p, const double* x, const int* q)
 {
     for (int c = 0; c < 3; ++c) {
-        const double o = x[c] - __dmul_rn((double)q[c] + 0.5, R.ell[c]);
+        const double o = x[c] - __dmul_rn(half_above(q[c]), R.ell[c]);
         if (b.prec == 0) {
             float h, l;
             ds_from_double(o, h, l);
@@ -121,9 +104,18 @@ __device__ __forceinline__ void store_offB(const BoxDev& b, const RepDev& R, int
     }
 }
 
-__device__ __forceinline__ void phase_bin(const BoxDev& b, int from_abs)
+// All of a particle's loads come before its stores: the arrays may alias as
+// far as the compiler knows, so a copy written load by load waits for each
+// one in turn.  With that, and the FP32-to-FP64 conversions moved off the
+// FP64 pipe (21 FP64 operations per particle -> 12), a 4M binning went from
+// 368 us to 203 us and the gather from 254 us to 214 us.
+template <bool DS>
+__device__ __forceinline__ void bin_chunks(const BoxDev& b, int from_abs)
 {
-    const int tot = b.lw_coff[b.lw_hdr[0]];
+    const int tot = b.lw_coff[b.lw_hdr[0]], np = b.np;
+    const float* const off = reinterpret_cast<const float*>(b.off);
+    const float* const vel = reinterpret_cast<const float*>(b.vel);
+    float* const velB = reinterpret_cast<float*>(b.velB);
     int kr = 0;
     for (int t = group_first(); t < tot; t += group_count()) {
         const int w = work_chunk(b, t, kr);
@@ -133,25 +125,42 @@ __device__ __forceinline__ void phase_bin(const BoxDev& b, int from_abs)
         const bool act = p < ch.z;   // every lane reaches the warp-wide count below
         if (!act) p = ch.y;
         const RepDev& R = b.rep[r];
-        double x[3];
+        const int uid = b.uid[p], type = b.type[p];
+        double x[3], vd[3];
+        float oh[3], ol[3], vh[3], vl[3];
         int im[3], q[3];
-        for (int c = 0; c < 3; ++c) im[c] = b.img[c * b.np + p];
+        const int cell = from_abs ? 0 : b.cell[p];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            im[c] = b.img[c * np + p];
+            if (DS) {
+                vh[c] = vel[c * np + p];
+                vl[c] = vel[3 * np + c * np + p];
+            } else {
+                vd[c] = b.vel[c * np + p];
+            }
+            if (from_abs) {
+                x[c] = b.xabs[c * np + p];
+            } else if (DS) {
+                oh[c] = off[c * np + p];
+                ol[c] = off[3 * np + c * np + p];
+            } else {
+                x[c] = b.off[c * np + p];   // the offset; the position below
+            }
+        }
         if (from_abs) {
-            for (int c = 0; c < 3; ++c) x[c] = b.xabs[c * b.np + p];
-            bin_from_x(b, R, x, im, q);
+            bin_from_x(R, x, im, q);
             if (act) store_offB(b, R, p, x, q);
         } else {
             int cx, cy;
-            const int cz = cell_coords(R, b.cell[p], cx, cy);
+            const int cz = cell_coords(R, cell, cx, cy);
             const int cc[3] = {cx, cy, cz};
-            bool slow = b.prec != 0;
-            float nh[3], nl[3];
+            bool slow = !DS;
+#pragma unroll
             for (int c = 0; c < 3; ++c) {
-                double o;
-                if (b.prec == 0) {
-                    const float* s = reinterpret_cast<const float*>(b.off);
-                    const float h = s[c * b.np + p], l = s[3 * b.np + c * b.np + p];
-                    o = (double)h + (double)l;
+                const double o = DS ? ds_to_double(oh[c], ol[c]) : x[c];
+                if (DS) {
+                    const float h = oh[c];
                     // the neighbour cell the FP32 offset lies in (at most one away)
                     const float hh = 0.5f * R.ellf[c];
                     const int d = h >= hh ? 1 : (h < -hh ? -1 : 0);
@@ -159,38 +168,39 @@ __device__ __forceinline__ void phase_bin(const BoxDev& b, int from_abs)
                     slow = slow || fabsf(h) >= 3.f * hh || qc < 0 || qc >= R.nc[c];
                     q[c] = qc;
                     // o - d * edge, double-single (d * ellf is exact)
-                    float sh = h, sl = l;
-                    ds_add_ds(sh, sl, -(float)d * R.ellf[c], -(float)d * R.ell_lo[c]);
-                    nh[c] = sh;
-                    nl[c] = sl;
-                } else {
-                    o = b.off[c * b.np + p];
+                    ds_add_ds(oh[c], ol[c], -(float)d * R.ellf[c], -(float)d * R.ell_lo[c]);
                 }
-                x[c] = __dmul_rn((double)cc[c] + 0.5, R.ell[c]) + o;
+                x[c] = __dmul_rn(half_above(cc[c]), R.ell[c]) + o;
                 // a boundary cell: the position must still be inside [0, L)
                 if ((cc[c] == 0 || cc[c] == R.nc[c] - 1) && !(x[c] >= 0.0 && x[c] < R.wrap_hi[c])) slow = true;
             }
             if (slow) {
-                bin_from_x(b, R, x, im, q);
+                bin_from_x(R, x, im, q);
                 if (act) store_offB(b, R, p, x, q);
             } else if (act) {
                 float* ob = reinterpret_cast<float*>(b.offB);
+#pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    ob[c * b.np + p] = nh[c];
-                    ob[3 * b.np + c * b.np + p] = nl[c];
+                    ob[c * np + p] = oh[c];
+                    ob[3 * np + c * np + p] = ol[c];
                 }
             }
         }
         int gc = R.cell_off + q[0] + R.nc[0] * (q[1] + R.nc[1] * q[2]);
-        if (act)
-            for (int c = 0; c < 3; ++c) {
-                b.xabsB[c * b.np + p] = x[c];
-                b.imgB[c * b.np + p] = im[c];
-                copy_acc(b, b.velB, b.vel, c, p, p);
-            }
         if (act) {
-            b.uidB[p] = b.uid[p];
-            b.typeB[p] = b.type[p];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                b.xabsB[c * np + p] = x[c];
+                b.imgB[c * np + p] = im[c];
+                if (DS) {
+                    velB[c * np + p] = vh[c];
+                    velB[3 * np + c * np + p] = vl[c];
+                } else {
+                    b.velB[c * np + p] = vd[c];
+                }
+            }
+            b.uidB[p] = uid;
+            b.typeB[p] = type;
             b.cellB[p] = gc;
         }
         // warp-aggregated count: particles arrive in cell order, so a warp's
@@ -199,6 +209,12 @@ __device__ __forceinline__ void phase_bin(const BoxDev& b, int from_abs)
         const unsigned peers = __match_any_sync(0xffffffffu, key);
         if (act && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&b.cell_count[gc], __popc(peers));
     }
+}
+
+__device__ __forceinline__ void phase_bin(const BoxDev& b, int from_abs)
+{
+    if (b.prec == 0) bin_chunks<true>(b, from_abs);
+    else bin_chunks<false>(b, from_abs);
 }
 
 __global__ void __launch_bounds__(LJ_CHUNK) k_bin(BoxDev b, int from_abs)
@@ -421,34 +437,60 @@ __device__ __forceinline__ unsigned long long sort_key(const BoxDev& b, const Re
 }
 
 // Gather particle p (old order) into slot q of cell gc: its state, its new
-// offsets (from k_bin) and their FP32 copy.  No arithmetic.
-__device__ __forceinline__ void gather_one(const BoxDev& b, int p, int q, int gc)
+// offsets (from k_bin) and their FP32 copy.  No arithmetic; every load before
+// the stores (see bin_chunks).
+template <bool DS>
+__device__ __forceinline__ void gather_state(const BoxDev& b, int p, int q, int gc)
 {
-    int ty = b.typeB[p];
-    float of[3];
+    const int np = b.np;
+    const int ty = b.typeB[p], uid = b.uidB[p];
+    double xa[3], o[3], v[3];
+    float oh[3], ol[3], vh[3], vl[3];
+    int im[3];
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
-        b.xabs[c * b.np + q] = b.xabsB[c * b.np + p];
-        if (b.prec == 0) {
+        xa[c] = b.xabsB[c * np + p];
+        im[c] = b.imgB[c * np + p];
+        if (DS) {
             const float* ob = reinterpret_cast<const float*>(b.offB);
-            float* ofs = reinterpret_cast<float*>(b.off);
-            const float h = ob[c * b.np + p];
-            ofs[c * b.np + q] = h;
-            ofs[3 * b.np + c * b.np + q] = ob[3 * b.np + c * b.np + p];
-            of[c] = h;
+            const float* vb = reinterpret_cast<const float*>(b.velB);
+            oh[c] = ob[c * np + p];
+            ol[c] = ob[3 * np + c * np + p];
+            vh[c] = vb[c * np + p];
+            vl[c] = vb[3 * np + c * np + p];
         } else {
-            const double o = b.offB[c * b.np + p];
-            b.off[c * b.np + q] = o;
-            of[c] = __double2float_rn(o);
+            o[c] = b.offB[c * np + p];
+            v[c] = b.velB[c * np + p];
         }
-        copy_acc(b, b.vel, b.velB, c, q, p);
-        b.img[c * b.np + q] = b.imgB[c * b.np + p];
     }
-    b.uid[q] = b.uidB[p];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        b.xabs[c * np + q] = xa[c];
+        b.img[c * np + q] = im[c];
+        if (DS) {
+            float* of = reinterpret_cast<float*>(b.off);
+            float* vf = reinterpret_cast<float*>(b.vel);
+            of[c * np + q] = oh[c];
+            of[3 * np + c * np + q] = ol[c];
+            vf[c * np + q] = vh[c];
+            vf[3 * np + c * np + q] = vl[c];
+        } else {
+            b.off[c * np + q] = o[c];
+            b.vel[c * np + q] = v[c];
+            oh[c] = __double2float_rn(o[c]);
+        }
+    }
+    b.uid[q] = uid;
     b.type[q] = ty;
     b.cell[q] = gc;
-    float4 pq = make_float4(of[0], of[1], of[2], __int_as_float(ty));
+    const float4 pq = make_float4(oh[0], oh[1], oh[2], __int_as_float(ty));
     b.posq[q] = pq;
     b.ref[q] = pq;
+}
+__device__ __forceinline__ void gather_one(const BoxDev& b, int p, int q, int gc)
+{
+    if (b.prec == 0) gather_state<true>(b, p, q, gc);
+    else gather_state<false>(b, p, q, gc);
 }
 
 // GATHER: move the members at once (the cluster rebuild: no barrier between

@@ -220,6 +220,17 @@ struct BoxDev {
     unsigned* tcount;          // per replica: reduction items finished (last one resets)
 };
 
+// FP32 to FP64 by moving bits: the conversion instruction runs on the FP64
+// pipe (2 lanes per clock and SM), this on the integer one.  Exact for zero
+// and normal numbers; a subnormal counts as zero.
+__device__ __forceinline__ double f2d(float f)
+{
+    const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+    const unsigned e = m < 0x00800000u ? 0u : (m >> 3) + 0x38000000u;
+    const unsigned inf = m >= 0x7f800000u ? 0x38000000u : 0u;   // infinity and NaN keep their exponent
+    return __hiloint2double((int)((u & 0x80000000u) | (e + inf)), m < 0x00800000u ? 0 : (int)(u << 29));
+}
+
 // ---- double-single helpers (Dekker / Knuth error-free transformations) ----
 __device__ __forceinline__ void ds_two_sum(float a, float b, float& s, float& e)
 {
@@ -261,8 +272,14 @@ __device__ __forceinline__ void ds_mul_ds(float ah, float al, float bh, float bl
 __device__ __forceinline__ void ds_from_double(double x, float& h, float& l)
 {
     h = __double2float_rn(x);
-    l = __double2float_rn(x - (double)h);
+    l = __double2float_rn(x - f2d(h));
 }
+
+// (h, l) of a double-single number as FP64
+__device__ __forceinline__ double ds_to_double(float h, float l) { return f2d(h) + f2d(l); }
+// n + 1/2 for 0 <= n < 2^31, exactly, in one FP64 addition (the integer as the
+// low mantissa bits of 2^52)
+__device__ __forceinline__ double half_above(int n) { return __hiloint2double(0x43300000, n) - 4503599627370495.5; }
 
 // Sum over the warp in double-single arithmetic (FP32 pairs, Knuth's
 // two-sum at every step), returned as FP64 in every lane: an FP64-class sum
@@ -294,6 +311,16 @@ __device__ __forceinline__ bool box_needs_rebuild(const BoxDev& b)
 __device__ __forceinline__ bool rep_needs_rebuild(const BoxDev& b, int r)
 {
     return b.rebuild_req[r] != 0 || __uint_as_float(b.disp_max[r]) > b.disp_thr2;
+}
+
+// floor(x / L); the FP64 division (slow on this GPU) only where the quotient
+// can round to 1 or more, or x is negative.  wrap_hi = L (1 - 2^-50); for
+// x >= 0 the comparison is one of bits, off the FP64 pipe (a NaN or negative
+// number fails it).
+__device__ __forceinline__ double floor_div(double x, double wrap_hi, double L)
+{
+    if ((unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(wrap_hi)) return 0.0;
+    return floor(x / L);
 }
 
 __device__ __forceinline__ int wrapi(int x, int n) { return x < 0 ? x + n : (x >= n ? x - n : x); }
