@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_adj_pre(BoxDev b, double* lx, doub
                                                       float4* u_slot, double h, int pre)
 {
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        int4 ch = b.chunk[w];
+        int4 ch = chunk_of(b, w);
         int p = ch.y + (int)threadIdx.x;
         if (p >= ch.z) continue;
         size_t gu = (size_t)b.uid[p];
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const fl
     int cur_r = -1;
     float3 ell = make_float3(0.f, 0.f, 0.f);
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        const int4 ch = b.chunk[w];
+        const int4 ch = chunk_of(b, w);
         const int r = ch.x;
         if (r != cur_r) {                       // block-uniform
             const RepDev& R = b.rep[r];
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kHistThreads) k_pair_hist(BoxDev b, int nbins,
 #pragma unroll
     for (int q = 0; q < NB; ++q) ck[q] = ((float)(lane + 32 * q) + 0.5f) * rbin;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        const int4 ch = b.chunk[w];
+        const int4 ch = chunk_of(b, w);
         const RepDev& R = b.rep[ch.x];
         const float ex = R.ellf[0], ey = 0.25f * R.ellf[1], ez = 0.0625f * R.ellf[2];   // edges in the digits' units
         float hi[NB], lo[NB];
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_pair_hist_grad(BoxDev b, i
     int cur_r = -1;
     float ex = 0.f, ey = 0.f, ez = 0.f;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        const int4 ch = b.chunk[w];
+        const int4 ch = chunk_of(b, w);
         if (ch.x != cur_r) {   // block-uniform
             const RepDev& R = b.rep[ch.x];
             ex = R.ellf[0];

@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
     float3 ell = make_float3(b.ell1.x, 0.25f * b.ell1.y, 0.0625f * b.ell1.z);   // edges in the digits' units
     for (int it = blockIdx.x; it < b.nchunk * PARTS; it += gridDim.x) {
         const int w = it / PARTS, part = it % PARTS;
-        const int4 ch = b.chunk[w];
+        const int4 ch = chunk_of(b, w);
         const int r = ch.x;
         if (!SINGLE && r != cur_r) {            // block-uniform
             const RepDev& R = b.rep[r];
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
         }
         if (threadIdx.x == 0 && part == 0) {
             if (w == 0) *b.any_req = 0;         // the list update of this step has run
-            if (w == b.rep[r].chunk_off) {      // clear the replica's rebuild triggers
+            if (b.nrep == 1 ? w == 0 : w == b.rep[r].chunk_off) {      // clear the replica's rebuild triggers
                 b.disp_max[r] = 0u;
                 b.rebuild_req[r] = 0;
             }
@@ -798,7 +798,7 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
     float3 ell = make_float3(0.f, 0.f, 0.f);
     for (int it = blockIdx.x; it < b.nchunk * kF64Parts; it += gridDim.x) {
         const int w = it / kF64Parts, part = it % kF64Parts;
-        const int4 ch = b.chunk[w];
+        const int4 ch = chunk_of(b, w);
         const int r = ch.x;
         __syncthreads();   // the tables are complete; the previous item's sums are read
         if (r != cur_r) {  // block-uniform
@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
         }
         if (threadIdx.x == 0 && part == 0) {
             if (w == 0) *b.any_req = 0;
-            if (w == b.rep[r].chunk_off) {
+            if (b.nrep == 1 ? w == 0 : w == b.rep[r].chunk_off) {
                 b.disp_max[r] = 0u;
                 b.rebuild_req[r] = 0;
             }
@@ -922,17 +922,170 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
 
 // ---------------------------------------------------------------------------
 // All pairs (Sec. 4: the untruncated LJ interaction between all particles;
-// every cutoff infinite).  Work items are (chunk of 128 particles, slice of
-// the replica's particles): a block sums the chunk's forces over its slice
-// (LJ_TPP threads per particle, the slice's offsets staged through shared
-// memory in tiles) into b.ap_part, and the block that completes a chunk's
-// last slice (atomic count) adds the slices in slice order (deterministic).
-// With one cell per replica all offsets are from the box centre:
-// d = o_i - o_j - L rint((o_i - o_j) / L) is the minimum image.
+// every cutoff infinite).  With one cell per replica all offsets are from the
+// box centre: d = o_i - o_j - L rint((o_i - o_j) / L) is the minimum image.
+//
+// FP32: a warp holds two particles and its lanes take every 32nd particle of
+// the replica, so the pair arithmetic is packed over the two particles, the
+// positions are staged through shared memory by the block (all loads of a
+// tile in flight at once: streaming them through L1 a tile of 32 ahead waited
+// for L2 at every one, 21 us at N = 2,000) and read with one load per lane and
+// two pairs, and the sums meet in shuffles: no partial forces in memory and
+// nothing for a last block to add up.  The minimum image
+// rounds by adding and subtracting 1.5 * 2^23 (the rounding instruction runs
+// at an eighth of the FP32 rate, three per pair).  Bound: issue, ~17
+// instructions per pair; at N = 2,000, two warps per scheduler, latency.  Work
+// items are groups of 16 particles (a block), pf_stride of them per chunk; with
+// pf_stride 1 a block takes the chunk's eight groups in turn.
+// N = 2,000 with energies: 21.9 us with slices of the j range per chunk,
+// partial forces in memory and a last-block sum (its serial reads of 15 slices
+// were half of it), 10.6 us here; N = 32,000: 1,176 -> 895 us (FP32 pipe).
 // ---------------------------------------------------------------------------
-constexpr int kAllTile = 1024;
-constexpr int kAllThreads = LJ_CHUNK * LJ_TPP;
+constexpr int kAllWarps = 8;
+constexpr int kAllThreads = 32 * kAllWarps;
+constexpr int kAllGroup = 2 * kAllWarps;               // particles of a block pass
+constexpr int kAllGroups = LJ_CHUNK / kAllGroup;       // passes of a chunk
+constexpr int kAllTile = 2048;                         // positions staged at a time
+static_assert(kAllGroups == LJ_ALL_SHARES, "one (E_pot, W) share per group");
 
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+
+template <bool MONO, bool ENERGY>
+__global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
+{
+    __shared__ float4 s_lj[MONO ? 1 : LJ_MAXT * LJ_MAXT];   // c12, -c6, 2 eps sigma^6
+    __shared__ double s_red[2][kAllWarps];
+    __shared__ __align__(16) float4 s_pos[kAllTile];
+    const int nt = b.nt;
+    if (!MONO) {
+        const LJDev* lj = b.lj;
+        for (int k = threadIdx.x; k < nt * nt; k += blockDim.x)
+            s_lj[k] = make_float4(lj->c12[k], -lj->c6[k], 0.5f * lj->e6[k], 0.f);
+        __syncthreads();
+    }
+    const float c12 = MONO ? b.c1.x : 1.f, nh = b.nh_1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int parts = b.pf_stride;
+    const float2 M = dup2(12582912.0f), nM = dup2(-12582912.0f);   // 1.5 * 2^23
+    const float4* __restrict__ posq = b.posq;
+    for (int it = blockIdx.x; it < b.nchunk * parts; it += gridDim.x) {
+        const int w = it / parts;
+        const int4 ch = chunk_of(b, w);
+        const RepDev& R = b.rep[ch.x];
+        if (threadIdx.x == 0 && it % parts == 0) {
+            if (w == 0) *b.any_req = 0;         // the re-binning of this step has run
+            if (b.nrep == 1 ? w == 0 : w == R.chunk_off) {   // clear the replica's triggers
+                b.disp_max[ch.x] = 0u;
+                b.rebuild_req[ch.x] = 0;
+            }
+        }
+        // one cell: its edge is the box's (one replica: from the kernel parameters)
+        const float3 L = b.nrep == 1 ? b.ell1 : make_float3(R.ellf[0], R.ellf[1], R.ellf[2]);
+        const float2 ix = dup2(1.0f / L.x), iy = dup2(1.0f / L.y), iz = dup2(1.0f / L.z);
+        const float2 nLx = dup2(-L.x), nLy = dup2(-L.y), nLz = dup2(-L.z);
+        const int jb = b.nrep == 1 ? 0 : R.p_off, je = b.nrep == 1 ? b.n1 : R.p_off + R.n;
+        double esum = 0.0, wsum = 0.0;
+        for (int grp = it % parts; grp < kAllGroups; grp += parts) {
+            const int p = ch.y + grp * kAllGroup + 2 * warp;   // the warp's particles: p and p + 1
+            const bool one = p < ch.z, two = p + 1 < ch.z;     // warp-uniform
+            const float4 a = posq[one ? p : ch.y], c = posq[two ? p + 1 : ch.y];
+            const float2 nx = make_float2(-a.x, -c.x), ny = make_float2(-a.y, -c.y), nz = make_float2(-a.z, -c.z);
+            const int ta = __float_as_int(a.w) * nt, tc = __float_as_int(c.w) * nt;
+            float2 fx = dup2(0.f), fy = fx, fz = fx, vir = fx, eb = fx;
+            // particle j against the two, masked (the particle itself, lanes past the end) by m
+            auto pair = [&](const float4& q, bool masked, float2 m) {
+                float2 dx = __fadd2_rn(dup2(q.x), nx), dy = __fadd2_rn(dup2(q.y), ny), dz = __fadd2_rn(dup2(q.z), nz);
+                dx = __ffma2_rn(__fadd2_rn(__ffma2_rn(dx, ix, M), nM), nLx, dx);
+                dy = __ffma2_rn(__fadd2_rn(__ffma2_rn(dy, iy, M), nM), nLy, dy);
+                dz = __ffma2_rn(__fadd2_rn(__ffma2_rn(dz, iz, M), nM), nLz, dz);
+                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                float2 ri = make_float2(rcp_approx(r2.x), rcp_approx(r2.y));
+                if (masked) ri = make_float2(m.x != 0.f ? ri.x : 0.f, m.y != 0.f ? ri.y : 0.f);
+                const float2 r6 = __fmul2_rn(__fmul2_rn(ri, ri), ri);
+                float2 g;
+                if (MONO) {
+                    g = __fmul2_rn(r6, __fadd2_rn(r6, dup2(nh)));   // f r^2, over c12
+                    if (ENERGY) eb = __fadd2_rn(eb, r6);
+                } else {
+                    const int tj = __float_as_int(q.w);
+                    const float4 u = s_lj[ta + tj], v = s_lj[tc + tj];
+                    g = __fmul2_rn(r6, __ffma2_rn(make_float2(u.x, v.x), r6, make_float2(u.y, v.y)));
+                    if (ENERGY) eb = __ffma2_rn(make_float2(u.z, v.z), r6, eb);
+                }
+                const float2 f = __fmul2_rn(ri, g);
+                fx = __ffma2_rn(f, dx, fx);   // of -d: negated at the end
+                fy = __ffma2_rn(f, dy, fy);
+                fz = __ffma2_rn(f, dz, fz);
+                if (ENERGY) vir = __fadd2_rn(vir, g);
+            };
+            for (int t0 = jb; t0 < je; t0 += kAllTile) {
+                const int t1 = min(t0 + kAllTile, je);
+                __syncthreads();   // the previous tile is no longer read
+#pragma unroll
+                for (int t = 0; t < kAllTile / kAllThreads; ++t) {
+                    const int j = t0 + t * kAllThreads + (int)threadIdx.x;
+                    if (j < t1) s_pos[j - t0] = posq[j];
+                }
+                __syncthreads();
+                if (!one) continue;
+                // groups of 32: the two particles' own (both in one) and a
+                // partial last one are masked, the runs between them are not
+                const int full = t0 + ((t1 - t0) & ~31);
+                const int own = p >= t0 && p < t1 ? t0 + ((p - t0) & ~31) : t1;
+                auto run = [&](int a0, int a1) {
+#pragma unroll 4
+                    for (int j0 = a0; j0 < a1; j0 += 32) pair(s_pos[j0 - t0 + lane], false, dup2(1.f));
+                };
+                auto edge = [&](int j0) {
+                    const int j = j0 + lane;
+                    pair(s_pos[min(j, t1 - 1) - t0], true,
+                         make_float2(j < t1 && j != p ? 1.f : 0.f, j < t1 && j != p + 1 ? 1.f : 0.f));
+                };
+                run(t0, min(own, full));
+                if (own < t1) edge(own);
+                run(own + 32, full);
+                if (full < t1 && full != own) edge(full);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                fx = __fadd2_rn(fx, make_float2(__shfl_xor_sync(0xffffffffu, fx.x, o), __shfl_xor_sync(0xffffffffu, fx.y, o)));
+                fy = __fadd2_rn(fy, make_float2(__shfl_xor_sync(0xffffffffu, fy.x, o), __shfl_xor_sync(0xffffffffu, fy.y, o)));
+                fz = __fadd2_rn(fz, make_float2(__shfl_xor_sync(0xffffffffu, fz.x, o), __shfl_xor_sync(0xffffffffu, fz.y, o)));
+            }
+            if ((lane == 0 && one) || (lane == 1 && two)) {
+                const float sx = lane == 0 ? fx.x : fx.y, sy = lane == 0 ? fy.x : fy.y, sz = lane == 0 ? fz.x : fz.y;
+                b.force4[p + lane] = make_float4(-c12 * sx, -c12 * sy, -c12 * sz, 0.f);
+                if (!isfinite(sx + sy + sz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
+            }
+            if (ENERGY) {
+                // u = f r^2 / 12 - 2 eps (sigma / r)^6 (no cutoff, no shift)
+                const float wv = c12 * (vir.x + (two ? vir.y : 0.f));   // both 0 without a first particle
+                const float ev = fmaf(wv, 1.f / 12.f, (MONO ? -0.5f * b.c1.w : -1.f) * (eb.x + (two ? eb.y : 0.f)));
+                const float2 de = warp_sum_ds2(ev), dw = warp_sum_ds2(wv);
+                esum += (double)de.x + (double)de.y;
+                wsum += (double)dw.x + (double)dw.y;
+            }
+        }
+        if (ENERGY) {
+            __syncthreads();   // the previous item's sums are read
+            if (lane == 0) {
+                s_red[0][warp] = 0.5 * esum;   // each pair is seen from both ends
+                s_red[1][warp] = 0.5 * wsum;
+            }
+            __syncthreads();
+            if (threadIdx.x < 2) {
+                double t = 0.0;
+                for (int k = 0; k < kAllWarps; ++k) t += s_red[threadIdx.x][k];
+                b.part_f[2 * (size_t)it + threadIdx.x] = t;
+            }
+        }
+    }
+}
+
+// All pairs in FP64 (MD_PREC_FP64).  Work items are (chunk of 128 particles,
+// slice of the replica's particles): a block sums the chunk's forces over its
+// slice into b.ap_part64, and the block that completes a chunk's last slice
+// (atomic count) adds the slices in slice order (deterministic).
 __device__ __forceinline__ void slice_range(const RepDev& R, int js, int nslice, int& j0, int& j1)
 {
     const int len = (R.n + nslice - 1) / nslice;
@@ -956,124 +1109,8 @@ __device__ __forceinline__ bool last_slice(const BoxDev& b, int w, int* s_flag)
     return last;
 }
 
-template <bool MONO, bool ENERGY>
-__global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
-{
-    __shared__ float4 s_pos[kAllTile];
-    __shared__ float4 s_lj[LJ_MAXT * LJ_MAXT];   // c12, c6, e12, e6
-    __shared__ float s_esh[LJ_MAXT * LJ_MAXT];
-    __shared__ double s_red[2][32];
-    __shared__ int s_flag;
-    const LJDev* lj = b.lj;
-    const int nt = lj->nt;
-    for (int k = threadIdx.x; k < nt * nt; k += blockDim.x) {
-        s_lj[k] = make_float4(lj->c12[k], lj->c6[k], lj->e12[k], lj->e6[k]);
-        s_esh[k] = lj->shift[k];
-    }
-    const float4 mlj = make_float4(lj->c12[0], lj->c6[0], lj->e12[0], lj->e6[0]);
-    const float mesh = lj->shift[0];
-    const int grp = threadIdx.x / LJ_TPP, l4 = threadIdx.x % LJ_TPP;
-    const int nitem = b.nchunk * b.ap_js;
-    for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
-        const int w = it / b.ap_js, js = it % b.ap_js;
-        const int4 ch = b.chunk[w];
-        const RepDev& R = b.rep[ch.x];
-        if (threadIdx.x == 0 && js == 0) {
-            if (w == 0) *b.any_req = 0;         // the re-binning of this step has run
-            if (w == R.chunk_off) {             // clear the replica's triggers
-                b.disp_max[ch.x] = 0u;
-                b.rebuild_req[ch.x] = 0;
-            }
-        }
-        const float Lx = (float)R.L[0], Ly = (float)R.L[1], Lz = (float)R.L[2];
-        const float ix = (float)(1.0 / R.L[0]), iy = (float)(1.0 / R.L[1]), iz = (float)(1.0 / R.L[2]);
-        const int p = ch.y + grp;
-        const bool act = p < ch.z;
-        const float4 pi = b.posq[act ? p : ch.y];
-        const int tb = __float_as_int(pi.w) * nt;
-        float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f, vir = 0.f;
-        int j0, j1;
-        slice_range(R, js, b.ap_js, j0, j1);
-        for (int t0 = j0; t0 < j1; t0 += kAllTile) {
-            const int nj = min(kAllTile, j1 - t0);
-            __syncthreads();   // the previous tile is no longer read
-            for (int t = threadIdx.x; t < nj; t += blockDim.x) s_pos[t] = b.posq[t0 + t];
-            __syncthreads();
-            for (int t = l4; t < nj; t += LJ_TPP) {
-                const float4 pj = s_pos[t];
-                float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-                dx -= Lx * rintf(dx * ix);
-                dy -= Ly * rintf(dy * iy);
-                dz -= Lz * rintf(dz * iz);
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                float4 c;
-                float esh;
-                if (MONO) {
-                    c = mlj;
-                    esh = mesh;
-                } else {
-                    const int pp = tb + __float_as_int(pj.w);
-                    c = s_lj[pp];
-                    esh = ENERGY ? s_esh[pp] : 0.f;
-                }
-                const float r2i = rcp_approx(r2);
-                const float r6i = r2i * r2i * r2i;
-                float f = r2i * r6i * fmaf(c.x, r6i, -c.y);
-                const bool in = act && t0 + t != p;
-                f = in ? f : 0.f;
-                fx = fmaf(f, dx, fx);
-                fy = fmaf(f, dy, fy);
-                fz = fmaf(f, dz, fz);
-                if (ENERGY) {
-                    const float u = r6i * fmaf(c.z, r6i, -c.w) - esh;
-                    e += in ? u : 0.f;
-                    vir = fmaf(f, r2, vir);
-                }
-            }
-        }
-#pragma unroll
-        for (int o = LJ_TPP / 2; o > 0; o >>= 1) {
-            fx += __shfl_xor_sync(0xffffffffu, fx, o);
-            fy += __shfl_xor_sync(0xffffffffu, fy, o);
-            fz += __shfl_xor_sync(0xffffffffu, fz, o);
-        }
-        if (act && l4 == 0) b.ap_part[(size_t)js * b.np + p] = make_float4(fx, fy, fz, 0.f);
-        if (ENERGY) {
-            double de = 0.5 * (double)e, dw = 0.5 * (double)vir;
-            block_sum2(de, dw, s_red);
-            if (threadIdx.x == 0) {
-                b.ap_pe[2 * (size_t)it] = de;
-                b.ap_pe[2 * (size_t)it + 1] = dw;
-            }
-        }
-        if (last_slice(b, w, &s_flag)) {
-            for (int q = ch.y + (int)threadIdx.x; q < ch.z; q += blockDim.x) {
-                float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int k = 0; k < b.ap_js; ++k) {
-                    const float4 g = __ldcg(&b.ap_part[(size_t)k * b.np + q]);
-                    f.x += g.x;
-                    f.y += g.y;
-                    f.z += g.z;
-                }
-                b.force4[q] = f;
-                if (!isfinite(f.x + f.y + f.z)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
-            }
-            if (ENERGY && threadIdx.x == 0) {
-                double de = 0.0, dw = 0.0;
-                for (int k = 0; k < b.ap_js; ++k) {
-                    de += __ldcg(&b.ap_pe[2 * ((size_t)w * b.ap_js + k)]);
-                    dw += __ldcg(&b.ap_pe[2 * ((size_t)w * b.ap_js + k) + 1]);
-                }
-                b.part_f[2 * w] = de;
-                b.part_f[2 * w + 1] = dw;
-            }
-        }
-    }
-}
-
-// All pairs in FP64 (MD_PREC_FP64): the same work items, one thread per
-// particle, FP64 offsets staged through shared memory; partial forces in
-// b.ap_part64 (3 planes per slice).
+// One thread per particle, FP64 offsets staged through shared memory; partial
+// forces in b.ap_part64 (3 planes per slice).
 template <bool ENERGY>
 __global__ void __launch_bounds__(LJ_CHUNK) k_force_all_f64(BoxDev b)
 {
@@ -1088,7 +1125,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_force_all_f64(BoxDev b)
     const int nitem = b.nchunk * b.ap_js;
     for (int it = blockIdx.x; it < nitem; it += gridDim.x) {
         const int w = it / b.ap_js, js = it % b.ap_js;
-        const int4 ch = b.chunk[w];
+        const int4 ch = chunk_of(b, w);
         const RepDev& R = b.rep[ch.x];
         if (threadIdx.x == 0 && js == 0) {
             if (w == 0) *b.any_req = 0;

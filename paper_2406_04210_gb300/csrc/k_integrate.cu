@@ -23,28 +23,87 @@ __device__ __forceinline__ double warp_sum_d(double v)
     return v;
 }
 
-// Andersen-like collision of particle p after the finalize of step `step`
-// (see md_set_thermostat): true and the new velocity in g when word 0 of
-// philox((local user index, step lo, step hi, 0), seed + replica) is below
-// the threshold; Gaussians by Box-Muller.
-__device__ __forceinline__ bool tstat_collide(const BoxDev& b, const RepDev& R, int r, int p, long long step,
-                                              double g[3])
+// Andersen-like collision of particle u of replica r after the finalize of
+// step `step` (see md_set_thermostat): true and the new velocity in g when word 0 of
+// philox((u, step lo, step hi, 0), seed + replica) is below
+// the threshold; Gaussians by Box-Muller.  All lanes of the warp call it (act:
+// the lane has a particle).  The FP64 logarithm and the sine pair are long
+// dependent chains on a slow pipe, and few lanes collide in a step: up to
+// kFewHits of them are taken in turn by the whole warp, even lanes computing
+// the first Box-Muller pair and odd lanes the second at the same time.
+constexpr int kFewHits = 2;
+__device__ __forceinline__ void box_muller(unsigned w0, unsigned w1, double& rs, double& rc)
 {
-    const unsigned u = (unsigned)(b.uid[p] - R.u_off);
+    const double inv32 = 1.0 / 4294967296.0;
+    const double r = sqrt(-2.0 * log(((double)w0 + 0.5) * inv32));
+    double s, c;
+    sincospi(2.0 * (((double)w1 + 0.5) * inv32), &s, &c);
+    rs = r * s;
+    rc = r * c;
+}
+__device__ __forceinline__ bool tstat_collide(const BoxDev& b, const RepDev& R, int r, unsigned u, bool act,
+                                              long long step, double g[3])
+{
     const unsigned long long key = b.tstat_seed + (unsigned long long)r;
     const uint2 k = make_uint2((unsigned)key, (unsigned)(key >> 32));
     const unsigned slo = (unsigned)step, shi = (unsigned)((unsigned long long)step >> 32);
     const uint4 x = philox4x32_10(make_uint4(u, slo, shi, 0u), k);
-    if (!(x.x < b.tstat_thr)) return false;
-    const uint4 y = philox4x32_10(make_uint4(u, slo, shi, 1u), k);
+    const bool hit = act && x.x < b.tstat_thr;
+    unsigned todo = __ballot_sync(0xffffffffu, hit);
+    if (todo == 0u) return false;   // warp-uniform
+    uint4 y = make_uint4(0u, 0u, 0u, 0u);
+    if (hit) y = philox4x32_10(make_uint4(u, slo, shi, 1u), k);
     const double sd = sqrt(b.tstat_T[r]);
-    const double two_pi = 6.283185307179586476925286766559;
-    const double inv32 = 1.0 / 4294967296.0;
-    const double r1 = sqrt(-2.0 * log(((double)x.y + 0.5) * inv32)), a1 = two_pi * (((double)x.z + 0.5) * inv32);
-    const double r2 = sqrt(-2.0 * log(((double)y.x + 0.5) * inv32)), a2 = two_pi * (((double)y.y + 0.5) * inv32);
-    g[0] = sd * (r1 * cos(a1));
-    g[1] = sd * (r1 * sin(a1));
-    g[2] = sd * (r2 * cos(a2));
+    double rs, rc;
+    if (__popc(todo) <= kFewHits) {
+        const bool odd = (threadIdx.x & 1) != 0;
+        for (; todo; todo &= todo - 1u) {
+            const int src = __ffs(todo) - 1;
+            const unsigned a0 = __shfl_sync(0xffffffffu, x.y, src), a1 = __shfl_sync(0xffffffffu, x.z, src);
+            const unsigned b0 = __shfl_sync(0xffffffffu, y.x, src), b1 = __shfl_sync(0xffffffffu, y.y, src);
+            box_muller(odd ? b0 : a0, odd ? b1 : a1, rs, rc);
+            const double g0 = __shfl_sync(0xffffffffu, rc, 0), g1 = __shfl_sync(0xffffffffu, rs, 0);
+            const double g2 = __shfl_sync(0xffffffffu, rc, 1);
+            if ((int)(threadIdx.x & 31) == src) {
+                g[0] = sd * g0;
+                g[1] = sd * g1;
+                g[2] = sd * g2;
+            }
+        }
+    } else if (hit) {
+        box_muller(x.y, x.z, rs, rc);
+        g[0] = sd * rc;
+        g[1] = sd * rs;
+        box_muller(y.x, y.y, rs, rc);
+        g[2] = sd * rc;
+    }
+    return hit;
+}
+
+// The collisions of a graph's steps, drawn at its head: the FP64 chain above
+// would otherwise stand in every step's integrator (5.6 of 14.3 us at N =
+// 2,000), while here all steps and particles draw at once.
+__global__ void __launch_bounds__(LJ_CHUNK) k_tstat_draw(BoxDev b, int nsteps, unsigned* hit_bits, double* gs)
+{
+    for (int it = blockIdx.x; it < nsteps * b.nchunk; it += gridDim.x) {
+        const int step = it / b.nchunk, w = it % b.nchunk;
+        const int4 ch = chunk_of(b, w);
+        const RepDev& R = b.rep[ch.x];
+        const int q = ch.y + (int)threadIdx.x;   // slot before any sort
+        double g[3] = {0.0, 0.0, 0.0};
+        const bool hit = tstat_collide(b, R, ch.x, (unsigned)(q - R.p_off), q < ch.z, *b.step_ctr + step, g);
+        const unsigned bits = __ballot_sync(0xffffffffu, hit);
+        if ((threadIdx.x & 31) == 0 && q < ch.z) hit_bits[(size_t)step * (b.np / 32) + q / 32] = bits;
+        if (hit)
+            for (int c = 0; c < 3; ++c) gs[((size_t)step * b.np + q) * 3 + c] = g[c];
+    }
+}
+// the same, read back by the integrator
+__device__ __forceinline__ bool tstat_drawn(const BoxDev& b, const RepDev& R, int uid, int sidx, double g[3])
+{
+    const int q = b.nrep == 1 ? uid : R.p_off + (uid - R.u_off);
+    if (!((b.tstat_hit[(size_t)sidx * (b.np / 32) + q / 32] >> (q & 31)) & 1u)) return false;
+    for (int c = 0; c < 3; ++c) g[c] = b.tstat_g[((size_t)sidx * b.np + q) * 3 + c];
     return true;
 }
 
@@ -88,12 +147,21 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_integrate(BoxDev b, double dt, int
     float* offf = reinterpret_cast<float*>(b.off);
     float* velf = reinterpret_cast<float*>(b.vel);
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        int4 ch = b.chunk[w];
+        int4 ch = chunk_of(b, w);
         int r = ch.x;
         int p = ch.y + (int)threadIdx.x;
         double ek = 0.0;
         float ekf = 0.f;   // double-single state: FP32 per particle
         unsigned dmax = 0u;
+        // thermostat collision after the finalize of this step
+        double g[3] = {0.0, 0.0, 0.0};
+        bool hit = false;
+        if (TSTAT && MODE != LJ_STEP_FIRST) {
+            const RepDev& R = b.rep[r];
+            const int uid = p < ch.z ? b.uid[p] : 0;
+            if (b.tstat_hit) hit = p < ch.z && tstat_drawn(b, R, uid, sidx, g);
+            else hit = tstat_collide(b, R, r, (unsigned)(uid - R.u_off), p < ch.z, *b.step_ctr + sidx, g);
+        }
         if (p < ch.z) {
             // every load before the stores (the arrays may alias as far as
             // the compiler knows: a load behind a store waits its turn)
@@ -128,11 +196,6 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_integrate(BoxDev b, double dt, int
                 F[2] = f4.z;
             }
             float o[3];
-            // thermostat collision after the finalize of this step
-            double g[3] = {0.0, 0.0, 0.0};
-            bool hit = false;
-            if (TSTAT && MODE != LJ_STEP_FIRST)
-                hit = tstat_collide(b, b.rep[r], r, p, *b.step_ctr + sidx, g);
             if (ACC == 0) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
@@ -235,7 +298,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_upload(BoxDev b, const double* pos
 {
     const int np = b.np;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        int4 ch = b.chunk[w];
+        int4 ch = chunk_of(b, w);
         int p = ch.y + (int)threadIdx.x;
         if (p >= ch.z) continue;
         const RepDev& R = b.rep[ch.x];
@@ -281,7 +344,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_download(BoxDev b, double* pos, do
 {
     const int np = b.np;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        int4 ch = b.chunk[w];
+        int4 ch = chunk_of(b, w);
         int p = ch.y + (int)threadIdx.x;
         if (p >= ch.z) continue;
         const RepDev& R = b.rep[ch.x];
@@ -334,7 +397,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_force_out(BoxDev b, double* f)
 {
     const int np = b.np;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        int4 ch = b.chunk[w];
+        int4 ch = chunk_of(b, w);
         int p = ch.y + (int)threadIdx.x;
         if (p >= ch.z) continue;
         size_t gu = (size_t)b.uid[p];
@@ -354,7 +417,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_get_nlist(BoxDev b, int* count, lo
 {
     const int np = b.np;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        int4 ch = b.chunk[w];
+        int4 ch = chunk_of(b, w);
         int p = ch.y + (int)threadIdx.x;
         if (p >= ch.z) continue;
         long long gu = b.uid[p];
@@ -387,6 +450,12 @@ __global__ void k_step_advance(long long* ctr, long long n)
     if (blockIdx.x == 0 && threadIdx.x == 0) *ctr += n;
 }
 }  // namespace
+
+cudaError_t launch_tstat_draw(const BoxDev& b, int nsteps, unsigned* hit, double* g, Launch l)
+{
+    k_tstat_draw<<<l.grid, LJ_CHUNK, 0, l.s>>>(b, nsteps, hit, g);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_step_advance(long long* ctr, long long n, cudaStream_t s)
 {
@@ -427,7 +496,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_materialize(BoxDev b)
 {
     const int np = b.np;
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        int4 ch = b.chunk[w];
+        int4 ch = chunk_of(b, w);
         int p = ch.y + (int)threadIdx.x;
         if (p >= ch.z) continue;
         const RepDev& R = b.rep[ch.x];

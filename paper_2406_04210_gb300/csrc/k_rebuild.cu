@@ -38,16 +38,22 @@ __device__ __forceinline__ int cell_coords(const RepDev& R, int gc, int& cx, int
     return t / R.nc[1];
 }
 
+// How many there are, of chunks and of cells (one replica: all of its own).
+__device__ __forceinline__ int work_chunks(const BoxDev& b) { return b.nrep == 1 ? b.nchunk : b.lw_coff[b.lw_hdr[0]]; }
+__device__ __forceinline__ int work_cells(const BoxDev& b) { return b.nrep == 1 ? b.ncell : b.lw_off[b.lw_hdr[0]]; }
+
 // Cell (chunk) t of the concatenation of the rebuilding replicas' cells
 // (particle chunks), from k_list_work's lists; kr is the replica index of the
 // caller's previous t (t only grows).
 __device__ __forceinline__ int work_cell(const BoxDev& b, int t, int& kr)
 {
+    if (b.nrep == 1) return t;
     while (t >= b.lw_off[kr + 1]) ++kr;
     return b.rep[b.lw_rep[kr]].cell_off + (t - b.lw_off[kr]);
 }
 __device__ __forceinline__ int work_chunk(const BoxDev& b, int t, int& kr)
 {
+    if (b.nrep == 1) return t;
     while (t >= b.lw_coff[kr + 1]) ++kr;
     return b.rep[b.lw_rep[kr]].chunk_off + (t - b.lw_coff[kr]);
 }
@@ -112,14 +118,14 @@ __device__ __forceinline__ void store_offB(const BoxDev& b, const RepDev& R, int
 template <bool DS>
 __device__ __forceinline__ void bin_chunks(const BoxDev& b, int from_abs)
 {
-    const int tot = b.lw_coff[b.lw_hdr[0]], np = b.np;
+    const int tot = work_chunks(b), np = b.np;
     const float* const off = reinterpret_cast<const float*>(b.off);
     const float* const vel = reinterpret_cast<const float*>(b.vel);
     float* const velB = reinterpret_cast<float*>(b.velB);
     int kr = 0;
     for (int t = group_first(); t < tot; t += group_count()) {
         const int w = work_chunk(b, t, kr);
-        int4 ch = b.chunk[w];
+        int4 ch = chunk_of(b, w);
         int r = ch.x;
         int p = ch.y + group_thread();
         const bool act = p < ch.z;   // every lane reaches the warp-wide count below
@@ -331,10 +337,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_add(BoxDev b, const int4*
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void phase_scatter(const BoxDev& b)
 {
-    const int tot = b.lw_coff[b.lw_hdr[0]];
+    const int tot = work_chunks(b);
     int kr = 0;
     for (int t = group_first(); t < tot; t += group_count()) {
-        int4 ch = b.chunk[work_chunk(b, t, kr)];
+        int4 ch = chunk_of(b, work_chunk(b, t, kr));
         int p = ch.y + group_thread();
         const bool act = p < ch.z;
         // warp-aggregated slot claims: one atomic per distinct cell of the
@@ -500,11 +506,11 @@ __device__ __forceinline__ void phase_rank(const BoxDev& b)
 {
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
-    const int total = b.lw_off[b.lw_hdr[0]];
+    const int total = work_cells(b);
     int kr = 0;
     for (int t = blockIdx.x * wpb + (threadIdx.x >> 5); t < total; t += gridDim.x * wpb) {
         const int gc = work_cell(b, t, kr);
-        const RepDev& R = b.rep[b.lw_rep[kr]];
+        const RepDev& R = b.rep[b.nrep == 1 ? 0 : b.lw_rep[kr]];
         int s0 = b.cell_start[gc];
         int n = b.cell_end[gc] - s0;
         for (int base = 0; base < n; base += 32) {
@@ -536,10 +542,10 @@ __global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
     if (b.all_pairs) {
         // one cell holds the whole replica and no list needs an order: a
         // particle's slot is its index inside the replica, one thread each
-        const int tot = b.lw_coff[b.lw_hdr[0]];
+        const int tot = work_chunks(b);
         int kr = 0;
         for (int t = blockIdx.x; t < tot; t += gridDim.x) {
-            const int4 ch = b.chunk[work_chunk(b, t, kr)];
+            const int4 ch = chunk_of(b, work_chunk(b, t, kr));
             const RepDev& R = b.rep[ch.x];
             for (int s = ch.y + (int)threadIdx.x; s < ch.z; s += blockDim.x) {
                 if (s == R.p_off) atomicAdd(&b.nbuild[ch.x], 1ull);   // a re-binning
@@ -555,10 +561,10 @@ __global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
 __global__ void __launch_bounds__(LJ_CHUNK) k_gather(BoxDev b)
 {
     if (b.all_pairs || !box_needs_rebuild(b)) return;
-    const int tot = b.lw_coff[b.lw_hdr[0]];
+    const int tot = work_chunks(b);
     int kr = 0;
     for (int t = blockIdx.x; t < tot; t += gridDim.x) {
-        const int4 ch = b.chunk[work_chunk(b, t, kr)];
+        const int4 ch = chunk_of(b, work_chunk(b, t, kr));
         const int s = ch.y + (int)threadIdx.x;
         if (s >= ch.z) continue;
         const int p = b.perm[s];
@@ -942,11 +948,11 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
     const float4* __restrict__ posq = b.posq;
     int longest = 0;
     const int nwarp = gridDim.x * kLaneWarps;
-    const int total = b.lw_off[b.lw_hdr[0]] * G;
+    const int total = work_cells(b) * G;
     int kr = 0;
     for (int t = blockIdx.x * kLaneWarps + warp; t < total; t += nwarp) {
         const int gc = work_cell(b, t / G, kr);
-        const int r = b.lw_rep[kr];
+        const int r = b.nrep == 1 ? 0 : b.lw_rep[kr];
         const RepDev& R = b.rep[r];
         const int cs = b.cell_start[gc], n = b.cell_end[gc] - cs;
         if (lane == 0 && t % G == 0 && gc == R.cell_off) atomicAdd(&b.nbuild[r], 1ull);

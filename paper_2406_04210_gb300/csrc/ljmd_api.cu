@@ -113,6 +113,8 @@ struct md_box {
     bool all_pairs = false;
     double tstat_rate = 0.0;
     double* d_tstat_T = nullptr;
+    char* d_tstat_draws = nullptr;   // the collisions of a graph's steps, drawn at its head
+    size_t tstat_draw_bytes = 0;
     long long* d_step_ctr = nullptr;
     // tuning
     int min_capacity = 0;
@@ -280,7 +282,10 @@ void apply_force_kernel(md_box* b)
     b->d.force_tiles = tiles ? 1 : 0;
     const bool spread = list32 && !tiles && spread_force(b);
     b->d.force_spread = spread ? 1 : 0;
-    b->d.pf_stride = b->all_pairs                ? 1
+    // all pairs, FP32: a block per 16 particles (LJ_ALL_SHARES per chunk), or,
+    // where the chunks alone are several per SM, per chunk
+    const int all = b->prec == MD_PREC_FP64 || b->chunks.size() > 1024 ? 1 : LJ_ALL_SHARES;
+    b->d.pf_stride = b->all_pairs                ? all
                      : b->prec == MD_PREC_FP64 ? LJ_F64_WARPS
                      : spread                    ? LJ_SPREAD_SHARES
                                                  : LJ_FORCE_WARPS;
@@ -298,7 +303,9 @@ Launch lforce(md_box* b)
     }
     int per_sm = b->force_per_sm > 0 ? b->force_per_sm : (b->prec == 2 ? 12 : 6);
     // the FP64 list kernel's items are quarters of a chunk
-    const int items = b->d.nchunk * (b->all_pairs ? std::max(1, b->d.ap_js) : b->prec == MD_PREC_FP64 ? LJ_F64_WARPS : 1);
+    int per_chunk = b->prec == MD_PREC_FP64 ? LJ_F64_WARPS : 1;
+    if (b->all_pairs) per_chunk = b->prec == MD_PREC_FP64 ? std::max(1, b->d.ap_js) : b->d.pf_stride;
+    const int items = b->d.nchunk * per_chunk;
     return Launch{std::max(1, std::min(items, b->nsm * per_sm)), 0, b->stream};
 }
 Launch llist(md_box* b)
@@ -806,6 +813,25 @@ BoxDev tape_view(md_box* b, int m)
     return v;
 }
 
+// The thermostat's draws of n steps ahead of them, while they fit 64 MiB (N =
+// 27,000 for 100 steps; beyond, the draw is a small part of a step anyway).
+size_t tstat_velocity_bytes(md_box* b, int64_t n) { return (size_t)n * (size_t)b->np * 3 * sizeof(double); }
+bool tstat_ahead(md_box* b, int64_t n) { return tstat_velocity_bytes(b, n) <= ((size_t)64 << 20); }
+
+md_status ensure_tstat(md_box* b, int64_t n)
+{
+    if (!b->d.tstat_thr || !tstat_ahead(b, n)) return MD_OK;
+    const size_t need = al256(tstat_velocity_bytes(b, n)) + (size_t)n * (size_t)b->np / 8;
+    if (b->tstat_draw_bytes >= need) return MD_OK;
+    invalidate_graphs(b);   // graphs hold the pointer
+    dev_release(b, b->d_tstat_draws);
+    b->d_tstat_draws = nullptr;
+    b->tstat_draw_bytes = 0;
+    CKS(dev_alloc(b, &b->d_tstat_draws, need, false));
+    b->tstat_draw_bytes = need;
+    return MD_OK;
+}
+
 md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* ring, GraphEnt* ge,
                         bool tape = false)
 {
@@ -827,6 +853,18 @@ md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* rin
         return cudaEventRecordWithFlags(ge->ev[2 * k + end], st, cudaEventRecordExternal);
     };
     BoxDev set[2] = {b->d, b->d};
+    if (b->d.tstat_thr && !tape && tstat_ahead(b, n)) {
+        unsigned* hit = reinterpret_cast<unsigned*>(b->d_tstat_draws + al256(tstat_velocity_bytes(b, n)));
+        double* g = reinterpret_cast<double*>(b->d_tstat_draws);
+        const int items = (int)n * b->d.nchunk;
+        CK(b, launch_tstat_draw(b->d, (int)n, hit, g,
+                                Launch{std::max(1, std::min(items, b->nsm * 8)), LJ_CHUNK, b->stream}));
+        b->launches += 1;
+        for (BoxDev& v : set) {
+            v.tstat_hit = hit;
+            v.tstat_g = g;
+        }
+    }
     set[1].part_f += b->pf_cap;
     set[1].part_k += LJ_KIN_WARPS * std::max<size_t>(1, b->chunks.size());
     bool pending[2] = {false, false};   // reductions not joined yet, by set
@@ -1075,6 +1113,7 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
     b->nrep = nrep;
     b->ntot = ntot;
     b->np = (int)std::max<int64_t>(np, 32);
+    b->d.n1 = (int)ntot;
     b->ustream = static_cast<cudaStream_t>(stream);
     cudaGetDevice(&b->device);
     cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, b->device);
@@ -1288,7 +1327,7 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
     b->all_pairs = all_pairs;
     b->d.all_pairs = all_pairs ? 1 : 0;
     apply_force_kernel(b);   // the force kernel and its (E_pot, W) shares
-    if (all_pairs && !b->d.ap_cnt) {
+    if (all_pairs && b->prec == MD_PREC_FP64 && !b->d.ap_cnt) {
         // j slices per chunk: enough work items to fill the GPU, each slice
         // at least ~128 particles
         int nmax = 1;
@@ -1296,8 +1335,7 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
         const int nch = std::max(1, (int)b->chunks.size());
         const int js = std::max(1, std::min((b->nsm * 4 + nch - 1) / nch, std::max(1, nmax / 128)));
         b->d.ap_js = js;
-        CKS(dev_alloc(b, &b->d.ap_part, (size_t)js * b->np, false));
-        if (b->prec == MD_PREC_FP64) CKS(dev_alloc(b, &b->d.ap_part64, (size_t)js * 3 * b->np, false));
+        CKS(dev_alloc(b, &b->d.ap_part64, (size_t)js * 3 * b->np, false));
         CKS(dev_alloc(b, &b->d.ap_pe, 2 * (size_t)js * nch, false));
         CKS(dev_alloc(b, &b->d.ap_cnt, nch));
     }
@@ -1462,6 +1500,7 @@ md_status md_integrate(md_box* b, double dt, int64_t nsteps, int32_t ckpt_every,
     const int energy = thermo_out ? 1 : 0;
     const int64_t chunk = record ? ckpt_every : b->chunk_steps;
     if (energy) CKS(ensure_thermo(b, std::min(nsteps, chunk)));
+    CKS(ensure_tstat(b, std::min(nsteps, chunk)));
     bool out_dev = energy && is_device_ptr(thermo_out);
     int64_t done = 0;
     int retries = 0;

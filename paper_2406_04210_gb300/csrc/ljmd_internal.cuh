@@ -47,6 +47,7 @@
 #define LJ_KIN_WARPS (LJ_CHUNK / 32)   // E_kin shares per chunk (one per warp of the integrator)
 #define LJ_SPREAD_THREADS 64   // threads of its small work items (16 particles)
 #define LJ_SPREAD_SHARES (LJ_CHUNK * 4 / 32)   // their (E_pot, W) shares per chunk: one per warp
+#define LJ_ALL_SHARES 8         // (E_pot, W) shares per chunk of the FP32 all-pairs kernel (one per 16 particles)
 #define LJ_THERMO_THREADS 256  // threads of the energy reduction
 #define LJ_THERMO_CHUNKS 256   // chunks of one energy-reduction item
 #define LJ_LIST_THREADS 256    // threads of the list-build kernel
@@ -128,6 +129,7 @@ struct LJDev {
 // Everything a kernel needs, passed by value.
 struct BoxDev {
     int nrep, np, nchunk, ncell;
+    int n1;                    // one replica: its particles
     int K;                     // list capacity (slots per particle; a multiple of LJ_ROW_BLOCK)
     int prec;                  // md_precision
     int nt;                    // species count
@@ -197,6 +199,11 @@ struct BoxDev {
     unsigned tstat_thr;
     unsigned long long tstat_seed;
     const double* tstat_T;
+    // collisions drawn ahead for the steps of a graph (null: drawn in the
+    // integrator): per step np / 32 words of hit bits and np new velocities,
+    // by slot before any sort (p_off + index inside the replica)
+    const unsigned* tstat_hit;
+    const double* tstat_g;
     long long* step_ctr;       // steps since md_set_thermostat (device word)
     int all_pairs;             // every cutoff infinite: forces over all pairs, no lists
     int force_tiles;           // FP32 list forces by the tiled kernel (k_force_tile_f32)
@@ -204,14 +211,14 @@ struct BoxDev {
     const int4* brick;         // its work items: (replica, first cell x, y, z) of bricks of up to
     int nbrick;                // rep.br[0] x br[1] x br[2] cells
     int order;                 // order inside a cell: 0 z runs (LJ_ORDER_ZRUN), 1 Morton sub-cells
-    int ap_js;                 // all pairs: slices of the j range per chunk
-    float4* ap_part;           // [slice][slot] partial FP32 forces
+    int ap_js;                 // all pairs, FP64: slices of the j range per chunk
     double* ap_part64;         // [slice][3][slot] partial FP64 forces
     double* ap_pe;             // [chunk * ap_js + slice][2] partial E_pot, W
     unsigned* ap_cnt;          // per chunk: slices done (the last one resets)
     // per-chunk FP64 partial sums
     double* part_f;            // [(chunk*pf_stride + q)*2 + 0] = E_pot share, [+1] = W share
-    int pf_stride;             // (E_pot, W) shares per chunk: one per warp of the list kernels, 1 for all pairs
+    int pf_stride;             // (E_pot, W) shares per chunk: one per warp of the list kernels, one per work
+                               // item of the all-pairs kernels
     int pf_ds;                 // 1: each share is a double-single pair (hi, lo floats in the double's
                                // 8 bytes: the FP32 list kernels), 0: a double; the tiled kernel
                                // leaves pf_stride shares per brick instead of per chunk
@@ -311,6 +318,14 @@ __device__ __forceinline__ bool box_needs_rebuild(const BoxDev& b)
 __device__ __forceinline__ bool rep_needs_rebuild(const BoxDev& b, int r)
 {
     return b.rebuild_req[r] != 0 || __uint_as_float(b.disp_max[r]) > b.disp_thr2;
+}
+
+// Particle work item w: one replica's follow from the index, sparing its
+// kernels a dependent load before the first useful one.
+__device__ __forceinline__ int4 chunk_of(const BoxDev& b, int w)
+{
+    if (b.nrep == 1) return make_int4(0, w * LJ_CHUNK, min((w + 1) * LJ_CHUNK, b.n1), w);
+    return b.chunk[w];
 }
 
 // floor(x / L); the FP64 division (slow on this GPU) only where the quotient
@@ -592,6 +607,8 @@ cudaError_t launch_pair_hist_grad(const BoxDev& b, int nbins, double rhist, doub
 // cond: condition of the step graph's list-update node, set when a build is due (0: none)
 cudaError_t launch_integrate(const BoxDev& b, int mode, int energy, double dt, int sidx,
                              cudaGraphConditionalHandle cond, Launch l);
+// the thermostat's collisions of the next nsteps steps into hit and g
+cudaError_t launch_tstat_draw(const BoxDev& b, int nsteps, unsigned* hit, double* g, Launch l);
 cudaError_t launch_step_advance(long long* ctr, long long n, cudaStream_t s);
 cudaError_t launch_upload(const BoxDev& b, const double* pos, const double* vel,
                           const int* type, int set_vel, Launch l);
