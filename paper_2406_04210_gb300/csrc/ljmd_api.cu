@@ -1376,6 +1376,7 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
         h.dsig[k] = sigma[k];
     }
     CK(b, cudaMemcpyAsync(b->d_lj, &h, sizeof h, cudaMemcpyHostToDevice, b->stream));
+    const BoxDev before = b->d;
     b->nt = nt;
     b->d.nt = nt;
     b->d.c1 = make_float4(h.c12[0], h.c6[0], h.e12[0], h.e6[0]);
@@ -1394,6 +1395,11 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
     d.band = (float)(1.5e-4 * rl * rl);
     double thr = 0.5 * skin - 2e-6;
     d.disp_thr2 = thr > 0 ? (float)(thr * thr) : 0.0f;
+    // captured step graphs hold these by value
+    auto same4 = [](const float4& x, const float4& y) { return x.x == y.x && x.y == y.y && x.z == y.z && x.w == y.w; };
+    if (before.nt != d.nt || !same4(before.c1, d.c1) || before.rc2_1 != d.rc2_1 || before.esh_1 != d.esh_1 ||
+        before.nh_1 != d.nh_1 || before.kap_1 != d.kap_1 || before.rl2 != d.rl2 || before.disp_thr2 != d.disp_thr2)
+        invalidate_graphs(b);
     if (grid_changes) CKS(make_grid(b));
     b->lj_set = true;
     b->rec_valid = false;
