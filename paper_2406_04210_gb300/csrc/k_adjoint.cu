@@ -27,51 +27,246 @@ __device__ __forceinline__ double warp_sum_d(double v)
     return v;
 }
 
-// u (user order, FP64 n x 3) -> slot order FP32 for the HVP kernel, after
-// the adjoint half-update of this step:
+// The tape of a replayed segment: state m's FP32 offsets in slot m, its slot ->
+// user map and lists in slot idx[m] (the state at which they were last built).
+struct TapeLists {
+    const int* uid;
+    const int* count;
+    const uint32_t* nbr;
+};
+__device__ __forceinline__ TapeLists tape_lists(const Tape& t, int m)
+{
+    const char* s = t.base + (size_t)t.idx[m] * t.stride;
+    return TapeLists{reinterpret_cast<const int*>(s + t.o_uid), reinterpret_cast<const int*>(s + t.o_cnt),
+                     reinterpret_cast<const uint32_t*>(s + t.o_nbr)};
+}
+__device__ __forceinline__ const float4* tape_posq(const Tape& t, int m)
+{
+    return reinterpret_cast<const float4*>(t.base + (size_t)m * t.stride);
+}
+
+// State m of the replay into the tape, between the step's list update and its
+// force kernel: the offsets always, the maps and lists only when this step
+// built them (the box-wide rebuild word is still up) or it is the segment's
+// first.  (Copied at every step the lists were 28 MB of traffic each at N =
+// 32,000, behind four copy nodes per step.)
+__global__ void __launch_bounds__(256) k_tape_save(BoxDev b, Tape t, int m)
+{
+    const bool fresh = m == 0 || *b.any_req != 0;
+    char* s = t.base + (size_t)m * t.stride;
+    const int i0 = blockIdx.x * blockDim.x + threadIdx.x, di = gridDim.x * blockDim.x;
+    for (int i = i0; i < b.np; i += di) {
+        reinterpret_cast<float4*>(s)[i] = b.posq[i];
+        if (fresh) {
+            reinterpret_cast<int*>(s + t.o_uid)[i] = b.uid[i];
+            reinterpret_cast<int*>(s + t.o_cnt)[i] = b.nbr_count[i];
+        }
+    }
+    if (fresh) {
+        const uint4* from = reinterpret_cast<const uint4*>(b.nbr);
+        uint4* to = reinterpret_cast<uint4*>(s + t.o_nbr);
+        const size_t n = (size_t)b.np * (size_t)b.K / 4;
+#pragma unroll 4
+        for (size_t i = i0; i < n; i += di) to[i] = from[i];
+    }
+    if (i0 == 0) t.idx[m] = fresh ? m : t.idx[m - 1];
+}
+
+// The particles' offsets and adjoint vectors u side by side, 32 bytes each (a
+// neighbour's two are one sector), u from the adjoint state (user order, FP64
+// n x 3) after the half-update of this step:
 //   pre = 1: lx <- lx - h/2 g;  lv <- lv + h lx;  u = lv   (then HVP of u)
 //   pre = 0: u = lv                                         (first state)
-__global__ void __launch_bounds__(LJ_CHUNK) k_adj_pre(BoxDev b, double* lx, double* lv, const double* g,
-                                                      float4* u_slot, double h, int pre)
+__global__ void __launch_bounds__(LJ_CHUNK) k_adj_pre(BoxDev b, Tape t, int m, double* lx, double* lv, const double* g,
+                                                      float4* pu, double h, int pre)
 {
+    const TapeLists T = tape_lists(t, m);
+    const float4* posq = tape_posq(t, m);
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
-        int4 ch = chunk_of(b, w);
-        int p = ch.y + (int)threadIdx.x;
+        const int4 ch = chunk_of(b, w);
+        const int p = ch.y + (int)threadIdx.x;
         if (p >= ch.z) continue;
-        size_t gu = (size_t)b.uid[p];
-        float uf[3];
+        const float4 pq = posq[p];
+        const size_t gu = (size_t)T.uid[p];
+        double v[3], x[3], gg[3];   // every load before the stores
+#pragma unroll
         for (int c = 0; c < 3; ++c) {
-            double v = lv[3 * gu + c];
-            if (pre) {
-                double x = lx[3 * gu + c] - 0.5 * h * g[3 * gu + c];
-                lx[3 * gu + c] = x;
-                v = v + h * x;
-                lv[3 * gu + c] = v;
-            }
-            uf[c] = (float)v;
+            v[c] = lv[3 * gu + c];
+            x[c] = pre ? lx[3 * gu + c] : 0.0;
+            gg[c] = pre ? g[3 * gu + c] : 0.0;
         }
-        u_slot[p] = make_float4(uf[0], uf[1], uf[2], 0.f);
+        if (pre) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                x[c] = x[c] - 0.5 * h * gg[c];
+                v[c] = v[c] + h * x[c];
+                lx[3 * gu + c] = x[c];
+                lv[3 * gu + c] = v[c];
+            }
+        }
+        pu[2 * (size_t)p] = pq;
+        pu[2 * (size_t)p + 1] = make_float4((float)v[0], (float)v[1], (float)v[2], 0.f);
     }
 }
 
-// HVP and parameter-gradient terms at one state, LJ_TPP threads per particle
-// (as the force kernel), with the adjoint update that follows it:
+// Sums of k_hvp_mono over a thread's pairs in units of c12 = 48 eps sigma^12,
+// with a = -d_ij, b = u_j - u_i: h = sum A (a.b) a - f b = -(H u)_i, and the
+// two moments of the parameter terms, x = sum r^-14 (u_i.a), y = sum r^-8 (u_i.a).
+struct HvpSums {
+    float hx, hy, hz;
+    float2 x, y;
+};
+
+// Two pairs: separations one by one, everything from r^2 on as FP32 pairs.  In
+// units of c12, with nh = -c6 / c12: f = r^-8 (r^-6 + nh), A = r^-10 (14 r^-6 +
+// 8 nh); the cutoff masks 1 / r^2, so a pair beyond it adds zeros.
+__device__ __forceinline__ void hvp_pair2(unsigned e0, const float4& q0, const float4& u0, unsigned e1,
+                                          const float4& q1, const float4& u1, const float4& pi, const float4& ui,
+                                          const float3& ell, float nh, float rc2, HvpSums& S)
+{
+    const float ax0 = fmaf(entry_unit<0>(e0), ell.x, q0.x - pi.x), ax1 = fmaf(entry_unit<0>(e1), ell.x, q1.x - pi.x);
+    const float ay0 = fmaf(entry_unit<1>(e0), ell.y, q0.y - pi.y), ay1 = fmaf(entry_unit<1>(e1), ell.y, q1.y - pi.y);
+    const float az0 = fmaf(entry_unit<2>(e0), ell.z, q0.z - pi.z), az1 = fmaf(entry_unit<2>(e1), ell.z, q1.z - pi.z);
+    const float2 ax = make_float2(ax0, ax1), ay = make_float2(ay0, ay1), az = make_float2(az0, az1);
+    const float2 bx = make_float2(u0.x - ui.x, u1.x - ui.x), by = make_float2(u0.y - ui.y, u1.y - ui.y),
+                 bz = make_float2(u0.z - ui.z, u1.z - ui.z);
+    const float2 r2 = __ffma2_rn(ax, ax, __ffma2_rn(ay, ay, __fmul2_rn(az, az)));
+    const float2 in = make_float2(r2.x < rc2 ? 1.f : 0.f, r2.y < rc2 ? 1.f : 0.f);
+    const float2 ri = __fmul2_rn(make_float2(rcp_approx(r2.x), rcp_approx(r2.y)), in);
+    const float2 r6 = __fmul2_rn(__fmul2_rn(ri, ri), ri);
+    const float2 r8 = __fmul2_rn(ri, r6);
+    const float2 f = __fmul2_rn(r8, __fadd2_rn(r6, make_float2(nh, nh)));
+    const float2 A = __fmul2_rn(__fmul2_rn(ri, r8), __ffma2_rn(make_float2(14.f, 14.f), r6, make_float2(8.f * nh, 8.f * nh)));
+    const float2 ab = __ffma2_rn(ax, bx, __ffma2_rn(ay, by, __fmul2_rn(az, bz)));
+    const float2 t = __fmul2_rn(A, ab);
+    const float2 nf = make_float2(-f.x, -f.y);
+    const float2 hx = __ffma2_rn(t, ax, __fmul2_rn(nf, bx)), hy = __ffma2_rn(t, ay, __fmul2_rn(nf, by)),
+                 hz = __ffma2_rn(t, az, __fmul2_rn(nf, bz));
+    S.hx += hx.x + hx.y;
+    S.hy += hy.x + hy.y;
+    S.hz += hz.x + hz.y;
+    const float2 ua = __ffma2_rn(make_float2(ui.x, ui.x), ax,
+                                 __ffma2_rn(make_float2(ui.y, ui.y), ay, __fmul2_rn(make_float2(ui.z, ui.z), az)));
+    const float2 v = __fmul2_rn(r8, ua);
+    S.x = __ffma2_rn(r6, v, S.x);
+    S.y = __fadd2_rn(S.y, v);
+}
+
+// HVP and parameter-gradient terms at one state, one species, with the
+// adjoint update that follows it:
 //   g <- H u (user order, FP64);  lx <- lx - h/2 g   (when upd)
-// part_g[chunk * 2P + 0..P-1] accumulates weight * sum lam.dF/deps and
-// [P..2P-1] weight * sum lam.dF/dsigma per symmetric type pair (P = nt * nt
-// slots; the (a, b) and (b, a) terms both land in the slot of min/max) over
-// the states of the reverse sweep; one reduction at its end.  MONO keeps the
-// two sums in registers and accumulates one pair per warp and chunk,
-// part_g[(chunk * LJ_FORCE_WARPS + warp) * 2 + 0/1], with no block barrier
-// (deterministic); otherwise shared-memory atomics, one 2P row per chunk.
-template <bool MONO>
-__global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const float4* __restrict__ u_slot,
+// part_g[2 q], [2 q + 1] accumulate weight * sum lam.dF/deps and lam.dF/dsigma
+// over the states of the reverse sweep, q one row per warp and work item (no
+// block barrier; deterministic), reduced once at its end.
+// Rows, work items and threads per particle as in k_force_f32 (chunks, or 16
+// particles by 64 threads in small boxes), pairs two at a time.  Bound at N =
+// 32,000: the serial row's latency; 36 us with one entry in flight per thread,
+// 17 us (64 registers, so that 2,000 items are one wave: 96 took 22).
+template <int THREADS, int RES>
+__global__ void __launch_bounds__(THREADS, RES) k_hvp_mono(BoxDev b, Tape tp, int m, const float4* __restrict__ pu,
+                                                           double* lx, double* g, double h, int upd,
+                                                           const double* weight, double* part_g)
+{
+    constexpr int PASS = THREADS / LJ_TPP;
+    constexpr int PARTS = THREADS == LJ_SPREAD_THREADS ? LJ_CHUNK / PASS : 1;
+    constexpr int OWN = LJ_CHUNK / PARTS;
+    const TapeLists T = tape_lists(tp, m);
+    const float c12 = b.c1.x, nh = b.nh_1, rc2 = b.rc2_1;
+    const float inv_eps = b.lj->inv_eps[0], inv_sig = b.lj->inv_sig[0];
+    const int K = b.K;
+    const int grp = threadIdx.x / LJ_TPP, l4 = threadIdx.x % LJ_TPP;
+    const unsigned sent = entry_make(13, b.np);
+    float3 ell = make_float3(b.ell1.x, 0.25f * b.ell1.y, 0.0625f * b.ell1.z);   // edges in the digits' units
+    for (int it = blockIdx.x; it < b.nchunk * PARTS; it += gridDim.x) {
+        const int w = it / PARTS, part = it % PARTS;
+        const int4 ch = chunk_of(b, w);
+        if (b.nrep > 1) {
+            const RepDev& R = b.rep[ch.x];
+            ell = make_float3(R.ellf[0], 0.25f * R.ellf[1], 0.0625f * R.ellf[2]);
+        }
+        HvpSums S;
+        S.x = S.y = make_float2(0.f, 0.f);
+        const int first = ch.y + part * OWN, last = min(first + OWN, ch.z);
+        for (int base = first; base < last; base += PASS) {
+            const int p = base + grp;
+            const bool act = p < last;
+            float4 pi = make_float4(0.f, 0.f, 0.f, 0.f), ui = pi;
+            int cnt = 0;
+            size_t gu = 0;
+            const uint4* L = reinterpret_cast<const uint4*>(T.nbr + (size_t)K * p) + l4;
+            uint4 cur = make_uint4(0u, 0u, 0u, 0u);
+            if (act) {
+                pi = pu[2 * (size_t)p];
+                ui = pu[2 * (size_t)p + 1];
+                cnt = min(T.count[p], K);
+                gu = 3 * (size_t)T.uid[p] + l4;
+                cur = __ldcs(L);   // the row's first block (K >= 16 slots), in flight with the count
+            }
+            const bool out = act && l4 < 3;
+            const double lx0 = out && upd ? lx[gu] : 0.0;   // this thread's component of the update
+            const int nblk = (cnt + LJ_ROW_BLOCK - 1) / LJ_ROW_BLOCK;
+            S.hx = S.hy = S.hz = 0.f;
+            auto block4 = [&](const uint4& q) {
+                const float4* n0 = pu + 2 * (size_t)entry_slot(q.x);
+                const float4* n1 = pu + 2 * (size_t)entry_slot(q.y);
+                const float4* n2 = pu + 2 * (size_t)entry_slot(q.z);
+                const float4* n3 = pu + 2 * (size_t)entry_slot(q.w);
+                const float4 p0 = __ldg(n0), v0 = __ldg(n0 + 1), p1 = __ldg(n1), v1 = __ldg(n1 + 1);
+                const float4 p2 = __ldg(n2), v2 = __ldg(n2 + 1), p3 = __ldg(n3), v3 = __ldg(n3 + 1);
+                hvp_pair2(q.x, p0, v0, q.y, p1, v1, pi, ui, ell, nh, rc2, S);
+                hvp_pair2(q.z, p2, v2, q.w, p3, v3, pi, ui, ell, nh, rc2, S);
+            };
+            if (nblk > 0) {
+                for (int blk = 1; blk < nblk; ++blk) {
+                    const uint4 nxt = __ldcs(L + blk * LJ_TPP);   // in flight during this block
+                    block4(cur);
+                    cur = nxt;
+                }
+                const int lim = cnt - ((nblk - 1) * LJ_ROW_BLOCK + 4 * l4);   // entries past the count: the sentinel
+                cur.x = lim > 0 ? cur.x : sent;
+                cur.y = lim > 1 ? cur.y : sent;
+                cur.z = lim > 2 ? cur.z : sent;
+                cur.w = lim > 3 ? cur.w : sent;
+                block4(cur);
+            }
+#pragma unroll
+            for (int o = LJ_TPP / 2; o > 0; o >>= 1) {
+                S.hx += __shfl_xor_sync(0xffffffffu, S.hx, o);
+                S.hy += __shfl_xor_sync(0xffffffffu, S.hy, o);
+                S.hz += __shfl_xor_sync(0xffffffffu, S.hz, o);
+            }
+            if (out) {
+                const double hv = (double)(-c12 * (l4 == 0 ? S.hx : (l4 == 1 ? S.hy : S.hz)));
+                g[gu] = hv;
+                if (upd) lx[gu] = lx0 - 0.5 * h * hv;
+            }
+        }
+        // u_i.dF/deps and u_i.dF/dsigma from the moments
+        const float x = S.x.x + S.x.y, y = nh * (S.y.x + S.y.y);
+        const float2 de = warp_sum_ds2(-c12 * inv_eps * (x + y));
+        const float2 ds = warp_sum_ds2(-6.f * c12 * inv_sig * fmaf(2.f, x, y));
+        if ((threadIdx.x & 31) == 0) {
+            const double wgt = *weight;
+            const size_t q = (size_t)it * (THREADS / 32) + (threadIdx.x >> 5);
+            const double e0 = part_g[2 * q], s0 = part_g[2 * q + 1];
+            part_g[2 * q] = e0 + wgt * ((double)de.x + (double)de.y);
+            part_g[2 * q + 1] = s0 + wgt * ((double)ds.x + (double)ds.y);
+        }
+    }
+}
+
+// The same for several species: part_g[chunk * 2P + 0..P-1] accumulates weight
+// * sum lam.dF/deps and [P..2P-1] weight * sum lam.dF/dsigma per symmetric type
+// pair (P = nt * nt slots; the (a, b) and (b, a) terms both land in the slot of
+// min/max), summed per chunk in shared memory.
+__global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, Tape tp, int m, const float4* __restrict__ pu,
                                                               double* lx, double* g, double h, int upd,
                                                               const double* weight, double* part_g)
 {
     __shared__ float4 s_c[LJ_MAXT * LJ_MAXT];     // c12, c6, a12, a6
     __shared__ float4 s_g[LJ_MAXT * LJ_MAXT];     // g12, g6, 1/eps, rc2
     __shared__ float s_acc[2 * LJ_MAXT * LJ_MAXT];
+    const TapeLists T = tape_lists(tp, m);
     const LJDev* lj = b.lj;
     const int nt = lj->nt;
     const int P = nt * nt;
@@ -79,12 +274,8 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const fl
         s_c[k] = make_float4(lj->c12[k], lj->c6[k], lj->a12[k], lj->a6[k]);
         s_g[k] = make_float4(lj->g12[k], lj->g6[k], lj->inv_eps[k], lj->rc2[k]);
     }
-    __syncthreads();   // the pair tables are complete
-    const float4 mc = make_float4(lj->c12[0], lj->c6[0], lj->a12[0], lj->a6[0]);
-    const float4 mg = make_float4(lj->g12[0], lj->g6[0], lj->inv_eps[0], lj->rc2[0]);
     const int K = b.K;
     const int grp = threadIdx.x / LJ_TPP, l8 = threadIdx.x % LJ_TPP;
-    const float4* __restrict__ posq = b.posq;
     int cur_r = -1;
     float3 ell = make_float3(0.f, 0.f, 0.f);
     for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
@@ -95,45 +286,34 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const fl
             ell = make_float3(R.ellf[0], 0.25f * R.ellf[1], 0.0625f * R.ellf[2]);   // edges in the digits' units
             cur_r = r;
         }
-        if (!MONO) {   // per-chunk species-pair sums in shared memory
-            __syncthreads();
-            for (int k = threadIdx.x; k < 2 * P; k += blockDim.x) s_acc[k] = 0.f;
-            __syncthreads();
-        }
-        float ge = 0.f, gs = 0.f;
+        __syncthreads();
+        for (int k = threadIdx.x; k < 2 * P; k += blockDim.x) s_acc[k] = 0.f;
+        __syncthreads();
         for (int base = ch.y; base < ch.z; base += LJ_FORCE_THREADS / LJ_TPP) {
             const int p = base + grp;
             const bool act = p < ch.z;
             float4 pi = make_float4(0.f, 0.f, 0.f, 0.f), ui = pi;
             int cnt = 0;
             if (act) {
-                pi = posq[p];
-                ui = u_slot[p];
-                cnt = min(b.nbr_count[p], K);
+                pi = pu[2 * (size_t)p];
+                ui = pu[2 * (size_t)p + 1];
+                cnt = min(T.count[p], K);
             }
             const int ti = __float_as_int(pi.w);
-            const uint32_t* L = b.nbr + (size_t)K * p;
+            const uint32_t* L = T.nbr + (size_t)K * p;
             float hx = 0.f, hy = 0.f, hz = 0.f;
             for (int s = l8; s < cnt; s += LJ_TPP) {
                 const unsigned ent = __ldcs(L + s);
-                const int j = (int)entry_slot(ent);
-                const float4 pj = __ldg(posq + j);
-                const float4 uj = __ldg(u_slot + j);
+                const size_t j = entry_slot(ent);
+                const float4 pj = __ldg(pu + 2 * j);
+                const float4 uj = __ldg(pu + 2 * j + 1);
                 // d = (o_i - o_j) - (dx, dy, dz) * ell, one rounding per component
                 const float dx = fmaf(-entry_unit<0>(ent), ell.x, pi.x - pj.x);
                 const float dy = fmaf(-entry_unit<1>(ent), ell.y, pi.y - pj.y);
                 const float dz = fmaf(-entry_unit<2>(ent), ell.z, pi.z - pj.z);
                 const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                float4 c, gg;
-                int pp = 0;
-                if (MONO) {
-                    c = mc;
-                    gg = mg;
-                } else {
-                    pp = ti * nt + __float_as_int(pj.w);
-                    c = s_c[pp];
-                    gg = s_g[pp];
-                }
+                const int tj = __float_as_int(pj.w);
+                const float4 c = s_c[ti * nt + tj], gg = s_g[ti * nt + tj];
                 const bool in = r2 < gg.w;
                 const float r2i = rcp_approx(r2);
                 const float r6i = r2i * r2i * r2i;
@@ -148,16 +328,10 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const fl
                 hy = fmaf(Adu, dy, fmaf(-f, uy, hy));
                 hz = fmaf(Adu, dz, fmaf(-f, uz, hz));
                 const float ld = fmaf(ui.x, dx, fmaf(ui.y, dy, ui.z * dz));
-                const float dsg = in ? r2i * r6i * fmaf(gg.x, r6i, -gg.y) * ld : 0.f;
-                const float dep = f * gg.z * ld;
-                if (MONO) {
-                    ge += dep;
-                    gs += dsg;
-                } else if (in) {
-                    const int a = ti, bb = __float_as_int(pj.w);
-                    const int q = (a < bb ? a : bb) * nt + (a < bb ? bb : a);
-                    atomicAdd(&s_acc[q], dep);
-                    atomicAdd(&s_acc[P + q], dsg);
+                if (in) {
+                    const int q = (ti < tj ? ti : tj) * nt + (ti < tj ? tj : ti);
+                    atomicAdd(&s_acc[q], f * gg.z * ld);
+                    atomicAdd(&s_acc[P + q], r2i * r6i * fmaf(gg.x, r6i, -gg.y) * ld);
                 }
             }
 #pragma unroll
@@ -167,7 +341,7 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const fl
                 hz += __shfl_xor_sync(0xffffffffu, hz, o);
             }
             if (act && l8 == 0) {
-                const size_t gu = (size_t)b.uid[p];
+                const size_t gu = (size_t)T.uid[p];
                 const double hv[3] = {hx, hy, hz};
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
@@ -177,19 +351,8 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_hvp_f32(BoxDev b, const fl
             }
         }
         const double wgt = *weight;
-        if (MONO) {
-            // one (d/deps, d/dsigma) share per warp and chunk (no block barrier)
-            const double de = warp_sum_ds(ge), ds = warp_sum_ds(gs);   // double-single warp sums
-            if ((threadIdx.x & 31) == 0) {
-                const size_t q = (size_t)w * LJ_FORCE_WARPS + (threadIdx.x >> 5);
-                part_g[2 * q] += wgt * de;
-                part_g[2 * q + 1] += wgt * ds;
-            }
-        } else {
-            __syncthreads();
-            for (int k = threadIdx.x; k < 2 * P; k += blockDim.x)
-                part_g[2 * (size_t)P * w + k] += wgt * (double)s_acc[k];
-        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < 2 * P; k += blockDim.x) part_g[2 * (size_t)P * w + k] += wgt * (double)s_acc[k];
     }
 }
 
@@ -436,18 +599,28 @@ __global__ void __launch_bounds__(LJ_FORCE_THREADS) k_pair_hist_grad(BoxDev b, i
 
 }  // namespace
 
-cudaError_t launch_adj_pre(const BoxDev& b, double* lx, double* lv, const double* g, float4* u_slot, double h,
-                           int pre, Launch l)
+cudaError_t launch_tape_save(const BoxDev& b, const Tape& t, int m, Launch l)
 {
-    k_adj_pre<<<l.grid, LJ_CHUNK, 0, l.s>>>(b, lx, lv, g, u_slot, h, pre);
+    k_tape_save<<<l.grid, 256, 0, l.s>>>(b, t, m);
     return cudaGetLastError();
 }
 
-cudaError_t launch_hvp(const BoxDev& b, const float4* u_slot, double* lx, double* g, double h, int upd,
-                       const double* weight, double* part_g, Launch l)
+cudaError_t launch_adj_pre(const BoxDev& b, const Tape& t, int m, double* lx, double* lv, const double* g, float4* pu,
+                           double h, int pre, Launch l)
 {
-    if (b.nt == 1) k_hvp_f32<true><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b, u_slot, lx, g, h, upd, weight, part_g);
-    else k_hvp_f32<false><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b, u_slot, lx, g, h, upd, weight, part_g);
+    k_adj_pre<<<l.grid, LJ_CHUNK, 0, l.s>>>(b, t, m, lx, lv, g, pu, h, pre);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hvp(const BoxDev& b, const Tape& t, int m, const float4* pu, double* lx, double* g, double h,
+                       int upd, const double* weight, double* part_g, int spread, Launch l)
+{
+    if (b.nt != 1)
+        k_hvp_f32<<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b, t, m, pu, lx, g, h, upd, weight, part_g);
+    else if (spread)
+        k_hvp_mono<LJ_SPREAD_THREADS, 16><<<l.grid, LJ_SPREAD_THREADS, 0, l.s>>>(b, t, m, pu, lx, g, h, upd, weight, part_g);
+    else
+        k_hvp_mono<LJ_FORCE_THREADS, 3><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b, t, m, pu, lx, g, h, upd, weight, part_g);
     return cudaGetLastError();
 }
 

@@ -153,6 +153,12 @@ struct md_box {
     char* d_tape = nullptr;
     size_t tape_step_bytes = 0;
     int tape_cap = 0;
+    int* d_tape_idx = nullptr;
+    // graphs of md_adjoint: the reverse sweep's four forms, then the replay
+    cudaGraphExec_t adj_exec[5] = {};
+    int64_t adj_kernels[5] = {};
+    int adj_k = 0;
+    double adj_h = 0.0;
     double* d_parth = nullptr;
     double* d_hist = nullptr;
     int hist_cap = 0;
@@ -251,6 +257,10 @@ void invalidate_graphs(md_box* b)
         for (auto e : g.ev) cudaEventDestroy(e);
     }
     b->graphs.clear();
+    for (auto& e : b->adj_exec) {
+        if (e) cudaGraphExecDestroy(e);
+        e = nullptr;
+    }
 }
 
 Launch lch(md_box* b) { return Launch{std::max(1, std::min((int)b->d.nchunk, b->nsm * 12)), LJ_CHUNK, b->stream}; }
@@ -782,35 +792,26 @@ md_status snapshot(md_box* b, bool restore)
 // With `ge` set, events bracket every phase of every step (profiling).
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Copy the state a Hessian-vector product needs (FP32 offsets, slot -> user
-// map, lists) into tape slot m.
-md_status tape_save(md_box* b, int m)
+// Tape slot of one state: FP32 offsets, slot -> user map, list lengths, lists.
+Tape tape_of(md_box* b)
 {
     const size_t np = (size_t)b->np;
-    char* t = b->d_tape + (size_t)m * b->tape_step_bytes;
-    CK(b, cudaMemcpyAsync(t, b->d.posq, np * 16, cudaMemcpyDeviceToDevice, b->stream));
-    t += al256(np * 16);
-    CK(b, cudaMemcpyAsync(t, b->d.uid, np * 4, cudaMemcpyDeviceToDevice, b->stream));
-    t += al256(np * 4);
-    CK(b, cudaMemcpyAsync(t, b->d.nbr_count, np * 4, cudaMemcpyDeviceToDevice, b->stream));
-    t += al256(np * 4);
-    CK(b, cudaMemcpyAsync(t, b->d.nbr, np * (size_t)b->d.K * 4, cudaMemcpyDeviceToDevice, b->stream));
-    return MD_OK;
+    Tape t;
+    t.base = b->d_tape;
+    t.o_uid = al256(np * 16);
+    t.o_cnt = t.o_uid + al256(np * 4);
+    t.o_nbr = t.o_cnt + al256(np * 4);
+    t.stride = t.o_nbr + al256(np * (size_t)b->d.K * 4);
+    t.idx = b->d_tape_idx;
+    return t;
 }
 
-BoxDev tape_view(md_box* b, int m)
+md_status tape_save(md_box* b, int m)
 {
-    const size_t np = (size_t)b->np;
-    BoxDev v = b->d;
-    char* t = b->d_tape + (size_t)m * b->tape_step_bytes;
-    v.posq = reinterpret_cast<float4*>(t);
-    t += al256(np * 16);
-    v.uid = reinterpret_cast<int*>(t);
-    t += al256(np * 4);
-    v.nbr_count = reinterpret_cast<int*>(t);
-    t += al256(np * 4);
-    v.nbr = reinterpret_cast<uint32_t*>(t);
-    return v;
+    const int blocks = (b->np + 255) / 256;
+    CK(b, launch_tape_save(b->d, tape_of(b), m, Launch{std::max(1, std::min(std::max(blocks, b->nsm * 4), b->nsm * 8)), 256, b->stream}));
+    b->launches += 1;
+    return MD_OK;
 }
 
 // The thermostat's draws of n steps ahead of them, while they fit 64 MiB (N =
@@ -897,12 +898,12 @@ md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* rin
         if (cond) CKS(cond_node(b, cond));
         else if (!b->all_pairs) CKS(enqueue_rebuild(b, 0));   // all pairs: the drift keeps offsets wrapped
         CK(b, mark(s, 1, 1, b->stream));
+        if (tape) CKS(tape_save(b, (int)s + 1));   // before the force kernel takes the rebuild word down
         CK(b, join((int)(s & 1)));
         CK(b, mark(s, 2, 0, b->stream));
         CK(b, launch_force(set[s & 1], energy, lforce(b)));
         CK(b, mark(s, 2, 1, b->stream));
         b->launches += 1;
-        if (tape) CKS(tape_save(b, (int)s + 1));
     }
     CK(b, join(0));
     CK(b, join(1));
@@ -1358,6 +1359,7 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
         h.g12[k] = (float)(576.0 * eps[k] * s6 * s6 / sg);
         h.g6[k] = (float)(144.0 * eps[k] * s6 / sg);
         h.inv_eps[k] = (float)(1.0 / eps[k]);
+        h.inv_sig[k] = (float)(1.0 / sg);
         h.c12[k] = (float)(48.0 * eps[k] * s6 * s6);
         h.c6[k] = (float)(24.0 * eps[k] * s6);
         h.e12[k] = (float)(4.0 * eps[k] * s6 * s6);
@@ -1597,19 +1599,27 @@ md_status md_adjoint(md_box* b, const double* lam_x_T, const double* lam_v_T, do
         CKS(dev_alloc(b, &b->d_lx, n3));
         CKS(dev_alloc(b, &b->d_lv, n3));
         CKS(dev_alloc(b, &b->d_g, n3));
-        CKS(dev_alloc(b, &b->d_u, np));
+        CKS(dev_alloc(b, &b->d_u, 2 * (np + 1)));
+        static const float4 far[2] = {{LJ_SENTINEL_OFF, LJ_SENTINEL_OFF, LJ_SENTINEL_OFF, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        CK(b, cudaMemcpyAsync(b->d_u + 2 * np, far, sizeof far, cudaMemcpyHostToDevice, b->stream));   // the sentinel
         CKS(dev_alloc(b, &b->d_theta, 2 * LJ_MAXT * LJ_MAXT));
         CKS(dev_alloc(b, &b->d_wts, 3));
         CKS(dev_alloc(b, &b->d_partg, 2 * (size_t)LJ_MAXT * LJ_MAXT * std::max<size_t>(1, b->chunks.size())));
     }
-    size_t step_bytes = al256(np * 16) + 2 * al256(np * 4) + al256(np * (size_t)b->d.K * 4);
+    const size_t step_bytes = tape_of(b).stride;
     if (b->tape_step_bytes != step_bytes || b->tape_cap < k + 1) {
+        invalidate_graphs(b);   // graphs hold the pointers
         dev_release(b, b->d_tape);
+        dev_release(b, b->d_tape_idx);
         b->d_tape = nullptr;
+        b->d_tape_idx = nullptr;
+        b->tape_cap = 0;
         CKS(dev_alloc(b, &b->d_tape, step_bytes * (size_t)(k + 1), false));
+        CKS(dev_alloc(b, &b->d_tape_idx, (size_t)(k + 1), false));
         b->tape_step_bytes = step_bytes;
         b->tape_cap = k + 1;
     }
+    const Tape tp = tape_of(b);
     const double wts[3] = {0.5 * h, h, 1.0};   // state weights, then the final reduction's
     CK(b, cudaMemcpyAsync(b->d_wts, wts, sizeof wts, cudaMemcpyHostToDevice, b->stream));
     CK(b, cudaMemsetAsync(b->d_theta, 0, sizeof(double) * 2 * LJ_MAXT * LJ_MAXT, b->stream));
@@ -1626,60 +1636,62 @@ md_status md_adjoint(md_box* b, const double* lam_x_T, const double* lam_v_T, do
     CK(b, cudaStreamSynchronize(b->stream));   // host inputs staged before reuse
     // keep the current (end of run) state; restored at the end
     CKS(snapshot(b, false));
-    Launch l = lch(b);
-    Launch lf = lforce(b);
-    // parameter-gradient rows: one per chunk, one per warp and chunk for one species
-    const int nchunk = (int)b->chunks.size() * (P == 1 ? LJ_FORCE_WARPS : 1);
+    const Launch l = lch(b);
+    // the HVP kernel's work items follow the force kernel's rule
+    const int spread = P == 1 && spread_force(b) ? 1 : 0;
+    const int items = b->d.nchunk * (spread ? LJ_CHUNK * LJ_TPP / LJ_SPREAD_THREADS : 1);
+    const Launch lf{std::max(1, std::min(items, b->nsm * (spread ? 32 : 6))), 0, b->stream};
+    // parameter-gradient rows: one per chunk, one per warp and item for one species
+    const int nrow = (int)b->chunks.size() * (P != 1 ? 1 : spread ? LJ_SPREAD_SHARES : LJ_FORCE_WARPS);
     const int twoP = 2 * P;
     // The replay of a segment (k recorded steps keeping the tape) and its
     // reverse sweep have the same launches for every segment: each is
-    // captured once into a CUDA graph and launched per segment.  The reverse
-    // sweep has four forms: the last segment also starts from the final
-    // state's HVP, and the first weights its last term by h/2.
-    struct Graphs {
-        cudaGraphExec_t g[5] = {};
-        int64_t kernels[5] = {};
-        ~Graphs()
-        {
-            for (auto e : g)
-                if (e) cudaGraphExecDestroy(e);
+    // captured into a CUDA graph once and launched per segment, and kept with
+    // the step graphs for the next call (capturing and instantiating them was
+    // a quarter of a 40-step gradient at N = 32,000).  The reverse sweep has
+    // four forms: the last segment also starts from the final state's HVP,
+    // and the first weights its last term by h/2.
+    if (b->adj_k != k || b->adj_h != h) {
+        for (auto& e : b->adj_exec) {
+            if (e) cudaGraphExecDestroy(e);
+            e = nullptr;
         }
-    } graphs;
+        b->adj_k = k;
+        b->adj_h = h;
+    }
     auto capture = [&](int slot, auto&& fn) -> md_status {
         const int64_t l0 = b->launches;
         CK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
         md_status st = fn();
         cudaGraph_t graph = nullptr;
         cudaError_t ce = cudaStreamEndCapture(b->stream, &graph);
-        graphs.kernels[slot] = b->launches - l0;
+        b->adj_kernels[slot] = b->launches - l0;
         b->launches = l0;
         if (st != MD_OK) {
             if (graph) cudaGraphDestroy(graph);
             return st;
         }
         if (ce != cudaSuccess) return cuda_fail(b, ce, "cudaStreamEndCapture");
-        ce = cudaGraphInstantiate(&graphs.g[slot], graph, 0);
+        ce = cudaGraphInstantiate(&b->adj_exec[slot], graph, 0);
         cudaGraphDestroy(graph);
-        if (ce != cudaSuccess) return cuda_fail(b, ce, "cudaGraphInstantiate");
+        if (ce != cudaSuccess) {
+            b->adj_exec[slot] = nullptr;
+            return cuda_fail(b, ce, "cudaGraphInstantiate");
+        }
         return MD_OK;
     };
     auto launch = [&](int slot) -> md_status {
-        CK(b, cudaGraphLaunch(graphs.g[slot], b->stream));
-        b->launches += graphs.kernels[slot];
+        CK(b, cudaGraphLaunch(b->adj_exec[slot], b->stream));
+        b->launches += b->adj_kernels[slot];
         return MD_OK;
     };
     auto reverse = [&](bool last, bool first) -> md_status {
         for (int m = k; m >= 0; --m) {
-            BoxDev v = tape_view(b, m);
-            if (m == k) {
-                if (!last) continue;   // this state's HVP was done at m = 0 of the next segment
-                CK(b, launch_adj_pre(v, b->d_lx, b->d_lv, b->d_g, b->d_u, h, 0, l));
-                CK(b, launch_hvp(v, b->d_u, b->d_lx, b->d_g, h, 0, b->d_wts, b->d_partg, lf));
-            } else {
-                CK(b, launch_adj_pre(v, b->d_lx, b->d_lv, b->d_g, b->d_u, h, 1, l));
-                CK(b, launch_hvp(v, b->d_u, b->d_lx, b->d_g, h, 1, b->d_wts + ((first && m == 0) ? 0 : 1),
-                                 b->d_partg, lf));
-            }
+            if (m == k && !last) continue;   // this state's HVP was done at m = 0 of the next segment
+            const int upd = m == k ? 0 : 1;
+            CK(b, launch_adj_pre(b->d, tp, m, b->d_lx, b->d_lv, b->d_g, b->d_u, h, upd, l));
+            CK(b, launch_hvp(b->d, tp, m, b->d_u, b->d_lx, b->d_g, h, upd,
+                             b->d_wts + (m == k || (first && m == 0) ? 0 : 1), b->d_partg, spread, lf));
             b->launches += 2;
         }
         return MD_OK;
@@ -1690,7 +1702,7 @@ md_status md_adjoint(md_box* b, const double* lam_x_T, const double* lam_v_T, do
         CKS(clear_err(b));
         CKS(replay_lists(b));
         CKS(tape_save(b, 0));
-        if (!graphs.g[4]) CKS(capture(4, [&]() { return enqueue_steps(b, k, h, 0, nullptr, nullptr, true); }));
+        if (!b->adj_exec[4]) CKS(capture(4, [&]() { return enqueue_steps(b, k, h, 0, nullptr, nullptr, true); }));
         CKS(launch(4));
         unsigned long long runs = 0;
         CK(b, cudaMemcpyAsync(&runs, b->d_cond_runs, sizeof runs, cudaMemcpyDeviceToHost, b->stream));
@@ -1700,10 +1712,10 @@ md_status md_adjoint(md_box* b, const double* lam_x_T, const double* lam_v_T, do
         b->cond_runs_seen = runs;
         if (e2[0]) return fail(b, MD_ERR_CAPACITY, "md_adjoint: replay of a segment failed");
         const int form = (c == C - 1 ? 1 : 0) | (c == 0 ? 2 : 0);
-        if (!graphs.g[form]) CKS(capture(form, [&]() { return reverse(c == C - 1, c == 0); }));
+        if (!b->adj_exec[form]) CKS(capture(form, [&]() { return reverse(c == C - 1, c == 0); }));
         CKS(launch(form));
     }
-    CK(b, launch_param_reduce(b->d_partg, nchunk, twoP, b->d_wts + 2, b->d_theta, b->stream));
+    CK(b, launch_param_reduce(b->d_partg, nrow, twoP, b->d_wts + 2, b->d_theta, b->stream));
     b->launches += 1;
     // outputs
     bool dx = is_device_ptr(lam_x_0), dv = is_device_ptr(lam_v_0);

@@ -118,7 +118,7 @@ struct LJDev {
     // Hessian and parameter-derivative coefficients (adjoint):
     // A = r2i^2 r6i (a12 r6i - a6); dF/dsigma coefficient r2i r6i (g12 r6i - g6)
     float a12[LJ_MAXT * LJ_MAXT], a6[LJ_MAXT * LJ_MAXT], g12[LJ_MAXT * LJ_MAXT], g6[LJ_MAXT * LJ_MAXT];
-    float inv_eps[LJ_MAXT * LJ_MAXT];
+    float inv_eps[LJ_MAXT * LJ_MAXT], inv_sig[LJ_MAXT * LJ_MAXT];
     float sig2[LJ_MAXT * LJ_MAXT], eps48[LJ_MAXT * LJ_MAXT], eps4[LJ_MAXT * LJ_MAXT];
     float rc2[LJ_MAXT * LJ_MAXT], shift[LJ_MAXT * LJ_MAXT];
     double dsig2[LJ_MAXT * LJ_MAXT], deps48[LJ_MAXT * LJ_MAXT], deps4[LJ_MAXT * LJ_MAXT];
@@ -590,12 +590,20 @@ cudaError_t launch_thermo(const BoxDev& b, double* out, int with_kin, Launch l);
 int force_tile_blocks_per_sm(int mono);   // resident blocks of the tiled force kernel
 
 // k_adjoint.cu
-cudaError_t launch_adj_pre(const BoxDev& b, double* lx, double* lv, const double* g, float4* u_slot, double h,
-                           int pre, Launch l);
-// HVP of u at the state of b, g <- H u, lx <- lx - h/2 g (when upd), and
+struct Tape {
+    char* base;                // slots of `stride` bytes, one per state
+    size_t stride;
+    size_t o_uid, o_cnt, o_nbr;   // slot layout: offsets (at 0), slot -> user map, list lengths, lists
+    int* idx;                  // per state: the slot holding its map and lists
+};
+cudaError_t launch_tape_save(const BoxDev& b, const Tape& t, int m, Launch l);
+// pu: (FP32 offset, u) per slot, one more than np (the sentinel)
+cudaError_t launch_adj_pre(const BoxDev& b, const Tape& t, int m, double* lx, double* lv, const double* g, float4* pu,
+                           double h, int pre, Launch l);
+// HVP of u at tape state m, g <- H u, lx <- lx - h/2 g (when upd), and
 // part_g += *weight * the state's parameter-gradient shares
-cudaError_t launch_hvp(const BoxDev& b, const float4* u_slot, double* lx, double* g, double h, int upd,
-                       const double* weight, double* part_g, Launch l);
+cudaError_t launch_hvp(const BoxDev& b, const Tape& t, int m, const float4* pu, double* lx, double* g, double h,
+                       int upd, const double* weight, double* part_g, int spread, Launch l);
 cudaError_t launch_param_reduce(const double* part_g, int nchunk, int twoP, const double* weight,
                                 double* theta_grad, cudaStream_t s);
 cudaError_t launch_pair_hist(const BoxDev& b, int nbins, double rhist, double width, double rmax, double* part_h,
