@@ -53,6 +53,15 @@ int round_up(int64_t x, int64_t m) { return (int)(((x + m - 1) / m) * m); }
 
 }  // namespace
 
+// Small results come back through the box's pinned buffer: a copy to it is
+// asynchronous, where one to pageable memory makes the driver stage it and
+// wait each time.
+struct PinnedBack {
+    int err[4];
+    unsigned long long runs;
+    double th[1];   // 4 per replica
+};
+
 struct md_box {
     int device = 0;
     int nsm = 152;
@@ -162,6 +171,7 @@ struct md_box {
     double* d_parth = nullptr;
     double* d_hist = nullptr;
     int hist_cap = 0;
+    PinnedBack* pin = nullptr;   // pinned host memory
     std::string err;
 };
 
@@ -358,11 +368,10 @@ md_status enter(md_box* b)
     return MD_OK;
 }
 
-// Finish: wait for the box's work; the caller's stream is ordered after it.
+// Finish: wait for the box's work (so that whatever the caller queues next,
+// on any stream, comes after it).
 md_status leave(md_box* b)
 {
-    CK(b, cudaEventRecord(b->ev, b->stream));
-    CK(b, cudaStreamWaitEvent(b->ustream, b->ev, 0));
     CK(b, cudaStreamSynchronize(b->stream));
     return MD_OK;
 }
@@ -385,10 +394,17 @@ md_status input_ptr(md_box* b, const void* src, size_t bytes, const void** dev, 
     return MD_OK;
 }
 
+md_status queue_err(md_box* b)
+{
+    CK(b, cudaMemcpyAsync(b->pin->err, b->d.err, 3 * sizeof(int), cudaMemcpyDeviceToHost, b->stream));
+    return MD_OK;
+}
+
 md_status read_err(md_box* b, int* err2)
 {
-    CK(b, cudaMemcpyAsync(err2, b->d.err, 3 * sizeof(int), cudaMemcpyDeviceToHost, b->stream));
+    CKS(queue_err(b));
     CK(b, cudaStreamSynchronize(b->stream));
+    std::memcpy(err2, b->pin->err, 3 * sizeof(int));
     return MD_OK;
 }
 
@@ -511,11 +527,9 @@ md_status enqueue_force(md_box* b, int energy, double* thermo_out_dev)
 
 md_status set_all_rebuild(md_box* b)
 {
-    std::vector<int> ones(b->nrep, 1);
-    CK(b, cudaMemcpyAsync(b->d.rebuild_req, ones.data(), sizeof(int) * b->nrep,
-                          cudaMemcpyHostToDevice, b->stream));
-    CK(b, cudaMemcpyAsync(b->d.any_req, ones.data(), sizeof(int), cudaMemcpyHostToDevice, b->stream));
-    CK(b, cudaStreamSynchronize(b->stream));   // `ones` is pageable and local
+    // any nonzero word asks for a build
+    CK(b, cudaMemsetAsync(b->d.rebuild_req, 1, sizeof(int) * b->nrep, b->stream));
+    CK(b, cudaMemsetAsync(b->d.any_req, 1, sizeof(int), b->stream));
     return MD_OK;
 }
 
@@ -1166,6 +1180,8 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
         // that work queued on the caller's stream still uses, and the box
         // clears and fills it on its own stream
         CKS(enter(b));
+        CK(b, cudaHostAlloc(reinterpret_cast<void**>(&b->pin), sizeof(PinnedBack) + 4 * sizeof(double) * (size_t)nrep,
+                            cudaHostAllocDefault));
         BoxDev& d = b->d;
         copy_reps_to(b, d);
         size_t np3 = 3 * (size_t)b->np;
@@ -1276,6 +1292,7 @@ md_status md_box_destroy(md_box* b)
     invalidate_graphs(b);
     for (auto& a : b->allocs) raw_free(b, a.p);
     b->allocs.clear();
+    if (b->pin) cudaFreeHost(b->pin);
     if (b->ev) cudaEventDestroy(b->ev);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
     for (cudaEvent_t ev : b->ev_join)
@@ -1468,12 +1485,10 @@ md_status md_force(md_box* b, double* force_out, double* epot, double* virial)
             CK(b, cudaMemcpyAsync(force_out, b->d_stage, fb, cudaMemcpyDeviceToHost, b->stream));
         }
     }
-    std::vector<double> th(4 * (size_t)b->nrep);
-    CK(b, cudaMemcpyAsync(th.data(), b->d_thermo, sizeof(double) * th.size(), cudaMemcpyDeviceToHost,
-                          b->stream));
+    const double* th = b->pin->th;
+    CK(b, cudaMemcpyAsync(b->pin->th, b->d_thermo, 4 * sizeof(double) * b->nrep, cudaMemcpyDeviceToHost, b->stream));
     int e2[3];
-    CKS(read_err(b, e2));
-    CKS(leave(b));
+    CKS(read_err(b, e2));   // waits for everything above
     for (int r = 0; r < b->nrep; ++r) {
         if (epot) epot[r] = th[4 * r + 0];
         if (virial) virial[r] = th[4 * r + 2];
@@ -1525,11 +1540,17 @@ md_status md_integrate(md_box* b, double dt, int64_t nsteps, int32_t ckpt_every,
         cudaGraphExec_t g;
         CKS(get_graph(b, n, dt, energy, &g));
         CK(b, cudaGraphLaunch(g, b->stream));
-        unsigned long long runs = 0;
-        CK(b, cudaMemcpyAsync(&runs, b->d_cond_runs, sizeof runs, cudaMemcpyDeviceToHost, b->stream));
+        if (energy && out_dev)   // ahead of the wait; a repeated graph writes it again
+            CK(b, cudaMemcpyAsync(thermo_out + (size_t)done * b->nrep * 4, b->d_thermo, sizeof(double) * n * b->nrep * 4,
+                                  cudaMemcpyDeviceToDevice, b->stream));
+        b->pin->runs = b->cond_runs_seen;
+        if (b->use_cond)
+            CK(b, cudaMemcpyAsync(&b->pin->runs, b->d_cond_runs, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                  b->stream));
         int e2[3];
         CKS(read_err(b, e2));
         // rebuild sequences the step graph's IF nodes ran
+        const unsigned long long runs = b->pin->runs;
         b->launches += (int64_t)(runs - b->cond_runs_seen) * rebuild_kernels(b, true);
         b->cond_runs_seen = runs;
         for (auto& ge : b->graphs)
@@ -1562,12 +1583,9 @@ md_status md_integrate(md_box* b, double dt, int64_t nsteps, int32_t ckpt_every,
             CKS(leave(b));
             return fail(b, MD_ERR_NONFINITE, "md_integrate: non-finite force");
         }
-        if (energy) {
-            size_t cnt = (size_t)n * b->nrep * 4;
-            double* dst = thermo_out + (size_t)done * b->nrep * 4;
-            CK(b, cudaMemcpyAsync(dst, b->d_thermo, sizeof(double) * cnt,
-                                  out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, b->stream));
-        }
+        if (energy && !out_dev)
+            CK(b, cudaMemcpyAsync(thermo_out + (size_t)done * b->nrep * 4, b->d_thermo, sizeof(double) * n * b->nrep * 4,
+                                  cudaMemcpyDeviceToHost, b->stream));
         done += n;
         b->steps += n;
     }
@@ -1704,10 +1722,13 @@ md_status md_adjoint(md_box* b, const double* lam_x_T, const double* lam_v_T, do
         CKS(tape_save(b, 0));
         if (!b->adj_exec[4]) CKS(capture(4, [&]() { return enqueue_steps(b, k, h, 0, nullptr, nullptr, true); }));
         CKS(launch(4));
-        unsigned long long runs = 0;
-        CK(b, cudaMemcpyAsync(&runs, b->d_cond_runs, sizeof runs, cudaMemcpyDeviceToHost, b->stream));
+        b->pin->runs = b->cond_runs_seen;
+        if (b->use_cond)
+            CK(b, cudaMemcpyAsync(&b->pin->runs, b->d_cond_runs, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                  b->stream));
         int e2[3];
         CKS(read_err(b, e2));
+        const unsigned long long runs = b->pin->runs;
         b->launches += (int64_t)(runs - b->cond_runs_seen) * rebuild_kernels(b, true);   // the replay's rebuilds
         b->cond_runs_seen = runs;
         if (e2[0]) return fail(b, MD_ERR_CAPACITY, "md_adjoint: replay of a segment failed");

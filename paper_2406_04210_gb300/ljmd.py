@@ -196,8 +196,9 @@ class Box:
         pv, kv = _ptr(vel)
         pt, kt = _ptr(type)
         h = ctypes.c_void_p()
+        self._stream = _stream_handle(stream)
         st = L.md_batch_create(ctypes.byref(h), nrep, n.ctypes.data, box.ctypes.data, pt, pp,
-                               pv, PREC[precision], _stream_handle(stream))
+                               pv, PREC[precision], self._stream)
         if st != 0:
             raise MDError(st, "md_batch_create failed")
         self._h = h
@@ -515,6 +516,7 @@ class TrajectoryFn:
             class _F(torch.autograd.Function):
                 @staticmethod
                 def forward(ctx, x0, v0, eps, sigma, box, dt, nsteps, ckpt_every):
+                    _order(box, x0)
                     box.set_lj(float(eps), float(sigma), box._rcut, box._skin, True)
                     box.set_state(x0.detach().contiguous(), v0.detach().contiguous())
                     box.integrate(dt, nsteps, thermo=False, ckpt_every=ckpt_every)
@@ -534,15 +536,28 @@ class TrajectoryFn:
                                          "run's record (another forward, state or parameter change)")
                     gx = torch.zeros_like(gv) if gx is None else gx.contiguous()
                     gv = torch.zeros_like(gx) if gv is None else gv.contiguous()
-                    lx0, lv0, ge, gs = box.adjoint(gx, gv)
-                    dev = gx.device
-                    return (torch.from_numpy(lx0).to(dev), torch.from_numpy(lv0).to(dev),
-                            torch.tensor(ge[0, 0], dtype=torch.float64, device=dev),
-                            torch.tensor(gs[0, 0], dtype=torch.float64, device=dev),
-                            None, None, None, None)
+                    _order(box, gx)
+                    # the gradients stay on the GPU (one species: 1 x 1 parameter gradients)
+                    lx0, lv0 = torch.empty_like(gx), torch.empty_like(gv)
+                    ge, gs = np.zeros((1, 1)), np.zeros((1, 1))
+                    box._check(box._lib.md_adjoint(box._h, gx.data_ptr(), gv.data_ptr(), lx0.data_ptr(),
+                                                   lv0.data_ptr(), ge.ctypes.data, gs.ctypes.data), "md_adjoint")
+                    theta = torch.tensor([ge[0, 0], gs[0, 0]], dtype=torch.float64, device=gx.device)
+                    return lx0, lv0, theta[0], theta[1], None, None, None, None
 
             cls._fn = _F
         return cls._fn.apply(*args)
+
+
+def _order(box, t):
+    """The box's calls are ordered after the stream it was made on: wait for
+    the current stream where that is another one (its tensors, and the memory
+    new tensors get, may still be in use there)."""
+    torch = _torch()
+    if t.is_cuda:
+        s = torch.cuda.current_stream(t.device)
+        if s.cuda_stream != (box._stream or 0):
+            s.synchronize()
 
 
 def _holds(box, x, tol=1e-8):
@@ -550,9 +565,12 @@ def _holds(box, x, tol=1e-8):
     `tol`, minimum image: a list rebuild re-centres the stored offsets, which
     moves the positions by rounding only)."""
     torch = _torch()
+    _order(box, x)
     cur = torch.empty((box.n_total, 3), dtype=torch.float64, device=x.device)
     box._check(box._lib.md_get_state(box._h, cur.data_ptr(), None, None), "md_get_state")
-    L = torch.as_tensor(np.repeat(box.box, box.n, axis=0), dtype=torch.float64, device=x.device)
+    L = torch.as_tensor(box.box, dtype=torch.float64, device=x.device)   # (1, 3) broadcasts
+    if box.nrep > 1:
+        L = torch.repeat_interleave(L, torch.as_tensor(box.n, device=x.device), dim=0)
     d = cur - x.detach().to(torch.float64).reshape(-1, 3)
     d = d - L * torch.round(d / L)
     if d.numel() and float(d.abs().max()) > tol:
@@ -587,9 +605,13 @@ class PairHistLossFn:
                 def backward(ctx, g):
                     nbins, rhist, width, rmax = ctx.args
                     _holds(ctx.box, ctx.saved_tensors[0])
-                    coef = 2.0 * ctx.diff / nbins * float(g)
-                    _, grad = ctx.box.pair_hist(nbins, rhist, width, rmax, coef=coef)
-                    return (torch.from_numpy(grad).to(g.device), None, None, None, None, None, None)
+                    coef = np.ascontiguousarray(2.0 * ctx.diff / nbins * float(g))
+                    width = rhist / nbins if width is None else width
+                    grad = torch.empty((ctx.box.n_total, 3), dtype=torch.float64, device=g.device)
+                    ctx.box._check(ctx.box._lib.md_pair_hist(
+                        ctx.box._h, int(nbins), float(rhist), float(width), float(rmax), coef.ctypes.data, None,
+                        grad.data_ptr()), "md_pair_hist")
+                    return grad, None, None, None, None, None, None
 
             cls._fn = _F
         return cls._fn.apply(*args)
