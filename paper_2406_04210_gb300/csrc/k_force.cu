@@ -751,37 +751,154 @@ __device__ __forceinline__ double rcp_f64(double x)
     return fma(y, fma(e, e, e), y);
 }
 
+// ---- 64-bit integer pair arithmetic of one species (k_force_f64) ----
+// The FP64 pipe has 2 lanes per clock and SM; a 64 x 64 -> 128-bit product
+// takes the integer pipes ~5 clocks per warp against 16 for one FP64
+// instruction.  So the pair terms are block fixed-point numbers whose common
+// exponents are set, per particle and queue drain, by the closest queued
+// pair (from the FP32 scan): R = r^2 (units of 2^(sR - 2q)) is at least 2^lam
+// for all of them, and
+//   Y  = 2^(62 + lam) / R             t   = 1 / r^2 = Y 2^tau
+//   T2 = Y^2 2^-62, T3 = T2 Y 2^-62   t^3 = T3 2^(124 + 3 tau)
+//   T4 = T2^2 2^-62                   t^4 = T4 2^(186 + 4 tau)
+//   g  = (T3 >> u) - Kg               t^3 - K, K = 1 / (2 sigma^6), units 2^(u + 124 + 3 tau)
+//   f  = T4 |g| 2^-(63 - z)           f / c12 = t^4 (t^3 - K)
+// are all below 2^62 and lose at most ~2^-57 of the closest pair's term.
+// Forces and the virial are summed as 128-bit integers (no rounding at all)
+// and turned into FP64 once per particle and drain.  Against exact rational
+// arithmetic, errors are 2.6e-17 of S_i = sum |F_ij| at liquid densities
+// (FP64 arithmetic: 1e-16).  Pairs closer than 2^-4.5 of the cutoff take the
+// FP64 loop.
+typedef unsigned long long u64;
+typedef unsigned __int128 u128;
+
+struct FxSums {
+    __int128 x, y, z, w;   // sum f d, sum t^3 g
+    u128 b;                // sum T3 >> u
+};
+
+// acc += sign * a * c, sign -1 where neg is ~0
+__device__ __forceinline__ void fx_mac(__int128& acc, u64 a, u64 c, long long neg)
+{
+    const u128 m = (u128)(__int128)neg;
+    acc += (__int128)((((u128)a * c) ^ m) - m);
+}
+__device__ __forceinline__ u64 fx_mul62(u64 a, u64 c) { return (u64)(((u128)a * c) >> 62); }
+
+// Exponents of a drain, from the FP32 square r2m of its smallest distance.
+struct FxScale {
+    int lam, tau, u, z;
+    u64 Kg;
+    float ys;   // 2^(lam - 2)
+    __device__ __forceinline__ bool set(const FxDev& fx, float r2m)
+    {
+        const float r = r2m * 0.9990234f;   // below the exact value, whatever the FP32 rounding
+        const int e = (int)(__float_as_uint(r) >> 23) - 127;
+        lam = e + 2 * fx.q - fx.sR;
+        if (lam < 54 || lam > 62 || !(r > 1.0e-37f)) return false;
+        z = (int)(7.0f * __log2f(__uint_as_float((__float_as_uint(r) & 0x007fffffu) | 0x3f800000u)));
+        z = min(max(z, 0), 6);
+        tau = 2 * fx.q - fx.sR - 62 - lam;
+        const int xk = fx.Ke - 124 - 3 * tau;
+        u = min(max(0, xk + 3), 63);
+        Kg = u - xk < 64 ? fx.Km >> (u - xk) : 0ull;   // u - xk >= 3
+        ys = __uint_as_float((unsigned)(lam - 2 + 127) << 23);
+        return xk <= 60;
+    }
+};
+
+// The pair at integer separation (dx, dy, dz).
+template <bool ENERGY>
+__device__ __forceinline__ bool fx_pair(const FxDev& fx, const FxScale& c, long long dx, long long dy, long long dz, FxSums& S)
+{
+    const long long nx = dx >> 63, ny = dy >> 63, nz = dz >> 63;
+    const u64 ax = (u64)((dx ^ nx) - nx), ay = (u64)((dy ^ ny) - ny), az = (u64)((dz ^ nz) - nz);
+    const u64 R = (u64)(((u128)ax * ax + (u128)ay * ay + (u128)az * az) >> fx.sR);
+    if (R >= fx.Rc) return false;
+    // Y: the FP32 reciprocal of R's upper word, then Y (1 + e + e^2)
+    const unsigned rh = (unsigned)(R >> 32), rl = (unsigned)R;
+    const unsigned y0 = (unsigned)(rcp_approx((float)rh) * c.ys);
+    const int s1 = c.lam - 34;   // 20 .. 28
+    const long long e = -(long long)((((u64)rh * y0) << (32 - s1)) + (((u64)rl * y0) >> s1));   // 2^64 (1 - R Y / 2^(62 + lam))
+    const int eh = (int)(e >> 16);
+    const long long cc = e + (((long long)eh * eh) >> 32);
+    const u64 Y = ((u64)y0 << 32) + (u64)((long long)(int)(cc >> 32) * (long long)(int)y0) + __umulhi((unsigned)cc, y0);
+    const u64 T2 = fx_mul62(Y, Y), T3 = fx_mul62(T2, Y), T4 = fx_mul62(T2, T2);
+    const u64 T3u = T3 >> c.u;
+    const long long g = (long long)(T3u - c.Kg), ng = g >> 63;
+    const u64 ag = (u64)((g ^ ng) - ng);
+    const u64 f = (u64)(((u128)T4 * ag) >> (63 - c.z));
+    fx_mac(S.x, f, ax, ng ^ nx);
+    fx_mac(S.y, f, ay, ng ^ ny);
+    fx_mac(S.z, f, az, ng ^ nz);
+    if (ENERGY) {
+        const u128 m = (u128)(__int128)ng;
+        S.w += (__int128)(((((u128)T3 * ag) >> 8) ^ m) - m);
+        S.b += T3u;
+    }
+    return true;
+}
+
+__device__ __forceinline__ __int128 fx_shfl_add(__int128 v, int o)
+{
+    const u64 lo = (u64)v, hi = (u64)((u128)v >> 64);
+    const u64 l2 = __shfl_xor_sync(0xffffffffu, lo, o), h2 = __shfl_xor_sync(0xffffffffu, hi, o);
+    return v + (__int128)(((u128)h2 << 64) | l2);
+}
+// 2^n for -1022 <= n <= 1023
+__device__ __forceinline__ double exp2_int(int n) { return __hiloint2double((n + 1023) << 20, 0); }
+// a 2^n for normal a: the exponent bits moved or, where the result would not
+// be normal, two multiplications
+__device__ __forceinline__ double scale_exp2(double a, int n)
+{
+    const int hi = __double2hiint(a), ex = ((hi >> 20) & 0x7ff) + n;
+    if (ex > 0 && ex < 2047) return __hiloint2double(hi + (n << 20), __double2loint(a));
+    return a * exp2_int(n >> 1) * exp2_int(n - (n >> 1));
+}
+// v a 2^n
+__device__ __forceinline__ double fx_to_double(__int128 v, double a, int n)
+{
+    return fma((double)(long long)(v >> 64), 18446744073709551616.0, (double)(u64)v) * scale_exp2(a, n);
+}
+
 // FP64 pair force (MD_PREC_FP64).  Bound: the FP64 pipe, 2 lanes per clock
-// and SM (64 times fewer than FP32), so what counts is the FP64 instructions
-// per list entry.  LJ_TPP threads per particle scan its row in blocks of 16
-// entries with the FP32 offsets and queue, in shared memory, the entries
-// whose FP32 distance can lie within the cutoff (28 % of a row with skin 0.3
-// does not); the same threads then take the queued entries in FP64: offsets
-// gathered from global memory, the reciprocal by rcp_f64, powers of r^-2 with
+// and SM (64 times fewer than FP32), where FP64 arithmetic is used, the
+// integer multipliers where it is not.  TPP threads per particle scan its
+// row with the FP32 offsets, four entries each and the next four in flight,
+// and queue, in shared memory, the entries whose FP32 distance can lie within
+// the cutoff (28 % of a row with skin 0.3 does not); the same threads then
+// take the queued entries: one species in 64-bit integers (above; offsets
+// from b.offx), else in FP64, the reciprocal by rcp_f64, powers of r^-2 with
 // the pair constants folded, the cutoff decided on r^2's bits: 23 FP64
 // instructions per pair within the cutoff with energies, against ~35 per list
 // entry for a thread per particle with a division.  Work items are quarters
 // of a chunk (32 particles per block), so that 4,000 particles reach 125 SMs.
-// N = 256,000, energies: 1177 us -> 688 us; N = 4,000: a step 127 us -> 48 us.
-constexpr int kF64Parts = LJ_CHUNK * LJ_TPP / LJ_F64_THREADS;   // work items per chunk
+// N = 256,000, energies: 1177 us -> 688 us in FP64, 307 us in integers;
+// N = 4,000: a step 127 us -> 48 us in FP64, 28 us in integers.
+// TPP: 4, or 16 in one-species boxes of at most an item per SM
+// (BoxDev::f64_wide).
+constexpr int kF64Parts = LJ_F64_WARPS;                         // work items, and (E_pot, W) shares, per chunk
 constexpr int kF64Own = LJ_CHUNK / kF64Parts;                   // particles of a work item
-constexpr int kF64Scan = 96;                                    // entries scanned between two drains of the queue
-constexpr int kF64Queue = kF64Scan + 4;                         // a particle's queue (stride 4 banks)
-static_assert(kF64Parts == LJ_F64_WARPS, "one (E_pot, W) share per work item fills a chunk's shares");
-template <bool MONO, bool ENERGY>
-__global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
+template <bool MONO, bool ENERGY, int TPP, int RES>
+__global__ void __launch_bounds__(kF64Own * TPP, RES) k_force_f64(BoxDev b)
 {
+    constexpr int kWarps = kF64Own * TPP / 32;
+    constexpr int kF64Scan = TPP == 4 ? 96 : 128;               // entries scanned between two drains of the queue
+    constexpr int kF64Queue = kF64Scan + 4;                     // a particle's queue (stride 4 banks)
     __shared__ double s_ell[3][4];                     // digit (0, 1, 2) of an entry -> shift (-1, 0, 1) * edge
+    __shared__ long long s_ellx[3][4];                 // the same as integers
     __shared__ uint32_t s_q[kF64Own * kF64Queue];
     __shared__ double2 s_c[LJ_MAXT * LJ_MAXT];         // 48 eps sigma^12, 24 eps sigma^6
     __shared__ double2 s_e[LJ_MAXT * LJ_MAXT];         // 4 eps sigma^12, 4 eps sigma^6
     __shared__ double s_sh[LJ_MAXT * LJ_MAXT];         // energy shift
     __shared__ unsigned long long s_rc2[LJ_MAXT * LJ_MAXT];   // rc^2 (its bits)
     __shared__ float s_near[LJ_MAXT * LJ_MAXT];        // FP32 r^2 below which an entry is queued
-    __shared__ double s_red[2][LJ_F64_WARPS];
+    __shared__ double s_red[2][kWarps];
     const LJDev* lj = b.lj;
-    const int nt = lj->nt;
+    const int nt = b.nt;
     const int np = b.np;
+    const float near1 = b.fx.near;
+    const bool fxon = MONO && b.fx.on;   // integer arithmetic; the tables serve its FP64 loop's rare pairs
     for (int k = threadIdx.x; k < nt * nt; k += blockDim.x) {
         const double s2 = lj->dsig2[k], s6 = s2 * s2 * s2, e4 = lj->deps4[k];
         s_c[k] = make_double2(12.0 * e4 * s6 * s6, 6.0 * e4 * s6);
@@ -791,7 +908,7 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
         s_near[k] = (float)lj->drc2[k] + b.band;       // the margin of the list build's FP64 recheck
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int grp = threadIdx.x / LJ_TPP, l4 = threadIdx.x % LJ_TPP;
+    const int grp = threadIdx.x / TPP, l4 = threadIdx.x % TPP;
     uint32_t* const q = s_q + grp * kF64Queue;
     const float4* __restrict__ posq = b.posq;
     int cur_r = -1;
@@ -803,8 +920,19 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
         __syncthreads();   // the tables are complete; the previous item's sums are read
         if (r != cur_r) {  // block-uniform
             const RepDev& R = b.rep[r];
-            ell = make_float3(R.ellf[0], 0.25f * R.ellf[1], 0.0625f * R.ellf[2]);   // edges in the digits' units
-            if (threadIdx.x < 9) s_ell[threadIdx.x / 3][threadIdx.x % 3] = (double)((int)threadIdx.x % 3 - 1) * R.ell[threadIdx.x / 3];
+            // edges in the digits' units
+            if (b.nrep == 1) ell = make_float3(b.ell1.x, 0.25f * b.ell1.y, 0.0625f * b.ell1.z);
+            else ell = make_float3(R.ellf[0], 0.25f * R.ellf[1], 0.0625f * R.ellf[2]);
+            if (threadIdx.x < 9) {
+                const int c = threadIdx.x / 3, d = (int)threadIdx.x % 3 - 1;
+                if (!fxon || b.nrep > 1) {
+                    const double sh = (double)d * R.ell[c];
+                    s_ell[c][d + 1] = sh;
+                    if (MONO) s_ellx[c][d + 1] = __double2ll_rn(sh * b.fx.scale);
+                } else {
+                    s_ellx[c][d + 1] = (long long)d * (c == 0 ? b.fx.ell[0] : (c == 1 ? b.fx.ell[1] : b.fx.ell[2]));
+                }
+            }
             __syncthreads();
             cur_r = r;
         }
@@ -819,9 +947,15 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
         const bool act = p < ch.z;
         const int pa = act ? p : ch.y;
         const float4 pi = posq[pa];
-        const double xi = b.off[pa], yi = b.off[np + pa], zi = b.off[2 * np + pa];
         const int tb = MONO ? 0 : __float_as_int(pi.w) * nt;
         const int cnt = act ? min(b.nbr_count[p], b.K) : 0;
+        long long xf = 0, yf = 0, zf = 0;
+        if (fxon) {
+            xf = b.offx[pa];
+            yf = b.offx[np + pa];
+            zf = b.offx[2 * np + pa];
+        }
+        bool summed = true;   // MONO: no FP64 partial sums of the four threads (their totals stand in threads 0..3)
         const uint4* row = reinterpret_cast<const uint4*>(b.nbr + (size_t)b.K * pa) + l4;
         double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0, vir = 0.0;
         int npair = 0;   // MONO: pairs within the cutoff (the shift is added once, at the end)
@@ -829,10 +963,14 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
         const int top = __reduce_max_sync(0xffffffffu, cnt);
         for (int s0 = 0; s0 < top; s0 += kF64Scan) {
             int nq = 0;   // queued entries of the particle (the same in its four lanes)
-            for (int s = s0; s < min(s0 + kF64Scan, top); s += LJ_ROW_BLOCK) {
-                uint4 ent = make_uint4(0u, 0u, 0u, 0u);
+            float r2m = 3.0e38f;   // the smallest FP32 r^2 among them
+            const int s1 = min(s0 + kF64Scan, top);
+            uint4 nxt = make_uint4(0u, 0u, 0u, 0u);
+            if (cnt > s0 + 4 * l4) nxt = __ldcs(row + s0 / 4);
+            for (int s = s0; s < s1; s += 4 * TPP) {
+                const uint4 ent = nxt;
                 const int lim = cnt - (s + 4 * l4);   // entries of this thread in the block
-                if (lim > 0) ent = __ldcs(row + s / 4);
+                if (s + 4 * TPP < s1 && lim > 4 * TPP) nxt = __ldcs(row + s / 4 + TPP);   // the next block, in flight
                 const uint32_t en[4] = {ent.x, ent.y, ent.z, ent.w};
                 bool in[4];
                 int c = 0;
@@ -845,29 +983,101 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
                         const float dy = fmaf(-entry_unit<1>(en[u]), ell.y, pi.y - pj.y);
                         const float dz = fmaf(-entry_unit<2>(en[u]), ell.z, pi.z - pj.z);
                         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        in[u] = r2 < s_near[MONO ? 0 : tb + __float_as_int(pj.w)];
+                        in[u] = r2 < (MONO ? near1 : s_near[tb + __float_as_int(pj.w)]);
+                        if (MONO && in[u]) r2m = fminf(r2m, r2);
                     }
                     c += in[u] ? 1 : 0;
                 }
                 int incl = c;
 #pragma unroll
-                for (int o = 1; o < LJ_TPP; o <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, incl, o, LJ_TPP);
+                for (int o = 1; o < TPP; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, incl, o, TPP);
                     if (l4 >= o) incl += t;
                 }
                 int at = nq + incl - c;
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (in[u]) q[at++] = en[u];
-                nq += __shfl_sync(0xffffffffu, incl, LJ_TPP - 1, LJ_TPP);
+                nq += __shfl_sync(0xffffffffu, incl, TPP - 1, TPP);
             }
             __syncwarp();
-            for (int t = l4; t < nq; t += LJ_TPP) {
+            int todo = nq;   // entries for the FP64 loop
+            if (fxon) {
+#pragma unroll
+                for (int o = 1; o < TPP; o <<= 1) r2m = fminf(r2m, __shfl_xor_sync(0xffffffffu, r2m, o));
+                FxScale c;
+                FxSums S;
+                S.x = S.y = S.z = S.w = 0;
+                S.b = 0;
+                const bool fits = nq > 0 && c.set(b.fx, r2m);
+                if (fits) {
+                    // the next entry's offsets are loaded while one is computed
+                    long long px = 0, py = 0, pz = 0;
+                    uint32_t ent = 0;
+                    auto fetch = [&](int t) {
+                        ent = q[t];
+                        const int j = (int)entry_slot(ent);
+                        px = __ldg(&b.offx[j]);
+                        py = __ldg(&b.offx[np + j]);
+                        pz = __ldg(&b.offx[2 * np + j]);
+                    };
+                    if (l4 < nq) fetch(l4);
+                    for (int t = l4; t < nq; t += TPP) {
+                        const long long dx = (xf - px) - s_ellx[0][ent & 3u];
+                        const long long dy = (yf - py) - s_ellx[1][(ent >> 2) & 3u];
+                        const long long dz = (zf - pz) - s_ellx[2][(ent >> 4) & 3u];
+                        if (t + TPP < nq) fetch(t + TPP);
+                        if (fx_pair<ENERGY>(b.fx, c, dx, dy, dz, S) && ENERGY) ++npair;
+                    }
+                    todo = 0;
+                }
+#pragma unroll
+                for (int o = 1; o < TPP; o <<= 1) {
+                    S.x = fx_shfl_add(S.x, o);
+                    S.y = fx_shfl_add(S.y, o);
+                    S.z = fx_shfl_add(S.z, o);
+                    if (ENERGY) {
+                        S.w = fx_shfl_add(S.w, o);
+                        S.b = (u128)fx_shfl_add((__int128)S.b, o);
+                    }
+                }
+                if (fits) {   // thread 0, 1, 2: its component of the force; 3: the virial and the energy
+                    const int g3 = c.u + 124 + 3 * c.tau;   // exponent of g
+                    const __int128 v = l4 == 0 ? S.x : (l4 == 1 ? S.y : (l4 == 2 ? S.z : S.w));
+                    const int n = l4 < 3 ? 63 - c.z + 186 + 4 * c.tau + g3 - b.fx.q : 8 + 124 + 3 * c.tau + g3;
+                    const double d = fx_to_double(v, b.fx.c12, n);
+                    fx = l4 == 0 ? fx + d : fx;
+                    fy = l4 == 1 ? fy + d : fy;
+                    fz = l4 == 2 ? fz + d : fz;
+                    if (ENERGY && l4 == 3) {
+                        vir += d;
+                        e += fma(d, 1.0 / 12.0, -fx_to_double((__int128)S.b, b.fx.hb, g3));
+                    }
+                }
+            }
+            if (todo > 0) summed = false;
+            double xi = 0.0, yi = 0.0, zi = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;   // the FP64 loop's
+            if (todo > 0) {
+                xi = b.off[pa];
+                yi = b.off[np + pa];
+                zi = b.off[2 * np + pa];
+                if (fxon && b.nrep == 1) {
+                    ex = b.rep[0].ell[0];
+                    ey = b.rep[0].ell[1];
+                    ez = b.rep[0].ell[2];
+                } else {
+                    ex = s_ell[0][2];
+                    ey = s_ell[1][2];
+                    ez = s_ell[2][2];
+                }
+            }
+            for (int t = l4; t < todo; t += TPP) {
                 const uint32_t ent = q[t];
                 const int j = (int)entry_slot(ent);
-                const double dx = (xi - __ldg(&b.off[j])) - s_ell[0][ent & 3u];
-                const double dy = (yi - __ldg(&b.off[np + j])) - s_ell[1][(ent >> 2) & 3u];
-                const double dz = (zi - __ldg(&b.off[2 * np + j])) - s_ell[2][(ent >> 4) & 3u];
+                const int gx = (int)(ent & 3u) - 1, gy = (int)((ent >> 2) & 3u) - 1, gz = (int)((ent >> 4) & 3u) - 1;
+                const double dx = (xi - __ldg(&b.off[j])) - (gx == 0 ? 0.0 : (gx > 0 ? ex : -ex));
+                const double dy = (yi - __ldg(&b.off[np + j])) - (gy == 0 ? 0.0 : (gy > 0 ? ey : -ey));
+                const double dz = (zi - __ldg(&b.off[2 * np + j])) - (gz == 0 ? 0.0 : (gz > 0 ? ez : -ez));
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 const int pp = MONO ? 0 : tb + __ldg(&b.type[j]);
                 // r2 < rc2 on their bits (neither is negative), not on the FP64 pipe; a NaN fails
@@ -894,26 +1104,40 @@ __global__ void __launch_bounds__(LJ_F64_THREADS) k_force_f64(BoxDev b)
             }
             __syncwarp();   // the queue is read before it fills again
         }
+        const bool partial = !fxon || __any_sync(0xffffffffu, !summed);   // warp-uniform
+        if (partial) {
 #pragma unroll
-        for (int o = LJ_TPP / 2; o > 0; o >>= 1) {
-            fx += __shfl_xor_sync(0xffffffffu, fx, o);
-            fy += __shfl_xor_sync(0xffffffffu, fy, o);
-            fz += __shfl_xor_sync(0xffffffffu, fz, o);
+            for (int o = TPP / 2; o > 0; o >>= 1) {
+                fx += __shfl_xor_sync(0xffffffffu, fx, o);
+                fy += __shfl_xor_sync(0xffffffffu, fy, o);
+                fz += __shfl_xor_sync(0xffffffffu, fz, o);
+            }
         }
         if (act && l4 < 3) b.force64[(size_t)l4 * np + p] = l4 == 0 ? fx : (l4 == 1 ? fy : fz);
-        if (act && l4 == 3 && !isfinite(fx + fy + fz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
+        if (act && !isfinite(fx + fy + fz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
         if (ENERGY) {
             // one (E_pot, W) share per work item
-            if (MONO) e -= (double)npair * s_sh[0];
-            const double de = warp_sum_d(0.5 * e), dw = warp_sum_d(0.5 * vir);
-            if (lane == 0) {
-                s_red[0][warp] = de;
-                s_red[1][warp] = dw;
+            if (partial) {
+                if (MONO) e -= (double)npair * s_sh[0];
+                const double de = warp_sum_d(0.5 * e), dw = warp_sum_d(0.5 * vir);
+                if (lane == 0) {
+                    s_red[0][warp] = de;
+                    s_red[1][warp] = dw;
+                }
+            } else {   // every particle's sums stand in its thread 3: the energy in 2, then both summed at once
+#pragma unroll
+                for (int o = 1; o < TPP; o <<= 1) npair += __shfl_xor_sync(0xffffffffu, npair, o);
+                const double e3 = __shfl_down_sync(0xffffffffu, e - (double)npair * s_sh[0], 1);
+                double q2 = l4 == 2 ? e3 : vir;
+#pragma unroll
+                for (int o = TPP; o < 32; o <<= 1) q2 += __shfl_xor_sync(0xffffffffu, q2, o);
+                if (lane == 2) s_red[0][warp] = 0.5 * q2;
+                if (lane == 3) s_red[1][warp] = 0.5 * q2;
             }
             __syncthreads();
             if (threadIdx.x < 2) {
                 double t = s_red[threadIdx.x][0];
-                for (int k = 1; k < LJ_F64_WARPS; ++k) t += s_red[threadIdx.x][k];
+                for (int k = 1; k < kWarps; ++k) t += s_red[threadIdx.x][k];
                 b.part_f[2 * (size_t)it + threadIdx.x] = t;
             }
         }
@@ -1363,12 +1587,16 @@ cudaError_t launch_force(const BoxDev& b, int energy, Launch l)
         return cudaGetLastError();
     }
     if (b.prec == 2) {
-        if (b.nt == 1) {
-            if (energy) k_force_f64<true, true><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
-            else k_force_f64<true, false><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
+        const int wide = 16 * kF64Own, narrow = 4 * kF64Own;
+        if (b.nt == 1 && b.f64_wide) {
+            if (energy) k_force_f64<true, true, 16, 1><<<l.grid, wide, 0, l.s>>>(b);
+            else k_force_f64<true, false, 16, 1><<<l.grid, wide, 0, l.s>>>(b);
+        } else if (b.nt == 1) {   // 4 blocks resident: 5 and 6 (fewer registers) took 5 and 9 % longer at N = 256,000
+            if (energy) k_force_f64<true, true, 4, 4><<<l.grid, narrow, 0, l.s>>>(b);
+            else k_force_f64<true, false, 4, 4><<<l.grid, narrow, 0, l.s>>>(b);
         } else {
-            if (energy) k_force_f64<false, true><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
-            else k_force_f64<false, false><<<l.grid, LJ_F64_THREADS, 0, l.s>>>(b);
+            if (energy) k_force_f64<false, true, 4, 8><<<l.grid, narrow, 0, l.s>>>(b);
+            else k_force_f64<false, false, 4, 8><<<l.grid, narrow, 0, l.s>>>(b);
         }
     } else if (b.force_tiles) {
         cudaError_t e = tile_kernel_attrs();

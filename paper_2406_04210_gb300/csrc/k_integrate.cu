@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_integrate(BoxDev b, double dt, int
                         double x = od3[c] + dt * v;
                         if (b.all_pairs) wrap_d(b, b.rep[r], c, p, x);
                         b.off[c * np + p] = x;
+                        if (FORCE64 && b.offx) b.offx[c * np + p] = __double2ll_rn(x * b.fx.scale);
                         o[c] = __double2float_rn(x);
                     }
                     b.vel[c * np + p] = v;
@@ -527,6 +528,24 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_materialize(BoxDev b)
     }
 }
 }  // namespace
+
+namespace {
+__global__ void __launch_bounds__(LJ_CHUNK) k_fix(BoxDev b)
+{
+    for (int w = blockIdx.x; w < b.nchunk; w += gridDim.x) {
+        const int4 ch = chunk_of(b, w);
+        const int p = ch.y + (int)threadIdx.x;
+        if (p >= ch.z) continue;
+        for (int c = 0; c < 3; ++c) b.offx[c * b.np + p] = __double2ll_rn(b.off[c * b.np + p] * b.fx.scale);
+    }
+}
+}  // namespace
+
+cudaError_t launch_fix(const BoxDev& b, Launch l)
+{
+    k_fix<<<l.grid, LJ_CHUNK, 0, l.s>>>(b);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_materialize(const BoxDev& b, Launch l)
 {

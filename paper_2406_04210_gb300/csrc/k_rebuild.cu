@@ -483,6 +483,7 @@ __device__ __forceinline__ void gather_state(const BoxDev& b, int p, int q, int 
         } else {
             b.off[c * np + q] = o[c];
             b.vel[c * np + q] = v[c];
+            if (b.offx) b.offx[c * np + q] = __double2ll_rn(o[c] * b.fx.scale);
             oh[c] = __double2float_rn(o[c]);
         }
     }

@@ -171,6 +171,8 @@ struct md_box {
     double* d_parth = nullptr;
     double* d_hist = nullptr;
     int hist_cap = 0;
+    double eps0 = 1.0, sigma0 = 1.0, rcut0 = 0.0, shift0 = 0.0;   // the first pair's parameters
+    long long* d_offx = nullptr; // offsets as integers (FP64 precision, one species)
     PinnedBack* pin = nullptr;   // pinned host memory
     std::string err;
 };
@@ -302,6 +304,11 @@ void apply_force_kernel(md_box* b)
     b->d.force_tiles = tiles ? 1 : 0;
     const bool spread = list32 && !tiles && spread_force(b);
     b->d.force_spread = spread ? 1 : 0;
+    // FP64, one species: 16 threads per particle while the quarter-chunk items
+    // leave an SM at most one block (N <= 4,800), 4 beyond.  Force kernel,
+    // 16 against 4: N = 1,000 18.3 / 21.2 us, N = 4,000 18.5 / 21.4 us,
+    // N = 8,000 31.0 / 24.4 us.
+    b->d.f64_wide = (int)b->chunks.size() * LJ_F64_WARPS <= b->nsm ? 1 : 0;
     // all pairs, FP32: a block per 16 particles (LJ_ALL_SHARES per chunk), or,
     // where the chunks alone are several per SM, per chunk
     const int all = b->prec == MD_PREC_FP64 || b->chunks.size() > 1024 ? 1 : LJ_ALL_SHARES;
@@ -683,6 +690,49 @@ md_status make_grid(md_box* b)
     return MD_OK;
 }
 
+// Scales of the integer pair arithmetic (k_force_f64): offsets stay below 2^61
+// (they are at most an edge or so), r^2 below the cutoff in [2^62, 2^63).
+md_status setup_fx(md_box* b)
+{
+    const double eps = b->eps0, sigma = b->sigma0, rcut = b->rcut0, shift = b->shift0;
+    FxDev fx{};
+    long long* const had = b->d.offx;
+    const bool on = b->prec == MD_PREC_FP64 && !b->all_pairs && b->nt == 1;
+    if (on) {
+        double ell = 0.0;
+        for (const RepDev& R : b->reps)
+            for (double e : R.ell) ell = std::max(ell, e);
+        const double rc2 = rcut * rcut, s2 = sigma * sigma, s6 = s2 * s2 * s2;
+        fx.q = 61 - (int)std::ceil(std::log2(4.0 * ell));
+        fx.sR = std::max(0, (int)std::ceil(std::log2(rc2 * 1.001)) + 2 * fx.q - 63);
+        int e;
+        fx.Km = (unsigned long long)std::ldexp(std::frexp(0.5 / s6, &e), 64);
+        fx.Ke = e - 64;
+        const double rcu = std::ldexp(rc2, 2 * fx.q - fx.sR);
+        fx.Rc = rcu < 9.2e18 ? (unsigned long long)rcu : 0ull;
+        fx.scale = std::ldexp(1.0, fx.q);
+        fx.c12 = 48.0 * eps * s6 * s6;
+        fx.hb = 2.0 * eps * s6;
+        fx.shift = shift;
+        fx.near = (float)rc2 + b->d.band;   // the margin of the list build's FP64 recheck
+        if (b->nrep == 1)
+            for (int c = 0; c < 3; ++c) fx.ell[c] = std::llrint(std::ldexp(b->reps[0].ell[c], fx.q));
+        // exponents far from those of reduced or SI units stay with FP64, and
+        // cells over 32 cutoffs wide (a huge skin): the FP32 offsets would not
+        // give the closest pair's distance to the 5e-4 that FxScale assumes
+        fx.on = ell <= 32.0 * rcut && std::abs(fx.q) < 200 && std::abs(fx.Ke) < 700 && fx.Rc != 0ull && std::isfinite(fx.c12) && fx.c12 > 1e-250 ? 1 : 0;
+    }
+    if (fx.on && !b->d_offx && dev_alloc(b, &b->d_offx, 3 * (size_t)b->np) != MD_OK) fx.on = 0;   // no room: FP64
+    b->d.offx = fx.on ? b->d_offx : nullptr;
+    const FxDev& o = b->d.fx;
+    if (had != b->d.offx || o.on != fx.on || o.q != fx.q || o.sR != fx.sR || o.Ke != fx.Ke || o.Km != fx.Km ||
+        o.Rc != fx.Rc || o.c12 != fx.c12 || o.hb != fx.hb || o.shift != fx.shift || o.near != fx.near ||
+        o.ell[0] != fx.ell[0] || o.ell[1] != fx.ell[1] || o.ell[2] != fx.ell[2])
+        invalidate_graphs(b);   // graphs hold them by value
+    b->d.fx = fx;
+    return MD_OK;
+}
+
 // Rebuild all replicas now (forced), regrowing the lists until they fit,
 // then recompute the forces.
 md_status full_rebuild(md_box* b)
@@ -744,6 +794,7 @@ static md_status apply_layout(md_box* b, double scale, int order)
             b->fresh_abs = true;
         }
         CKS(make_grid(b));
+        CKS(setup_fx(b));   // scaled by the cells' edges
     }
     b->rec_valid = false;
     return full_rebuild(b);
@@ -982,6 +1033,10 @@ md_status replay_lists(md_box* b)
         b->launches += 1;
     }
     CK(b, launch_list(b, b->stream));
+    if (b->d.offx) {   // the restored offsets as integers
+        CK(b, launch_fix(b->d, lch(b)));
+        b->launches += 1;
+    }
     CK(b, launch_force(b->d, 0, lforce(b)));
     b->launches += 2;
     return MD_OK;
@@ -1420,6 +1475,11 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
         before.nh_1 != d.nh_1 || before.kap_1 != d.kap_1 || before.rl2 != d.rl2 || before.disp_thr2 != d.disp_thr2)
         invalidate_graphs(b);
     if (grid_changes) CKS(make_grid(b));
+    b->eps0 = eps[0];
+    b->sigma0 = sigma[0];
+    b->rcut0 = rcut[0];
+    b->shift0 = h.dshift[0];
+    CKS(setup_fx(b));
     b->lj_set = true;
     b->rec_valid = false;
     CKS(full_rebuild(b));

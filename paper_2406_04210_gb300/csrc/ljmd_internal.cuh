@@ -126,6 +126,19 @@ struct LJDev {
     double deps[LJ_MAXT * LJ_MAXT], dsig[LJ_MAXT * LJ_MAXT];
 };
 
+// ---- one-species FP64 pair forces in 64-bit integers (k_force_f64) ----
+// Offsets as multiples of 2^-q (exact where FP64 holds them), r^2 as a
+// multiple of 2^(sR - 2q) below 2^63, K = 1 / (2 sigma^6) = Km 2^Ke.
+struct FxDev {
+    int on, q, sR, Ke;
+    unsigned long long Km;
+    unsigned long long Rc;     // rc^2 in units of R
+    double scale;              // 2^q
+    double c12, hb, shift;     // 48 eps sigma^12, 2 eps sigma^6, energy shift
+    float near;                // FP32 r^2 below which an entry is queued
+    long long ell[3];          // one replica: the cell edges in units of 2^-q
+};
+
 // Everything a kernel needs, passed by value.
 struct BoxDev {
     int nrep, np, nchunk, ncell;
@@ -162,6 +175,8 @@ struct BoxDev {
     double* xabs;              // xabs[c*np + p]: positions of the last build
     float4* force4;            // FP32 forces (mixed modes)
     double* force64;           // FP64 forces (FP64 mode), force64[c*np + p]
+    FxDev fx;                  // FP64 mode, one species: integer pair arithmetic
+    long long* offx;           // and the offsets as integers, offx[c*np + p] (null: not used)
     // old-order copies during a rebuild
     double* xabsB;
     double* offB;              // new offsets from the new cell centre (layout of `off`), from k_bin
@@ -207,6 +222,7 @@ struct BoxDev {
     long long* step_ctr;       // steps since md_set_thermostat (device word)
     int all_pairs;             // every cutoff infinite: forces over all pairs, no lists
     int force_tiles;           // FP32 list forces by the tiled kernel (k_force_tile_f32)
+    int f64_wide;              // FP64 list forces of one species with 16 threads per particle
     int force_spread;          // FP32 list forces by k_force_f32's small work items
     const int4* brick;         // its work items: (replica, first cell x, y, z) of bricks of up to
     int nbrick;                // rep.br[0] x br[1] x br[2] cells
@@ -623,5 +639,6 @@ cudaError_t launch_upload(const BoxDev& b, const double* pos, const double* vel,
 cudaError_t launch_download(const BoxDev& b, double* pos, double* vel, int* img, Launch l);
 cudaError_t launch_force_out(const BoxDev& b, double* f, Launch l);
 cudaError_t launch_materialize(const BoxDev& b, Launch l);
+cudaError_t launch_fix(const BoxDev& b, Launch l);   // offx from off
 cudaError_t launch_get_nlist(const BoxDev& b, int* count, long long* nbr, long long cap,
                              double* pos, Launch l);
