@@ -319,6 +319,24 @@ void apply_force_kernel(md_box* b)
     b->d.pf_ds = list32 ? 1 : 0;
 }
 
+// Grid of the force kernels over `items` work items.  Automatic, FP32 lists:
+// a block per item, handed out in order as blocks finish, so that the SMs work
+// on neighbouring chunks at a time (a fixed stride lets them drift apart, and
+// the neighbours' data leaves L2): 6 blocks per SM against all, one species
+// with energies, N = 256,000 47.3 / 45.4 us, 1M 147.7 / 138.6, 4M 565 / 508.
+// With several species a block loads the pair tables first: 6 per SM to
+// 640,000 particles (the mixture, N = 256,000 74.1 / 77.1 us, 1M 246 / 244).
+int force_grid(md_box* b, int items)
+{
+    int per_sm = b->force_per_sm;
+    if (per_sm <= 0) {
+        if (b->prec == MD_PREC_FP64) per_sm = 12;
+        else if (b->all_pairs || (b->nt > 1 && items <= 5000)) per_sm = 6;
+        else return std::max(1, items);
+    }
+    return std::max(1, std::min(items, b->nsm * per_sm));
+}
+
 Launch lforce(md_box* b)
 {
     if (b->d.force_tiles)   // persistent: the resident blocks, bricks handed out in a grid stride
@@ -328,12 +346,10 @@ Launch lforce(md_box* b)
         const int items = b->d.nchunk * (LJ_CHUNK * LJ_TPP / LJ_SPREAD_THREADS);
         return Launch{std::max(1, std::min(items, b->nsm * 32)), 0, b->stream};
     }
-    int per_sm = b->force_per_sm > 0 ? b->force_per_sm : (b->prec == 2 ? 12 : 6);
     // the FP64 list kernel's items are quarters of a chunk
     int per_chunk = b->prec == MD_PREC_FP64 ? LJ_F64_WARPS : 1;
     if (b->all_pairs) per_chunk = b->prec == MD_PREC_FP64 ? std::max(1, b->d.ap_js) : b->d.pf_stride;
-    const int items = b->d.nchunk * per_chunk;
-    return Launch{std::max(1, std::min(items, b->nsm * per_sm)), 0, b->stream};
+    return Launch{force_grid(b, b->d.nchunk * per_chunk), 0, b->stream};
 }
 Launch llist(md_box* b)
 {
@@ -351,7 +367,12 @@ bool lanes_list(md_box* b)
 cudaError_t launch_list(md_box* b, cudaStream_t s)
 {
     if (lanes_list(b)) {
-        const int per_sm = b->list_per_sm > 0 ? b->list_per_sm : 8;   // resident blocks (64 registers, 27 KB)
+        // 8 resident blocks (64 registers, 27 KB); one replica, four rounds of
+        // them, handed out in order (see force_grid; more would cost the early
+        // exits of the steps that keep their lists): forced update at 1M 868 ->
+        // 829 us, 4M 3151 -> 2956, 256,000 281 -> 282.  Several replicas: each
+        // block walks the rebuilding replicas' list.
+        const int per_sm = b->list_per_sm > 0 ? b->list_per_sm : (b->nrep == 1 ? 32 : 8);
         const int warps = LJ_LANE_THREADS / 32;
         // four lanes per particle where a warp per cell leaves schedulers
         // idle: forced update (with host overhead) at N = 4,000 160 -> 134 us,
@@ -901,7 +922,9 @@ md_status ensure_tstat(md_box* b, int64_t n)
 md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* ring, GraphEnt* ge,
                         bool tape = false)
 {
-    Launch l = lch(b);
+    Launch l = lch(b), li = l;
+    // handed out in order (see force_grid): N = 4M 107 -> 98 us with energies, 95 -> 91 without
+    li.grid = std::max(1, std::min((int)b->d.nchunk, b->nsm * 32));
     // The energy reduction of step s reads the force shares of step s and the
     // kinetic shares of the integrate after it.  It runs on a branch (side
     // stream) beside the list update and the next force: the shares have two
@@ -945,7 +968,7 @@ md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* rin
         cudaGraphConditionalHandle cond = 0;
         if (s < n) CKS(cond_begin(b, &cond));
         const int prev = (int)((s + 1) & 1);   // the set of step s - 1
-        CK(b, launch_integrate(set[prev], mode, s == 0 ? 0 : energy, dt, (int)(s > 0 ? s - 1 : 0), cond, l));
+        CK(b, launch_integrate(set[prev], mode, s == 0 ? 0 : energy, dt, (int)(s > 0 ? s - 1 : 0), cond, li));
         CK(b, mark(s, 0, 1, b->stream));
         b->launches += 1;
         if (s > 0 && energy) {
@@ -2158,7 +2181,7 @@ md_status md_autotune(md_box* b, int32_t reps, int32_t t[4])
         // the list build's grid again, at the chosen layout and kernel
         float best_g = 1e30f;
         int best_gl = b->list_per_sm;
-        for (int lc : {3, 4, 6, 8, 12, 16, 24}) {
+        for (int lc : {3, 4, 6, 8, 12, 16, 24, 32}) {
             b->list_per_sm = lc;
             float ms = 0.f;
             CKS(time_launches(b, reps, [&]() -> md_status {
@@ -2345,8 +2368,7 @@ extern "C" md_status md_force_noalloc(md_box* b, double* force_out, double* epot
     CKS(clear_err(b));
     Launch lf = lforce(b);
     if (b->d.force_tiles) {   // the chunk kernel's grid
-        const int per_sm = b->force_per_sm > 0 ? b->force_per_sm : 6;
-        lf.grid = std::max(1, std::min((int)v.nchunk, b->nsm * per_sm));
+        lf.grid = force_grid(b, (int)v.nchunk);
     }
     CK(b, launch_force(v, 1, lf));
     CK(b, launch_thermo(v, th, 0, lthermo(b)));

@@ -1,0 +1,36 @@
+"""The launch grids chosen by size (a block per work item, or a few per SM) do
+not change any bit: forces, energies and lists of the automatic grids against
+fixed ones, at chunk counts around the SMs' blocks and for the mixture."""
+import numpy as np
+import pytest
+
+from paper_2406_04210_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ljmd():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2406_04210_gb300 import build, ljmd as m
+    build.build()
+    m.load()
+    return m
+
+
+@pytest.mark.parametrize("species,n", [(1, 65537), (1, 116737), (1, 160001), (2, 70000)])
+def test_grids_do_not_change_results(ljmd, species, n):
+    s = inputs.fcc_subset_system(n, 0.8, 0.7, seed=n) if species == 1 else inputs.binary_random_system(n, seed=2)
+    a, b = ljmd.from_system(s), ljmd.from_system(s)
+    b.set_tuning(force_blocks_per_sm=3, list_blocks_per_sm=5)
+    b.neighbour_update(True)
+    for x, y in zip(a.force(), b.force()):
+        np.testing.assert_array_equal(x, y)
+    ca, na, _ = a.nlist()
+    cb, nb, _ = b.nlist()
+    np.testing.assert_array_equal(ca, cb)
+    assert all((na[i, :c] == nb[i, :c]).all() for i, c in enumerate(ca))
+    for x, y in zip(a.integrate(0.001, 5), b.integrate(0.001, 5)):
+        np.testing.assert_array_equal(x, y)
