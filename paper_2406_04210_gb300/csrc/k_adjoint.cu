@@ -243,14 +243,10 @@ __global__ void __launch_bounds__(THREADS, RES) k_hvp_mono(BoxDev b, Tape tp, in
         }
         // u_i.dF/deps and u_i.dF/dsigma from the moments
         const float x = S.x.x + S.x.y, y = nh * (S.y.x + S.y.y);
-        const float2 de = warp_sum_ds2(-c12 * inv_eps * (x + y));
-        const float2 ds = warp_sum_ds2(-6.f * c12 * inv_sig * fmaf(2.f, x, y));
-        if ((threadIdx.x & 31) == 0) {
-            const double wgt = *weight;
-            const size_t q = (size_t)it * (THREADS / 32) + (threadIdx.x >> 5);
-            const double e0 = part_g[2 * q], s0 = part_g[2 * q + 1];
-            part_g[2 * q] = e0 + wgt * ((double)de.x + (double)de.y);
-            part_g[2 * q + 1] = s0 + wgt * ((double)ds.x + (double)ds.y);
+        const float2 d = warp_sum2_ds2(-c12 * inv_eps * (x + y), -6.f * c12 * inv_sig * fmaf(2.f, x, y));
+        if ((threadIdx.x & 15) == 0) {
+            const size_t q = (size_t)it * (THREADS / 16) + (threadIdx.x >> 4);
+            part_g[q] += *weight * ((double)d.x + (double)d.y);
         }
     }
 }

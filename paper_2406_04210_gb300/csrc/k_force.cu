@@ -321,11 +321,10 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
             // pair itself (pf_ds), halved exactly; the reduction converts
             const float vir = c12 * (S.w.x + S.w.y);
             const float e = fmaf(vir, 1.f / 12.f, (MONO ? -0.5f * b.c1.w : -1.f) * (S.b.x + S.b.y));
-            const float2 de = warp_sum_ds2(e), dw = warp_sum_ds2(vir);
-            if ((threadIdx.x & 31) == 0) {
-                const size_t q = (size_t)it * (THREADS / 32) + (threadIdx.x >> 5);
-                reinterpret_cast<float4*>(b.part_f)[q] =
-                    make_float4(0.5f * de.x, 0.5f * de.y, 0.5f * dw.x, 0.5f * dw.y);
+            const float2 d = warp_sum2_ds2(e, vir);
+            if ((threadIdx.x & 15) == 0) {
+                const size_t q = (size_t)it * (THREADS / 16) + (threadIdx.x >> 4);
+                reinterpret_cast<float2*>(b.part_f)[q] = make_float2(0.5f * d.x, 0.5f * d.y);
             }
         }
     }
@@ -732,10 +731,10 @@ __global__ void __launch_bounds__(LJ_BRICK_THREADS + 32, 4) k_force_tile_f32(Box
             // (zeros where the warp had no particle): the warp sum in
             // double-single, stored as the (hi, lo) pair, halved exactly
             // (each pair is in two rows of a full list)
-            const float2 de = warp_sum_ds2(e_acc), dw = warp_sum_ds2(w_acc);
-            if (lane == 0)
-                reinterpret_cast<float4*>(b.part_f)[(size_t)bi * kBrickWarps + warp] =
-                    make_float4(0.5f * de.x, 0.5f * de.y, 0.5f * dw.x, 0.5f * dw.y);
+            const float2 d = warp_sum2_ds2(e_acc, w_acc);
+            if ((lane & 15) == 0)
+                reinterpret_cast<float2*>(b.part_f)[2 * ((size_t)bi * kBrickWarps + warp) + (lane >> 4)] =
+                    make_float2(0.5f * d.x, 0.5f * d.y);
         }
         mbar_arrive1(&s_empty[buf]);   // every consumer thread: its reads of the buffer precede this
     }
@@ -1208,7 +1207,7 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
         const float2 ix = dup2(1.0f / L.x), iy = dup2(1.0f / L.y), iz = dup2(1.0f / L.z);
         const float2 nLx = dup2(-L.x), nLy = dup2(-L.y), nLz = dup2(-L.z);
         const int jb = b.nrep == 1 ? 0 : R.p_off, je = b.nrep == 1 ? b.n1 : R.p_off + R.n;
-        double esum = 0.0, wsum = 0.0;
+        double sum = 0.0;   // E_pot in the lanes below 16, W in the others
         for (int grp = it % parts; grp < kAllGroups; grp += parts) {
             const int p = ch.y + grp * kAllGroup + 2 * warp;   // the warp's particles: p and p + 1
             const bool one = p < ch.z, two = p + 1 < ch.z;     // warp-uniform
@@ -1285,17 +1284,13 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
                 // u = f r^2 / 12 - 2 eps (sigma / r)^6 (no cutoff, no shift)
                 const float wv = c12 * (vir.x + (two ? vir.y : 0.f));   // both 0 without a first particle
                 const float ev = fmaf(wv, 1.f / 12.f, (MONO ? -0.5f * b.c1.w : -1.f) * (eb.x + (two ? eb.y : 0.f)));
-                const float2 de = warp_sum_ds2(ev), dw = warp_sum_ds2(wv);
-                esum += (double)de.x + (double)de.y;
-                wsum += (double)dw.x + (double)dw.y;
+                const float2 d = warp_sum2_ds2(ev, wv);
+                sum += (double)d.x + (double)d.y;
             }
         }
         if (ENERGY) {
             __syncthreads();   // the previous item's sums are read
-            if (lane == 0) {
-                s_red[0][warp] = 0.5 * esum;   // each pair is seen from both ends
-                s_red[1][warp] = 0.5 * wsum;
-            }
+            if ((lane & 15) == 0) s_red[lane >> 4][warp] = 0.5 * sum;   // each pair is seen from both ends
             __syncthreads();
             if (threadIdx.x < 2) {
                 double t = 0.0;

