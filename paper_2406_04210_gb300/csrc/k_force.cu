@@ -213,6 +213,7 @@ static_assert(LJ_TPP * 4 == LJ_ROW_BLOCK, "a row block is one 16-byte load per t
 template <bool MONO, bool ENERGY, bool SINGLE, int THREADS, int RES>
 __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
 {
+    await_previous();
     constexpr int TPP = LJ_TPP;
     constexpr bool SPREAD = THREADS == LJ_SPREAD_THREADS;
     constexpr int PASS = THREADS / TPP;                       // particles of a pass
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
     const float c12 = MONO ? b.c1.x : 1.f, nh = b.nh_1, kap = b.kap_1, mrc2 = b.rc2_1;
     const int K = b.K;
     const int grp = threadIdx.x / TPP, lt = threadIdx.x % TPP;
-    const float4* __restrict__ posq = b.posq;
+    const float4* posq = b.posq;
     const unsigned sent = entry_make(13, b.np);
     int cur_r = -1;
     float3 ell = make_float3(b.ell1.x, 0.25f * b.ell1.y, 0.0625f * b.ell1.z);   // edges in the digits' units
@@ -272,10 +273,10 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
             S.fx = S.fy = S.fz = 0.f;
             // four entries: four gathers in flight
             auto block4 = [&](const uint4& q) {
-                const float4 p0 = __ldg(posq + entry_slot(q.x));
-                const float4 p1 = __ldg(posq + entry_slot(q.y));
-                const float4 p2 = __ldg(posq + entry_slot(q.z));
-                const float4 p3 = __ldg(posq + entry_slot(q.w));
+                const float4 p0 = posq[entry_slot(q.x)];
+                const float4 p1 = posq[entry_slot(q.y)];
+                const float4 p2 = posq[entry_slot(q.z)];
+                const float4 p3 = posq[entry_slot(q.w)];
                 if (SPREAD) {
                     pair2_f32<MONO, ENERGY>(q.x, p0, q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
                     pair2_f32<MONO, ENERGY>(q.z, p2, q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
@@ -487,7 +488,7 @@ __global__ void __launch_bounds__(LJ_BRICK_THREADS + 32, 4) k_force_tile_f32(Box
     __syncthreads();   // the block's only barrier: the roles part here
     const uint32_t X0 = (uint32_t)__cvta_generic_to_shared(s_dyn);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float4* __restrict__ posq = b.posq;
+    const float4* posq = b.posq;
 
     if (warp == kBrickWarps) {
         // ---------------- producer ----------------
@@ -696,7 +697,7 @@ __global__ void __launch_bounds__(LJ_BRICK_THREADS + 32, 4) k_force_tile_f32(Box
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
                         const unsigned ek = (!last || lim > kk) ? q[kk] : sent_ent;
-                        const float4 pj = __ldg(posq + entry_slot(ek));
+                        const float4 pj = posq[entry_slot(ek)];
                         pair_f32<MONO, ENERGY>(ek, pj, pi, ti, ell_digit, s_lj, s_rc2, s_esh, nt, mlj, mrc2, mesh, fx,
                                                fy, fz, e, vir);
                     }
@@ -881,6 +882,7 @@ constexpr int kF64Own = LJ_CHUNK / kF64Parts;                   // particles of 
 template <bool MONO, bool ENERGY, int TPP, int RES>
 __global__ void __launch_bounds__(kF64Own * TPP, RES) k_force_f64(BoxDev b)
 {
+    await_previous();
     constexpr int kWarps = kF64Own * TPP / 32;
     constexpr int kF64Scan = TPP == 4 ? 96 : 128;               // entries scanned between two drains of the queue
     constexpr int kF64Queue = kF64Scan + 4;                     // a particle's queue (stride 4 banks)
@@ -909,7 +911,7 @@ __global__ void __launch_bounds__(kF64Own * TPP, RES) k_force_f64(BoxDev b)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = threadIdx.x / TPP, l4 = threadIdx.x % TPP;
     uint32_t* const q = s_q + grp * kF64Queue;
-    const float4* __restrict__ posq = b.posq;
+    const float4* posq = b.posq;
     int cur_r = -1;
     float3 ell = make_float3(0.f, 0.f, 0.f);
     for (int it = blockIdx.x; it < b.nchunk * kF64Parts; it += gridDim.x) {
@@ -977,7 +979,7 @@ __global__ void __launch_bounds__(kF64Own * TPP, RES) k_force_f64(BoxDev b)
                 for (int u = 0; u < 4; ++u) {
                     in[u] = false;
                     if (u < lim) {
-                        const float4 pj = __ldg(posq + entry_slot(en[u]));
+                        const float4 pj = posq[entry_slot(en[u])];
                         const float dx = fmaf(-entry_unit<0>(en[u]), ell.x, pi.x - pj.x);
                         const float dy = fmaf(-entry_unit<1>(en[u]), ell.y, pi.y - pj.y);
                         const float dz = fmaf(-entry_unit<2>(en[u]), ell.z, pi.z - pj.z);
@@ -1016,9 +1018,9 @@ __global__ void __launch_bounds__(kF64Own * TPP, RES) k_force_f64(BoxDev b)
                     auto fetch = [&](int t) {
                         ent = q[t];
                         const int j = (int)entry_slot(ent);
-                        px = __ldg(&b.offx[j]);
-                        py = __ldg(&b.offx[np + j]);
-                        pz = __ldg(&b.offx[2 * np + j]);
+                        px = b.offx[j];
+                        py = b.offx[np + j];
+                        pz = b.offx[2 * np + j];
                     };
                     if (l4 < nq) fetch(l4);
                     for (int t = l4; t < nq; t += TPP) {
@@ -1074,11 +1076,11 @@ __global__ void __launch_bounds__(kF64Own * TPP, RES) k_force_f64(BoxDev b)
                 const uint32_t ent = q[t];
                 const int j = (int)entry_slot(ent);
                 const int gx = (int)(ent & 3u) - 1, gy = (int)((ent >> 2) & 3u) - 1, gz = (int)((ent >> 4) & 3u) - 1;
-                const double dx = (xi - __ldg(&b.off[j])) - (gx == 0 ? 0.0 : (gx > 0 ? ex : -ex));
-                const double dy = (yi - __ldg(&b.off[np + j])) - (gy == 0 ? 0.0 : (gy > 0 ? ey : -ey));
-                const double dz = (zi - __ldg(&b.off[2 * np + j])) - (gz == 0 ? 0.0 : (gz > 0 ? ez : -ez));
+                const double dx = (xi - b.off[j]) - (gx == 0 ? 0.0 : (gx > 0 ? ex : -ex));
+                const double dy = (yi - b.off[np + j]) - (gy == 0 ? 0.0 : (gy > 0 ? ey : -ey));
+                const double dz = (zi - b.off[2 * np + j]) - (gz == 0 ? 0.0 : (gz > 0 ? ez : -ez));
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                const int pp = MONO ? 0 : tb + __ldg(&b.type[j]);
+                const int pp = MONO ? 0 : tb + b.type[j];
                 // r2 < rc2 on their bits (neither is negative), not on the FP64 pipe; a NaN fails
                 if ((unsigned long long)__double_as_longlong(r2) < s_rc2[pp]) {
                     const double2 c = s_c[pp];
@@ -1176,6 +1178,7 @@ __device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
 template <bool MONO, bool ENERGY>
 __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
 {
+    await_previous();
     __shared__ float4 s_lj[MONO ? 1 : LJ_MAXT * LJ_MAXT];   // c12, -c6, 2 eps sigma^6
     __shared__ double s_red[2][kAllWarps];
     __shared__ __align__(16) float4 s_pos[kAllTile];
@@ -1190,7 +1193,7 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int parts = b.pf_stride;
     const float2 M = dup2(12582912.0f), nM = dup2(-12582912.0f);   // 1.5 * 2^23
-    const float4* __restrict__ posq = b.posq;
+    const float4* posq = b.posq;
     for (int it = blockIdx.x; it < b.nchunk * parts; it += gridDim.x) {
         const int w = it / parts;
         const int4 ch = chunk_of(b, w);
@@ -1333,6 +1336,7 @@ __device__ __forceinline__ bool last_slice(const BoxDev& b, int w, int* s_flag)
 template <bool ENERGY>
 __global__ void __launch_bounds__(LJ_CHUNK) k_force_all_f64(BoxDev b)
 {
+    await_previous();
     constexpr int kT = 512;
     __shared__ double s_x[kT], s_y[kT], s_z[kT];
     __shared__ int s_t[kT];
@@ -1568,33 +1572,34 @@ static cudaError_t tile_kernel_attrs()
 
 cudaError_t launch_force(const BoxDev& b, int energy, Launch l)
 {
+    cudaError_t e = cudaSuccess;
     if (b.all_pairs) {
         if (b.prec == 2) {
-            if (energy) k_force_all_f64<true><<<l.grid, LJ_CHUNK, 0, l.s>>>(b);
-            else k_force_all_f64<false><<<l.grid, LJ_CHUNK, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_all_f64<true>, l.grid, LJ_CHUNK, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_all_f64<false>, l.grid, LJ_CHUNK, 0, l.s, l.early, b);
         } else if (b.nt == 1) {
-            if (energy) k_force_all_f32<true, true><<<l.grid, kAllThreads, 0, l.s>>>(b);
-            else k_force_all_f32<true, false><<<l.grid, kAllThreads, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_all_f32<true, true>, l.grid, kAllThreads, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_all_f32<true, false>, l.grid, kAllThreads, 0, l.s, l.early, b);
         } else {
-            if (energy) k_force_all_f32<false, true><<<l.grid, kAllThreads, 0, l.s>>>(b);
-            else k_force_all_f32<false, false><<<l.grid, kAllThreads, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_all_f32<false, true>, l.grid, kAllThreads, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_all_f32<false, false>, l.grid, kAllThreads, 0, l.s, l.early, b);
         }
-        return cudaGetLastError();
+        return e;
     }
     if (b.prec == 2) {
         const int wide = 16 * kF64Own, narrow = 4 * kF64Own;
         if (b.nt == 1 && b.f64_wide) {
-            if (energy) k_force_f64<true, true, 16, 1><<<l.grid, wide, 0, l.s>>>(b);
-            else k_force_f64<true, false, 16, 1><<<l.grid, wide, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_f64<true, true, 16, 1>, l.grid, wide, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_f64<true, false, 16, 1>, l.grid, wide, 0, l.s, l.early, b);
         } else if (b.nt == 1) {   // 4 blocks resident: 5 and 6 (fewer registers) took 5 and 9 % longer at N = 256,000
-            if (energy) k_force_f64<true, true, 4, 4><<<l.grid, narrow, 0, l.s>>>(b);
-            else k_force_f64<true, false, 4, 4><<<l.grid, narrow, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_f64<true, true, 4, 4>, l.grid, narrow, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_f64<true, false, 4, 4>, l.grid, narrow, 0, l.s, l.early, b);
         } else {
-            if (energy) k_force_f64<false, true, 4, 8><<<l.grid, narrow, 0, l.s>>>(b);
-            else k_force_f64<false, false, 4, 8><<<l.grid, narrow, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_f64<false, true, 4, 8>, l.grid, narrow, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_f64<false, false, 4, 8>, l.grid, narrow, 0, l.s, l.early, b);
         }
     } else if (b.force_tiles) {
-        cudaError_t e = tile_kernel_attrs();
+        e = tile_kernel_attrs();
         if (e != cudaSuccess) return e;
         const int th = LJ_BRICK_THREADS + 32;
         const size_t dm = 2 * tile_buf_bytes(true), dx = 2 * tile_buf_bytes(false);
@@ -1608,26 +1613,26 @@ cudaError_t launch_force(const BoxDev& b, int energy, Launch l)
     } else if (b.force_spread) {
         const int th = LJ_SPREAD_THREADS;
         if (b.nt == 1 && b.nrep == 1) {
-            if (energy) k_force_f32<true, true, true, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
-            else k_force_f32<true, false, true, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_f32<true, true, true, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_f32<true, false, true, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
         } else if (b.nt == 1) {
-            if (energy) k_force_f32<true, true, false, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
-            else k_force_f32<true, false, false, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_f32<true, true, false, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_f32<true, false, false, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
         } else {
-            if (energy) k_force_f32<false, true, false, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
-            else k_force_f32<false, false, false, LJ_SPREAD_THREADS, 1><<<l.grid, th, 0, l.s>>>(b);
+            if (energy) e = launch_kernel(k_force_f32<false, true, false, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_f32<false, false, false, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
         }
     } else if (b.nt == 1 && b.nrep == 1) {
-        if (energy) k_force_f32<true, true, true, LJ_FORCE_THREADS, 8><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
-        else k_force_f32<true, false, true, LJ_FORCE_THREADS, 8><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        if (energy) e = launch_kernel(k_force_f32<true, true, true, LJ_FORCE_THREADS, 8>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
+        else e = launch_kernel(k_force_f32<true, false, true, LJ_FORCE_THREADS, 8>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
     } else if (b.nt == 1) {
-        if (energy) k_force_f32<true, true, false, LJ_FORCE_THREADS, 8><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
-        else k_force_f32<true, false, false, LJ_FORCE_THREADS, 8><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        if (energy) e = launch_kernel(k_force_f32<true, true, false, LJ_FORCE_THREADS, 8>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
+        else e = launch_kernel(k_force_f32<true, false, false, LJ_FORCE_THREADS, 8>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
     } else {
-        if (energy) k_force_f32<false, true, false, LJ_FORCE_THREADS, 6><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
-        else k_force_f32<false, false, false, LJ_FORCE_THREADS, 6><<<l.grid, LJ_FORCE_THREADS, 0, l.s>>>(b);
+        if (energy) e = launch_kernel(k_force_f32<false, true, false, LJ_FORCE_THREADS, 6>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
+        else e = launch_kernel(k_force_f32<false, false, false, LJ_FORCE_THREADS, 6>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
     }
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Resident blocks per SM of the tiled force kernel (its persistent grid).

@@ -139,6 +139,7 @@ template <int ACC, bool FORCE64, int MODE, bool ENERGY, bool TSTAT>
 __global__ void __launch_bounds__(LJ_CHUNK) k_integrate(BoxDev b, double dt, int sidx,
                                                         cudaGraphConditionalHandle cond)
 {
+    await_previous();
     const int np = b.np;
     const double hdt = 0.5 * dt;
     float dt_h, dt_l;
@@ -273,8 +274,8 @@ cudaError_t launch_integrate_t(const BoxDev& b, int mode, int energy, double dt,
 {
 #define LJ_INT_CASE(M, E)                                                                       \
     do {                                                                                        \
-        if (b.tstat_thr) k_integrate<ACC, FORCE64, M, E, true><<<l.grid, LJ_CHUNK, 0, l.s>>>(b, dt, sidx, cond);  \
-        else k_integrate<ACC, FORCE64, M, E, false><<<l.grid, LJ_CHUNK, 0, l.s>>>(b, dt, sidx, cond);            \
+        return launch_kernel(b.tstat_thr ? k_integrate<ACC, FORCE64, M, E, true> : k_integrate<ACC, FORCE64, M, E, false>, \
+                             l.grid, LJ_CHUNK, 0, l.s, l.early, b, dt, sidx, cond);                     \
     } while (0)
     if (mode == LJ_STEP_FIRST) LJ_INT_CASE(LJ_STEP_FIRST, false);
     else if (mode == LJ_STEP_MID) {
@@ -285,7 +286,6 @@ cudaError_t launch_integrate_t(const BoxDev& b, int mode, int energy, double dt,
         else LJ_INT_CASE(LJ_STEP_LAST, false);
     }
 #undef LJ_INT_CASE
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

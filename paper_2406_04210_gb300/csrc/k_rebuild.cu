@@ -225,6 +225,7 @@ __device__ __forceinline__ void phase_bin(const BoxDev& b, int from_abs)
 
 __global__ void __launch_bounds__(LJ_CHUNK) k_bin(BoxDev b, int from_abs)
 {
+    await_previous();
     if (box_needs_rebuild(b)) phase_bin(b, from_abs);
 }
 
@@ -323,12 +324,14 @@ __device__ __forceinline__ void phase_scan_add(const BoxDev& b, const int4* tile
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(BoxDev b, const int4* tiles, int ntiles, int* tile_sum)
 {
+    await_previous();
     if (box_needs_rebuild(b)) phase_scan_tiles<kScanThreads>(b, tiles, ntiles, tile_sum);
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_add(BoxDev b, const int4* tiles, int ntiles,
                                                             const int* tile_sum)
 {
+    await_previous();
     if (box_needs_rebuild(b)) phase_scan_add(b, tiles, ntiles, tile_sum);
 }
 
@@ -357,6 +360,7 @@ __device__ __forceinline__ void phase_scatter(const BoxDev& b)
 
 __global__ void __launch_bounds__(LJ_CHUNK) k_scatter(BoxDev b)
 {
+    await_previous();
     if (box_needs_rebuild(b)) phase_scatter(b);
 }
 
@@ -397,6 +401,7 @@ __device__ __forceinline__ void phase_list_work(const BoxDev& b)   // one block
 
 __global__ void __launch_bounds__(1024) k_list_work(BoxDev b, unsigned long long* runs)
 {
+    await_previous();
     if (!box_needs_rebuild(b)) return;
     phase_list_work(b);
     if (runs && threadIdx.x == 0) *runs += 1ull;   // launch accounting of a conditional rebuild
@@ -539,6 +544,7 @@ __device__ __forceinline__ void phase_rank(const BoxDev& b)
 
 __global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
 {
+    await_previous();
     if (!box_needs_rebuild(b)) return;
     if (b.all_pairs) {
         // one cell holds the whole replica and no list needs an order: a
@@ -561,6 +567,7 @@ __global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
 
 __global__ void __launch_bounds__(LJ_CHUNK) k_gather(BoxDev b)
 {
+    await_previous();
     if (b.all_pairs || !box_needs_rebuild(b)) return;
     const int tot = work_chunks(b);
     int kr = 0;
@@ -920,6 +927,7 @@ __device__ __forceinline__ float lane_t(const float4& pi, const float4& q, float
 template <int G>
 __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
 {
+    await_previous();
     if (!box_needs_rebuild(b)) return;
     constexpr int P = 32 / G;    // particles of a pass
     constexpr int T = 32 / G;    // candidates of a batch that a lane tests
@@ -946,7 +954,7 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
     uint32_t* const re = s_ce[warp];
     const float rl2 = b.rl2f, band = b.band;
     const float rcull = rl2 + band + 1e-3f;   // staging margin for the rounding of the shifted offsets
-    const float4* __restrict__ posq = b.posq;
+    const float4* posq = b.posq;
     int longest = 0;
     const int nwarp = gridDim.x * kLaneWarps;
     const int total = work_cells(b) * G;
@@ -1177,6 +1185,7 @@ __device__ __forceinline__ void cluster_barrier()
 __global__ void __launch_bounds__(kClusterThreads) k_rebuild_cluster(BoxDev b, int from_abs, const int4* tiles,
                                                                       int ntiles, int* tile_sum)
 {
+    await_previous();
     if (!box_needs_rebuild(b)) return;   // the same word for every block: none is left waiting
     if (b.nrep > 1) {   // one replica: its work lists never change
         if (blockIdx.x == 0) phase_list_work(b);
@@ -1200,33 +1209,27 @@ static_assert(kClusterThreads % LJ_CHUNK == 0, "whole groups");
 
 cudaError_t launch_bin(const BoxDev& b, int from_abs, Launch l)
 {
-    k_bin<<<l.grid, LJ_CHUNK, 0, l.s>>>(b, from_abs);
-    return cudaGetLastError();
+    return launch_kernel(k_bin, l.grid, LJ_CHUNK, 0, l.s, l.early, b, from_abs);
 }
 
 cudaError_t launch_scan_tiles(const BoxDev& b, const int4* tiles, int ntiles, int* tile_sum,
                               Launch l)
 {
-    k_scan_tiles<<<l.grid, kScanThreads, 0, l.s>>>(b, tiles, ntiles, tile_sum);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(k_scan_tiles, l.grid, kScanThreads, 0, l.s, l.early, b, tiles, ntiles, tile_sum);
     if (e != cudaSuccess || ntiles <= b.nrep) return e;   // one tile per replica: finished
-    k_scan_add<<<l.grid, kScanThreads, 0, l.s>>>(b, tiles, ntiles, tile_sum);
-    return cudaGetLastError();
+    return launch_kernel(k_scan_add, l.grid, kScanThreads, 0, l.s, l.early, b, tiles, ntiles, tile_sum);
 }
 
 cudaError_t launch_scatter(const BoxDev& b, Launch l)
 {
-    k_scatter<<<l.grid, LJ_CHUNK, 0, l.s>>>(b);
-    return cudaGetLastError();
+    return launch_kernel(k_scatter, l.grid, LJ_CHUNK, 0, l.s, l.early, b);
 }
 
 cudaError_t launch_sortgather(const BoxDev& b, Launch l, Launch lg)
 {
-    k_sortgather<<<l.grid, 256, 0, l.s>>>(b);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(k_sortgather, l.grid, 256, 0, l.s, l.early, b);
     if (e != cudaSuccess || b.all_pairs) return e;
-    k_gather<<<lg.grid, LJ_CHUNK, 0, lg.s>>>(b);
-    return cudaGetLastError();
+    return launch_kernel(k_gather, lg.grid, LJ_CHUNK, 0, lg.s, lg.early, b);
 }
 
 cudaError_t launch_nlist(const BoxDev& b, Launch l)
@@ -1242,18 +1245,16 @@ cudaError_t launch_nlist(const BoxDev& b, Launch l)
     return cudaGetLastError();
 }
 
-cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s)
+cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s, bool early)
 {
-    k_list_work<<<1, 1024, 0, s>>>(b, runs);
-    return cudaGetLastError();
+    return launch_kernel(k_list_work, 1, 1024, 0, s, early, b, runs);
 }
 
 cudaError_t launch_nlist_lanes(const BoxDev& b, int per_particle, Launch l)
 {
     const size_t dyn = (size_t)LJ_LANE_THREADS * kLaneRow * sizeof(uint32_t);   // the row buffers: below 48 KB
-    if (per_particle == 4) k_nlist_lanes<4><<<l.grid, LJ_LANE_THREADS, dyn, l.s>>>(b);
-    else k_nlist_lanes<1><<<l.grid, LJ_LANE_THREADS, dyn, l.s>>>(b);
-    return cudaGetLastError();
+    return launch_kernel(per_particle == 4 ? k_nlist_lanes<4> : k_nlist_lanes<1>, l.grid, LJ_LANE_THREADS, dyn, l.s,
+                         l.early, b);
 }
 
 // Whether this GPU holds the cluster (16 blocks is beyond the portable 8).
@@ -1277,18 +1278,20 @@ bool cluster_rebuild_fits()
 }
 
 cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles, int* tile_sum,
-                                   cudaStream_t s)
+                                   cudaStream_t s, bool early)
 {
     cudaLaunchConfig_t c{};
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = kClusterBlocks;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kClusterBlocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     c.gridDim = dim3(kClusterBlocks);
     c.blockDim = dim3(kClusterThreads);
     c.stream = s;
-    c.attrs = &at;
-    c.numAttrs = 1;
+    c.attrs = at;
+    c.numAttrs = early ? 2 : 1;
     return cudaLaunchKernelEx(&c, k_rebuild_cluster, b, from_abs, tiles, ntiles, tile_sum);
 }
 

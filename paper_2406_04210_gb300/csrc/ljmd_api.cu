@@ -65,6 +65,7 @@ struct PinnedBack {
 struct md_box {
     int device = 0;
     int nsm = 152;
+    bool early = false;        // step kernels by programmatic launches (while a step graph is captured)
     cudaStream_t ustream = nullptr;
     cudaStream_t stream = nullptr;
     cudaEvent_t ev = nullptr;
@@ -364,7 +365,7 @@ bool lanes_list(md_box* b)
     return b->list_kernel != MD_LIST_QUADS;
 }
 
-cudaError_t launch_list(md_box* b, cudaStream_t s)
+cudaError_t launch_list(md_box* b, cudaStream_t s, bool early = false)
 {
     if (lanes_list(b)) {
         // 8 resident blocks (64 registers, 27 KB); one replica, four rounds of
@@ -380,7 +381,7 @@ cudaError_t launch_list(md_box* b, cudaStream_t s)
         const int g = b->d.ncell <= 2048 ? 4 : 1;
         return launch_nlist_lanes(
             b->d, g,
-            Launch{std::max(1, std::min((b->d.ncell * g + warps - 1) / warps, b->nsm * per_sm)), LJ_LANE_THREADS, s});
+            Launch{std::max(1, std::min((b->d.ncell * g + warps - 1) / warps, b->nsm * per_sm)), LJ_LANE_THREADS, s, early});
     }
     Launch l = llist(b);
     l.s = s;
@@ -466,22 +467,37 @@ bool cluster_rebuild(md_box* b)
     return b->np <= kClusterSlots;
 }
 
+// Programmatic launches inside a step graph (Launch::early): a kernel's blocks
+// are placed while the previous kernel drains, which takes ~0.5 us off each of
+// the step's launches.  The rebuild kernels, which usually exit at once,
+// always; the list kernel with one replica (several: 604 against 629 us a step
+// of 512); the integrator and the force in boxes of up to 64 chunks only: in
+// larger ones blocks placed early land unevenly on the SMs (N = 100,000: the
+// force's early launch makes a step 43 -> 61 us).  Us a step with energies,
+// none / rebuild kernels / all four: N = 4,000 12.6 / 11.8 / 10.9, 8,000 12.3
+// / 11.4 / 10.9, 16,000 14.5 / 13.8 / 14.9; none / rebuild kernels: 100,000
+// 43.7 / 40.0, 256,000 78.5 / 74.1, 1M 216 / 212.  Not in profiled graphs
+// (events stand between the kernels) or with conditional nodes.
+bool early_step(md_box* b) { return b->early && b->chunks.size() <= 64; }
+
 // runs: counts the sequence's executions (the body of a conditional node)
 md_status enqueue_rebuild_kernels(md_box* b, int from_abs, cudaStream_t s, unsigned long long* runs)
 {
-    auto on = [s](Launch l) {
+    const bool early = b->early && !runs;
+    auto on = [s, early](Launch l) {
         l.s = s;
+        l.early = early;
         return l;
     };
     Launch l = on(lch(b));
     // the cells and chunks the rebuild kernels visit (one replica's never change: make_grid)
-    if (runs || b->nrep > 1) CK(b, launch_list_work(b->d, runs, s));
+    if (runs || b->nrep > 1) CK(b, launch_list_work(b->d, runs, s, early));
     CK(b, launch_bin(b->d, from_abs, l));
-    Launch lt{std::max(1, std::min((int)b->tiles.size(), b->nsm * 8)), 0, s};
+    Launch lt{std::max(1, std::min((int)b->tiles.size(), b->nsm * 8)), 0, s, early};
     CK(b, launch_scan_tiles(b->d, b->d_tiles, (int)b->tiles.size(), b->d_tile_sum, lt));
     CK(b, launch_scatter(b->d, l));
     CK(b, launch_sortgather(b->d, on(b->all_pairs ? lch(b) : lcell(b)), l));
-    if (!b->all_pairs) CK(b, launch_list(b, s));
+    if (!b->all_pairs) CK(b, launch_list(b, s, early && b->nrep == 1));
     b->launches += rebuild_kernels(b, runs != nullptr);
     return MD_OK;
 }
@@ -489,8 +505,8 @@ md_status enqueue_rebuild_kernels(md_box* b, int from_abs, cudaStream_t s, unsig
 md_status enqueue_rebuild(md_box* b, int from_abs)
 {
     if (!cluster_rebuild(b)) return enqueue_rebuild_kernels(b, from_abs, b->stream, nullptr);
-    CK(b, launch_rebuild_cluster(b->d, from_abs, b->d_tiles, (int)b->tiles.size(), b->d_tile_sum, b->stream));
-    CK(b, launch_list(b, b->stream));
+    CK(b, launch_rebuild_cluster(b->d, from_abs, b->d_tiles, (int)b->tiles.size(), b->d_tile_sum, b->stream, b->early));
+    CK(b, launch_list(b, b->stream, b->early && b->nrep == 1));
     b->launches += 2;
     return MD_OK;
 }
@@ -968,6 +984,7 @@ md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* rin
         cudaGraphConditionalHandle cond = 0;
         if (s < n) CKS(cond_begin(b, &cond));
         const int prev = (int)((s + 1) & 1);   // the set of step s - 1
+        li.early = s > 0 && early_step(b);
         CK(b, launch_integrate(set[prev], mode, s == 0 ? 0 : energy, dt, (int)(s > 0 ? s - 1 : 0), cond, li));
         CK(b, mark(s, 0, 1, b->stream));
         b->launches += 1;
@@ -989,7 +1006,9 @@ md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* rin
         if (tape) CKS(tape_save(b, (int)s + 1));   // before the force kernel takes the rebuild word down
         CK(b, join((int)(s & 1)));
         CK(b, mark(s, 2, 0, b->stream));
-        CK(b, launch_force(set[s & 1], energy, lforce(b)));
+        Launch lf = lforce(b);
+        lf.early = early_step(b);
+        CK(b, launch_force(set[s & 1], energy, lf));
         CK(b, mark(s, 2, 1, b->stream));
         b->launches += 1;
     }
@@ -1052,7 +1071,7 @@ md_status replay_lists(md_box* b)
 {
     CKS(set_all_rebuild(b));
     if (b->nrep > 1) {
-        CK(b, launch_list_work(b->d, nullptr, b->stream));
+        CK(b, launch_list_work(b->d, nullptr, b->stream, false));
         b->launches += 1;
     }
     CK(b, launch_list(b, b->stream));
@@ -1085,7 +1104,9 @@ md_status get_graph(md_box* b, int64_t n, double dt, int energy, cudaGraphExec_t
         cudaGraph_t graph = nullptr;
         int64_t l0 = b->launches;
         CK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+        b->early = !b->profiling && !b->use_cond;
         md_status st = enqueue_steps(b, n, dt, energy, b->d_thermo, b->profiling ? &ge : nullptr);
+        b->early = false;
         cudaError_t ce = cudaStreamEndCapture(b->stream, &graph);
         ge.kernels = b->launches - l0;
         b->launches = l0;

@@ -340,6 +340,17 @@ __device__ __forceinline__ double warp_sum_ds(float x)
     return (double)s.x + (double)s.y;
 }
 
+// First statement of the kernels of a step: the previous kernel's results are
+// complete and visible (it has no effect after an ordinary launch), and the
+// next kernel's blocks may become resident beside this one's; they wait here.
+// No load may be of the read-only kind (ld.global.nc) in such a kernel: the
+// compiler may move those above.
+__device__ __forceinline__ void await_previous()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Cheap block-level early exit of the rebuild kernels: nothing to do unless
 // the integrator or the host raised the box-wide request word.
 __device__ __forceinline__ bool box_needs_rebuild(const BoxDev& b)
@@ -598,7 +609,26 @@ struct Launch {
     int grid;
     int block;
     cudaStream_t s;
+    bool early = false;   // programmatic launch: the kernel begins with await_previous()
 };
+
+// Launch a kernel that begins with await_previous(); early: its blocks may
+// become resident while the previous kernel of the stream still runs.
+template <class... P, class... A>
+inline cudaError_t launch_kernel(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s, bool early, A... a)
+{
+    cudaLaunchConfig_t c{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&c, k, static_cast<P>(a)...);
+}
 
 // k_rebuild.cu
 cudaError_t launch_bin(const BoxDev& b, int from_abs, Launch l);
@@ -611,10 +641,10 @@ cudaError_t launch_nlist(const BoxDev& b, Launch l);
 // one warp per cell (per_particle 1) or per quarter of its particles (4 lanes per particle)
 cudaError_t launch_nlist_lanes(const BoxDev& b, int per_particle, Launch l);
 // one block; before the cell kernels; counts its executions with work in *runs (nullable)
-cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s);
+cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s, bool early);
 // binning, sort and gather in one launch of one cluster (small boxes)
 cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles, int* tile_sum,
-                                   cudaStream_t s);
+                                   cudaStream_t s, bool early);
 bool cluster_rebuild_fits();
 // k_force.cu
 cudaError_t launch_force(const BoxDev& b, int energy, Launch l);
