@@ -109,13 +109,26 @@ struct PairSums {
     float2 w, b;
 };
 
+// The pair constants of a particle with species 0 and with species 1 (TWO: boxes
+// of two species).  Chosen by selects: the table's two shared-memory loads per
+// pair share the L1 data pipe, which bounds the kernel, with the gathers.  The
+// 1.2-density mixture with / without energies, table -> selects: N = 256,000
+// 74.3 / 67.9 -> 64.0 / 59.3 us, 1M 241 / 217 -> 208 / 189, 32,000 20.7 / 18.2
+// -> 18.4 / 17.0.  The row's ten constants take registers: five blocks of 256
+// per SM with energies (six: 1M 223 us), six without.
+struct RowConsts {
+    float4 c0, c1;   // c12, -c6, 2 eps sigma^6, shift
+    float r0, r1;    // rc^2
+};
+
 // Two pair terms: the separations one by one, everything from r^2 on as FP32
 // pairs.  The cutoff masks 1/r^2 (times 1 or 0), so that every term of a pair
 // beyond it, the sentinel's too, is 0.
-template <bool MONO, bool ENERGY>
+template <bool MONO, bool ENERGY, bool TWO>
 __device__ __forceinline__ void pair2_f32(unsigned e0, const float4& q0, unsigned e1, const float4& q1,
                                           const float4& pi, int tb, const float3& ell, const float4* s_lj,
-                                          const float* s_rc2, float nh, float kap, float mrc2, PairSums& S)
+                                          const float* s_rc2, float nh, float kap, float mrc2, const RowConsts& rc,
+                                          PairSums& S)
 {
     const float2 a0 = neg_d_xy(e0, q0, pi, ell), a1 = neg_d_xy(e1, q1, pi, ell);
     const float2 az = make_float2(fmaf(entry_unit<2>(e0), ell.z, q0.z - pi.z), fmaf(entry_unit<2>(e1), ell.z, q1.z - pi.z));
@@ -126,12 +139,12 @@ __device__ __forceinline__ void pair2_f32(unsigned e0, const float4& q0, unsigne
         rc2 = make_float2(mrc2, mrc2);
     } else {
         const int p0 = tb + __float_as_int(q0.w), p1 = tb + __float_as_int(q1.w);
-        const float4 c0 = s_lj[p0], c1 = s_lj[p1];
+        const float4 c0 = TWO ? (p0 & 1 ? rc.c1 : rc.c0) : s_lj[p0], c1 = TWO ? (p1 & 1 ? rc.c1 : rc.c0) : s_lj[p1];
         c12 = make_float2(c0.x, c1.x);
         nc6 = make_float2(c0.y, c1.y);
         hb = make_float2(c0.z, c1.z);
         esh = make_float2(c0.w, c1.w);
-        rc2 = make_float2(s_rc2[p0], s_rc2[p1]);
+        rc2 = TWO ? make_float2(p0 & 1 ? rc.r1 : rc.r0, p1 & 1 ? rc.r1 : rc.r0) : make_float2(s_rc2[p0], s_rc2[p1]);
     }
     const float2 in = make_float2(r2.x < rc2.x ? 1.f : 0.f, r2.y < rc2.y ? 1.f : 0.f);
     const float2 ri = __fmul2_rn(make_float2(rcp_approx(r2.x), rcp_approx(r2.y)), in);
@@ -155,10 +168,10 @@ __device__ __forceinline__ void pair2_f32(unsigned e0, const float4& q0, unsigne
 // One pair term, the same sums, in scalar arithmetic: more instructions, but it
 // fits the 32 registers of eight blocks of 256 per SM (packed operands and
 // constants take register pairs).
-template <bool MONO, bool ENERGY>
+template <bool MONO, bool ENERGY, bool TWO>
 __device__ __forceinline__ void pair1_f32(unsigned e0, const float4& q0, const float4& pi, int tb, const float3& ell,
                                           const float4* s_lj, const float* s_rc2, float nh, float kap, float mrc2,
-                                          PairSums& S)
+                                          const RowConsts& rc, PairSums& S)
 {
     const float2 a0 = neg_d_xy(e0, q0, pi, ell);
     const float az = fmaf(entry_unit<2>(e0), ell.z, q0.z - pi.z);
@@ -168,8 +181,14 @@ __device__ __forceinline__ void pair1_f32(unsigned e0, const float4& q0, const f
     float rc2 = mrc2;
     if (!MONO) {
         const int p0 = tb + __float_as_int(q0.w);
-        c = s_lj[p0];
-        rc2 = s_rc2[p0];
+        if (TWO) {   // tb is even
+            const bool o = __float_as_int(q0.w) != 0;
+            c = make_float4(o ? rc.c1.x : rc.c0.x, o ? rc.c1.y : rc.c0.y, o ? rc.c1.z : rc.c0.z, o ? rc.c1.w : rc.c0.w);
+            rc2 = o ? rc.r1 : rc.r0;
+        } else {
+            c = s_lj[p0];
+            rc2 = s_rc2[p0];
+        }
     }
     const bool in = r2 < rc2;
     const float ri = in ? rcp_approx(r2) : 0.f;
@@ -201,7 +220,7 @@ __device__ __forceinline__ void pair1_f32(unsigned e0, const float4& q0, const f
 // at 256k, fewer resident warps), nor rows in the order of slot mod 8 (fewer
 // bank conflicts, more lines: 44.7 us, but 662 us against 588 at 4M) moved, so
 // resident warps matter most: 32 registers and eight blocks per SM for one
-// species, 40 and six for several.  With the digits below the slot and the
+// species, 40 and six for several (two: see RowConsts).  With the digits below the slot and the
 // energy from sums the force needs anyway: 4M with energies 589 -> 573 us,
 // without 529 -> 515, the 256k mixture 78.6 -> 75.3.  SPREAD: the serial row
 // (five dependent blocks), on every SM instead of a few: N = 4,000 16.4 -> 9.0
@@ -210,7 +229,7 @@ __device__ __forceinline__ void pair1_f32(unsigned e0, const float4& q0, const f
 // parameters.  SINGLE (MONO and one replica): the cell edge from the
 // parameters too.  One (E_pot, W) share per warp and item.
 static_assert(LJ_TPP * 4 == LJ_ROW_BLOCK, "a row block is one 16-byte load per thread of a particle");
-template <bool MONO, bool ENERGY, bool SINGLE, int THREADS, int RES>
+template <bool MONO, bool ENERGY, bool SINGLE, int THREADS, int RES, bool TWO = false>
 __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
 {
     await_previous();
@@ -270,6 +289,13 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
             }
             const int nblk = (cnt + 4 * TPP - 1) / (4 * TPP);
             const int tb = MONO ? 0 : __float_as_int(pi.w) * b.nt;
+            RowConsts rc;
+            if (TWO) {
+                rc.c0 = s_lj[tb];
+                rc.c1 = s_lj[tb + 1];
+                rc.r0 = s_rc2[tb];
+                rc.r1 = s_rc2[tb + 1];
+            }
             S.fx = S.fy = S.fz = 0.f;
             // four entries: four gathers in flight
             auto block4 = [&](const uint4& q) {
@@ -278,13 +304,13 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
                 const float4 p2 = posq[entry_slot(q.z)];
                 const float4 p3 = posq[entry_slot(q.w)];
                 if (SPREAD) {
-                    pair2_f32<MONO, ENERGY>(q.x, p0, q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
-                    pair2_f32<MONO, ENERGY>(q.z, p2, q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
+                    pair2_f32<MONO, ENERGY, TWO>(q.x, p0, q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
+                    pair2_f32<MONO, ENERGY, TWO>(q.z, p2, q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
                 } else {
-                    pair1_f32<MONO, ENERGY>(q.x, p0, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
-                    pair1_f32<MONO, ENERGY>(q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
-                    pair1_f32<MONO, ENERGY>(q.z, p2, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
-                    pair1_f32<MONO, ENERGY>(q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, S);
+                    pair1_f32<MONO, ENERGY, TWO>(q.x, p0, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
+                    pair1_f32<MONO, ENERGY, TWO>(q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
+                    pair1_f32<MONO, ENERGY, TWO>(q.z, p2, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
+                    pair1_f32<MONO, ENERGY, TWO>(q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
                 }
             };
             if (nblk > 0) {
@@ -1618,6 +1644,9 @@ cudaError_t launch_force(const BoxDev& b, int energy, Launch l)
         } else if (b.nt == 1) {
             if (energy) e = launch_kernel(k_force_f32<true, true, false, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
             else e = launch_kernel(k_force_f32<true, false, false, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
+        } else if (b.nt == 2) {
+            if (energy) e = launch_kernel(k_force_f32<false, true, false, LJ_SPREAD_THREADS, 1, true>, l.grid, th, 0, l.s, l.early, b);
+            else e = launch_kernel(k_force_f32<false, false, false, LJ_SPREAD_THREADS, 1, true>, l.grid, th, 0, l.s, l.early, b);
         } else {
             if (energy) e = launch_kernel(k_force_f32<false, true, false, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
             else e = launch_kernel(k_force_f32<false, false, false, LJ_SPREAD_THREADS, 1>, l.grid, th, 0, l.s, l.early, b);
@@ -1628,6 +1657,9 @@ cudaError_t launch_force(const BoxDev& b, int energy, Launch l)
     } else if (b.nt == 1) {
         if (energy) e = launch_kernel(k_force_f32<true, true, false, LJ_FORCE_THREADS, 8>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
         else e = launch_kernel(k_force_f32<true, false, false, LJ_FORCE_THREADS, 8>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
+    } else if (b.nt == 2) {
+        if (energy) e = launch_kernel(k_force_f32<false, true, false, LJ_FORCE_THREADS, 5, true>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
+        else e = launch_kernel(k_force_f32<false, false, false, LJ_FORCE_THREADS, 6, true>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
     } else {
         if (energy) e = launch_kernel(k_force_f32<false, true, false, LJ_FORCE_THREADS, 6>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);
         else e = launch_kernel(k_force_f32<false, false, false, LJ_FORCE_THREADS, 6>, l.grid, LJ_FORCE_THREADS, 0, l.s, l.early, b);

@@ -325,14 +325,15 @@ void apply_force_kernel(md_box* b)
 // on neighbouring chunks at a time (a fixed stride lets them drift apart, and
 // the neighbours' data leaves L2): 6 blocks per SM against all, one species
 // with energies, N = 256,000 47.3 / 45.4 us, 1M 147.7 / 138.6, 4M 565 / 508.
-// With several species a block loads the pair tables first: 6 per SM to
-// 640,000 particles (the mixture, N = 256,000 74.1 / 77.1 us, 1M 246 / 244).
+// With tables (three species and more) a block loads them first: 6 per SM to
+// 640,000 particles (measured with the mixture's tables, N = 256,000 74.1 / 77.1
+// us, 1M 246 / 244).
 int force_grid(md_box* b, int items)
 {
     int per_sm = b->force_per_sm;
     if (per_sm <= 0) {
         if (b->prec == MD_PREC_FP64) per_sm = 12;
-        else if (b->all_pairs || (b->nt > 1 && items <= 5000)) per_sm = 6;
+        else if (b->all_pairs || (b->nt > 2 && items <= 5000)) per_sm = 6;
         else return std::max(1, items);
     }
     return std::max(1, std::min(items, b->nsm * per_sm));
