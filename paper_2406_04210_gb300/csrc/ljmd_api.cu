@@ -1785,7 +1785,9 @@ md_status md_adjoint(md_box* b, const double* lam_x_T, const double* lam_v_T, do
     auto capture = [&](int slot, auto&& fn) -> md_status {
         const int64_t l0 = b->launches;
         CK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+        b->early = !b->use_cond;   // the replayed steps (see early_step)
         md_status st = fn();
+        b->early = false;
         cudaGraph_t graph = nullptr;
         cudaError_t ce = cudaStreamEndCapture(b->stream, &graph);
         b->adj_kernels[slot] = b->launches - l0;
