@@ -896,7 +896,7 @@ __global__ void __launch_bounds__(LJ_LIST_THREADS, 3) k_nlist(BoxDev b)
 // entries of its hits to its own row buffer in shared memory (no ballots:
 // every lane owns its buffer), from which whole pieces of four entries go out
 // with 16-byte stores.  Pairs within `band` of rl^2 are re-decided in FP64 as
-// in k_nlist (checked per batch: the smallest |r^2 - rl^2| tells whether any
+// in k_nlist (checked per half batch: the smallest |r^2 - rl^2| tells whether any
 // pair lies in the band).  d_ij and r^2 are computed as FP32 pairs.
 // G = 1 where the cells fill the GPU (launch_list's rule); what bounds it
 // then: issue (74 % of peak) and the shared-memory pipe (65 %), ~310
@@ -912,8 +912,11 @@ __global__ void __launch_bounds__(LJ_LIST_THREADS, 3) k_nlist(BoxDev b)
 constexpr int kLaneWarps = LJ_LANE_THREADS / 32;
 constexpr int kRing = 64;   // staged candidates per warp: < 32 waiting + one chunk
 // Entries a lane holds in shared memory: fewer than 4 not yet written out, and
-// a batch's 32 / G on top (flushed when less room is left), so the rows'
-// shared memory does not grow with the capacity K.
+// half a batch's 32 / G on top (flushed when less room is left), so the rows'
+// shared memory does not grow with the capacity K.  Looked at once a batch,
+// the buffers were written out two or three entries at a time: forced update
+// at 256,000 281 -> 269 us, at 4M 2956 -> 2839 (quarters: 277 and 2983; buffers
+// of 32 or 48 entries: 2917 and 2883).
 constexpr int kLaneRow = 40;
 
 // r^2 - rl^2 of the pair (i, candidate q = o_j + shift), rounded as in the
@@ -1036,16 +1039,16 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
                 cnt = rest;
             };
             // test the 32 staged candidates from head on against the lane's
-            // particle and append the hits
-            auto batch = [&]() {
-                if (__any_sync(0xffffffffu, cnt > kLaneRow - T)) flush();
+            // particle and append the hits, half of them between two looks at
+            // the buffers (which so fill further before they are written out)
+            auto half_batch = [&](int h0) {
+                if (__any_sync(0xffffffffu, cnt > kLaneRow - T / 2)) flush();
                 const int c0 = cnt;
-                const int h0 = (int)(head & (kRing - 1)) + T * sub;
                 // branch-free, two candidates per step with FP32-pair
                 // arithmetic on t = r^2 - rl^2: every candidate's entry is
                 // written to the next free slot (32-bit shared address), which
                 // advances only on a hit
-                float near = 1.0e30f;   // smallest |t| of the batch
+                float near = 1.0e30f;   // smallest |t| of the half
                 uint32_t wa = (uint32_t)__cvta_generic_to_shared(row + 32 * cnt);
                 const float2 px = make_float2(-pi.x, -pi.x), py = make_float2(-pi.y, -pi.y),
                              pz = make_float2(-pi.z, -pi.z), nrl = make_float2(-rl2, -rl2);
@@ -1060,8 +1063,8 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
                     asm volatile("st.shared.u32 [%0], %1;" ::"r"(wa), "r"(e1));
                     if ((t2.y < band) & (e1 != self)) wa += 128u;
                 };
-#pragma unroll 2
-                for (int u = 0; u < T; u += 4) {
+#pragma unroll
+                for (int u = 0; u < T / 2; u += 4) {
                     const float4 qx = *reinterpret_cast<const float4*>(rx + h0 + u);
                     const float4 qy = *reinterpret_cast<const float4*>(ry + h0 + u);
                     const float4 qz = *reinterpret_cast<const float4*>(rz + h0 + u);
@@ -1072,7 +1075,7 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
                 asm volatile("" ::: "memory");   // the stores above stay above
                 __syncwarp();
                 cnt = (int)((wa - (uint32_t)__cvta_generic_to_shared(row)) >> 7);
-                // FP64 decision of the batch's accepted pairs near rl (rare)
+                // FP64 decision of the half's accepted pairs near rl (rare)
                 if (near <= band) {
                     int w = c0;
                     const int e = cnt;
@@ -1086,6 +1089,10 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
                     }
                     cnt = w;
                 }
+            };
+            auto batch = [&]() {
+#pragma unroll 1
+                for (int h = 0; h < T; h += T / 2) half_batch((int)(head & (kRing - 1)) + T * sub + h);
                 head += 32u;
             };
             // chunk iterator over the neighbour cells: (k, j0), 32 slots at a time
