@@ -1460,6 +1460,12 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_force_all_f64(BoxDev b)
     }
 }
 
+// A share of the FP32 forces: its (hi, lo) pair, stored where a double stands.
+__device__ __forceinline__ double ds_bits_to_double(double v)
+{
+    return f2d(__int_as_float(__double2loint(v))) + f2d(__int_as_float(__double2hiint(v)));
+}
+
 // E_pot, E_kin, W, T per replica from the per-chunk partial sums, in a
 // fixed order (deterministic): each block of LJ_THERMO_THREADS sums one item
 // (a run of up to LJ_THERMO_CHUNKS chunks of one replica, pf_stride
@@ -1467,37 +1473,43 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_force_all_f64(BoxDev b)
 // of one item is written out by its block directly; otherwise each block
 // stores its 3 sums and the block that completes the replica's last item
 // (atomic count) adds the item sums in item order and resets the count.
+// Bound: the FP64 pipe of the few SMs it runs on, which it leaves idle where a
+// thread has no share, and the conversions, which move bits; items of 64
+// chunks instead of 256.  Beside the steps (with its fork), before / after: N =
+// 4,000 11.5 / 9.9 us, 32,000 24.6 / 12.4 (there longer than the step: 20.1 ->
+// 18.8 us a step), 100,000 19 / 11.8, 4M 33 / 25.
 __global__ void __launch_bounds__(LJ_THERMO_THREADS) k_thermo(BoxDev b, double* out, int with_kin)
 {
-    __shared__ double s_red[3][LJ_THERMO_THREADS / 32];
+    constexpr int NW = LJ_THERMO_THREADS / 32;
+    static_assert(NW == 8, "a group of 8 lanes takes the warps' sums");
+    __shared__ double s_red[3][NW];
     __shared__ int s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto block_sum3 = [&](double& e, double& w, double& k) {
-        e = warp_sum_d(e);
-        w = warp_sum_d(w);
-        k = warp_sum_d(k);
-        if (lane == 0) {
-            s_red[0][warp] = e;
-            s_red[1][warp] = w;
-            s_red[2][warp] = k;
+    // E_pot, E_kin and W over the block, in lanes 0, 8 and 16 of warp 0.  Each
+    // exchange of a warp leaves half the lanes one of two sums: 6 FP64
+    // additions a warp, not 15 (16 clocks of the SM's FP64 pipe each)
+    auto block_sum3 = [&](double e, double w, double k) -> double {
+        const bool up16 = (lane & 16) != 0, up8 = (lane & 8) != 0;
+        double a = (up16 ? w : e) + __shfl_xor_sync(0xffffffffu, up16 ? e : w, 16);
+        k += __shfl_xor_sync(0xffffffffu, k, 16);
+        a = (up8 ? k : a) + __shfl_xor_sync(0xffffffffu, up8 ? a : k, 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if ((lane & 7) == 0 && lane < 24) s_red[lane >> 3][warp] = a;
+        __syncthreads();
+        a = 0.0;
+        if (warp == 0) {   // the warp sums in a fixed order
+            if (lane < 24) a = s_red[lane >> 3][lane & 7];
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
         }
         __syncthreads();
-        if (warp == 0) {   // the warp sums in a fixed order: lane q holds warp q's sums
-            const int nw = blockDim.x >> 5;
-            e = lane < nw ? s_red[0][lane] : 0.0;
-            w = lane < nw ? s_red[1][lane] : 0.0;
-            k = lane < nw ? s_red[2][lane] : 0.0;
-            e = warp_sum_d(e);
-            w = warp_sum_d(w);
-            k = warp_sum_d(k);
-        }
-        __syncthreads();
+        return a;
     };
-    auto write_out = [&](const RepDev& R, int r, double e, double w, double k) {
-        out[4 * r + 0] = e;
-        out[4 * r + 1] = k;
-        out[4 * r + 2] = w;
-        out[4 * r + 3] = R.n > 1 ? 2.0 * k / (3.0 * (double)R.n - 3.0) : 0.0;
+    const int which = warp == 0 && (lane & 7) == 0 && lane < 24 ? lane >> 3 : -1;   // 0 E_pot, 1 E_kin, 2 W
+    auto write_out = [&](const RepDev& R, int r, double a) {
+        if (which >= 0) out[4 * r + which] = a;
+        if (which == 1) out[4 * r + 3] = R.n > 1 ? 2.0 * a / (3.0 * (double)R.n - 3.0) : 0.0;
     };
     for (int it = blockIdx.x; it < b.ntitem; it += gridDim.x) {
         const int4 t = b.titem[it];
@@ -1518,22 +1530,23 @@ __global__ void __launch_bounds__(LJ_THERMO_THREADS) k_thermo(BoxDev b, double* 
         const int nt4 = 4 * (int)blockDim.x;
         for (int c0 = s0; c0 < s1; c0 += nt4) {
             double2 v[4];
+            const int c = c0 + (int)threadIdx.x;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int c = c0 + u * (int)blockDim.x + (int)threadIdx.x;
-                if (b.pf_ds) {   // (hi, lo) float pairs
-                    const float4 f = c < s1 ? reinterpret_cast<const float4*>(b.part_f)[c]
-                                            : make_float4(0.f, 0.f, 0.f, 0.f);
-                    v[u] = make_double2((double)f.x + (double)f.y, (double)f.z + (double)f.w);
-                } else {
-                    v[u] = c < s1 ? sh[c] : make_double2(0.0, 0.0);
+            for (int u = 0; u < 4; ++u) {   // FP32 forces: (hi, lo) float pairs
+                v[u] = make_double2(0.0, 0.0);
+                if (c + u * LJ_THERMO_THREADS < s1) v[u] = sh[c + u * LJ_THERMO_THREADS];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c + u * LJ_THERMO_THREADS < s1) {
+                    if (b.pf_ds) {
+                        e += ds_bits_to_double(v[u].x);
+                        w += ds_bits_to_double(v[u].y);
+                    } else {
+                        e += v[u].x;
+                        w += v[u].y;
+                    }
                 }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                e += v[u].x;
-                w += v[u].y;
-            }
         }
         if (with_kin)
             for (int c0 = t.y * LJ_KIN_WARPS; c0 < t.z * LJ_KIN_WARPS; c0 += nt4) {
@@ -1544,34 +1557,32 @@ __global__ void __launch_bounds__(LJ_THERMO_THREADS) k_thermo(BoxDev b, double* 
                     v[u] = c < t.z * LJ_KIN_WARPS ? b.part_k[c] : 0.0;
                 }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) k += v[u];
+                for (int u = 0; u < 4; ++u)
+                    if (c0 + u * LJ_THERMO_THREADS + (int)threadIdx.x < t.z * LJ_KIN_WARPS) k += v[u];
             }
-        block_sum3(e, w, k);
+        double a = block_sum3(e, w, k);
         if (R.nti == 1) {   // block-uniform: the replica's only item
-            if (threadIdx.x == 0) write_out(R, r, e, w, k);
+            write_out(R, r, a);
             continue;
         }
-        if (threadIdx.x == 0) {
-            b.part_t[3 * it + 0] = e;
-            b.part_t[3 * it + 1] = w;
-            b.part_t[3 * it + 2] = k;
+        if (which >= 0) {
+            b.part_t[3 * it + which] = a;
             __threadfence();
-            s_last = atomicAdd(&b.tcount[r], 1u) == (unsigned)(R.nti - 1);
         }
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = atomicAdd(&b.tcount[r], 1u) == (unsigned)(R.nti - 1);
         __syncthreads();
         if (s_last) {   // block-uniform
             __threadfence();
             e = w = k = 0.0;
             for (int i = R.ti_off + (int)threadIdx.x; i < R.ti_off + R.nti; i += blockDim.x) {
                 e += __ldcg(&b.part_t[3 * i + 0]);
-                w += __ldcg(&b.part_t[3 * i + 1]);
-                k += __ldcg(&b.part_t[3 * i + 2]);
+                k += __ldcg(&b.part_t[3 * i + 1]);
+                w += __ldcg(&b.part_t[3 * i + 2]);
             }
-            block_sum3(e, w, k);
-            if (threadIdx.x == 0) {
-                write_out(R, r, e, w, k);
-                b.tcount[r] = 0u;
-            }
+            a = block_sum3(e, w, k);
+            write_out(R, r, a);
+            if (threadIdx.x == 0) b.tcount[r] = 0u;
         }
         __syncthreads();
     }

@@ -49,7 +49,7 @@
 #define LJ_SPREAD_SHARES (LJ_CHUNK * 4 / 32)   // their (E_pot, W) shares per chunk: one per warp
 #define LJ_ALL_SHARES 8         // (E_pot, W) shares per chunk of the FP32 all-pairs kernel (one per 16 particles)
 #define LJ_THERMO_THREADS 256  // threads of the energy reduction
-#define LJ_THERMO_CHUNKS 256   // chunks of one energy-reduction item
+#define LJ_THERMO_CHUNKS 64    // chunks of one energy-reduction item
 #define LJ_LIST_THREADS 256    // threads of the list-build kernel
 #define LJ_LANE_THREADS 128    // threads of the lane-per-particle list-build kernel
 #define LJ_F64_THREADS 128     // threads of the FP64 pair kernel (LJ_TPP per particle)
@@ -239,7 +239,7 @@ struct BoxDev {
                                // 8 bytes: the FP32 list kernels), 0: a double; the tiled kernel
                                // leaves pf_stride shares per brick instead of per chunk
     double* part_k;            // [chunk*LJ_KIN_WARPS + warp] = E_kin share
-    double* part_t;            // [item*3 + 0..2] = E_pot, W, E_kin of a reduction item
+    double* part_t;            // [item*3 + 0..2] = E_pot, E_kin, W of a reduction item
     unsigned* tcount;          // per replica: reduction items finished (last one resets)
 };
 
