@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_scatter(BoxDev b)
 // k_list_work: the work of a rebuild, one block.  The rebuilding replicas in
 // order, with the prefixes of their cell and particle-chunk counts, so that
 // the per-cell kernels (k_sortgather, k_nlist_lanes) and the per-chunk ones
-// (k_bin, k_scatter, k_gather) stride over those cells and chunks only: a step
+// (k_bin, k_scatter) stride over those cells and chunks only: a step
 // in which a few replicas of many rebuild does not walk (and test) every cell
 // and chunk of the batch.  Launched first in every rebuild sequence.
 // ---------------------------------------------------------------------------
@@ -415,11 +415,14 @@ __global__ void __launch_bounds__(1024) k_list_work(BoxDev b, unsigned long long
 // every neighbour cell, the contiguous run of candidates within reach along
 // z.  The alternative layout (order 1) sorts a cell by a space-filling curve
 // over its 4 x 4 x 4 sub-cells first (Sec. 3: particles are sorted for
-// locality); the list build then takes whole neighbour cells.  The ranks are
-// written as each member's final slot (dst); k_gather then
-// moves the state, the new cell-relative offsets (computed by k_bin) and
-// their FP32 copy into the sorted arrays, one thread per particle.  (All
-// pairs: one cell per replica, no order; k_sortgather gathers directly.)
+// locality); the list build then takes whole neighbour cells.  The lane that
+// ranked a member moves its state, the new cell-relative offsets (computed by
+// k_bin) and their FP32 copy to its slot.  (All pairs: one cell per replica,
+// no order.)  Bound: DRAM and the latency of the gathered loads, all issued
+// before the stores.  A kernel of its own for the gather, one thread per
+// particle, had all its lanes busy (a cell fills 18 of 32), but read the keys'
+// lines again and was one more launch in every step: forced update at 256,000
+// 271 -> 262 us, at 4M 2837 -> 2771; a step at 100,000 39.4 -> 38.0 us.
 // ---------------------------------------------------------------------------
 // FP32 offset from the new cell centre, as posq will hold it (offB, from k_bin)
 __device__ __forceinline__ float offB32(const BoxDev& b, int c, int p)
@@ -505,9 +508,7 @@ __device__ __forceinline__ void gather_one(const BoxDev& b, int p, int q, int gc
     else gather_state<false>(b, p, q, gc);
 }
 
-// GATHER: move the members at once (the cluster rebuild: no barrier between
-// the ranks and the gather); otherwise the ranks go to dst for k_gather.
-template <bool GATHER>
+// Rank the members of the cells and move them to their slots.
 __device__ __forceinline__ void phase_rank(const BoxDev& b)
 {
     const int lane = threadIdx.x & 31;
@@ -534,10 +535,7 @@ __device__ __forceinline__ void phase_rank(const BoxDev& b)
                     rank += (kt < key) ? 1 : 0;
                 }
             }
-            if (idx < n) {
-                if (GATHER) gather_one(b, p, s0 + rank, gc);
-                else b.dst[s0 + idx] = s0 + rank;
-            }
+            if (idx < n) gather_one(b, p, s0 + rank, gc);
         }
     }
 }
@@ -562,22 +560,7 @@ __global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
         }
         return;
     }
-    phase_rank<false>(b);
-}
-
-__global__ void __launch_bounds__(LJ_CHUNK) k_gather(BoxDev b)
-{
-    await_previous();
-    if (b.all_pairs || !box_needs_rebuild(b)) return;
-    const int tot = work_chunks(b);
-    int kr = 0;
-    for (int t = blockIdx.x; t < tot; t += gridDim.x) {
-        const int4 ch = chunk_of(b, work_chunk(b, t, kr));
-        const int s = ch.y + (int)threadIdx.x;
-        if (s >= ch.z) continue;
-        const int p = b.perm[s];
-        gather_one(b, p, b.dst[s], b.cellB[p]);
-    }
+    phase_rank(b);
 }
 
 // ---------------------------------------------------------------------------
@@ -1208,7 +1191,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_rebuild_cluster(BoxDev b, i
     }
     phase_scatter(b);
     cluster_barrier();
-    phase_rank<true>(b);
+    phase_rank(b);
 }
 static_assert(kClusterThreads % LJ_CHUNK == 0, "whole groups");
 
@@ -1232,11 +1215,9 @@ cudaError_t launch_scatter(const BoxDev& b, Launch l)
     return launch_kernel(k_scatter, l.grid, LJ_CHUNK, 0, l.s, l.early, b);
 }
 
-cudaError_t launch_sortgather(const BoxDev& b, Launch l, Launch lg)
+cudaError_t launch_sortgather(const BoxDev& b, Launch l)
 {
-    cudaError_t e = launch_kernel(k_sortgather, l.grid, 256, 0, l.s, l.early, b);
-    if (e != cudaSuccess || b.all_pairs) return e;
-    return launch_kernel(k_gather, lg.grid, LJ_CHUNK, 0, lg.s, lg.early, b);
+    return launch_kernel(k_sortgather, l.grid, 256, 0, l.s, l.early, b);
 }
 
 cudaError_t launch_nlist(const BoxDev& b, Launch l)

@@ -449,11 +449,11 @@ md_status clear_err(md_box* b)
 // ------------------------------------------------------------------------
 // Kernels of one separate rebuild sequence (work lists where `runs` or several
 // replicas ask, bin, scan, its second pass where a replica has several tiles,
-// scatter, rank, gather, list; all pairs: binning only re-wraps and
+// scatter, rank and gather, list; all pairs: binning only re-wraps and
 // re-centres).
 int rebuild_kernels(md_box* b, bool runs)
 {
-    return (b->all_pairs ? 4 : 6) + ((int)b->tiles.size() > b->nrep ? 1 : 0) + (runs || b->nrep > 1 ? 1 : 0);
+    return (b->all_pairs ? 4 : 5) + ((int)b->tiles.size() > b->nrep ? 1 : 0) + (runs || b->nrep > 1 ? 1 : 0);
 }
 
 // Binning, sort and gather as one cluster launch (k_rebuild_cluster) instead
@@ -497,7 +497,7 @@ md_status enqueue_rebuild_kernels(md_box* b, int from_abs, cudaStream_t s, unsig
     Launch lt{std::max(1, std::min((int)b->tiles.size(), b->nsm * 8)), 0, s, early};
     CK(b, launch_scan_tiles(b->d, b->d_tiles, (int)b->tiles.size(), b->d_tile_sum, lt));
     CK(b, launch_scatter(b->d, l));
-    CK(b, launch_sortgather(b->d, on(b->all_pairs ? lch(b) : lcell(b)), l));
+    CK(b, launch_sortgather(b->d, on(b->all_pairs ? lch(b) : lcell(b))));
     if (!b->all_pairs) CK(b, launch_list(b, s, early && b->nrep == 1));
     b->launches += rebuild_kernels(b, runs != nullptr);
     return MD_OK;
@@ -1322,7 +1322,6 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
         CKS(dev_alloc(b, &d.typeB, b->np));
         CKS(dev_alloc(b, &d.cellB, b->np));
         CKS(dev_alloc(b, &d.perm, b->np));
-        CKS(dev_alloc(b, &d.dst, b->np));
         CKS(dev_alloc(b, &d.nbr_count, b->np));
         CKS(dev_alloc(b, &d.disp_max, nrep));
         CKS(dev_alloc(b, &d.rebuild_req, nrep));

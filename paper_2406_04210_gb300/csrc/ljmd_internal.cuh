@@ -194,7 +194,6 @@ struct BoxDev {
     int* typeB;
     int* cellB;
     int* perm;                 // slot -> old index, during a rebuild
-    int* dst;                  // slot of perm -> final slot (ranked in its cell), during a rebuild
     // cells
     int* cell_count;
     int* cell_start;
@@ -636,7 +635,7 @@ cudaError_t launch_scan_tiles(const BoxDev& b, const int4* tiles, int ntiles, in
                               Launch l);
 int ljmd_scan_tile_cells();
 cudaError_t launch_scatter(const BoxDev& b, Launch l);
-cudaError_t launch_sortgather(const BoxDev& b, Launch l, Launch lg);   // rank (l), then gather (lg) unless all pairs
+cudaError_t launch_sortgather(const BoxDev& b, Launch l);
 cudaError_t launch_nlist(const BoxDev& b, Launch l);
 // one warp per cell (per_particle 1) or per quarter of its particles (4 lanes per particle)
 cudaError_t launch_nlist_lanes(const BoxDev& b, int per_particle, Launch l);
