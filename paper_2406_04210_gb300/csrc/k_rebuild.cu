@@ -9,8 +9,8 @@
 // whole sequence can sit in a CUDA graph and cost one early exit per kernel
 // when no replica needs it.
 //
-// Sequence: k_bin (new cell of every particle, counts) -> k_scan_tiles +
-// k_scan_add (exclusive scan of the counts per replica) -> k_scatter (slot
+// Sequence: k_bin (new cell of every particle, counts) -> k_scan
+// (exclusive scan of the counts per replica) -> k_scatter (slot
 // per particle) -> k_sortgather (order inside each cell by FP32 z offset,
 // ties by user index, so the layout is a deterministic function of the
 // positions; gather into the sorted arrays) -> k_nlist (27-cell search,
@@ -23,7 +23,7 @@
 
 namespace {
 
-constexpr int kScanThreads = 128;
+constexpr int kScanThreads = 256;
 constexpr int kScanTile = 2048;   // cells per scan tile
 // The cluster rebuild: one cluster of 16 blocks (the most a cluster may hold)
 constexpr int kClusterBlocks = 16;
@@ -230,13 +230,12 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_bin(BoxDev b, int from_abs)
 }
 
 // ---------------------------------------------------------------------------
-// Exclusive scan of cell counts inside each replica, in two passes over
-// tiles of kScanTile cells, runs of consecutive cells per thread:
-// k_scan_tiles writes the tile-local prefix into cell_start and the tile
-// total into tile_sum; k_scan_add adds the totals of the replica's earlier
-// tiles plus the replica's first slot.  A replica of one tile is finished by
-// the first pass.  tiles[t] = (rep, first cell, end cell, first tile of the
-// replica).
+// Exclusive scan of cell counts inside each replica: a block per tile of
+// kScanTile cells, a run of consecutive cells per thread; it first sums the
+// counts of the replica's earlier tiles itself (from L2; at 4M the last of 101
+// tiles reads 0.8 MB), which costs the few builds less than a second pass, a
+// launch in every step: a step at N = 100,000 38.0 -> 36.6 us.  tiles[t] =
+// (rep, first cell, end cell, first tile of the replica).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int block_excl_scan(int v, int* s_warp, int& total)
 {
@@ -268,71 +267,46 @@ __device__ __forceinline__ int block_excl_scan(int v, int* s_warp, int& total)
     return r;
 }
 
-// cell c starts at slot s: its range is open for k_scatter (cell_end is the
-// cursor; it ends at start + count), its count is ready for the next build
-__device__ __forceinline__ void cell_open(const BoxDev& b, int c, int s)
-{
-    b.cell_start[c] = s;
-    b.cell_end[c] = s;
-    b.cell_count[c] = 0;
-}
-
 template <int THREADS>
-__device__ __forceinline__ void phase_scan_tiles(const BoxDev& b, const int4* tiles, int ntiles, int* tile_sum)
+__device__ __forceinline__ void phase_scan(const BoxDev& b, const int4* tiles, int ntiles)
 {
-    constexpr int kScanPer = kScanTile / THREADS;   // cells per thread
+    constexpr int PER = kScanTile / THREADS;   // cells per thread
     __shared__ int s_warp[33];
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int4 tl = tiles[t];
         if (!rep_needs_rebuild(b, tl.x)) continue;   // block-uniform
-        const int c0 = tl.y + (int)threadIdx.x * kScanPer;
-        int v[kScanPer], sum = 0;
+        const int c0 = tl.y + (int)threadIdx.x * PER;
+        int v[PER], sum = 0, part = 0, total;
 #pragma unroll
-        for (int u = 0; u < kScanPer; ++u) {
+        for (int u = 0; u < PER; ++u) {
             v[u] = c0 + u < tl.z ? b.cell_count[c0 + u] : 0;
             sum += v[u];
         }
-        int total;
-        int ex = block_excl_scan(sum, s_warp, total);
-        const bool whole = tl.z - tl.y == b.rep[tl.x].ncell;
-        if (whole) ex += b.rep[tl.x].p_off;
+        for (int c = b.rep[tl.x].cell_off + (int)threadIdx.x; c < tl.y; c += 8 * THREADS) {
+            int x[8];
 #pragma unroll
-        for (int u = 0; u < kScanPer; ++u) {
-            if (c0 + u < tl.z) {
-                if (whole) cell_open(b, c0 + u, ex);
-                else b.cell_start[c0 + u] = ex;
+            for (int u = 0; u < 8; ++u) x[u] = c + u * THREADS < tl.y ? b.cell_count[c + u * THREADS] : 0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) part += x[u];
+        }
+        int before = 0;
+        if (t != tl.w) block_excl_scan(part, s_warp, before);   // block-uniform
+        int ex = block_excl_scan(sum, s_warp, total) + before + b.rep[tl.x].p_off;
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            if (c0 + u < tl.z) {   // the range is open for k_scatter (cell_end is the cursor; it ends at start + count)
+                b.cell_start[c0 + u] = ex;
+                b.cell_end[c0 + u] = ex;
             }
             ex += v[u];
         }
-        if (threadIdx.x == 0) tile_sum[t] = total;
     }
 }
 
-__device__ __forceinline__ void phase_scan_add(const BoxDev& b, const int4* tiles, int ntiles, const int* tile_sum)
-{
-    __shared__ int s_warp[33];
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int4 tl = tiles[t];
-        if (!rep_needs_rebuild(b, tl.x) || tl.z - tl.y == b.rep[tl.x].ncell) continue;   // block-uniform
-        int part = 0, before;
-        for (int u = tl.w + (int)threadIdx.x; u < t; u += blockDim.x) part += tile_sum[u];
-        block_excl_scan(part, s_warp, before);
-        before += b.rep[tl.x].p_off;
-        for (int c = tl.y + (int)threadIdx.x; c < tl.z; c += blockDim.x) cell_open(b, c, b.cell_start[c] + before);
-    }
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_tiles(BoxDev b, const int4* tiles, int ntiles, int* tile_sum)
+__global__ void __launch_bounds__(kScanThreads) k_scan(BoxDev b, const int4* tiles, int ntiles)
 {
     await_previous();
-    if (box_needs_rebuild(b)) phase_scan_tiles<kScanThreads>(b, tiles, ntiles, tile_sum);
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_scan_add(BoxDev b, const int4* tiles, int ntiles,
-                                                            const int* tile_sum)
-{
-    await_previous();
-    if (box_needs_rebuild(b)) phase_scan_add(b, tiles, ntiles, tile_sum);
+    if (box_needs_rebuild(b)) phase_scan<kScanThreads>(b, tiles, ntiles);
 }
 
 // ---------------------------------------------------------------------------
@@ -520,6 +494,7 @@ __device__ __forceinline__ void phase_rank(const BoxDev& b)
         const RepDev& R = b.rep[b.nrep == 1 ? 0 : b.lw_rep[kr]];
         int s0 = b.cell_start[gc];
         int n = b.cell_end[gc] - s0;
+        if (lane == 0) b.cell_count[gc] = 0;   // for the next build
         for (int base = 0; base < n; base += 32) {
             int idx = base + lane;
             int p = idx < n ? b.perm[s0 + idx] : -1;
@@ -553,7 +528,10 @@ __global__ void __launch_bounds__(256) k_sortgather(BoxDev b)
             const int4 ch = chunk_of(b, work_chunk(b, t, kr));
             const RepDev& R = b.rep[ch.x];
             for (int s = ch.y + (int)threadIdx.x; s < ch.z; s += blockDim.x) {
-                if (s == R.p_off) atomicAdd(&b.nbuild[ch.x], 1ull);   // a re-binning
+                if (s == R.p_off) {
+                    atomicAdd(&b.nbuild[ch.x], 1ull);   // a re-binning
+                    b.cell_count[R.cell_off] = 0;       // for the next one
+                }
                 const int p = b.perm[s];
                 gather_one(b, p, R.p_off + (b.uidB[p] - R.u_off), R.cell_off);
             }
@@ -1173,7 +1151,7 @@ __device__ __forceinline__ void cluster_barrier()
 }
 
 __global__ void __launch_bounds__(kClusterThreads) k_rebuild_cluster(BoxDev b, int from_abs, const int4* tiles,
-                                                                      int ntiles, int* tile_sum)
+                                                                      int ntiles)
 {
     await_previous();
     if (!box_needs_rebuild(b)) return;   // the same word for every block: none is left waiting
@@ -1183,12 +1161,8 @@ __global__ void __launch_bounds__(kClusterThreads) k_rebuild_cluster(BoxDev b, i
     }
     phase_bin(b, from_abs);
     cluster_barrier();
-    phase_scan_tiles<kClusterThreads>(b, tiles, ntiles, tile_sum);
+    phase_scan<kClusterThreads>(b, tiles, ntiles);
     cluster_barrier();
-    if (ntiles > b.nrep) {   // some replica has more than one tile
-        phase_scan_add(b, tiles, ntiles, tile_sum);
-        cluster_barrier();
-    }
     phase_scatter(b);
     cluster_barrier();
     phase_rank(b);
@@ -1202,12 +1176,9 @@ cudaError_t launch_bin(const BoxDev& b, int from_abs, Launch l)
     return launch_kernel(k_bin, l.grid, LJ_CHUNK, 0, l.s, l.early, b, from_abs);
 }
 
-cudaError_t launch_scan_tiles(const BoxDev& b, const int4* tiles, int ntiles, int* tile_sum,
-                              Launch l)
+cudaError_t launch_scan(const BoxDev& b, const int4* tiles, int ntiles, Launch l)
 {
-    cudaError_t e = launch_kernel(k_scan_tiles, l.grid, kScanThreads, 0, l.s, l.early, b, tiles, ntiles, tile_sum);
-    if (e != cudaSuccess || ntiles <= b.nrep) return e;   // one tile per replica: finished
-    return launch_kernel(k_scan_add, l.grid, kScanThreads, 0, l.s, l.early, b, tiles, ntiles, tile_sum);
+    return launch_kernel(k_scan, l.grid, kScanThreads, 0, l.s, l.early, b, tiles, ntiles);
 }
 
 cudaError_t launch_scatter(const BoxDev& b, Launch l)
@@ -1265,7 +1236,7 @@ bool cluster_rebuild_fits()
     return ok;
 }
 
-cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles, int* tile_sum,
+cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles,
                                    cudaStream_t s, bool early)
 {
     cudaLaunchConfig_t c{};
@@ -1280,7 +1251,7 @@ cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* ti
     c.stream = s;
     c.attrs = at;
     c.numAttrs = early ? 2 : 1;
-    return cudaLaunchKernelEx(&c, k_rebuild_cluster, b, from_abs, tiles, ntiles, tile_sum);
+    return cudaLaunchKernelEx(&c, k_rebuild_cluster, b, from_abs, tiles, ntiles);
 }
 
 int ljmd_scan_tile_cells() { return kScanTile; }

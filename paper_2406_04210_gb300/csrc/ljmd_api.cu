@@ -105,7 +105,6 @@ struct md_box {
     std::vector<int4> bricks;  // work items of the tiled force kernel: (replica, first cell x, y, z)
     size_t pf_cap = 0;         // doubles of one of the two sets of d.part_f
     int4* d_brick = nullptr;
-    int* d_tile_sum = nullptr;
     int* d_type_user = nullptr;
     double* d_thermo = nullptr;
     int64_t thermo_cap = 0;    // doubles
@@ -448,12 +447,11 @@ md_status clear_err(md_box* b)
 // Rebuild / force sequences
 // ------------------------------------------------------------------------
 // Kernels of one separate rebuild sequence (work lists where `runs` or several
-// replicas ask, bin, scan, its second pass where a replica has several tiles,
-// scatter, rank and gather, list; all pairs: binning only re-wraps and
-// re-centres).
+// replicas ask, bin, scan, scatter, rank and gather, list; all pairs: binning
+// only re-wraps and re-centres).
 int rebuild_kernels(md_box* b, bool runs)
 {
-    return (b->all_pairs ? 4 : 5) + ((int)b->tiles.size() > b->nrep ? 1 : 0) + (runs || b->nrep > 1 ? 1 : 0);
+    return (b->all_pairs ? 4 : 5) + (runs || b->nrep > 1 ? 1 : 0);
 }
 
 // Binning, sort and gather as one cluster launch (k_rebuild_cluster) instead
@@ -495,7 +493,7 @@ md_status enqueue_rebuild_kernels(md_box* b, int from_abs, cudaStream_t s, unsig
     if (runs || b->nrep > 1) CK(b, launch_list_work(b->d, runs, s, early));
     CK(b, launch_bin(b->d, from_abs, l));
     Launch lt{std::max(1, std::min((int)b->tiles.size(), b->nsm * 8)), 0, s, early};
-    CK(b, launch_scan_tiles(b->d, b->d_tiles, (int)b->tiles.size(), b->d_tile_sum, lt));
+    CK(b, launch_scan(b->d, b->d_tiles, (int)b->tiles.size(), lt));
     CK(b, launch_scatter(b->d, l));
     CK(b, launch_sortgather(b->d, on(b->all_pairs ? lch(b) : lcell(b))));
     if (!b->all_pairs) CK(b, launch_list(b, s, early && b->nrep == 1));
@@ -506,7 +504,7 @@ md_status enqueue_rebuild_kernels(md_box* b, int from_abs, cudaStream_t s, unsig
 md_status enqueue_rebuild(md_box* b, int from_abs)
 {
     if (!cluster_rebuild(b)) return enqueue_rebuild_kernels(b, from_abs, b->stream, nullptr);
-    CK(b, launch_rebuild_cluster(b->d, from_abs, b->d_tiles, (int)b->tiles.size(), b->d_tile_sum, b->stream, b->early));
+    CK(b, launch_rebuild_cluster(b->d, from_abs, b->d_tiles, (int)b->tiles.size(), b->stream, b->early));
     CK(b, launch_list(b, b->stream, b->early && b->nrep == 1));
     b->launches += 2;
     return MD_OK;
@@ -680,7 +678,6 @@ md_status make_grid(md_box* b)
     dev_release(b, b->d_tiles);
     dev_release(b, b->d_brick);
     b->d_brick = nullptr;
-    dev_release(b, b->d_tile_sum);
     d.cell_count = d.cell_start = d.cell_end = nullptr;
     d.cell_rep = nullptr;
     CKS(dev_alloc(b, &d.cell_count, d.ncell));
@@ -697,7 +694,6 @@ md_status make_grid(md_box* b)
     }
     d.cell_rep = cr;
     CKS(dev_alloc(b, &b->d_tiles, b->tiles.size(), false));
-    CKS(dev_alloc(b, &b->d_tile_sum, b->tiles.size()));
     CK(b, cudaMemcpyAsync(b->d_tiles, b->tiles.data(), sizeof(int4) * b->tiles.size(),
                           cudaMemcpyHostToDevice, b->stream));
     CKS(dev_alloc(b, &b->d_brick, b->bricks.size(), false));

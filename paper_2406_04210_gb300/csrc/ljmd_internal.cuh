@@ -631,8 +631,7 @@ inline cudaError_t launch_kernel(void (*k)(P...), int grid, int block, size_t sm
 
 // k_rebuild.cu
 cudaError_t launch_bin(const BoxDev& b, int from_abs, Launch l);
-cudaError_t launch_scan_tiles(const BoxDev& b, const int4* tiles, int ntiles, int* tile_sum,
-                              Launch l);
+cudaError_t launch_scan(const BoxDev& b, const int4* tiles, int ntiles, Launch l);
 int ljmd_scan_tile_cells();
 cudaError_t launch_scatter(const BoxDev& b, Launch l);
 cudaError_t launch_sortgather(const BoxDev& b, Launch l);
@@ -642,7 +641,7 @@ cudaError_t launch_nlist_lanes(const BoxDev& b, int per_particle, Launch l);
 // one block; before the cell kernels; counts its executions with work in *runs (nullable)
 cudaError_t launch_list_work(const BoxDev& b, unsigned long long* runs, cudaStream_t s, bool early);
 // binning, sort and gather in one launch of one cluster (small boxes)
-cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles, int* tile_sum,
+cudaError_t launch_rebuild_cluster(const BoxDev& b, int from_abs, const int4* tiles, int ntiles,
                                    cudaStream_t s, bool early);
 bool cluster_rebuild_fits();
 // k_force.cu
