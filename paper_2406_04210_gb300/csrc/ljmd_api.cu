@@ -456,10 +456,11 @@ int rebuild_kernels(md_box* b, bool runs)
 
 // Binning, sort and gather as one cluster launch (k_rebuild_cluster) instead
 // of the separate kernels: boxes whose stages 16 blocks get through faster
-// than the launches cost.  Per step, separate against cluster: N = 4,000
-// 33.4 / 28.1 us, N = 32,000 (the list update's phase) 22.5 / 19.0 us,
-// N = 100,000 61.4 / 69.6 us.
-constexpr int kClusterSlots = 32768;
+// than the launches cost.  Us a step with energies, separate against cluster:
+// N = 8,000 13.4 / 10.8, 24,000 17.5 / 15.8, 48,000 24.8 / 23.2, 64,000 27.7 /
+// 26.7 (where the 16 SMs' build, an order of magnitude longer than on all,
+// takes that back in hotter runs).
+constexpr int kClusterSlots = 49152;
 bool cluster_rebuild(md_box* b)
 {
     if (b->all_pairs || !b->cluster_ok) return false;

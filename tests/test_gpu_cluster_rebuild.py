@@ -2,7 +2,7 @@
 step graphs the same stages run as separate kernels.  Both must give the same
 trajectories and energies bit for bit: one scan tile and two (over 2048
 cells), several replicas of uneven size, the largest boxes on the cluster path
-(32,768 slots) and the first beyond it, each precision."""
+(49,152 slots) and the first beyond it, each precision."""
 import numpy as np
 import pytest
 
@@ -24,6 +24,7 @@ def ljmd():
 
 @pytest.mark.parametrize("prec", ["mixed_ds", "mixed_fp64", "fp64"])
 @pytest.mark.parametrize("sizes,rho,rcut", [((300,), 0.8, 2.5), ((32768,), 0.7, 2.2), ((32769,), 0.7, 2.2),
+                                            ((49152,), 0.7, 2.2), ((49153,), 0.7, 2.2),
                                             ((500, 4001, 977), 0.8, 2.5)])
 def test_cluster_and_separate_rebuilds_agree(ljmd, sizes, rho, rcut, prec):
     ss = [inputs.fcc_subset_system(n, rho, 2.0, seed=n, rcut=rcut) for n in sizes]

@@ -29,7 +29,8 @@ def _run(make, profiled, dt, steps):
 
 
 @pytest.mark.parametrize("n,prec", [(500, "mixed_ds"), (8192, "mixed_ds"), (8193, "mixed_ds"), (8192, "fp64"),
-                                    (20000, "mixed_fp64"), (40000, "mixed_ds"), (140000, "mixed_ds")])
+                                    (20000, "mixed_fp64"), (40000, "mixed_ds"),
+                                    (49152, "mixed_ds"), (49153, "mixed_ds"), (140000, "mixed_ds")])
 def test_one_box(ljmd, n, prec):
     s = inputs.fcc_subset_system(n, 0.8, 3.0, seed=n)
     for x, y in zip(*(_run(lambda: ljmd.from_system(s, prec), prof, 0.003, 30) for prof in (False, True))):
