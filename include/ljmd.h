@@ -224,8 +224,9 @@ md_status md_pair_hist(md_box* b, int32_t nbins, double rhist, double width,
  * a static device array of 524,288 doubles (4 MiB) that every GPU loading
  * the library holds until the process exits; boxes needing more (16 doubles
  * per 128 particles with FP32 forces, 8 all-FP64, 2 in the all-pairs form,
- * + 4 per replica; about 4.19M particles for one box) are rejected with
- * MD_ERR_ARG and a message.  The first call on a device looks up that array's address
+ * + 4 per replica; about 4.19M particles for one box; boxes of up to 512 and
+ * 1,024 such chunks use 32 and, all pairs, 16, far inside it) are rejected
+ * with MD_ERR_ARG and a message.  The first call on a device looks up that array's address
  * (cudaGetSymbolAddress); make that first call before any stream capture.
  * All calls share the one array and overwrite what they use, so calls whose
  * GPU work overlaps (on different streams or boxes) race.
@@ -323,12 +324,12 @@ md_status md_get_layout(md_box* b, double* cell_scale, int32_t* order);
  *                  quads of particles with the candidates spread over its
  *                  lanes (each neighbour cell narrowed to its z-run within
  *                  reach under MD_ORDER_ZRUN)
- *   MD_LIST_LANES  one warp per cell, one lane per particle of the cell; the
- *                  warp stages each candidate once (dropping those beyond
+ *   MD_LIST_LANES  one warp per cell, one lane per particle of the cell (four
+ *                  in boxes of up to 2,048 cells); the warp stages each candidate once (dropping those beyond
  *                  the list radius of the cell's box) and every lane tests
  *                  it against its own particle; each lane's row is buffered
- *                  in shared memory as 16-bit codes (48 per lane) and
- *                  written out in 16-entry blocks
+ *                  in shared memory (40 entries per lane) and written out in
+ *                  pieces of four
  *   MD_LIST_AUTO   (default) MD_LIST_LANES
  * The setting takes effect at the next list build. */
 enum { MD_LIST_AUTO = 0, MD_LIST_QUADS = 1, MD_LIST_LANES = 2 };
@@ -354,7 +355,7 @@ md_status md_get_list_kernel(md_box* b, int32_t* kind);
  *                    reported as MD_ERR_TIMEOUT by the call)
  *   MD_FORCE_AUTO    (default) MD_FORCE_CHUNKS until md_autotune times both
  *                    and sets the faster one
- * On the 4M-particle fluid the chunk kernel is the faster (0.54 against
+ * On the 4M-particle fluid the chunk kernel is the faster (0.50 against
  * 0.65 ms per launch on GB300).  The FP64 precision and the all-pairs form
  * have kernels of their own and ignore the setting.  md_force_noalloc always
  * uses MD_FORCE_CHUNKS.  The setting takes effect at the next force
@@ -365,12 +366,12 @@ md_status md_set_force_kernel(md_box* b, int32_t kind);
 md_status md_get_force_kernel(md_box* b, int32_t* kind);
 
 /* Step graphs: with on = 1 the list update of each captured step is a
- * conditional (IF) node, so steps without a list build launch one tiny kernel
- * instead of the rebuild sequence; with on = 0 (default) the rebuild kernels
- * are captured unconditionally and exit early when no build is due.  Results
- * are the same bit for bit.  On GB300 the node costs ~4.5 us per step more
- * than the early exits (measured at N = 2,000 and 97,556), so it pays only
- * in launch count.  Profilers cannot look inside graphs with conditional
+ * conditional (IF) node whose condition the integrator sets, so steps without
+ * a list build skip the rebuild sequence; with on = 0 (default) the rebuild
+ * kernels are captured unconditionally, launched programmatically, and exit
+ * early when no build is due.  Results are the same bit for bit.  On GB300 the
+ * node costs more per step than the early exits (~4.5 us against seven plain
+ * ones at N = 2,000 and 97,556), so it pays only in launch count.  Profilers cannot look inside graphs with conditional
  * nodes.  If the runtime refuses the node the box falls back to on = 0 by
  * itself; md_get_graph_conditional reads the mode in use. */
 md_status md_set_graph_conditional(md_box* b, int32_t on);

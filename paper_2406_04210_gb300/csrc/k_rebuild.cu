@@ -1136,8 +1136,8 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
 // k_rebuild_cluster: binning, sort and gather of small boxes in one launch,
 // by one thread-block cluster whose blocks meet at the hardware's cluster
 // barrier between the stages.  A step without a build then pays two early
-// exits (this and the list build) instead of eight, and a build no launches
-// between the stages; the list build stays a kernel of its own, as it wants
+// exits (this and the list build) instead of five (eight when this was
+// measured first), and a build no launches between the stages; the list build stays a kernel of its own, as it wants
 // every SM.  (One cooperative launch for everything, with grid barriers, was
 // measured first: its launch inside a step graph cost nearly what the early
 // exits had, 32.7 us a step at N = 4,000 against 34.3.)

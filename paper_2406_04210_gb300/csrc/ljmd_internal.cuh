@@ -10,26 +10,28 @@
 //     MD_PREC_MIXED_DS the offsets and velocities are double-single pairs
 //     (hi, lo) of FP32; otherwise FP64.
 //   * posq[p] = (float offset x, y, z, type bits) feeds the FP32 pair kernels.
-//   * pair work is done per "segment": a run of up to S consecutive cells
-//     along x inside one row (cy, cz) of a replica.  Its particles are one
-//     contiguous slot range, and the 27-cell neighbourhood of all its cells
-//     is the "tile": 9 rows x (S + 2) cells, i.e. at most 18 contiguous slot
-//     ranges ("pieces"), staged in shared memory.
+//   * the quad list kernel works per "segment": a run of up to S consecutive
+//     cells along x inside one row (cy, cz) of a replica.  Its particles are
+//     one contiguous slot range, and the 27-cell neighbourhood of all its
+//     cells is the "tile": 9 rows x (S + 2) cells, i.e. at most 18 contiguous
+//     slot ranges ("pieces"), staged in shared memory.  The lane list kernel
+//     (the default) works per cell.
 //   * Verlet lists (Sec. 3) are 32-bit entries: the slot j in bits 31-6 and the
 //     image shift of j's cell relative to i's cell as three 2-bit digits
 //     (dz+1, dy+1, dx+1 in bits 5-4, 3-2, 1-0), so
 //     d_ij = (o_i - o_j) - (dx, dy, dz) * cell edge, decoded with integer and
 //     FP32 arithmetic (no table): low digits fall inside an FP32 mantissa by
-//     one and-or each, where digits above the slot took a shift more.  The stencil code k = 9(dz+1) + 3(dy+1) +
-//     (dx+1) orders the 27 cells.
+//     one and-or each, where digits above the slot took a shift more.  The
+//     stencil code k = 9(dz+1) + 3(dy+1) + (dx+1) orders the 27 cells.
 //     Entry s of particle p is nbr[p K + s] (K a multiple of 16): the FP32
 //     force kernel reads a row in blocks of 16 entries, one 16-byte load per
 //     thread of the particle; entries past the count are never written, and
 //     the kernel replaces them by the sentinel slot np in the last block.
-//   * the list build works per segment with the tile staged in shared memory;
-//     the pair-force kernels work per 128-particle chunk, 4 threads per
-//     particle, and gather neighbour offsets through L1 (the 64 particles of a
-//     block pass are consecutive, so they share one 27-cell neighbourhood).
+//   * the pair-force kernels work per 128-particle chunk, or a part of one, 4
+//     threads per particle, and gather neighbour offsets through L1 (the
+//     particles of an item are consecutive, so they share one 27-cell
+//     neighbourhood).
+//   * MD_PREC_FP64 with one species: offx, the offsets as 64-bit integers.
 #pragma once
 
 #include <cuda_runtime.h>
