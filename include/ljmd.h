@@ -283,8 +283,7 @@ md_status md_get_info(md_box* b, md_info* out);
  * configurations per device; here they are set or timed per box), t[4]:
  *   t[0] blocks per SM of the pair-force kernels  (0 = default: by form and
  *        size, a block per work item for FP32 lists of one species)
- *   t[1] blocks per SM of the list build          (0 = default: lanes 32, 8 with
- *        several replicas; quads 6)
+ *   t[1] blocks per SM of the list build          (0 = default: lanes 32, quads 6)
  *   t[2] cells per list-build segment, <= 16      (0 = automatic: ~1400
  *        particles per 27-cell tile)
  *   t[3] neighbour-list slots per particle       (0 = automatic: fitted to

@@ -368,12 +368,11 @@ bool lanes_list(md_box* b)
 cudaError_t launch_list(md_box* b, cudaStream_t s, bool early = false)
 {
     if (lanes_list(b)) {
-        // 8 resident blocks (64 registers, 27 KB); one replica, four rounds of
-        // them, handed out in order (see force_grid; more would cost the early
-        // exits of the steps that keep their lists): forced update at 1M 868 ->
-        // 829 us, 4M 3151 -> 2956, 256,000 281 -> 282.  Several replicas: each
-        // block walks the rebuilding replicas' list.
-        const int per_sm = b->list_per_sm > 0 ? b->list_per_sm : (b->nrep == 1 ? 32 : 8);
+        // 8 resident blocks (64 registers, 27 KB), four rounds of them, handed
+        // out in order (see force_grid; more would cost the early exits of the
+        // steps that keep their lists): forced update at 1M 868 -> 829 us, 4M
+        // 3151 -> 2956, 256,000 281 -> 282; a step of 512 replicas 610 -> 600.
+        const int per_sm = b->list_per_sm > 0 ? b->list_per_sm : 32;
         const int warps = LJ_LANE_THREADS / 32;
         // four lanes per particle where a warp per cell leaves schedulers
         // idle: forced update (with host overhead) at N = 4,000 160 -> 134 us,
