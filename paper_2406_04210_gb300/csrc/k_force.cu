@@ -1463,7 +1463,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_force_all_f64(BoxDev b)
 // A share of the FP32 forces: its (hi, lo) pair, stored where a double stands.
 __device__ __forceinline__ double ds_bits_to_double(double v)
 {
-    return f2d(__int_as_float(__double2loint(v))) + f2d(__int_as_float(__double2hiint(v)));
+    return f2d_exact(__int_as_float(__double2loint(v))) + f2d_exact(__int_as_float(__double2hiint(v)));
 }
 
 // E_pot, E_kin, W, T per replica from the per-chunk partial sums, in a
@@ -1478,7 +1478,8 @@ __device__ __forceinline__ double ds_bits_to_double(double v)
 // chunks instead of 256.  Beside the steps (with its fork), before / after: N =
 // 4,000 11.5 / 9.9 us, 32,000 24.6 / 12.4 (there longer than the step: 20.1 ->
 // 18.8 us a step), 100,000 19 / 11.8, 4M 33 / 25.
-__global__ void __launch_bounds__(LJ_THERMO_THREADS) k_thermo(BoxDev b, double* out, int with_kin)
+// Block `bid` of `nb`; host (nullable): the same in host memory.
+__device__ __forceinline__ void thermo_items(const BoxDev& b, double* out, double* host, int with_kin, int bid, int nb)
 {
     constexpr int NW = LJ_THERMO_THREADS / 32;
     static_assert(NW == 8, "a group of 8 lanes takes the warps' sums");
@@ -1509,9 +1510,10 @@ __global__ void __launch_bounds__(LJ_THERMO_THREADS) k_thermo(BoxDev b, double* 
     const int which = warp == 0 && (lane & 7) == 0 && lane < 24 ? lane >> 3 : -1;   // 0 E_pot, 1 E_kin, 2 W
     auto write_out = [&](const RepDev& R, int r, double a) {
         if (which >= 0) out[4 * r + which] = a;
+        if (which >= 0 && host) host[4 * r + which] = a;
         if (which == 1) out[4 * r + 3] = R.n > 1 ? 2.0 * a / (3.0 * (double)R.n - 3.0) : 0.0;
     };
-    for (int it = blockIdx.x; it < b.ntitem; it += gridDim.x) {
+    for (int it = bid; it < b.ntitem; it += nb) {
         const int4 t = b.titem[it];
         const int r = t.x;
         const RepDev& R = b.rep[r];
@@ -1585,6 +1587,45 @@ __global__ void __launch_bounds__(LJ_THERMO_THREADS) k_thermo(BoxDev b, double* 
             if (threadIdx.x == 0) b.tcount[r] = 0u;
         }
         __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(LJ_THERMO_THREADS) k_thermo(BoxDev b, double* out, int with_kin)
+{
+    thermo_items(b, out, nullptr, with_kin, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// What follows the force kernel of a single evaluation, in one launch: blocks
+// below nred reduce the energies, the others write the forces in user order
+// (f nullable), and the energies and the error words go straight to pinned
+// host memory.  Latency-bound: as two kernels and two copies, each waiting for
+// the one before, they were a fifth of a call: N = 4,000 64.6 -> 50.1 us.
+__global__ void __launch_bounds__(LJ_THERMO_THREADS) k_force_finish(BoxDev b, double* out, double* f, double* host_th,
+                                                                    int* host_err, int nred)
+{
+    if ((int)blockIdx.x < nred) {
+        if (blockIdx.x == 0 && threadIdx.x < 3) host_err[threadIdx.x] = b.err[threadIdx.x];
+        thermo_items(b, out, host_th, 0, (int)blockIdx.x, nred);
+        return;
+    }
+    constexpr int PER = LJ_THERMO_THREADS / LJ_CHUNK;   // chunks a block takes at a time
+    const int np = b.np;
+    for (int w = PER * ((int)blockIdx.x - nred) + (int)threadIdx.x / LJ_CHUNK; w < b.nchunk;
+         w += PER * ((int)gridDim.x - nred)) {
+        const int4 ch = chunk_of(b, w);
+        const int p = ch.y + (int)threadIdx.x % LJ_CHUNK;
+        if (p >= ch.z) continue;
+        const size_t gu = (size_t)b.uid[p];
+        if (b.prec == 2) {
+            double q[3];
+            for (int c = 0; c < 3; ++c) q[c] = b.force64[c * np + p];
+            for (int c = 0; c < 3; ++c) f[3 * gu + c] = q[c];
+        } else {
+            const float4 q = b.force4[p];
+            f[3 * gu + 0] = f2d_exact(q.x);
+            f[3 * gu + 1] = f2d_exact(q.y);
+            f[3 * gu + 2] = f2d_exact(q.z);
+        }
     }
 }
 
@@ -1693,6 +1734,13 @@ int force_tile_blocks_per_sm(int mono)
         o = (e == cudaSuccess && v > 0) ? v : 2;
     }
     return o > 0 ? o : 2;
+}
+
+cudaError_t launch_force_finish(const BoxDev& b, double* out, double* f, double* host_th, int* host_err, int nred,
+                                Launch l)
+{
+    k_force_finish<<<nred + l.grid, LJ_THERMO_THREADS, 0, l.s>>>(b, out, f, host_th, host_err, nred);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_thermo(const BoxDev& b, double* out, int with_kin, Launch l)

@@ -174,6 +174,7 @@ struct md_box {
     double eps0 = 1.0, sigma0 = 1.0, rcut0 = 0.0, shift0 = 0.0;   // the first pair's parameters
     long long* d_offx = nullptr; // offsets as integers (FP64 precision, one species)
     PinnedBack* pin = nullptr;   // pinned host memory
+    PinnedBack* pin_dev = nullptr;   // and its device address
     std::string err;
 };
 
@@ -1278,6 +1279,7 @@ md_status md_batch_create(md_box** out, int32_t nrep, const int64_t* n, const do
         CKS(enter(b));
         CK(b, cudaHostAlloc(reinterpret_cast<void**>(&b->pin), sizeof(PinnedBack) + 4 * sizeof(double) * (size_t)nrep,
                             cudaHostAllocDefault));
+        CK(b, cudaHostGetDevicePointer(reinterpret_cast<void**>(&b->pin_dev), b->pin, 0));
         BoxDev& d = b->d;
         copy_reps_to(b, d);
         size_t np3 = 3 * (size_t)b->np;
@@ -1574,21 +1576,21 @@ md_status md_force(md_box* b, double* force_out, double* epot, double* virial)
     CKS(enter(b));
     CKS(ensure_thermo(b, 1));
     CKS(clear_err(b));
-    CKS(enqueue_force(b, 1, b->d_thermo));
-    if (force_out && b->ntot > 0) {
-        size_t fb = sizeof(double) * 3 * (size_t)b->ntot;
-        if (is_device_ptr(force_out)) {
-            CK(b, launch_force_out(b->d, force_out, lch(b)));
-        } else {
-            CKS(ensure_stage(b, fb));
-            CK(b, launch_force_out(b->d, static_cast<double*>(b->d_stage), lch(b)));
-            CK(b, cudaMemcpyAsync(force_out, b->d_stage, fb, cudaMemcpyDeviceToHost, b->stream));
-        }
-    }
+    const bool want = force_out && b->ntot > 0, dev = want && is_device_ptr(force_out);
+    const size_t fb = sizeof(double) * 3 * (size_t)b->ntot;
+    if (want && !dev) CKS(ensure_stage(b, fb));
+    CKS(enqueue_force(b, 1, nullptr));
+    // the reduction beside the output, their results straight into the pinned page
+    Launch lo = lch(b);
+    lo.grid = want ? (lo.grid + 1) / 2 : 0;   // two chunks per block
+    CK(b, launch_force_finish(b->d, b->d_thermo, dev ? force_out : static_cast<double*>(b->d_stage), b->pin_dev->th,
+                              b->pin_dev->err, lthermo(b).grid, lo));
+    b->launches += 1;
+    if (want && !dev) CK(b, cudaMemcpyAsync(force_out, b->d_stage, fb, cudaMemcpyDeviceToHost, b->stream));
+    CK(b, cudaStreamSynchronize(b->stream));
     const double* th = b->pin->th;
-    CK(b, cudaMemcpyAsync(b->pin->th, b->d_thermo, 4 * sizeof(double) * b->nrep, cudaMemcpyDeviceToHost, b->stream));
     int e2[3];
-    CKS(read_err(b, e2));   // waits for everything above
+    std::memcpy(e2, b->pin->err, sizeof e2);
     for (int r = 0; r < b->nrep; ++r) {
         if (epot) epot[r] = th[4 * r + 0];
         if (virial) virial[r] = th[4 * r + 2];

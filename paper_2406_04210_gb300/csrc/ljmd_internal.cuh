@@ -255,6 +255,13 @@ __device__ __forceinline__ double f2d(float f)
     return __hiloint2double((int)((u & 0x80000000u) | (e + inf)), m < 0x00800000u ? 0 : (int)(u << 29));
 }
 
+// The same, exact for subnormals too (their conversion is a branch away).
+__device__ __forceinline__ double f2d_exact(float f)
+{
+    const unsigned m = __float_as_uint(f) & 0x7fffffffu;
+    return m != 0u && m < 0x00800000u ? (double)f : f2d(f);
+}
+
 // ---- double-single helpers (Dekker / Knuth error-free transformations) ----
 __device__ __forceinline__ void ds_two_sum(float a, float b, float& s, float& e)
 {
@@ -649,6 +656,9 @@ bool cluster_rebuild_fits();
 // k_force.cu
 cudaError_t launch_force(const BoxDev& b, int energy, Launch l);
 cudaError_t launch_thermo(const BoxDev& b, double* out, int with_kin, Launch l);
+// the reduction (nred blocks), the forces in user order (l.grid blocks; f null: 0) and the error words to the host
+cudaError_t launch_force_finish(const BoxDev& b, double* out, double* f, double* host_th, int* host_err, int nred,
+                                Launch l);
 int force_tile_blocks_per_sm(int mono);   // resident blocks of the tiled force kernel
 
 // k_adjoint.cu
