@@ -915,14 +915,25 @@ md_status tape_save(md_box* b, int m)
 }
 
 // The thermostat's draws of n steps ahead of them, while they fit 64 MiB (N =
-// 27,000 for 100 steps; beyond, the draw is a small part of a step anyway).
+// 27,000 for 100 steps; beyond, the draw is a small part of a step anyway):
+// np velocities and np hit bits per step.
 size_t tstat_velocity_bytes(md_box* b, int64_t n) { return (size_t)n * (size_t)b->np * 3 * sizeof(double); }
-bool tstat_ahead(md_box* b, int64_t n) { return tstat_velocity_bytes(b, n) <= ((size_t)64 << 20); }
+size_t tstat_bytes(md_box* b, int64_t n) { return al256(tstat_velocity_bytes(b, n)) + (size_t)n * (size_t)b->np / 8; }
+bool tstat_fits(md_box* b, int64_t n) { return tstat_velocity_bytes(b, n) <= ((size_t)64 << 20); }
 
+// Whether a graph of n steps draws ahead: decided for each graph by the buffer
+// it would write (a run's last graph may be short enough where its others are
+// not); without the room the integrator draws.
+bool tstat_ahead(md_box* b, int64_t n)
+{
+    return b->d.tstat_thr && tstat_fits(b, n) && b->d_tstat_draws && b->tstat_draw_bytes >= tstat_bytes(b, n);
+}
+
+// Room for the draws of a graph of n steps, before its capture.
 md_status ensure_tstat(md_box* b, int64_t n)
 {
-    if (!b->d.tstat_thr || !tstat_ahead(b, n)) return MD_OK;
-    const size_t need = al256(tstat_velocity_bytes(b, n)) + (size_t)n * (size_t)b->np / 8;
+    if (!b->d.tstat_thr || !tstat_fits(b, n)) return MD_OK;
+    const size_t need = tstat_bytes(b, n);
     if (b->tstat_draw_bytes >= need) return MD_OK;
     invalidate_graphs(b);   // graphs hold the pointer
     dev_release(b, b->d_tstat_draws);
@@ -956,7 +967,7 @@ md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* rin
         return cudaEventRecordWithFlags(ge->ev[2 * k + end], st, cudaEventRecordExternal);
     };
     BoxDev set[2] = {b->d, b->d};
-    if (b->d.tstat_thr && !tape && tstat_ahead(b, n)) {
+    if (!tape && tstat_ahead(b, n)) {
         unsigned* hit = reinterpret_cast<unsigned*>(b->d_tstat_draws + al256(tstat_velocity_bytes(b, n)));
         double* g = reinterpret_cast<double*>(b->d_tstat_draws);
         const int items = (int)n * b->d.nchunk;
@@ -1625,7 +1636,6 @@ md_status md_integrate(md_box* b, double dt, int64_t nsteps, int32_t ckpt_every,
     const int energy = thermo_out ? 1 : 0;
     const int64_t chunk = record ? ckpt_every : b->chunk_steps;
     if (energy) CKS(ensure_thermo(b, std::min(nsteps, chunk)));
-    CKS(ensure_tstat(b, std::min(nsteps, chunk)));
     bool out_dev = energy && is_device_ptr(thermo_out);
     int64_t done = 0;
     int retries = 0;
@@ -1639,6 +1649,7 @@ md_status md_integrate(md_box* b, double dt, int64_t nsteps, int32_t ckpt_every,
         b->fresh_abs = false;   // offsets advance; xabs keeps the last build
         CKS(clear_err(b));
         CKS(snapshot(b, false));
+        CKS(ensure_tstat(b, n));   // each graph's own: the last one may be the only one that fits
         cudaGraphExec_t g;
         CKS(get_graph(b, n, dt, energy, &g));
         CK(b, cudaGraphLaunch(g, b->stream));

@@ -84,3 +84,16 @@ def test_collisions_drawn_ahead_equal_those_drawn_step_by_step(ljmd, rate):
             b.integrate(0.002, steps, thermo=False)
         out.append(b.get_state())
     np.testing.assert_allclose(out[1][1], out[0][1], rtol=0, atol=1e-9)
+
+
+@pytest.mark.parametrize("calls", [(150,), (10, 150), (10, 140)])
+def test_a_short_last_graph_draws_ahead_where_the_others_do_not(ljmd, calls):
+    # 30,000 particles: 100 steps' draws exceed 64 MiB, those of the last 40 or 50 fit
+    s = inputs.fcc_subset_system(30000, 0.8, 0.7, seed=3)
+    out = []
+    for steps in (calls, (10,) * (sum(calls) // 10)):
+        b = ljmd.from_system(s).set_thermostat(1.3, 20.0, seed=6)
+        for n in steps:
+            b.integrate(0.002, n, thermo=False)
+        out.append(b.get_state())
+    np.testing.assert_allclose(out[1][1], out[0][1], rtol=0, atol=1e-9)
