@@ -109,20 +109,22 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_adj_pre(BoxDev b, Tape t, int m, d
     }
 }
 
-// Sums of k_hvp_mono over a thread's pairs in units of c12 = 48 eps sigma^12,
-// with a = -d_ij, b = u_j - u_i: h = sum A (a.b) a - f b = -(H u)_i, and the
-// two moments of the parameter terms, x = sum r^-14 (u_i.a), y = sum r^-8 (u_i.a).
+// Sums of k_hvp_mono over a thread's pairs in units of c6 = 24 eps sigma^6, with
+// a = -d_ij, b = u_j - u_i and q = 2 (sigma / r)^6 - 1: h = sum A (a.b) a - f b =
+// -(H u)_i, and the two moments of the parameter terms, x = sum q r^-8 (u_i.a),
+// y = sum r^-8 (u_i.a).
 struct HvpSums {
     float hx, hy, hz;
     float2 x, y;
 };
 
 // Two pairs: separations one by one, everything from r^2 on as FP32 pairs.  In
-// units of c12, with nh = -c6 / c12: f = r^-8 (r^-6 + nh), A = r^-10 (14 r^-6 +
-// 8 nh); the cutoff masks 1 / r^2, so a pair beyond it adds zeros.
+// units of c6, with tw = 2 sigma^6: q = tw r^-6 - 1, f = r^-8 q, A = r^-10 (14 q +
+// 6); the cutoff masks 1 / r^2, so a pair beyond it adds zeros.  (Units as in
+// the force kernel: r^-16 alone leaves the range of FP32 with the unit of length.)
 __device__ __forceinline__ void hvp_pair2(unsigned e0, const float4& q0, const float4& u0, unsigned e1,
                                           const float4& q1, const float4& u1, const float4& pi, const float4& ui,
-                                          const float3& ell, float nh, float rc2, HvpSums& S)
+                                          const float3& ell, float tw, float rc2, HvpSums& S)
 {
     const float ax0 = fmaf(entry_unit<0>(e0), ell.x, q0.x - pi.x), ax1 = fmaf(entry_unit<0>(e1), ell.x, q1.x - pi.x);
     const float ay0 = fmaf(entry_unit<1>(e0), ell.y, q0.y - pi.y), ay1 = fmaf(entry_unit<1>(e1), ell.y, q1.y - pi.y);
@@ -135,8 +137,9 @@ __device__ __forceinline__ void hvp_pair2(unsigned e0, const float4& q0, const f
     const float2 ri = __fmul2_rn(make_float2(rcp_approx(r2.x), rcp_approx(r2.y)), in);
     const float2 r6 = __fmul2_rn(__fmul2_rn(ri, ri), ri);
     const float2 r8 = __fmul2_rn(ri, r6);
-    const float2 f = __fmul2_rn(r8, __fadd2_rn(r6, make_float2(nh, nh)));
-    const float2 A = __fmul2_rn(__fmul2_rn(ri, r8), __ffma2_rn(make_float2(14.f, 14.f), r6, make_float2(8.f * nh, 8.f * nh)));
+    const float2 q = __ffma2_rn(make_float2(tw, tw), r6, make_float2(-1.f, -1.f));
+    const float2 f = __fmul2_rn(r8, q);
+    const float2 A = __fmul2_rn(__fmul2_rn(ri, r8), __ffma2_rn(make_float2(14.f, 14.f), q, make_float2(6.f, 6.f)));
     const float2 ab = __ffma2_rn(ax, bx, __ffma2_rn(ay, by, __fmul2_rn(az, bz)));
     const float2 t = __fmul2_rn(A, ab);
     const float2 nf = make_float2(-f.x, -f.y);
@@ -148,7 +151,7 @@ __device__ __forceinline__ void hvp_pair2(unsigned e0, const float4& q0, const f
     const float2 ua = __ffma2_rn(make_float2(ui.x, ui.x), ax,
                                  __ffma2_rn(make_float2(ui.y, ui.y), ay, __fmul2_rn(make_float2(ui.z, ui.z), az)));
     const float2 v = __fmul2_rn(r8, ua);
-    S.x = __ffma2_rn(r6, v, S.x);
+    S.x = __ffma2_rn(q, v, S.x);
     S.y = __fadd2_rn(S.y, v);
 }
 
@@ -171,7 +174,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_hvp_mono(BoxDev b, Tape tp, in
     constexpr int PARTS = THREADS == LJ_SPREAD_THREADS ? LJ_CHUNK / PASS : 1;
     constexpr int OWN = LJ_CHUNK / PARTS;
     const TapeLists T = tape_lists(tp, m);
-    const float c12 = b.c1.x, nh = b.nh_1, rc2 = b.rc2_1;
+    const float c6 = b.c1.y, tw = b.tw_1, rc2 = b.rc2_1;
     const float inv_eps = b.lj->inv_eps[0], inv_sig = b.lj->inv_sig[0];
     const int K = b.K;
     const int grp = threadIdx.x / LJ_TPP, l4 = threadIdx.x % LJ_TPP;
@@ -213,8 +216,8 @@ __global__ void __launch_bounds__(THREADS, RES) k_hvp_mono(BoxDev b, Tape tp, in
                 const float4* n3 = pu + 2 * (size_t)entry_slot(q.w);
                 const float4 p0 = __ldg(n0), v0 = __ldg(n0 + 1), p1 = __ldg(n1), v1 = __ldg(n1 + 1);
                 const float4 p2 = __ldg(n2), v2 = __ldg(n2 + 1), p3 = __ldg(n3), v3 = __ldg(n3 + 1);
-                hvp_pair2(q.x, p0, v0, q.y, p1, v1, pi, ui, ell, nh, rc2, S);
-                hvp_pair2(q.z, p2, v2, q.w, p3, v3, pi, ui, ell, nh, rc2, S);
+                hvp_pair2(q.x, p0, v0, q.y, p1, v1, pi, ui, ell, tw, rc2, S);
+                hvp_pair2(q.z, p2, v2, q.w, p3, v3, pi, ui, ell, tw, rc2, S);
             };
             if (nblk > 0) {
                 for (int blk = 1; blk < nblk; ++blk) {
@@ -236,14 +239,14 @@ __global__ void __launch_bounds__(THREADS, RES) k_hvp_mono(BoxDev b, Tape tp, in
                 S.hz += __shfl_xor_sync(0xffffffffu, S.hz, o);
             }
             if (out) {
-                const double hv = (double)(-c12 * (l4 == 0 ? S.hx : (l4 == 1 ? S.hy : S.hz)));
+                const double hv = (double)(-c6 * (l4 == 0 ? S.hx : (l4 == 1 ? S.hy : S.hz)));
                 g[gu] = hv;
                 if (upd) lx[gu] = lx0 - 0.5 * h * hv;
             }
         }
         // u_i.dF/deps and u_i.dF/dsigma from the moments
-        const float x = S.x.x + S.x.y, y = nh * (S.y.x + S.y.y);
-        const float2 d = warp_sum2_ds2(-c12 * inv_eps * (x + y), -6.f * c12 * inv_sig * fmaf(2.f, x, y));
+        const float x = S.x.x + S.x.y, y = S.y.x + S.y.y;
+        const float2 d = warp_sum2_ds2(-c6 * inv_eps * x, -6.f * c6 * inv_sig * fmaf(2.f, x, y));
         if ((threadIdx.x & 15) == 0) {
             const size_t q = (size_t)it * (THREADS / 16) + (threadIdx.x >> 4);
             part_g[q] += *weight * ((double)d.x + (double)d.y);

@@ -97,13 +97,16 @@ __device__ __forceinline__ void pair_f32(unsigned ent, const float4& pj, const f
     }
 }
 
-// Sums of k_force_f32 over a thread's pairs, in units of c12 = 48 eps sigma^12
-// for one species (applied at the end).  w = sum f r^2 (the virial).  The
-// energy needs no pair arithmetic of its own: with s6 = (sigma / r)^6,
+// Sums of k_force_f32 over a thread's pairs, in units of c6 = 24 eps sigma^6 for
+// one species (applied at the end).  w = sum f r^2 (the virial).  The energy
+// needs no pair arithmetic of its own: with s6 = (sigma / r)^6,
 //   u = 4 eps (s6^2 - s6) - shift = (f r^2) / 12 - (2 eps s6 + shift),
-// so b sums the second term (one species: over 2 eps sigma^6).  Each is two
-// partial sums (the two pairs of pair2_f32), which also halves what each
-// rounds.
+// so b sums the second term (one species: over 2 eps sigma^6).  w and b are
+// two partial sums each in pair2_f32 (its two pairs), one in pair1_f32.
+// f r^2 = c6 r^-6 (2 s6 - 1): the largest power formed is r^-8, so that the
+// unit of length has the room it has in the tables of several species (r^-14,
+// in units of 48 eps sigma^12, is subnormal from sigma = 400 and overflows
+// below 2e-3).
 struct PairSums {
     float fx, fy, fz;
     float2 w, b;
@@ -127,7 +130,7 @@ struct RowConsts {
 template <bool MONO, bool ENERGY, bool TWO>
 __device__ __forceinline__ void pair2_f32(unsigned e0, const float4& q0, unsigned e1, const float4& q1,
                                           const float4& pi, int tb, const float3& ell, const float4* s_lj,
-                                          const float* s_rc2, float nh, float kap, float mrc2, const RowConsts& rc,
+                                          const float* s_rc2, float tw, float kap, float mrc2, const RowConsts& rc,
                                           PairSums& S)
 {
     const float2 a0 = neg_d_xy(e0, q0, pi, ell), a1 = neg_d_xy(e1, q1, pi, ell);
@@ -136,6 +139,8 @@ __device__ __forceinline__ void pair2_f32(unsigned e0, const float4& q0, unsigne
     const float2 r2 = __ffma2_rn(az, az, make_float2(s0.x + s0.y, s1.x + s1.y));
     float2 c12, nc6, rc2, hb, esh;
     if (MONO) {
+        c12 = make_float2(tw, tw);
+        nc6 = make_float2(-1.f, -1.f);
         rc2 = make_float2(mrc2, mrc2);
     } else {
         const int p0 = tb + __float_as_int(q0.w), p1 = tb + __float_as_int(q1.w);
@@ -149,8 +154,7 @@ __device__ __forceinline__ void pair2_f32(unsigned e0, const float4& q0, unsigne
     const float2 in = make_float2(r2.x < rc2.x ? 1.f : 0.f, r2.y < rc2.y ? 1.f : 0.f);
     const float2 ri = __fmul2_rn(make_float2(rcp_approx(r2.x), rcp_approx(r2.y)), in);
     const float2 r6 = __fmul2_rn(__fmul2_rn(ri, ri), ri);
-    const float2 g =   // f r^2
-        __fmul2_rn(r6, MONO ? __fadd2_rn(r6, make_float2(nh, nh)) : __ffma2_rn(c12, r6, nc6));
+    const float2 g = __fmul2_rn(r6, __ffma2_rn(c12, r6, nc6));   // f r^2
     const float2 f = __fmul2_rn(ri, g);
     S.fx = fmaf(f.x, a0.x, S.fx);   // of -d: the sums are negated at the end
     S.fy = fmaf(f.x, a0.y, S.fy);
@@ -170,14 +174,14 @@ __device__ __forceinline__ void pair2_f32(unsigned e0, const float4& q0, unsigne
 // constants take register pairs).
 template <bool MONO, bool ENERGY, bool TWO>
 __device__ __forceinline__ void pair1_f32(unsigned e0, const float4& q0, const float4& pi, int tb, const float3& ell,
-                                          const float4* s_lj, const float* s_rc2, float nh, float kap, float mrc2,
+                                          const float4* s_lj, const float* s_rc2, float tw, float kap, float mrc2,
                                           const RowConsts& rc, PairSums& S)
 {
     const float2 a0 = neg_d_xy(e0, q0, pi, ell);
     const float az = fmaf(entry_unit<2>(e0), ell.z, q0.z - pi.z);
     const float2 s0 = __fmul2_rn(a0, a0);
     const float r2 = fmaf(az, az, s0.x + s0.y);
-    float4 c = make_float4(1.f, nh, 0.f, 0.f);
+    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
     float rc2 = mrc2;
     if (!MONO) {
         const int p0 = tb + __float_as_int(q0.w);
@@ -193,7 +197,7 @@ __device__ __forceinline__ void pair1_f32(unsigned e0, const float4& q0, const f
     const bool in = r2 < rc2;
     const float ri = in ? rcp_approx(r2) : 0.f;
     const float r6 = ri * ri * ri;
-    const float g = r6 * (MONO ? r6 + nh : fmaf(c.x, r6, c.y));   // f r^2
+    const float g = MONO ? fmaf(tw * r6, r6, -r6) : r6 * fmaf(c.x, r6, c.y);   // f r^2
     const float f = ri * g;
     S.fx = fmaf(f, a0.x, S.fx);   // of -d: the sums are negated at the end
     S.fy = fmaf(f, a0.y, S.fy);
@@ -248,8 +252,8 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
         }
         __syncthreads();   // the pair tables are complete (the block's only barrier)
     }
-    // one species: f r^2 = c12 r6 (r6 + nh), the energy's second term (e6 / 2) (r6 + kap)
-    const float c12 = MONO ? b.c1.x : 1.f, nh = b.nh_1, kap = b.kap_1, mrc2 = b.rc2_1;
+    // one species: f r^2 = c6 r6 (tw r6 - 1), the energy's second term (e6 / 2) (r6 + kap)
+    const float c6 = MONO ? b.c1.y : 1.f, tw = b.tw_1, kap = b.kap_1, mrc2 = b.rc2_1;
     const int K = b.K;
     const int grp = threadIdx.x / TPP, lt = threadIdx.x % TPP;
     const float4* posq = b.posq;
@@ -304,13 +308,13 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
                 const float4 p2 = posq[entry_slot(q.z)];
                 const float4 p3 = posq[entry_slot(q.w)];
                 if (SPREAD) {
-                    pair2_f32<MONO, ENERGY, TWO>(q.x, p0, q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
-                    pair2_f32<MONO, ENERGY, TWO>(q.z, p2, q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
+                    pair2_f32<MONO, ENERGY, TWO>(q.x, p0, q.y, p1, pi, tb, ell, s_lj, s_rc2, tw, kap, mrc2, rc, S);
+                    pair2_f32<MONO, ENERGY, TWO>(q.z, p2, q.w, p3, pi, tb, ell, s_lj, s_rc2, tw, kap, mrc2, rc, S);
                 } else {
-                    pair1_f32<MONO, ENERGY, TWO>(q.x, p0, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
-                    pair1_f32<MONO, ENERGY, TWO>(q.y, p1, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
-                    pair1_f32<MONO, ENERGY, TWO>(q.z, p2, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
-                    pair1_f32<MONO, ENERGY, TWO>(q.w, p3, pi, tb, ell, s_lj, s_rc2, nh, kap, mrc2, rc, S);
+                    pair1_f32<MONO, ENERGY, TWO>(q.x, p0, pi, tb, ell, s_lj, s_rc2, tw, kap, mrc2, rc, S);
+                    pair1_f32<MONO, ENERGY, TWO>(q.y, p1, pi, tb, ell, s_lj, s_rc2, tw, kap, mrc2, rc, S);
+                    pair1_f32<MONO, ENERGY, TWO>(q.z, p2, pi, tb, ell, s_lj, s_rc2, tw, kap, mrc2, rc, S);
+                    pair1_f32<MONO, ENERGY, TWO>(q.w, p3, pi, tb, ell, s_lj, s_rc2, tw, kap, mrc2, rc, S);
                 }
             };
             if (nblk > 0) {
@@ -335,7 +339,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
                 S.fz += __shfl_xor_sync(0xffffffffu, S.fz, o);
             }
             if (act && lt == 0) {
-                b.force4[p] = make_float4(-c12 * S.fx, -c12 * S.fy, -c12 * S.fz, 0.f);
+                b.force4[p] = make_float4(-c6 * S.fx, -c6 * S.fy, -c6 * S.fz, 0.f);
                 if (!isfinite(S.fx + S.fy + S.fz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
             }
         }
@@ -346,7 +350,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
             // sum): FP64-class precision on the FP32 pipe, since FP64 adds
             // are scarce on this GPU.  The share is stored as the (hi, lo)
             // pair itself (pf_ds), halved exactly; the reduction converts
-            const float vir = c12 * (S.w.x + S.w.y);
+            const float vir = c6 * (S.w.x + S.w.y);
             const float e = fmaf(vir, 1.f / 12.f, (MONO ? -0.5f * b.c1.w : -1.f) * (S.b.x + S.b.y));
             const float2 d = warp_sum2_ds2(e, vir);
             if ((threadIdx.x & 15) == 0) {
@@ -1215,11 +1219,25 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
             s_lj[k] = make_float4(lj->c12[k], -lj->c6[k], 0.5f * lj->e6[k], 0.f);
         __syncthreads();
     }
-    const float c12 = MONO ? b.c1.x : 1.f, nh = b.nh_1;
+    // one species: lengths over the power of two nearest sigma, where they are
+    // staged, and the energy in units of c12 = 48 eps sigma^12 of that length.
+    // (The list kernels' form, which needs no scale, costs an FMA with three
+    // packed register operands instead of an addition: N = 32,000 836 -> 870 us.)
+    const float4 one_c = b.all_1;   // 1 / length, c12, -c6 / c12, e6 / 2
+    const float c12 = MONO ? one_c.y : 1.f;
+    const float2 nh = dup2(one_c.z);
+    auto load = [&](int j) {
+        float4 q = b.posq[j];
+        if (MONO) {
+            q.x *= one_c.x;
+            q.y *= one_c.x;
+            q.z *= one_c.x;
+        }
+        return q;
+    };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int parts = b.pf_stride;
     const float2 M = dup2(12582912.0f), nM = dup2(-12582912.0f);   // 1.5 * 2^23
-    const float4* posq = b.posq;
     for (int it = blockIdx.x; it < b.nchunk * parts; it += gridDim.x) {
         const int w = it / parts;
         const int4 ch = chunk_of(b, w);
@@ -1232,7 +1250,8 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
             }
         }
         // one cell: its edge is the box's (one replica: from the kernel parameters)
-        const float3 L = b.nrep == 1 ? b.ell1 : make_float3(R.ellf[0], R.ellf[1], R.ellf[2]);
+        float3 L = b.nrep == 1 ? b.ell1 : make_float3(R.ellf[0], R.ellf[1], R.ellf[2]);
+        if (MONO) L = make_float3(L.x * one_c.x, L.y * one_c.x, L.z * one_c.x);
         const float2 ix = dup2(1.0f / L.x), iy = dup2(1.0f / L.y), iz = dup2(1.0f / L.z);
         const float2 nLx = dup2(-L.x), nLy = dup2(-L.y), nLz = dup2(-L.z);
         const int jb = b.nrep == 1 ? 0 : R.p_off, je = b.nrep == 1 ? b.n1 : R.p_off + R.n;
@@ -1240,7 +1259,7 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
         for (int grp = it % parts; grp < kAllGroups; grp += parts) {
             const int p = ch.y + grp * kAllGroup + 2 * warp;   // the warp's particles: p and p + 1
             const bool one = p < ch.z, two = p + 1 < ch.z;     // warp-uniform
-            const float4 a = posq[one ? p : ch.y], c = posq[two ? p + 1 : ch.y];
+            const float4 a = load(one ? p : ch.y), c = load(two ? p + 1 : ch.y);
             const float2 nx = make_float2(-a.x, -c.x), ny = make_float2(-a.y, -c.y), nz = make_float2(-a.z, -c.z);
             const int ta = __float_as_int(a.w) * nt, tc = __float_as_int(c.w) * nt;
             float2 fx = dup2(0.f), fy = fx, fz = fx, vir = fx, eb = fx;
@@ -1256,7 +1275,7 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
                 const float2 r6 = __fmul2_rn(__fmul2_rn(ri, ri), ri);
                 float2 g;
                 if (MONO) {
-                    g = __fmul2_rn(r6, __fadd2_rn(r6, dup2(nh)));   // f r^2, over c12
+                    g = __fmul2_rn(r6, __fadd2_rn(r6, nh));   // f r^2, over c12
                     if (ENERGY) eb = __fadd2_rn(eb, r6);
                 } else {
                     const int tj = __float_as_int(q.w);
@@ -1276,7 +1295,7 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
 #pragma unroll
                 for (int t = 0; t < kAllTile / kAllThreads; ++t) {
                     const int j = t0 + t * kAllThreads + (int)threadIdx.x;
-                    if (j < t1) s_pos[j - t0] = posq[j];
+                    if (j < t1) s_pos[j - t0] = load(j);
                 }
                 __syncthreads();
                 if (!one) continue;
@@ -1305,14 +1324,15 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
                 fz = __fadd2_rn(fz, make_float2(__shfl_xor_sync(0xffffffffu, fz.x, o), __shfl_xor_sync(0xffffffffu, fz.y, o)));
             }
             if ((lane == 0 && one) || (lane == 1 && two)) {
+                const float cf = MONO ? c12 * one_c.x : 1.f;
                 const float sx = lane == 0 ? fx.x : fx.y, sy = lane == 0 ? fy.x : fy.y, sz = lane == 0 ? fz.x : fz.y;
-                b.force4[p + lane] = make_float4(-c12 * sx, -c12 * sy, -c12 * sz, 0.f);
+                b.force4[p + lane] = make_float4(-cf * sx, -cf * sy, -cf * sz, 0.f);
                 if (!isfinite(sx + sy + sz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
             }
             if (ENERGY) {
                 // u = f r^2 / 12 - 2 eps (sigma / r)^6 (no cutoff, no shift)
                 const float wv = c12 * (vir.x + (two ? vir.y : 0.f));   // both 0 without a first particle
-                const float ev = fmaf(wv, 1.f / 12.f, (MONO ? -0.5f * b.c1.w : -1.f) * (eb.x + (two ? eb.y : 0.f)));
+                const float ev = fmaf(wv, 1.f / 12.f, (MONO ? -one_c.w : -1.f) * (eb.x + (two ? eb.y : 0.f)));
                 const float2 d = warp_sum2_ds2(ev, wv);
                 sum += (double)d.x + (double)d.y;
             }

@@ -1511,8 +1511,11 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
     b->d.esh_1 = h.shift[0];
     {
         const double s2 = sigma[0] * sigma[0], s6 = s2 * s2 * s2;
-        b->d.nh_1 = (float)(-0.5 / s6);
+        b->d.tw_1 = (float)(2.0 * s6);
         b->d.kap_1 = (float)(h.dshift[0] / (2.0 * eps[0] * s6));
+        const double u = std::exp2(std::min(100.0, std::max(-100.0, std::round(std::log2(sigma[0]))))), q = sigma[0] / u;
+        const double q6 = q * q * q * q * q * q;
+        b->d.all_1 = make_float4((float)(1.0 / u), (float)(48.0 * eps[0] * q6 * q6), (float)(-0.5 / q6), (float)(2.0 * eps[0] * q6));
     }
     b->skin = skin;
     b->rl = rl;
@@ -1524,8 +1527,8 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
     d.disp_thr2 = thr > 0 ? (float)(thr * thr) : 0.0f;
     // captured step graphs hold these by value
     auto same4 = [](const float4& x, const float4& y) { return x.x == y.x && x.y == y.y && x.z == y.z && x.w == y.w; };
-    if (before.nt != d.nt || !same4(before.c1, d.c1) || before.rc2_1 != d.rc2_1 || before.esh_1 != d.esh_1 ||
-        before.nh_1 != d.nh_1 || before.kap_1 != d.kap_1 || before.rl2 != d.rl2 || before.disp_thr2 != d.disp_thr2)
+    if (before.nt != d.nt || !same4(before.c1, d.c1) || !same4(before.all_1, d.all_1) || before.rc2_1 != d.rc2_1 || before.esh_1 != d.esh_1 ||
+        before.tw_1 != d.tw_1 || before.kap_1 != d.kap_1 || before.rl2 != d.rl2 || before.disp_thr2 != d.disp_thr2)
         invalidate_graphs(b);
     if (grid_changes) CKS(make_grid(b));
     b->eps0 = eps[0];
