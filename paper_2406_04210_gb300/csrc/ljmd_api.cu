@@ -124,6 +124,7 @@ struct md_box {
     double* d_tstat_T = nullptr;
     char* d_tstat_draws = nullptr;   // the collisions of a graph's steps, drawn at its head
     size_t tstat_draw_bytes = 0;
+    size_t tstat_refused = SIZE_MAX;   // the allocator refused this much for it
     long long* d_step_ctr = nullptr;
     // tuning
     int min_capacity = 0;
@@ -929,19 +930,20 @@ bool tstat_ahead(md_box* b, int64_t n)
     return b->d.tstat_thr && tstat_fits(b, n) && b->d_tstat_draws && b->tstat_draw_bytes >= tstat_bytes(b, n);
 }
 
-// Room for the draws of a graph of n steps, before its capture.
-md_status ensure_tstat(md_box* b, int64_t n)
+// Room for the draws of a graph of n steps, before its capture.  A refused
+// allocation is no error, as the integrators then draw; as much is not asked
+// for again before the next md_set_thermostat.
+void ensure_tstat(md_box* b, int64_t n)
 {
-    if (!b->d.tstat_thr || !tstat_fits(b, n)) return MD_OK;
+    if (!b->d.tstat_thr || !tstat_fits(b, n)) return;
     const size_t need = tstat_bytes(b, n);
-    if (b->tstat_draw_bytes >= need) return MD_OK;
+    if (b->tstat_draw_bytes >= need || need >= b->tstat_refused) return;
     invalidate_graphs(b);   // graphs hold the pointer
     dev_release(b, b->d_tstat_draws);
     b->d_tstat_draws = nullptr;
     b->tstat_draw_bytes = 0;
-    CKS(dev_alloc(b, &b->d_tstat_draws, need, false));
-    b->tstat_draw_bytes = need;
-    return MD_OK;
+    if (dev_alloc(b, &b->d_tstat_draws, need, false) == MD_OK) b->tstat_draw_bytes = need;
+    else b->tstat_refused = need;
 }
 
 md_status enqueue_steps(md_box* b, int64_t n, double dt, int energy, double* ring, GraphEnt* ge,
@@ -1558,6 +1560,7 @@ md_status md_set_thermostat(md_box* b, const double* T_bath, double rate, uint64
     b->tstat_rate = rate;
     b->d.tstat_seed = seed;
     b->d.tstat_thr = 0u;   // set per dt by md_integrate
+    b->tstat_refused = SIZE_MAX;
     b->rec_valid = false;
     invalidate_graphs(b);
     CKS(leave(b));   // T_bath may be pageable host memory
@@ -1652,7 +1655,7 @@ md_status md_integrate(md_box* b, double dt, int64_t nsteps, int32_t ckpt_every,
         b->fresh_abs = false;   // offsets advance; xabs keeps the last build
         CKS(clear_err(b));
         CKS(snapshot(b, false));
-        CKS(ensure_tstat(b, n));   // each graph's own: the last one may be the only one that fits
+        ensure_tstat(b, n);   // each graph's own: the last one may be the only one that fits
         cudaGraphExec_t g;
         CKS(get_graph(b, n, dt, energy, &g));
         CK(b, cudaGraphLaunch(g, b->stream));
