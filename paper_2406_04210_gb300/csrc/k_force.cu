@@ -1483,7 +1483,7 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_force_all_f64(BoxDev b)
 // A share of the FP32 forces: its (hi, lo) pair, stored where a double stands.
 __device__ __forceinline__ double ds_bits_to_double(double v)
 {
-    return f2d_exact(__int_as_float(__double2loint(v))) + f2d_exact(__int_as_float(__double2hiint(v)));
+    return f2d(__int_as_float(__double2loint(v))) + f2d(__int_as_float(__double2hiint(v)));
 }
 
 // E_pot, E_kin, W, T per replica from the per-chunk partial sums, in a
@@ -1642,9 +1642,9 @@ __global__ void __launch_bounds__(LJ_THERMO_THREADS) k_force_finish(BoxDev b, do
             for (int c = 0; c < 3; ++c) f[3 * gu + c] = q[c];
         } else {
             const float4 q = b.force4[p];
-            f[3 * gu + 0] = f2d_exact(q.x);
-            f[3 * gu + 1] = f2d_exact(q.y);
-            f[3 * gu + 2] = f2d_exact(q.z);
+            f[3 * gu + 0] = f2d(q.x);
+            f[3 * gu + 1] = f2d(q.y);
+            f[3 * gu + 2] = f2d(q.z);
         }
     }
 }

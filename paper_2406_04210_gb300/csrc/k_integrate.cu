@@ -373,12 +373,12 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_download(BoxDev b, double* pos, do
         cc[0] = local % R.nc[0];
         cc[1] = (local / R.nc[0]) % R.nc[1];
         cc[2] = local / (R.nc[0] * R.nc[1]);
+        if (b.prec == 0) {
+            ds_to_double3(fo, fo + 3, o);
+            ds_to_double3(fv, fv + 3, v);
+        }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            if (b.prec == 0) {
-                o[c] = ds_to_double(fo[c], fo[3 + c]);
-                v[c] = ds_to_double(fv[c], fv[3 + c]);
-            }
             double x = fma(half_above(cc[c]), R.ell[c], o[c]);
             int im = im3[c];
             const double L = R.L[c];

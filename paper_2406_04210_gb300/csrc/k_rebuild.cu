@@ -175,9 +175,10 @@ __device__ __forceinline__ void bin_chunks(const BoxDev& b, int from_abs)
             const int cz = cell_coords(R, cell, cx, cy);
             const int cc[3] = {cx, cy, cz};
             bool slow = !DS;
+            if (DS) ds_to_double3(oh, ol, x);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const double o = DS ? ds_to_double(oh[c], ol[c]) : x[c];
+                const double o = x[c];
                 if (DS) {
                     const float h = oh[c];
                     // the neighbour cell the FP32 offset lies in (at most one away)

@@ -246,22 +246,18 @@ struct BoxDev {
 };
 
 // FP32 to FP64 by moving bits: the conversion instruction runs on the FP64
-// pipe (2 lanes per clock and SM), this on the integer one.  Exact for zero
-// and normal numbers; a subnormal counts as zero.
-__device__ __forceinline__ double f2d(float f)
+// pipe (2 lanes per clock and SM), this on the integer one.  f2d_normal is
+// exact except that a subnormal counts as zero; f2d is exact (a subnormal
+// takes the instruction, a branch away).
+__device__ __forceinline__ bool is_subnormal(float f) { return (__float_as_uint(f) & 0x7fffffffu) - 1u < 0x007fffffu; }
+__device__ __forceinline__ double f2d_normal(float f)
 {
     const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
     const unsigned e = m < 0x00800000u ? 0u : (m >> 3) + 0x38000000u;
     const unsigned inf = m >= 0x7f800000u ? 0x38000000u : 0u;   // infinity and NaN keep their exponent
     return __hiloint2double((int)((u & 0x80000000u) | (e + inf)), m < 0x00800000u ? 0 : (int)(u << 29));
 }
-
-// The same, exact for subnormals too (their conversion is a branch away).
-__device__ __forceinline__ double f2d_exact(float f)
-{
-    const unsigned m = __float_as_uint(f) & 0x7fffffffu;
-    return m != 0u && m < 0x00800000u ? (double)f : f2d(f);
-}
+__device__ __forceinline__ double f2d(float f) { return is_subnormal(f) ? (double)f : f2d_normal(f); }
 
 // ---- double-single helpers (Dekker / Knuth error-free transformations) ----
 __device__ __forceinline__ void ds_two_sum(float a, float b, float& s, float& e)
@@ -304,11 +300,24 @@ __device__ __forceinline__ void ds_mul_ds(float ah, float al, float bh, float bl
 __device__ __forceinline__ void ds_from_double(double x, float& h, float& l)
 {
     h = __double2float_rn(x);
-    l = __double2float_rn(x - f2d(h));
+    // behind a subnormal h at most half of the smallest number is left, which rounds to 0
+    l = (__float_as_uint(h) & 0x7fffffffu) < 0x00800000u ? 0.f : __double2float_rn(x - f2d_normal(h));
 }
 
-// (h, l) of a double-single number as FP64
-__device__ __forceinline__ double ds_to_double(float h, float l) { return f2d(h) + f2d(l); }
+// (h, l) of three double-single numbers as FP64, with one branch for the
+// subnormal words among them
+__device__ __forceinline__ void ds_to_double3(const float* h, const float* l, double* o)
+{
+    bool sub = false;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sub = sub | is_subnormal(h[c]) | is_subnormal(l[c]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) o[c] = f2d_normal(h[c]) + f2d_normal(l[c]);
+    if (sub) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) o[c] = (double)h[c] + (double)l[c];
+    }
+}
 // n + 1/2 for 0 <= n < 2^31, exactly, in one FP64 addition (the integer as the
 // low mantissa bits of 2^52)
 __device__ __forceinline__ double half_above(int n) { return __hiloint2double(0x43300000, n) - 4503599627370495.5; }
