@@ -516,12 +516,12 @@ class TrajectoryFn:
             class _F(torch.autograd.Function):
                 @staticmethod
                 def forward(ctx, x0, v0, eps, sigma, box, dt, nsteps, ckpt_every):
-                    _order(box, x0)
+                    x, v = x0.detach().contiguous(), v0.detach().contiguous()
+                    _order(box, x)   # behind those copies
                     box.set_lj(float(eps), float(sigma), box._rcut, box._skin, True)
-                    box.set_state(x0.detach().contiguous(), v0.detach().contiguous())
+                    box.set_state(x, v)
                     box.integrate(dt, nsteps, thermo=False, ckpt_every=ckpt_every)
-                    xT = torch.empty_like(x0)
-                    vT = torch.empty_like(v0)
+                    xT, vT = torch.empty_like(x), torch.empty_like(v)
                     box._check(box._lib.md_get_state(box._h, xT.data_ptr(), vT.data_ptr(), None),
                                "md_get_state")
                     ctx.box = box

@@ -38,3 +38,34 @@ def test_box_made_behind_queued_work_in_reused_memory(ljmd):
         box = ljmd.Box(pos, s.box, vel).set_lj()
         f, e, w = box.force()
         assert np.array_equal(f, ref[0]) and np.array_equal(e, ref[1]) and np.array_equal(w, ref[2])
+
+
+@pytest.mark.parametrize("side", [False, True])
+def test_autograd_bridge_takes_transposed_tensors_on_any_stream(ljmd, side):
+    """x0 and v0 stored by component, written on the current stream behind
+    queued work, where the box was made on another one."""
+    import torch
+    from paper_2406_04210_gb300 import inputs
+    s = inputs.fcc_system(6, seed=12)
+    box = ljmd.from_system(s)
+    one = torch.tensor(1.0, dtype=torch.float64)
+    rng = np.random.default_rng(0)
+    gx, gv = (torch.tensor(rng.normal(size=s.pos.shape), device="cuda") for _ in range(2))
+
+    def run(x0, v0):
+        x0, v0, e, g = (t.detach().requires_grad_() for t in (x0, v0, one, one))
+        xT, vT = ljmd.TrajectoryFn.apply(x0, v0, e, g, box, s.dt, 4, 2)
+        ((xT * gx).sum() + (vT * gv).sum()).backward()
+        return [t.detach().cpu().numpy() for t in (xT, vT, x0.grad, v0.grad, e.grad, g.grad)]
+
+    pos, vel = (torch.tensor(a, device="cuda") for a in (s.pos, s.vel))
+    want = run(pos, vel)
+    slow = torch.ones(1 << 28, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream() if side else torch.cuda.current_stream()):
+        for _ in range(8):
+            slow.mul_(1.0)
+        got = run(pos.t().contiguous().t(), vel.t().contiguous().t())
+        torch.cuda.synchronize()
+    for w, g in zip(want, got):
+        np.testing.assert_array_equal(g, w)
