@@ -282,7 +282,9 @@ md_status md_get_info(md_box* b, md_info* out);
 /* Launch and layout tuning (Sec. 3 and Sec. 5: the paper determines launch
  * configurations per device; here they are set or timed per box), t[4]:
  *   t[0] blocks per SM of the pair-force kernels  (0 = default: by form and
- *        size, a block per work item for FP32 lists of one species)
+ *        size, a block per work item for FP32 lists of one species; in boxes
+ *        of up to 512 chunks, whose blocks are a quarter as large, t[0]
+ *        counts fours of them)
  *   t[1] blocks per SM of the list build          (0 = default: lanes 32, quads 6)
  *   t[2] cells per list-build segment, <= 16      (0 = automatic: ~1400
  *        particles per 27-cell tile)

@@ -345,9 +345,10 @@ Launch lforce(md_box* b)
     if (b->d.force_tiles)   // persistent: the resident blocks, bricks handed out in a grid stride
         return Launch{std::max(1, std::min((int)b->d.nbrick, b->nsm * force_tile_blocks_per_sm(b->d.nt == 1))), 0,
                       b->stream};
-    if (b->d.force_spread) {
+    if (b->d.force_spread) {   // t[0] counts blocks of 256 threads; automatic are 32 small blocks per SM
         const int items = b->d.nchunk * (LJ_CHUNK * LJ_TPP / LJ_SPREAD_THREADS);
-        return Launch{std::max(1, std::min(items, b->nsm * 32)), 0, b->stream};
+        const int per_sm = (b->force_per_sm > 0 ? b->force_per_sm : 8) * (LJ_FORCE_THREADS / LJ_SPREAD_THREADS);
+        return Launch{std::max(1, std::min(items, b->nsm * per_sm)), 0, b->stream};
     }
     // the FP64 list kernel's items are quarters of a chunk
     int per_chunk = b->prec == MD_PREC_FP64 ? LJ_F64_WARPS : 1;

@@ -34,3 +34,22 @@ def test_grids_do_not_change_results(ljmd, species, n):
     assert all((na[i, :c] == nb[i, :c]).all() for i, c in enumerate(ca))
     for x, y in zip(a.integrate(0.001, 5), b.integrate(0.001, 5)):
         np.testing.assert_array_equal(x, y)
+
+
+def test_small_boxes_follow_the_set_grid(ljmd):
+    # a quarter of a wave of small blocks per SM against all of them: the same forces, later
+    s = inputs.fcc_subset_system(60000, 0.8, 0.7, seed=5)
+    b = ljmd.from_system(s)
+    forces, ms = [], []
+    for per_sm in (0, 1):
+        b.set_tuning(force_blocks_per_sm=per_sm)
+        forces.append(b.force()[0])
+        b.integrate(0.001, 5)
+        b.set_profiling(True)
+        b.integrate(0.001, 20)
+        t, launches = b.profile()["force"]
+        b.set_profiling(False)
+        b.set_state(s.pos, s.vel)
+        ms.append(t / launches)
+    np.testing.assert_array_equal(*forces)
+    assert ms[1] > 1.3 * ms[0]
