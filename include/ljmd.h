@@ -378,8 +378,10 @@ md_status md_get_force_kernel(md_box* b, int32_t* kind);
 md_status md_set_graph_conditional(md_box* b, int32_t on);
 md_status md_get_graph_conditional(md_box* b, int32_t* on);
 
-/* Autotuner: times `reps` launches of the pair-force kernel for each
- * blocks-per-SM candidate, and `reps` forced list builds for each segment
+/* Autotuner: times `reps` launches of the pair-force kernel on its automatic
+ * grid and for each blocks-per-SM candidate (one replaces the automatic grid if
+ * it is 2 % faster; t[0] is then 0 only where no number of blocks per SM gives
+ * the automatic grid, beyond 32 work items per SM), and `reps` forced list builds for each segment
  * length (automatic choice +-2) x list blocks-per-SM candidate, at the
  * current positions; applies the fastest and returns it in t[4] (as
  * md_get_tuning).  It then times the cell layouts (cell_scale 1, 1.08, 1.15 and 1.22,

@@ -321,23 +321,25 @@ void apply_force_kernel(md_box* b)
     b->d.pf_ds = list32 ? 1 : 0;
 }
 
-// Grid of the force kernels over `items` work items.  Automatic, FP32 lists:
-// a block per item, handed out in order as blocks finish, so that the SMs work
-// on neighbouring chunks at a time (a fixed stride lets them drift apart, and
-// the neighbours' data leaves L2): 6 blocks per SM against all, one species
-// with energies, N = 256,000 47.3 / 45.4 us, 1M 147.7 / 138.6, 4M 565 / 508.
-// With tables (three species and more) a block loads them first: 6 per SM to
-// 640,000 particles (measured with the mixture's tables, N = 256,000 74.1 / 77.1
-// us, 1M 246 / 244).
+// Grid of the force kernels over `items` work items (but see lforce for the
+// small ones), as blocks per SM; 0 = a block per item.  FP32 lists: a block per
+// item, handed out in order as blocks finish, so that the SMs work on
+// neighbouring chunks at a time (a fixed stride lets them drift apart, and the
+// neighbours' data leaves L2): 6 blocks per SM against all, one species with
+// energies, N = 256,000 47.3 / 45.4 us, 1M 147.7 / 138.6, 4M 565 / 508.  With
+// tables (three species and more) a block loads them first: 6 per SM to 640,000
+// particles (measured with the mixture's tables, N = 256,000 74.1 / 77.1 us, 1M
+// 246 / 244).
+int automatic_per_sm(md_box* b, int items)
+{
+    if (b->prec == MD_PREC_FP64) return 12;
+    return b->all_pairs || (b->nt > 2 && items <= 5000) ? 6 : 0;
+}
+
 int force_grid(md_box* b, int items)
 {
-    int per_sm = b->force_per_sm;
-    if (per_sm <= 0) {
-        if (b->prec == MD_PREC_FP64) per_sm = 12;
-        else if (b->all_pairs || (b->nt > 2 && items <= 5000)) per_sm = 6;
-        else return std::max(1, items);
-    }
-    return std::max(1, std::min(items, b->nsm * per_sm));
+    const int per_sm = b->force_per_sm > 0 ? b->force_per_sm : automatic_per_sm(b, items);
+    return std::max(1, per_sm > 0 ? std::min(items, b->nsm * per_sm) : items);
 }
 
 Launch lforce(md_box* b)
@@ -2109,19 +2111,28 @@ md_status md_autotune(md_box* b, int32_t reps, int32_t t[4])
     if (!b || !b->lj_set || reps < 1) return fail(b, MD_ERR_ARG, "md_autotune: md_set_lj not called");
     if (b->all_pairs) return fail(b, MD_ERR_ARG, "md_autotune: not in the all-pairs form");
     CKS(enter(b));
-    // pair-force grid of the chunk kernel: blocks per SM (the tiled kernel
-    // runs its resident blocks)
-    const int fcand[] = {2, 3, 4, 6, 8, 12, 16, 24, 32};
+    // pair-force grid of the chunk kernel (the tiled kernel runs its resident
+    // blocks): the automatic one, or the fastest number of blocks per SM if
+    // that is faster by more than repeated timings differ (2 %).  The
+    // automatic grid is stored as a number where one gives it, else as 0.
     int best_f = b->force_per_sm > 0 ? b->force_per_sm : 6;
-    float best_ft = 1e30f;
-    for (int c : fcand) {
-        if (b->d.force_tiles) break;
-        b->force_per_sm = c;
-        float ms = 0.f;
-        CKS(time_launches(b, reps, [&]() -> md_status { return enqueue_force(b, 1, nullptr); }, &ms));
-        if (ms < best_ft) {
-            best_ft = ms;
-            best_f = c;
+    if (!b->d.force_tiles) {
+        const int fcand[] = {2, 3, 4, 6, 8, 12, 16, 24, 32};
+        b->force_per_sm = 0;
+        const int grid = lforce(b).grid;
+        best_f = b->d.force_spread ? 8 : automatic_per_sm(b, grid);
+        if (best_f == 0 && grid <= b->nsm * 32) best_f = 32;
+        float best_ft = 0.f;
+        CKS(time_launches(b, reps, [&]() -> md_status { return enqueue_force(b, 1, nullptr); }, &best_ft));
+        best_ft *= 0.98f;
+        for (int c : fcand) {
+            b->force_per_sm = c;
+            float ms = 0.f;
+            CKS(time_launches(b, reps, [&]() -> md_status { return enqueue_force(b, 1, nullptr); }, &ms));
+            if (ms < best_ft) {
+                best_ft = ms;
+                best_f = c;
+            }
         }
     }
     b->force_per_sm = best_f;

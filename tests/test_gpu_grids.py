@@ -53,3 +53,13 @@ def test_small_boxes_follow_the_set_grid(ljmd):
         ms.append(t / launches)
     np.testing.assert_array_equal(*forces)
     assert ms[1] > 1.3 * ms[0]
+
+
+def test_autotune_keeps_the_automatic_force_grid(ljmd):
+    # a block per chunk, more than 32 per SM: no candidate is 2 % faster (they are 1 to 10 % slower)
+    s = inputs.fcc_subset_system(1000000, 0.8442, 0.7, seed=6)
+    b = ljmd.from_system(s)
+    f0 = b.force()[0]
+    t = b.autotune(reps=10, cache=False)
+    assert t["force_blocks_per_sm"] == 0 == b.tuning()["force_blocks_per_sm"]
+    assert np.abs(b.force()[0] - f0).max() <= 1e-4 * np.abs(f0).max()
