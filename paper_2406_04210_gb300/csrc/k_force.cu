@@ -97,16 +97,19 @@ __device__ __forceinline__ void pair_f32(unsigned ent, const float4& pj, const f
     }
 }
 
-// Sums of k_force_f32 over a thread's pairs, in units of c6 = 24 eps sigma^6 for
-// one species (applied at the end).  w = sum f r^2 (the virial).  The energy
-// needs no pair arithmetic of its own: with s6 = (sigma / r)^6,
+// Sums of k_force_f32 over a thread's pairs, in units applied at the end: 24 eps
+// sigma^6 for one species, 12 for several (whose tables hold 4 eps sigma^12 and 2
+// eps sigma^6).  w = sum f r^2 (the virial).  The energy needs no pair arithmetic
+// of its own: with s6 = (sigma / r)^6,
 //   u = 4 eps (s6^2 - s6) - shift = (f r^2) / 12 - (2 eps s6 + shift),
-// so b sums the second term (one species: over 2 eps sigma^6).  w and b are
-// two partial sums each in pair2_f32 (its two pairs), one in pair1_f32.
-// f r^2 = c6 r^-6 (2 s6 - 1): the largest power formed is r^-8, so that the
-// unit of length has the room it has in the tables of several species (r^-14,
-// in units of 48 eps sigma^12, is subnormal from sigma = 400 and overflows
-// below 2e-3).
+// so b sums the second term, in units of 2 eps sigma^6 for one species.  In
+// these units it is w - b, with no constant that is rounded on its own (1/12 in
+// FP32 shifts every particle's energy by 3e-8 of w / 12 alike, which the sum over
+// the particles does not average out).  w and b are two partial sums each in
+// pair2_f32 (its two pairs), one in pair1_f32.
+// For one species f r^2 = c6 r^-6 (2 s6 - 1): the largest power formed is r^-8, so
+// that the unit of length has the room it has in the tables (r^-14, in units of
+// 48 eps sigma^12, is subnormal from sigma = 400 and overflows below 2e-3).
 struct PairSums {
     float fx, fy, fz;
     float2 w, b;
@@ -120,7 +123,7 @@ struct PairSums {
 // -> 18.4 / 17.0.  The row's ten constants take registers: five blocks of 256
 // per SM with energies (six: 1M 223 us), six without.
 struct RowConsts {
-    float4 c0, c1;   // c12, -c6, 2 eps sigma^6, shift
+    float4 c0, c1;   // 4 eps sigma^12, -2 eps sigma^6, 2 eps sigma^6, shift
     float r0, r1;    // rc^2
 };
 
@@ -242,18 +245,18 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
     constexpr int PASS = THREADS / TPP;                       // particles of a pass
     constexpr int PARTS = SPREAD ? LJ_CHUNK / PASS : 1;       // work items of a chunk
     constexpr int OWN = LJ_CHUNK / PARTS;                     // particles of an item
-    __shared__ float4 s_lj[MONO ? 1 : LJ_MAXT * LJ_MAXT];     // c12, -c6, 2 eps sigma^6, shift
+    __shared__ float4 s_lj[MONO ? 1 : LJ_MAXT * LJ_MAXT];     // 4 eps sigma^12, -2 eps sigma^6, 2 eps sigma^6, shift
     __shared__ float s_rc2[MONO ? 1 : LJ_MAXT * LJ_MAXT];
     if (!MONO) {
         const LJDev* lj = b.lj;
         for (int k = threadIdx.x; k < b.nt * b.nt; k += blockDim.x) {
-            s_lj[k] = make_float4(lj->c12[k], -lj->c6[k], 0.5f * lj->e6[k], lj->shift[k]);
+            s_lj[k] = make_float4(lj->e12[k], -0.5f * lj->e6[k], 0.5f * lj->e6[k], lj->shift[k]);
             s_rc2[k] = lj->rc2[k];
         }
         __syncthreads();   // the pair tables are complete (the block's only barrier)
     }
     // one species: f r^2 = c6 r6 (tw r6 - 1), the energy's second term (e6 / 2) (r6 + kap)
-    const float c6 = MONO ? b.c1.y : 1.f, tw = b.tw_1, kap = b.kap_1, mrc2 = b.rc2_1;
+    const float unit = MONO ? b.c1.y : 12.f, eunit = MONO ? 0.5f * b.c1.w : 1.f, tw = b.tw_1, kap = b.kap_1, mrc2 = b.rc2_1;
     const int K = b.K;
     const int grp = threadIdx.x / TPP, lt = threadIdx.x % TPP;
     const float4* posq = b.posq;
@@ -339,7 +342,7 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
                 S.fz += __shfl_xor_sync(0xffffffffu, S.fz, o);
             }
             if (act && lt == 0) {
-                b.force4[p] = make_float4(-c6 * S.fx, -c6 * S.fy, -c6 * S.fz, 0.f);
+                b.force4[p] = make_float4(-unit * S.fx, -unit * S.fy, -unit * S.fz, 0.f);
                 if (!isfinite(S.fx + S.fy + S.fz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
             }
         }
@@ -350,8 +353,8 @@ __global__ void __launch_bounds__(THREADS, RES) k_force_f32(BoxDev b)
             // sum): FP64-class precision on the FP32 pipe, since FP64 adds
             // are scarce on this GPU.  The share is stored as the (hi, lo)
             // pair itself (pf_ds), halved exactly; the reduction converts
-            const float vir = c6 * (S.w.x + S.w.y);
-            const float e = fmaf(vir, 1.f / 12.f, (MONO ? -0.5f * b.c1.w : -1.f) * (S.b.x + S.b.y));
+            const float w = S.w.x + S.w.y, vir = unit * w;
+            const float e = eunit * (w - (S.b.x + S.b.y));
             const float2 d = warp_sum2_ds2(e, vir);
             if ((threadIdx.x & 15) == 0) {
                 const size_t q = (size_t)it * (THREADS / 16) + (threadIdx.x >> 4);
@@ -1209,22 +1212,23 @@ template <bool MONO, bool ENERGY>
 __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
 {
     await_previous();
-    __shared__ float4 s_lj[MONO ? 1 : LJ_MAXT * LJ_MAXT];   // c12, -c6, 2 eps sigma^6
+    __shared__ float4 s_lj[MONO ? 1 : LJ_MAXT * LJ_MAXT];   // 4 eps sigma^12, -2 eps sigma^6, 2 eps sigma^6
     __shared__ double s_red[2][kAllWarps];
     __shared__ __align__(16) float4 s_pos[kAllTile];
     const int nt = b.nt;
     if (!MONO) {
         const LJDev* lj = b.lj;
         for (int k = threadIdx.x; k < nt * nt; k += blockDim.x)
-            s_lj[k] = make_float4(lj->c12[k], -lj->c6[k], 0.5f * lj->e6[k], 0.f);
+            s_lj[k] = make_float4(lj->e12[k], -0.5f * lj->e6[k], 0.5f * lj->e6[k], 0.f);
         __syncthreads();
     }
     // one species: lengths over the power of two nearest sigma, where they are
-    // staged, and the energy in units of c12 = 48 eps sigma^12 of that length.
+    // staged, and the sums in units of c12 = 48 eps sigma^12 of that length (12
+    // for several species, see PairSums).
     // (The list kernels' form, which needs no scale, costs an FMA with three
     // packed register operands instead of an addition: N = 32,000 836 -> 870 us.)
-    const float4 one_c = b.all_1;   // 1 / length, c12, -c6 / c12, e6 / 2
-    const float c12 = MONO ? one_c.y : 1.f;
+    const float4 one_c = b.all_1;   // 1 / length, c12, -c6 / c12, c12 / 12
+    const float unit = MONO ? one_c.y : 12.f;
     const float2 nh = dup2(one_c.z);
     auto load = [&](int j) {
         float4 q = b.posq[j];
@@ -1324,15 +1328,16 @@ __global__ void __launch_bounds__(kAllThreads) k_force_all_f32(BoxDev b)
                 fz = __fadd2_rn(fz, make_float2(__shfl_xor_sync(0xffffffffu, fz.x, o), __shfl_xor_sync(0xffffffffu, fz.y, o)));
             }
             if ((lane == 0 && one) || (lane == 1 && two)) {
-                const float cf = MONO ? c12 * one_c.x : 1.f;
+                const float cf = MONO ? unit * one_c.x : unit;
                 const float sx = lane == 0 ? fx.x : fx.y, sy = lane == 0 ? fy.x : fy.y, sz = lane == 0 ? fz.x : fz.y;
                 b.force4[p + lane] = make_float4(-cf * sx, -cf * sy, -cf * sz, 0.f);
                 if (!isfinite(sx + sy + sz)) atomicOr(&b.err[0], LJ_ERRBIT_NONFINITE);
             }
             if (ENERGY) {
-                // u = f r^2 / 12 - 2 eps (sigma / r)^6 (no cutoff, no shift)
-                const float wv = c12 * (vir.x + (two ? vir.y : 0.f));   // both 0 without a first particle
-                const float ev = fmaf(wv, 1.f / 12.f, (MONO ? -one_c.w : -1.f) * (eb.x + (two ? eb.y : 0.f)));
+                // u = f r^2 / 12 - 2 eps (sigma / r)^6 (no cutoff, no shift); one species: over c12 / 12,
+                // r6 (r6 + nh) + nh r6
+                const float wu = vir.x + (two ? vir.y : 0.f), bu = eb.x + (two ? eb.y : 0.f);   // 0 without a first particle
+                const float wv = unit * wu, ev = MONO ? one_c.w * fmaf(one_c.z, bu, wu) : wu - bu;
                 const float2 d = warp_sum2_ds2(ev, wv);
                 sum += (double)d.x + (double)d.y;
             }

@@ -1520,7 +1520,7 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
         b->d.kap_1 = (float)(h.dshift[0] / (2.0 * eps[0] * s6));
         const double u = std::exp2(std::min(100.0, std::max(-100.0, std::round(std::log2(sigma[0]))))), q = sigma[0] / u;
         const double q6 = q * q * q * q * q * q;
-        b->d.all_1 = make_float4((float)(1.0 / u), (float)(48.0 * eps[0] * q6 * q6), (float)(-0.5 / q6), (float)(2.0 * eps[0] * q6));
+        b->d.all_1 = make_float4((float)(1.0 / u), (float)(48.0 * eps[0] * q6 * q6), (float)(-0.5 / q6), (float)(4.0 * eps[0] * q6 * q6));
     }
     b->skin = skin;
     b->rl = rl;

@@ -154,7 +154,7 @@ struct BoxDev {
     // one species (nt == 1): its FP32 pair constants, read by the force
     // kernel from the kernel parameters (no registers held for them)
     float4 c1;                 // c12, c6, e12, e6
-    float4 all_1;              // all pairs: 1 / (the power of two nearest sigma), and c12, -c6 / c12, e6 / 2 in that length
+    float4 all_1;              // all pairs: 1 / (the power of two nearest sigma), and c12, -c6 / c12, c12 / 12 in that length
     float rc2_1, esh_1;
     float tw_1, kap_1;         // c12 / c6, shift / (e6 / 2)
     float3 ell1;               // one replica (nrep == 1): its cell edge, FP32
