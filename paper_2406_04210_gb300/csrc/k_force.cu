@@ -907,7 +907,7 @@ __device__ __forceinline__ double fx_to_double(__int128 v, double a, int n)
 // entry for a thread per particle with a division.  Work items are quarters
 // of a chunk (32 particles per block), so that 4,000 particles reach 125 SMs.
 // N = 256,000, energies: 1177 us -> 688 us in FP64, 307 us in integers;
-// N = 4,000: a step 127 us -> 48 us in FP64, 28 us in integers.
+// N = 4,000: a step 127 us -> 48 us in FP64, 26 us in integers.
 // TPP: 4, or 16 in one-species boxes of at most an item per SM
 // (BoxDev::f64_wide).
 constexpr int kF64Parts = LJ_F64_WARPS;                         // work items, and (E_pot, W) shares, per chunk

@@ -248,8 +248,10 @@ __global__ void __launch_bounds__(LJ_CHUNK) k_bin(BoxDev b, int from_abs)
 // kScanTile cells, a run of consecutive cells per thread; it first sums the
 // counts of the replica's earlier tiles itself (from L2; at 4M the last of 101
 // tiles reads 0.8 MB), which costs the few builds less than a second pass, a
-// launch in every step: a step at N = 100,000 38.0 -> 36.6 us.  tiles[t] =
-// (rep, first cell, end cell, first tile of the replica).
+// launch in every step: a step at N = 100,000 38.0 -> 36.6 us.  The reads grow
+// with the square of the tiles, which is not seen at 32M (a forced update takes
+// 0.65 ns per particle, 0.67 at 4M).  tiles[t] = (rep, first cell, end cell,
+// first tile of the replica).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int block_excl_scan(int v, int* s_warp, int& total)
 {
@@ -1150,13 +1152,11 @@ __global__ void __launch_bounds__(LJ_LANE_THREADS, 8) k_nlist_lanes(BoxDev b)
 // k_rebuild_cluster: binning, sort and gather of small boxes in one launch,
 // by one thread-block cluster whose blocks meet at the hardware's cluster
 // barrier between the stages.  A step without a build then pays two early
-// exits (this and the list build) instead of five (eight when this was
-// measured first), and a build no launches between the stages; the list build stays a kernel of its own, as it wants
-// every SM.  (One cooperative launch for everything, with grid barriers, was
-// measured first: its launch inside a step graph cost nearly what the early
-// exits had, 32.7 us a step at N = 4,000 against 34.3.)
-// A step of the N = 4,000 fluid: 33.4 us with the separate kernels, 28.1 us
-// with this; the launch rule has the other sizes.
+// exits (this and the list build) instead of five, and a build no launches
+// between the stages; the list build stays a kernel of its own, as it wants
+// every SM.  (A cooperative launch with grid barriers, which could hold the list
+// build too, costs ~8 us inside a step graph.)  The launch rule,
+// cluster_rebuild, has the times.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cluster_barrier()
 {
@@ -1169,7 +1169,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_rebuild_cluster(BoxDev b, i
 {
     await_previous();
     if (!box_needs_rebuild(b)) return;   // the same word for every block: none is left waiting
-    if (b.nrep > 1) {   // one replica: its work lists never change
+    if (b.nrep > 1) {   // one replica's work is all of its own
         if (blockIdx.x == 0) phase_list_work(b);
         cluster_barrier();
     }

@@ -172,7 +172,7 @@ struct md_box {
     double* d_parth = nullptr;
     double* d_hist = nullptr;
     int hist_cap = 0;
-    double eps0 = 1.0, sigma0 = 1.0, rcut0 = 0.0, shift0 = 0.0;   // the first pair's parameters
+    double eps0 = 1.0, sigma0 = 1.0, rcut0 = 0.0;   // the first pair's parameters
     long long* d_offx = nullptr; // offsets as integers (FP64 precision, one species)
     PinnedBack* pin = nullptr;   // pinned host memory
     PinnedBack* pin_dev = nullptr;   // and its device address
@@ -280,12 +280,13 @@ void invalidate_graphs(md_box* b)
 Launch lch(md_box* b) { return Launch{std::max(1, std::min((int)b->d.nchunk, b->nsm * 12)), LJ_CHUNK, b->stream}; }
 Launch lthermo(md_box* b) { return Launch{std::max(1, std::min(b->d.ntitem, b->nsm * 8)), LJ_THERMO_THREADS, b->stream}; }
 Launch lcell(md_box* b) { return Launch{std::max(1, std::min((b->d.ncell + 7) / 8, b->nsm * 8)), 256, b->stream}; }
-// The FP32 list-form force kernel and the layout of its (E_pot, W) shares:
-// the chunk kernel unless the tiled one is asked for (or chosen by
-// md_autotune).  The FP32 list
-// kernels leave one double-single share per warp and chunk (chunk kernel)
-// or brick (tiled kernel, LJ_BRICK_WARPS = LJ_FORCE_WARPS), the FP64 one an
-// FP64 share per warp and chunk, the all-pairs kernels one per chunk.
+// The FP32 list-form force kernel is the chunk kernel unless the tiled one is
+// asked for (or chosen by md_autotune).  (E_pot, W) shares, apply_force_kernel:
+// FP32 lists one double-single share per warp and work item, 16 per chunk with
+// small items, else 8 per chunk (tiled: per brick, LJ_BRICK_WARPS =
+// LJ_FORCE_WARPS); the FP64 list kernel an FP64 share per work item, 4 per
+// chunk; all pairs one per work item: FP32 8 per chunk up to 1,024 chunks, else
+// and in FP64 one.
 // Small work items of the FP32 list force (16 particles instead of 128): up
 // to 512 chunks, where the chunks leave SMs idle or a block's two serial
 // passes set the time.  In-graph with energies, chunks / small items: N =
@@ -462,8 +463,11 @@ int rebuild_kernels(md_box* b, bool runs)
 // of the separate kernels: boxes whose stages 16 blocks get through faster
 // than the launches cost.  Us a step with energies, separate against cluster:
 // N = 8,000 13.4 / 10.8, 24,000 17.5 / 15.8, 48,000 24.8 / 23.2, 64,000 27.7 /
-// 26.7 (where the 16 SMs' build, an order of magnitude longer than on all,
-// takes that back in hotter runs).
+// 26.7 (where the 16 SMs' build takes that back in hotter runs).  The line is
+// drawn for steps and holds for builds that the host asks for too, which have
+// no early exits to gain: md_neighbour_update, separate against cluster, N =
+// 4,000 107 / 101, 8,000 96 / 91, 16,000 96 / 103, 32,000 120 / 137, 49,000 123 /
+// 153.
 constexpr int kClusterSlots = 49152;
 bool cluster_rebuild(md_box* b)
 {
@@ -494,7 +498,7 @@ md_status enqueue_rebuild_kernels(md_box* b, int from_abs, cudaStream_t s, unsig
         return l;
     };
     Launch l = on(lch(b));
-    // the cells and chunks the rebuild kernels visit (one replica's never change: make_grid)
+    // the cells and chunks the rebuild kernels visit (one replica's are all of its own: there it only counts runs)
     if (runs || b->nrep > 1) CK(b, launch_list_work(b->d, runs, s, early));
     CK(b, launch_bin(b->d, from_abs, l));
     Launch lt{std::max(1, std::min((int)b->tiles.size(), b->nsm * 8)), 0, s, early};
@@ -704,8 +708,6 @@ md_status make_grid(md_box* b)
     CKS(dev_alloc(b, &b->d_brick, b->bricks.size(), false));
     CK(b, cudaMemcpyAsync(b->d_brick, b->bricks.data(), sizeof(int4) * b->bricks.size(),
                           cudaMemcpyHostToDevice, b->stream));
-    const int lw1[6] = {1, 0, 0, d.ncell, 0, d.nchunk};   // the work lists of one replica never change
-    if (b->nrep == 1) CK(b, cudaMemcpyAsync(d.lw_hdr, lw1, sizeof lw1, cudaMemcpyHostToDevice, b->stream));
     CK(b, cudaStreamSynchronize(b->stream));   // `bricks` may change before the copy would run
     d.brick = b->d_brick;
     d.nbrick = (int)b->bricks.size();
@@ -733,7 +735,7 @@ md_status make_grid(md_box* b)
 // (they are at most an edge or so), r^2 below the cutoff in [2^62, 2^63).
 md_status setup_fx(md_box* b)
 {
-    const double eps = b->eps0, sigma = b->sigma0, rcut = b->rcut0, shift = b->shift0;
+    const double eps = b->eps0, sigma = b->sigma0, rcut = b->rcut0;
     FxDev fx{};
     long long* const had = b->d.offx;
     const bool on = b->prec == MD_PREC_FP64 && !b->all_pairs && b->nt == 1;
@@ -752,7 +754,6 @@ md_status setup_fx(md_box* b)
         fx.scale = std::ldexp(1.0, fx.q);
         fx.c12 = 48.0 * eps * s6 * s6;
         fx.hb = 2.0 * eps * s6;
-        fx.shift = shift;
         fx.near = (float)rc2 + b->d.band;   // the margin of the list build's FP64 recheck
         if (b->nrep == 1)
             for (int c = 0; c < 3; ++c) fx.ell[c] = std::llrint(std::ldexp(b->reps[0].ell[c], fx.q));
@@ -765,7 +766,7 @@ md_status setup_fx(md_box* b)
     b->d.offx = fx.on ? b->d_offx : nullptr;
     const FxDev& o = b->d.fx;
     if (had != b->d.offx || o.on != fx.on || o.q != fx.q || o.sR != fx.sR || o.Ke != fx.Ke || o.Km != fx.Km ||
-        o.Rc != fx.Rc || o.c12 != fx.c12 || o.hb != fx.hb || o.shift != fx.shift || o.near != fx.near ||
+        o.Rc != fx.Rc || o.c12 != fx.c12 || o.hb != fx.hb || o.near != fx.near ||
         o.ell[0] != fx.ell[0] || o.ell[1] != fx.ell[1] || o.ell[2] != fx.ell[2])
         invalidate_graphs(b);   // graphs hold them by value
     b->d.fx = fx;
@@ -1539,7 +1540,6 @@ md_status md_set_lj(md_box* b, int32_t ntypes, const double* eps, const double* 
     b->eps0 = eps[0];
     b->sigma0 = sigma[0];
     b->rcut0 = rcut[0];
-    b->shift0 = h.dshift[0];
     CKS(setup_fx(b));
     b->lj_set = true;
     b->rec_valid = false;
@@ -2391,9 +2391,9 @@ extern "C" md_status md_force_noalloc(md_box* b, double* force_out, double* epot
     if (need > (size_t)LJMD_NOALLOC_DOUBLES) {
         char msg[240];
         snprintf(msg, sizeof msg,
-                 "md_force_noalloc: box needs %zu scratch doubles (16 per 128 particles with FP32 forces, 8 "
-                 "all-FP64, 2 for all pairs, + 4 per replica); the static scratch holds %d",
-                 need, LJMD_NOALLOC_DOUBLES);
+                 "md_force_noalloc: box needs %zu scratch doubles (%d per 128 particles in its form, + 4 per replica); "
+                 "the static scratch holds %d",
+                 need, 2 * v.pf_stride, LJMD_NOALLOC_DOUBLES);
         return fail(b, MD_ERR_ARG, msg);
     }
     if (!b->lj_set) return fail(b, MD_ERR_ARG, "md_force_noalloc: md_set_lj not called");

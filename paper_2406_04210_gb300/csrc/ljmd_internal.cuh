@@ -136,7 +136,7 @@ struct FxDev {
     unsigned long long Km;
     unsigned long long Rc;     // rc^2 in units of R
     double scale;              // 2^q
-    double c12, hb, shift;     // 48 eps sigma^12, 2 eps sigma^6, energy shift
+    double c12, hb;            // 48 eps sigma^12, 2 eps sigma^6
     float near;                // FP32 r^2 below which an entry is queued
     long long ell[3];          // one replica: the cell edges in units of 2^-q
 };
